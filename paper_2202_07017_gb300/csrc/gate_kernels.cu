@@ -27,6 +27,13 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Threads per block of a kernel with ITEMS units per thread: one-unit kernels
+// run with the block size of their launch (see shape_for).
+template <int ITEMS>
+__device__ __forceinline__ int block_threads() {
+  return ITEMS == 1 ? (int)blockDim.x : kThreads;
+}
+
 // ---- phase multiply variants ---------------------------------------------------
 enum { PK_GEN = 0, PK_NEG = 1, PK_I = 2, PK_MI = 3 };
 
@@ -63,12 +70,14 @@ template <typename I, int MK, int ITEMS, bool DITHER>
 __global__ void __launch_bounds__(kThreads)
     k1q_c64_pair(float4* __restrict__ psi, I n_units, Ins<I> ins, I tmask, I cmask,
                  int amp1_only, M2<float> g, uint32_t seed) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I lo[ITEMS];
   float4 a[ITEMS], b[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       lo[it] = insert_zeros(u, ins) | cmask;
       a[it] = psi[lo[it]];
@@ -77,7 +86,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       float4 x = a[it], y = b[it];
       if constexpr (DITHER) {
@@ -99,12 +108,14 @@ template <typename I, int MK, int ITEMS, bool DITHER>
 __global__ void __launch_bounds__(kThreads)
     k1q_c64_in(float4* __restrict__ psi, I n_units, Ins<I> ins, I cmask, M2<float> g,
                uint32_t seed) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I v[ITEMS];
   float4 a[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       v[it] = insert_zeros(u, ins) | cmask;
       a[it] = psi[v[it]];
@@ -112,7 +123,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       float4 x = a[it];
       if constexpr (DITHER)
@@ -129,12 +140,14 @@ template <typename I, int MK, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     k1q_c128_pair(double2* __restrict__ psi, I n_units, Ins<I> ins, I tmask, I cmask,
                   M2<double> g) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I lo[ITEMS];
   double2 a[ITEMS], b[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       lo[it] = insert_zeros(u, ins) | cmask;
       a[it] = psi[lo[it]];
@@ -143,7 +156,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       double2 x = a[it], y = b[it];
       mv2<MK>(g, x.x, x.y, y.x, y.y);
@@ -158,12 +171,14 @@ template <typename I, int PK, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     kphase_c64(float4* __restrict__ psi, I n_units, Ins<I> ins, I omask, int amp1_only,
                float c, float s) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I v[ITEMS];
   float4 a[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       v[it] = insert_zeros(u, ins) | omask;
       a[it] = psi[v[it]];
@@ -171,7 +186,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       float4 x = a[it];
       if (!amp1_only) rot<PK>(c, s, x.x, x.y);
@@ -185,12 +200,14 @@ template <typename I, int PK, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     kphase_c128(double2* __restrict__ psi, I n_units, Ins<I> ins, I omask, double c,
                 double s) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I v[ITEMS];
   double2 a[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       v[it] = insert_zeros(u, ins) | omask;
       a[it] = psi[v[it]];
@@ -198,7 +215,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       double2 x = a[it];
       rot<PK>(c, s, x.x, x.y);
@@ -214,12 +231,14 @@ template <typename I, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     kswap_c64_vv(float4* __restrict__ psi, I n_units, Ins<I> ins, I amask, I bmask, I cmask,
                  int amp1_only) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I p[ITEMS];
   float4 x[ITEMS], y[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       p[it] = insert_zeros(u, ins) | cmask;
       x[it] = psi[p[it] | bmask];
@@ -228,7 +247,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       float4 nx = y[it], ny = x[it];
       if (amp1_only) {
@@ -246,12 +265,14 @@ __global__ void __launch_bounds__(kThreads)
 template <typename I, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     kswap_c64_v0(float4* __restrict__ psi, I n_units, Ins<I> ins, I amask, I cmask) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I p[ITEMS];
   float4 x[ITEMS], y[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       p[it] = insert_zeros(u, ins) | cmask;
       x[it] = psi[p[it]];
@@ -260,7 +281,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       float4 v = x[it], w = y[it];
       const float tz = v.z, tw = v.w;
@@ -277,12 +298,14 @@ __global__ void __launch_bounds__(kThreads)
 template <typename I, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     kswap_c128(double2* __restrict__ psi, I n_units, Ins<I> ins, I amask, I bmask, I cmask) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
   I p[ITEMS];
   double2 x[ITEMS], y[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       p[it] = insert_zeros(u, ins) | cmask;
       x[it] = psi[p[it] | bmask];
@@ -291,7 +314,7 @@ __global__ void __launch_bounds__(kThreads)
   }
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I u = base + (I)(it * kThreads);
+    const I u = base + (I)(it * T);
     if (u < n_units) {
       psi[p[it] | bmask] = y[it];
       psi[p[it] | amask] = x[it];
@@ -311,10 +334,11 @@ template <int K, typename R, typename T2, typename I>
 __global__ void __launch_bounds__(kThreads)
     kgen(T2* __restrict__ psi, I n_units, Ins<I> ins, I cmask, const __grid_constant__ GenParams<K, R, I> p) {
   constexpr int D = 1 << K;
-  const I u = (I)blockIdx.x * (I)kThreads + (I)threadIdx.x;
+  const I u = (I)blockIdx.x * (I)block_threads<1>() + (I)threadIdx.x;
   if (u >= n_units) return;
   const I b = insert_zeros(u, ins) | cmask;
   R ar[D], ai[D];
+  grid_dependency_wait();
 #pragma unroll
   for (int t = 0; t < D; ++t) {
     const T2 v = psi[b | p.off[t]];
@@ -339,10 +363,12 @@ __global__ void __launch_bounds__(kThreads)
 
 template <typename I, int ITEMS>
 __global__ void kinit_c64(float4* __restrict__ psi, I n_vec, I bvec, int slot) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I v = base + (I)(it * kThreads);
+    const I v = base + (I)(it * T);
     if (v < n_vec) {
       float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
       if (v == bvec) {
@@ -355,10 +381,12 @@ __global__ void kinit_c64(float4* __restrict__ psi, I n_vec, I bvec, int slot) {
 
 template <typename I, int ITEMS>
 __global__ void kinit_c128(double2* __restrict__ psi, I n_vec, I bvec) {
-  const I base = (I)blockIdx.x * (I)(kThreads * ITEMS) + (I)threadIdx.x;
+  const int T = block_threads<ITEMS>();
+  const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
+  grid_dependency_wait();
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const I v = base + (I)(it * kThreads);
+    const I v = base + (I)(it * T);
     if (v < n_vec) psi[v] = make_double2(v == bvec ? 1.0 : 0.0, 0.0);
   }
 }
@@ -370,7 +398,7 @@ __global__ void kinit_c128(double2* __restrict__ psi, I n_vec, I bvec) {
 // ITEMS = 8 for both families brings the 1-qubit kernel from 5.9 to
 // 6.8 TB/s (the copy bandwidth) and the controlled-U1 kernel from 3.6 to
 // 6.6 TB/s; fewer vectors in flight leave HBM latency exposed.
-// SV_ITEMS_PAIR / SV_ITEMS_SINGLE (1, 2, 4, 8) override the defaults.
+// SV_ITEMS_PAIR / SV_ITEMS_SINGLE (1, 2, 4, 8) override the largest count.
 int env_items(const char* name, int dflt) {
   const char* e = getenv(name);
   const int x = e ? atoi(e) : dflt;
@@ -385,20 +413,38 @@ int items_single() {
   return v;
 }
 
+// Units per thread, threads per block and blocks of a launch over n_units.
+// Small states are bound by how many SMs work at all (a 2^12-amplitude
+// complex128 state in blocks of 256 x 8 pairs is one block, whose SM issues
+// two fp64 operations a clock), so the units per thread drop until every SM
+// has kFillBlocks blocks, and below that the blocks shrink to two warps.
+// Measured on GB300 (random layered circuits, a launch per gate): n = 12
+// complex128, depth 20, 7.11 -> 3.41 ms; n = 18 complex64, depth 20, 7.30 ->
+// 5.13 ms; the QFT at n = 20 1.12 -> 0.91 ms, at n = 26 21.9 ms either way.
+struct Shape {
+  int items, threads;
+  unsigned grid;
+};
+constexpr uint64_t kFillBlocks = 4;
+constexpr uint64_t kSmCount = 152;
+
+Shape shape_for(uint64_t n_units, int items) {
+  while (items > 1 && n_units < kFillBlocks * kSmCount * kThreads * items) items >>= 1;
+  int threads = kThreads;
+  if (items == 1)
+    while (threads > 64 && n_units < kSmCount * threads) threads >>= 1;
+  const uint64_t per = (uint64_t)threads * items;
+  return {items, threads, (unsigned)((n_units + per - 1) / per)};
+}
+
 template <typename F>
-void with_items(int items, F&& f) {
-  switch (items) {
+void with_items(const Shape& sh, F&& f) {
+  switch (sh.items) {
     case 1: f(std::integral_constant<int, 1>{}); break;
     case 2: f(std::integral_constant<int, 2>{}); break;
     case 8: f(std::integral_constant<int, 8>{}); break;
     default: f(std::integral_constant<int, 4>{}); break;
   }
-}
-
-template <typename I>
-unsigned grid_for(I n_units, int items) {
-  const uint64_t per = (uint64_t)kThreads * items;
-  return (unsigned)(((uint64_t)n_units + per - 1) / per);
 }
 
 bool is_zero(cd z) { return z.re == 0.0 && z.im == 0.0; }
@@ -420,11 +466,11 @@ int phase_kind(cd ph) {
 }
 
 template <typename... KArgs, typename... Args>
-void launch_k(void (*kern)(KArgs...), const char* name, unsigned grid, cudaStream_t st,
+void launch_k(void (*kern)(KArgs...), const char* name, const Shape& sh, cudaStream_t st,
               Args... args) {
-  if (grid == 0) return;
+  if (sh.grid == 0) return;
   ProfScope prof(st, name);
-  kern<<<grid, kThreads, 0, st>>>(args...);
+  launch_dependent(kern, sh.grid, sh.threads, 0, st, args...);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
@@ -452,13 +498,14 @@ void run_1q_c64(float4* psi, int n, cudaStream_t st, int t, int nc, const int* c
   if (t == 0) {
     Ins<I> ins = make_ins<I>(vpos);
     const I nu = I(1) << (n - 1 - (int)vpos.size());
-    with_items(items_single(), [&](auto it) {
+    const Shape sh = shape_for(nu, items_single());
+    with_items(sh, [&](auto it) {
       constexpr int IT = decltype(it)::value;
       if (seed)
-        launch_k(k1q_c64_in<I, MK, IT, true>, "k1q_c64_in", grid_for(nu, IT), st, psi, nu, ins,
+        launch_k(k1q_c64_in<I, MK, IT, true>, "k1q_c64_in", sh, st, psi, nu, ins,
                  cmask, g, seed);
       else
-        launch_k(k1q_c64_in<I, MK, IT, false>, "k1q_c64_in", grid_for(nu, IT), st, psi, nu, ins,
+        launch_k(k1q_c64_in<I, MK, IT, false>, "k1q_c64_in", sh, st, psi, nu, ins,
                  cmask, g, seed);
     });
   } else {
@@ -466,13 +513,14 @@ void run_1q_c64(float4* psi, int n, cudaStream_t st, int t, int nc, const int* c
     Ins<I> ins = make_ins<I>(vpos);
     const I tmask = I(1) << (t - 1);
     const I nu = I(1) << (n - 1 - (int)vpos.size());
-    with_items(items_pair(), [&](auto it) {
+    const Shape sh = shape_for(nu, items_pair());
+    with_items(sh, [&](auto it) {
       constexpr int IT = decltype(it)::value;
       if (seed)
-        launch_k(k1q_c64_pair<I, MK, IT, true>, "k1q_c64_pair", grid_for(nu, IT), st, psi, nu,
+        launch_k(k1q_c64_pair<I, MK, IT, true>, "k1q_c64_pair", sh, st, psi, nu,
                  ins, tmask, cmask, amp1_only, g, seed);
       else
-        launch_k(k1q_c64_pair<I, MK, IT, false>, "k1q_c64_pair", grid_for(nu, IT), st, psi, nu,
+        launch_k(k1q_c64_pair<I, MK, IT, false>, "k1q_c64_pair", sh, st, psi, nu,
                  ins, tmask, cmask, amp1_only, g, seed);
     });
   }
@@ -490,9 +538,10 @@ void run_1q_c128(double2* psi, int n, cudaStream_t st, int t, int nc, const int*
   Ins<I> ins = make_ins<I>(pos);
   const I tmask = I(1) << t;
   const I nu = I(1) << (n - (int)pos.size());
-  with_items(items_pair(), [&](auto it) {
+  const Shape sh = shape_for(nu, items_pair());
+    with_items(sh, [&](auto it) {
     constexpr int IT = decltype(it)::value;
-    launch_k(k1q_c128_pair<I, MK, IT>, "k1q_c128_pair", grid_for(nu, IT), st, psi, nu, ins,
+    launch_k(k1q_c128_pair<I, MK, IT>, "k1q_c128_pair", sh, st, psi, nu, ins,
              tmask, cmask, g);
   });
 }
@@ -534,9 +583,10 @@ void run_phase_pk(void* data, sv_dtype dt, int n, cudaStream_t st, const std::ve
     Ins<I> ins = make_ins<I>(vpos);
     const I nu = I(1) << (n - 1 - (int)vpos.size());
     const float c = (float)ph.re, s = (float)ph.im;
-    with_items(items_single(), [&](auto it) {
+    const Shape sh = shape_for(nu, items_single());
+    with_items(sh, [&](auto it) {
       constexpr int IT = decltype(it)::value;
-      launch_k(kphase_c64<I, PK, IT>, "kphase_c64", grid_for(nu, IT), st, psi, nu, ins, omask,
+      launch_k(kphase_c64<I, PK, IT>, "kphase_c64", sh, st, psi, nu, ins, omask,
                amp1_only, c, s);
     });
   } else {
@@ -545,9 +595,10 @@ void run_phase_pk(void* data, sv_dtype dt, int n, cudaStream_t st, const std::ve
     for (int b : bits) omask |= I(1) << b;
     Ins<I> ins = make_ins<I>(bits);
     const I nu = I(1) << (n - (int)bits.size());
-    with_items(items_single(), [&](auto it) {
+    const Shape sh = shape_for(nu, items_single());
+    with_items(sh, [&](auto it) {
       constexpr int IT = decltype(it)::value;
-      launch_k(kphase_c128<I, PK, IT>, "kphase_c128", grid_for(nu, IT), st, psi, nu, ins, omask,
+      launch_k(kphase_c128<I, PK, IT>, "kphase_c128", sh, st, psi, nu, ins, omask,
                ph.re, ph.im);
     });
   }
@@ -579,9 +630,10 @@ void run_swap(void* data, sv_dtype dt, int n, cudaStream_t st, int a, int b, int
       vpos.push_back(a - 1);
       Ins<I> ins = make_ins<I>(vpos);
       const I nu = I(1) << (n - 1 - (int)vpos.size());
-      with_items(items_pair(), [&](auto it) {
+      const Shape sh = shape_for(nu, items_pair());
+    with_items(sh, [&](auto it) {
         constexpr int IT = decltype(it)::value;
-        launch_k(kswap_c64_v0<I, IT>, "kswap_c64_v0", grid_for(nu, IT), st, psi, nu, ins, amask,
+        launch_k(kswap_c64_v0<I, IT>, "kswap_c64_v0", sh, st, psi, nu, ins, amask,
                  cmask);
       });
     } else {
@@ -590,9 +642,10 @@ void run_swap(void* data, sv_dtype dt, int n, cudaStream_t st, int a, int b, int
       vpos.push_back(b - 1);
       Ins<I> ins = make_ins<I>(vpos);
       const I nu = I(1) << (n - 1 - (int)vpos.size());
-      with_items(items_pair(), [&](auto it) {
+      const Shape sh = shape_for(nu, items_pair());
+    with_items(sh, [&](auto it) {
         constexpr int IT = decltype(it)::value;
-        launch_k(kswap_c64_vv<I, IT>, "kswap_c64_vv", grid_for(nu, IT), st, psi, nu, ins, amask,
+        launch_k(kswap_c64_vv<I, IT>, "kswap_c64_vv", sh, st, psi, nu, ins, amask,
                  bmask, cmask, amp1_only);
       });
     }
@@ -607,9 +660,10 @@ void run_swap(void* data, sv_dtype dt, int n, cudaStream_t st, int a, int b, int
     Ins<I> ins = make_ins<I>(pos);
     const I amask = I(1) << a, bmask = I(1) << b;
     const I nu = I(1) << (n - (int)pos.size());
-    with_items(items_pair(), [&](auto it) {
+    const Shape sh = shape_for(nu, items_pair());
+    with_items(sh, [&](auto it) {
       constexpr int IT = decltype(it)::value;
-      launch_k(kswap_c128<I, IT>, "kswap_c128", grid_for(nu, IT), st, psi, nu, ins, amask, bmask,
+      launch_k(kswap_c128<I, IT>, "kswap_c128", sh, st, psi, nu, ins, amask, bmask,
                cmask);
     });
   }
@@ -643,7 +697,7 @@ void run_gen_k(void* data, sv_dtype dt, int n, cudaStream_t st, const int* tp, i
   }
   Ins<I> ins = make_ins<I>(pos);
   const I nu = I(1) << (n - (int)pos.size());
-  const unsigned grid = grid_for(nu, 1);
+  const Shape grid = shape_for(nu, 1);
   if (dt == SV_C64)
     launch_k(kgen<K, float, float2, I>, "kgen_c64", grid, st, (float2*)data, nu, ins, cmask,
              gen_params<K, float, I>(tp, G));
@@ -755,28 +809,29 @@ sv_status launch_gate(void* data, sv_dtype dt, int n, cudaStream_t st, int k, co
   return check_launch("gate kernel");
 }
 
+namespace {
+template <typename I>
+void run_init(void* data, sv_dtype dt, int n, cudaStream_t st, uint64_t basis) {
+  // n >= 1: 2^(n-1) vectors of 2 complex64 amplitudes, 2^n of one complex128
+  const bool c64 = dt == SV_C64;
+  const I nu = I(1) << (c64 ? n - 1 : n);
+  const Shape sh = shape_for(nu, 4);
+  with_items(sh, [&](auto it) {
+    constexpr int IT = decltype(it)::value;
+    if (c64)
+      launch_k(kinit_c64<I, IT>, "kinit_c64", sh, st, (float4*)data, nu, (I)(basis >> 1),
+               (int)(basis & 1));
+    else
+      launch_k(kinit_c128<I, IT>, "kinit_c128", sh, st, (double2*)data, nu, (I)basis);
+  });
+}
+}  // namespace
+
 sv_status launch_init(void* data, sv_dtype dt, int n, cudaStream_t st, uint64_t basis) {
-  if (dt == SV_C64) {
-    const uint64_t nvec = uint64_t(1) << (n - 1);  // n >= 1: 2^(n-1) vectors of 2 amplitudes
-    if (use_32bit_index(n, dt)) {
-      const uint32_t nu = (uint32_t)nvec;
-      launch_k(kinit_c64<uint32_t, 4>, "kinit_c64", grid_for(nu, 4), st, (float4*)data, nu,
-               (uint32_t)(basis >> 1), (int)(basis & 1));
-    } else {
-      launch_k(kinit_c64<uint64_t, 4>, "kinit_c64", grid_for(nvec, 4), st, (float4*)data, nvec,
-               basis >> 1, (int)(basis & 1));
-    }
-  } else {
-    const uint64_t nvec = uint64_t(1) << n;
-    if (use_32bit_index(n, dt)) {
-      const uint32_t nu = (uint32_t)nvec;
-      launch_k(kinit_c128<uint32_t, 4>, "kinit_c128", grid_for(nu, 4), st, (double2*)data, nu,
-               (uint32_t)basis);
-    } else {
-      launch_k(kinit_c128<uint64_t, 4>, "kinit_c128", grid_for(nvec, 4), st, (double2*)data, nvec,
-               basis);
-    }
-  }
+  if (use_32bit_index(n, dt))
+    run_init<uint32_t>(data, dt, n, st, basis);
+  else
+    run_init<uint64_t>(data, dt, n, st, basis);
   return check_launch("init kernel");
 }
 

@@ -192,4 +192,33 @@ __device__ __forceinline__ double block_sum(double v) {
 
 bool use_32bit_index(int n, sv_dtype dt);
 
+// ---- dependent launches ----------------------------------------------------------
+// A kernel launched by launch_dependent may have its blocks set up while the
+// stream's previous kernel drains; it calls grid_dependency_wait before its
+// first access to device memory, which returns once everything earlier on the
+// stream has finished and is visible.  No kernel signals its dependents early,
+// so a block never occupies an SM that the previous kernel still needs.
+// Measured on GB300 for chains of one-gate kernels, against plain launches:
+// n = 12 complex128 (831 launches) 3.41 -> 1.62 ms, n = 18 complex64 5.13 ->
+// 2.47 ms, the QFT at n = 20 0.91 -> 0.43 ms and at n = 26 21.9 -> 20.9 ms.
+__device__ __forceinline__ void grid_dependency_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_dependent(void (*kern)(KArgs...), unsigned grid, unsigned threads,
+                                    size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+
 }  // namespace sv
