@@ -54,6 +54,7 @@ template <typename I, int PAULI>
 __global__ void __launch_bounds__(kRedThreads)
     kadj_c64_pair(float4* __restrict__ psi, float4* __restrict__ lam, I n_units, Ins<I> ins,
                   I tmask, I cmask, int amp1_only, M2<float> g, double* __restrict__ partials) {
+  grid_dependency_wait();
   Kahan32 acc;
   for (I u = (I)blockIdx.x * kRedThreads + threadIdx.x; u < n_units;
        u += (I)gridDim.x * kRedThreads) {
@@ -86,6 +87,7 @@ template <typename I, int PAULI>
 __global__ void __launch_bounds__(kRedThreads)
     kadj_c64_in(float4* __restrict__ psi, float4* __restrict__ lam, I n_units, Ins<I> ins,
                 I cmask, M2<float> g, double* __restrict__ partials) {
+  grid_dependency_wait();
   Kahan32 acc;
   for (I u = (I)blockIdx.x * kRedThreads + threadIdx.x; u < n_units;
        u += (I)gridDim.x * kRedThreads) {
@@ -107,6 +109,7 @@ template <typename I, int PAULI>
 __global__ void __launch_bounds__(kRedThreads)
     kadj_c128(double2* __restrict__ psi, double2* __restrict__ lam, I n_units, Ins<I> ins,
               I tmask, I cmask, M2<double> g, double* __restrict__ partials) {
+  grid_dependency_wait();
   double acc = 0.0;
   for (I u = (I)blockIdx.x * kRedThreads + threadIdx.x; u < n_units;
        u += (I)gridDim.x * kRedThreads) {
@@ -145,14 +148,14 @@ void run_adj(void* psi, void* lam, sv_dtype dt, int n, cudaStream_t st, int tp, 
     if (tp == 0) {
       Ins<I> ins = make_ins<I>(vpos);
       const I nu = I(1) << (n - 1 - (int)vpos.size());
-      kadj_c64_in<I, PAULI><<<grid, kRedThreads, 0, st>>>((float4*)psi, (float4*)lam, nu, ins,
-                                                          cmask, g, partials);
+      launch_dependent(kadj_c64_in<I, PAULI>, grid, kRedThreads, 0, st, (float4*)psi, (float4*)lam,
+                       nu, ins, cmask, g, partials);
     } else {
       vpos.push_back(tp - 1);
       Ins<I> ins = make_ins<I>(vpos);
       const I nu = I(1) << (n - 1 - (int)vpos.size());
-      kadj_c64_pair<I, PAULI><<<grid, kRedThreads, 0, st>>>(
-          (float4*)psi, (float4*)lam, nu, ins, I(1) << (tp - 1), cmask, amp1_only, g, partials);
+      launch_dependent(kadj_c64_pair<I, PAULI>, grid, kRedThreads, 0, st, (float4*)psi,
+                       (float4*)lam, nu, ins, I(1) << (tp - 1), cmask, amp1_only, g, partials);
     }
   } else {
     std::vector<int> pos{tp};
@@ -163,9 +166,8 @@ void run_adj(void* psi, void* lam, sv_dtype dt, int n, cudaStream_t st, int tp, 
     }
     Ins<I> ins = make_ins<I>(pos);
     const I nu = I(1) << (n - (int)pos.size());
-    kadj_c128<I, PAULI><<<grid, kRedThreads, 0, st>>>((double2*)psi, (double2*)lam, nu, ins,
-                                                      I(1) << tp, cmask, to_m2<double>(G),
-                                                      partials);
+    launch_dependent(kadj_c128<I, PAULI>, grid, kRedThreads, 0, st, (double2*)psi, (double2*)lam,
+                     nu, ins, I(1) << tp, cmask, to_m2<double>(G), partials);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }

@@ -30,6 +30,7 @@ struct DiagRun {
 // complex64 vectors (2 amplitudes), phases from an fp32 angle sum
 __global__ void __launch_bounds__(kEThreads)
     kdiag_c64(float4* __restrict__ psi, uint64_t nvec, const __grid_constant__ DiagRun D) {
+  grid_dependency_wait();
   constexpr int IT = 8;
   const uint64_t base = (uint64_t)blockIdx.x * (kEThreads * IT) + threadIdx.x;
   float4 v[IT];
@@ -64,6 +65,7 @@ __global__ void __launch_bounds__(kEThreads)
 
 __global__ void __launch_bounds__(kEThreads)
     kdiag_c128(double2* __restrict__ psi, uint64_t dim, const __grid_constant__ DiagRun D) {
+  grid_dependency_wait();
   constexpr int IT = 8;
   const uint64_t base = (uint64_t)blockIdx.x * (kEThreads * IT) + threadIdx.x;
   double2 v[IT];
@@ -92,6 +94,7 @@ template <typename R, typename T2>
 __global__ void __launch_bounds__(kEThreads)
     kpair(T2* __restrict__ psi, uint64_t npairs, uint64_t lowmask, uint64_t xm, uint64_t zm,
           R c, R kr, R ki) {
+  grid_dependency_wait();
   constexpr int IT = 8;
   const uint64_t base = (uint64_t)blockIdx.x * (kEThreads * IT) + threadIdx.x;
   uint64_t xs[IT];
@@ -149,6 +152,7 @@ template <typename R, typename T2, bool DIAG>
 __global__ void __launch_bounds__(kEThreads)
     kadj_pauli(T2* __restrict__ psi, T2* __restrict__ lam, uint64_t units, uint64_t lowmask,
                uint64_t xm, uint64_t zm, int ny, R c, R kr, R ki, double* __restrict__ partials) {
+  grid_dependency_wait();
   CompSum<R> acc;
   for (uint64_t u = (uint64_t)blockIdx.x * kEThreads + threadIdx.x; u < units;
        u += (uint64_t)gridDim.x * kEThreads) {
@@ -200,11 +204,11 @@ sv_status run_diag(const Target& s, const DiagRun& D) {
   if (s.dt == SV_C64) {
     const uint64_t nvec = uint64_t(1) << (s.n - 1);
     const unsigned g = (unsigned)((nvec + kEThreads * 8 - 1) / (kEThreads * 8));
-    kdiag_c64<<<g, kEThreads, 0, s.stream>>>((float4*)s.data, nvec, D);
+    launch_dependent(kdiag_c64, g, kEThreads, 0, s.stream, (float4*)s.data, nvec, D);
   } else {
     const uint64_t dim = uint64_t(1) << s.n;
     const unsigned g = (unsigned)((dim + kEThreads * 8 - 1) / (kEThreads * 8));
-    kdiag_c128<<<g, kEThreads, 0, s.stream>>>((double2*)s.data, dim, D);
+    launch_dependent(kdiag_c128, g, kEThreads, 0, s.stream, (double2*)s.data, dim, D);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("diagonal rotation kernel");
@@ -233,11 +237,11 @@ sv_status run_pair(const Target& s, uint64_t xm, uint64_t zm, double a) {
     double c32 = ca;
     cd k32{kr, ki};
     feedback_round_pair(&c32, &k32, s.rc ? &s.rc->drift : nullptr);
-    kpair<float, float2><<<g, kEThreads, 0, s.stream>>>((float2*)s.data, npairs, lowmask, xm, zm,
-                                                        (float)c32, (float)k32.re, (float)k32.im);
+    launch_dependent(kpair<float, float2>, g, kEThreads, 0, s.stream, (float2*)s.data, npairs,
+                     lowmask, xm, zm, (float)c32, (float)k32.re, (float)k32.im);
   } else {
-    kpair<double, double2><<<g, kEThreads, 0, s.stream>>>((double2*)s.data, npairs, lowmask, xm,
-                                                          zm, ca, kr, ki);
+    launch_dependent(kpair<double, double2>, g, kEThreads, 0, s.stream, (double2*)s.data, npairs,
+                     lowmask, xm, zm, ca, kr, ki);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("pair rotation kernel");
@@ -303,20 +307,20 @@ sv_status launch_adjoint_pauli(void* psi, void* lam, sv_dtype dt, int n, cudaStr
   ProfScope prof(st, dt == SV_C64 ? "kadj_pauli_c64" : "kadj_pauli_c128");
   if (dt == SV_C64) {
     if (diag)
-      kadj_pauli<float, float2, true><<<grid, kEThreads, 0, st>>>(
-          (float2*)psi, (float2*)lam, units, lowmask, xm, zm, ny, (float)c, (float)kr, (float)ki,
-          partials);
+      launch_dependent(kadj_pauli<float, float2, true>, grid, kEThreads, 0, st, (float2*)psi,
+                       (float2*)lam, units, lowmask, xm, zm, ny, (float)c, (float)kr, (float)ki,
+                       partials);
     else
-      kadj_pauli<float, float2, false><<<grid, kEThreads, 0, st>>>(
-          (float2*)psi, (float2*)lam, units, lowmask, xm, zm, ny, (float)c, (float)kr, (float)ki,
-          partials);
+      launch_dependent(kadj_pauli<float, float2, false>, grid, kEThreads, 0, st, (float2*)psi,
+                       (float2*)lam, units, lowmask, xm, zm, ny, (float)c, (float)kr, (float)ki,
+                       partials);
   } else {
     if (diag)
-      kadj_pauli<double, double2, true><<<grid, kEThreads, 0, st>>>(
-          (double2*)psi, (double2*)lam, units, lowmask, xm, zm, ny, c, kr, ki, partials);
+      launch_dependent(kadj_pauli<double, double2, true>, grid, kEThreads, 0, st, (double2*)psi,
+                       (double2*)lam, units, lowmask, xm, zm, ny, c, kr, ki, partials);
     else
-      kadj_pauli<double, double2, false><<<grid, kEThreads, 0, st>>>(
-          (double2*)psi, (double2*)lam, units, lowmask, xm, zm, ny, c, kr, ki, partials);
+      launch_dependent(kadj_pauli<double, double2, false>, grid, kEThreads, 0, st, (double2*)psi,
+                       (double2*)lam, units, lowmask, xm, zm, ny, c, kr, ki, partials);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   if (nparts) *nparts = grid;

@@ -666,6 +666,7 @@ template <typename R, int KGF>
 __global__ void __launch_bounds__(kFThreads, sizeof(R) == 4 ? 3 : 2)
     kfused(typename Cplx2<R>::T* __restrict__ psi, uint64_t n_blocks,
            const __grid_constant__ FusedParams<R> P) {
+  grid_dependency_wait();
   typedef typename Cplx2<R>::T V2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V2* sm = reinterpret_cast<V2*>(smem_raw);
@@ -831,6 +832,7 @@ __global__ void __launch_bounds__(kFThreads, MINB)
     mbar_init(barp, 1);
     fence_proxy_async_smem();
   }
+  grid_dependency_wait();  // the parameters are the only input so far
   __syncthreads();
   uint32_t parity = 0;
   for (uint64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
@@ -1186,6 +1188,7 @@ __global__ void __launch_bounds__(kFThreads, MINB)
     mbar_init(barp, 1);
     fence_proxy_async_smem();
   }
+  grid_dependency_wait();  // the parameters are the only input so far
   __syncthreads();
   uint32_t parity = 0;
   for (uint64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
@@ -1979,7 +1982,7 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint64_t grid = std::min<uint64_t>(nblk, (uint64_t)sms * res);
-    kern<<<(unsigned)grid, kFThreads, smem, st>>>(nblk, P);
+    launch_dependent(kern, (unsigned)grid, kFThreads, smem, st, nblk, P);
   } else {
     typename PassKernels<R>::Lsu kern = PassKernels<R>::lsu(kg);
     const size_t smem = (amp << P.m) + (sizeof(uint64_t) * (((size_t(1) << (P.m - P.L)) + 1) & ~size_t(1))) +
@@ -1990,8 +1993,8 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
       attr_set[kg] = true;
     }
     const uint64_t grid = std::min<uint64_t>(nblk, 152 * 16);
-    kern<<<(unsigned)grid, kFThreads, smem, st>>>(
-        reinterpret_cast<typename Cplx2<R>::T*>(data), nblk, P);
+    launch_dependent(kern, (unsigned)grid, kFThreads, smem, st,
+                     reinterpret_cast<typename Cplx2<R>::T*>(data), nblk, P);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("fused pass kernel");
@@ -2056,7 +2059,7 @@ sv_status run_adj_pass(void* psi, void* lam, int n, cudaStream_t st, const Fused
   const uint64_t nblk = uint64_t(1) << (n - P.m);
   const uint64_t grid = std::min<uint64_t>({nblk, (uint64_t)sms * res, (uint64_t)pstride});
   ProfScope prof(st, sizeof(R) == 4 ? "kfused_adj_c64" : "kfused_adj_c128");
-  kern<<<(unsigned)grid, kFThreads, smem, st>>>(nblk, P, partials, pstride);
+  launch_dependent(kern, (unsigned)grid, kFThreads, smem, st, nblk, P, partials, pstride);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("fused reverse pass kernel");
 }
@@ -2107,7 +2110,7 @@ sv_status selftest_wait(void* data, int n, cudaStream_t st) {
   const size_t smem = ((sizeof(R) * 2) << P.m) + 1024;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   const uint64_t nblk = uint64_t(1) << (n - P.m);
-  kern<<<(unsigned)std::min<uint64_t>(nblk, 152), kFThreads, smem, st>>>(nblk, P);
+  launch_dependent(kern, (unsigned)std::min<uint64_t>(nblk, 152), kFThreads, smem, st, nblk, P);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("bounded-wait self-test kernel");
 }

@@ -135,6 +135,7 @@ template <typename T2>
 __global__ void __launch_bounds__(kRedThreads)
     kprob_slices(const T2* __restrict__ psi, Ins<uint64_t> rest, const int* __restrict__ mpos,
                  int m, uint64_t per_bin, int slices, U128* __restrict__ partials) {
+  grid_dependency_wait();
   __shared__ U128 ws[kRedThreads / 32];
   const int r = blockIdx.x / slices, c = blockIdx.x % slices;
   uint64_t rbits = 0;
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(kRedThreads)
 // P(r) = (sum of the bin's slices) / 2^120, rounded to fp64
 __global__ void kprob_finish(const U128* __restrict__ partials, int slices, uint64_t bins,
                              double* __restrict__ out) {
+  grid_dependency_wait();
   const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= bins) return;
   U128 t = {0, 0};
@@ -180,6 +182,7 @@ __global__ void kprob_finish(const U128* __restrict__ partials, int slices, uint
 template <typename V>
 __global__ void __launch_bounds__(kRedThreads)
     kchunk_sums(const V* __restrict__ psi, int vbits, uint64_t K, U128* __restrict__ sums) {
+  grid_dependency_wait();
   const uint64_t k = (uint64_t)blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (k >= K) return;
@@ -202,6 +205,7 @@ __global__ void __launch_bounds__(kRedThreads)
 
 // inclusive prefix sums in place (exact, so any order gives the same values)
 __global__ void __launch_bounds__(1024) kscan(U128* __restrict__ v, uint64_t K) {
+  grid_dependency_wait();
   __shared__ U128 tot[1024];
   const uint64_t seg = (K + 1023) / 1024;
   const uint64_t a = threadIdx.x * seg, b = a + seg < K ? a + seg : K;
@@ -229,6 +233,7 @@ __global__ void __launch_bounds__(1024) kscan(U128* __restrict__ v, uint64_t K) 
 // totals[blockIdx.x].
 __global__ void __launch_bounds__(1024) kscan_local(U128* __restrict__ v, uint64_t K,
                                                     U128* __restrict__ totals) {
+  grid_dependency_wait();
   __shared__ U128 ws[32];
   const uint64_t i = (uint64_t)blockIdx.x * 1024 + threadIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -257,6 +262,7 @@ __global__ void __launch_bounds__(1024) kscan_local(U128* __restrict__ v, uint64
 // v[i] += inclusive prefix of the totals of the blocks before i's block
 __global__ void __launch_bounds__(1024) kscan_add(U128* __restrict__ v, uint64_t K,
                                                   const U128* __restrict__ scanned_totals) {
+  grid_dependency_wait();
   const uint64_t i = (uint64_t)blockIdx.x * 1024 + threadIdx.x;
   if (blockIdx.x == 0 || i >= K) return;
   v[i] = add128(v[i], scanned_totals[blockIdx.x - 1]);
@@ -268,6 +274,7 @@ __global__ void __launch_bounds__(kRedThreads)
     kshots(const T2* __restrict__ psi, int cbits, const U128* __restrict__ prefix, uint64_t K,
            const double* __restrict__ u, int64_t nshots, const int* __restrict__ mpos, int m,
            uint64_t* __restrict__ out) {
+  grid_dependency_wait();
   const int64_t s = (int64_t)blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (s >= nshots) return;
@@ -354,16 +361,17 @@ sv_status sv_probabilities(sv_state s, const int* qubits, int n_meas, double* ou
   {
     ProfScope prof(s->stream, "kprob_slices");
     if (s->dt == SV_C64)
-      kprob_slices<float2><<<(unsigned)nparts, kRedThreads, 0, s->stream>>>(
-          (const float2*)s->data, rest, dpos, m, per_bin, slices, parts);
+      launch_dependent(kprob_slices<float2>, (unsigned)nparts, kRedThreads, 0,
+                       s->stream, (const float2*)s->data, rest, dpos, m, per_bin, slices, parts);
     else
-      kprob_slices<double2><<<(unsigned)nparts, kRedThreads, 0, s->stream>>>(
-          (const double2*)s->data, rest, dpos, m, per_bin, slices, parts);
+      launch_dependent(kprob_slices<double2>, (unsigned)nparts, kRedThreads, 0,
+                       s->stream, (const double2*)s->data, rest, dpos, m, per_bin, slices, parts);
     g_launches.fetch_add(1, std::memory_order_relaxed);
   }
   {
     ProfScope prof(s->stream, "kprob_finish");
-    kprob_finish<<<(unsigned)((bins + 255) / 256), 256, 0, s->stream>>>(parts, slices, bins, dbins);
+    launch_dependent(kprob_finish, (unsigned)((bins + 255) / 256), 256, 0,
+                     s->stream, parts, slices, bins, dbins);
     g_launches.fetch_add(1, std::memory_order_relaxed);
   }
   st = check_launch("probabilities kernels");
@@ -410,22 +418,22 @@ sv_status sv_sample(sv_state s, const int* qubits, int n_meas, int64_t n_shots,
     ProfScope prof(s->stream, "kchunk_sums");
     const unsigned g = (unsigned)((K + kRedThreads / 32 - 1) / (kRedThreads / 32));
     if (s->dt == SV_C64)  // 2 amplitudes per 16-byte vector
-      kchunk_sums<float4><<<g, kRedThreads, 0, s->stream>>>((const float4*)s->data, cbits - 1,
-                                                            K, prefix);
+      launch_dependent(kchunk_sums<float4>, g, kRedThreads, 0,
+                       s->stream, (const float4*)s->data, cbits - 1, K, prefix);
     else
-      kchunk_sums<double2><<<g, kRedThreads, 0, s->stream>>>((const double2*)s->data, cbits, K,
-                                                             prefix);
+      launch_dependent(kchunk_sums<double2>, g, kRedThreads, 0,
+                       s->stream, (const double2*)s->data, cbits, K, prefix);
     g_launches.fetch_add(1, std::memory_order_relaxed);
   }
   {
     ProfScope prof(s->stream, "kscan");
     if (nb == 1) {
-      kscan<<<1, 1024, 0, s->stream>>>(prefix, K);
+      launch_dependent(kscan, 1, 1024, 0, s->stream, prefix, K);
       g_launches.fetch_add(1, std::memory_order_relaxed);
     } else {
-      kscan_local<<<(unsigned)nb, 1024, 0, s->stream>>>(prefix, K, btot);
-      kscan<<<1, 1024, 0, s->stream>>>(btot, nb);
-      kscan_add<<<(unsigned)nb, 1024, 0, s->stream>>>(prefix, K, btot);
+      launch_dependent(kscan_local, (unsigned)nb, 1024, 0, s->stream, prefix, K, btot);
+      launch_dependent(kscan, 1, 1024, 0, s->stream, btot, nb);
+      launch_dependent(kscan_add, (unsigned)nb, 1024, 0, s->stream, prefix, K, btot);
       g_launches.fetch_add(3, std::memory_order_relaxed);
     }
   }
@@ -433,11 +441,11 @@ sv_status sv_sample(sv_state s, const int* qubits, int n_meas, int64_t n_shots,
     ProfScope prof(s->stream, "kshots");
     const unsigned g = (unsigned)((n_shots + kRedThreads / 32 - 1) / (kRedThreads / 32));
     if (s->dt == SV_C64)
-      kshots<float2><<<g, kRedThreads, 0, s->stream>>>((const float2*)s->data, cbits, prefix, K,
-                                                       du, n_shots, dpos, m, dout);
+      launch_dependent(kshots<float2>, g, kRedThreads, 0,
+                       s->stream, (const float2*)s->data, cbits, prefix, K, du, n_shots, dpos, m, dout);
     else
-      kshots<double2><<<g, kRedThreads, 0, s->stream>>>((const double2*)s->data, cbits, prefix,
-                                                         K, du, n_shots, dpos, m, dout);
+      launch_dependent(kshots<double2>, g, kRedThreads, 0,
+                       s->stream, (const double2*)s->data, cbits, prefix, K, du, n_shots, dpos, m, dout);
     g_launches.fetch_add(1, std::memory_order_relaxed);
   }
   st = check_launch("sampling kernels");

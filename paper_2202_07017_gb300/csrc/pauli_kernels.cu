@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     mbar_init(barp[1], 1);
     fence_proxy_async_smem();
   }
+  grid_dependency_wait();
   __syncthreads();
   CompSum<R> acc;
   uint32_t parity[2] = {0, 0};
@@ -346,6 +347,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     }
     fence_proxy_async_smem();
   }
+  grid_dependency_wait();
   __syncthreads();
   CompSum<R> acc[kPG * kXGroups];
   // bit j: buffer j.  used: filled before (its refill waits until every warp
@@ -494,6 +496,7 @@ template <typename R>
 __global__ void __launch_bounds__(kDThreads, 3)
     kdiag_energy(const typename Cplx2P<R>::T* __restrict__ psi, const __grid_constant__ DiagDev<R> D,
                  double* __restrict__ partials) {
+  grid_dependency_wait();
   typedef typename Cplx2P<R>::T V2;
   constexpr bool C64 = sizeof(R) == 4;
   constexpr int NT = C64 ? 16 : 8;  // amplitudes of a tile
@@ -561,6 +564,7 @@ __global__ void __launch_bounds__(kDThreads, 2)
     kdiag_apply(typename Cplx2P<R>::T* __restrict__ out,
                 const typename Cplx2P<R>::T* __restrict__ psi, const __grid_constant__ DiagDev<R> D,
                 int accumulate, double* __restrict__ partials) {
+  grid_dependency_wait();
   typedef typename Cplx2P<R>::T V2;
   constexpr bool C64 = sizeof(R) == 4;
   constexpr int NT = C64 ? 16 : 8;  // amplitudes of a tile
@@ -1079,11 +1083,11 @@ sv_status expval_staged(sv_state s, const sv_pauli_sum* H, double* dst) {
   for (size_t i = 0; i < ndiag; ++i) {
     ProfScope prof(s->stream, c64 ? "kdiag_energy_c64" : "kdiag_energy_c128");
     if (c64)
-      kdiag_energy<float><<<dgrid, kDThreads, 0, s->stream>>>((const float2*)s->data, dfs[i],
-                                                               s->partials + total);
+      launch_dependent(kdiag_energy<float>, dgrid, kDThreads, 0,
+                       s->stream, (const float2*)s->data, dfs[i], s->partials + total);
     else
-      kdiag_energy<double><<<dgrid, kDThreads, 0, s->stream>>>((const double2*)s->data, dds[i],
-                                                                s->partials + total);
+      launch_dependent(kdiag_energy<double>, dgrid, kDThreads, 0,
+                       s->stream, (const double2*)s->data, dds[i], s->partials + total);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     st = check_launch("diagonal-term kernel");
     if (st) return st;
@@ -1095,23 +1099,23 @@ sv_status expval_staged(sv_state s, const sv_pauli_sum* H, double* dst) {
       ProfScope prof(s->stream, c64 ? "kpauli_xbits_c64" : "kpauli_xbits_c128");
       if (c64) {
         grid = grid_of((const void*)kpauli_xbits<float>, smem_x, kXBuf);
-        kpauli_xbits<float><<<(unsigned)grid, kPThreads, smem_x, s->stream>>>(
-            nblk, lean[i], s->partials + total, status);
+        launch_dependent(kpauli_xbits<float>, (unsigned)grid, kPThreads, smem_x,
+                         s->stream, nblk, lean[i], s->partials + total, status);
       } else {
         grid = grid_of((const void*)kpauli_xbits<double>, smem_x, kXBuf);
-        kpauli_xbits<double><<<(unsigned)grid, kPThreads, smem_x, s->stream>>>(
-            nblk, lean[i], s->partials + total, status);
+        launch_dependent(kpauli_xbits<double>, (unsigned)grid, kPThreads, smem_x,
+                         s->stream, nblk, lean[i], s->partials + total, status);
       }
     } else {
       ProfScope prof(s->stream, c64 ? "kpauli_energy_c64" : "kpauli_energy_c128");
       if (c64) {
         grid = grid_of((const void*)kpauli_energy<float>, smem, 2);
-        kpauli_energy<float><<<(unsigned)grid, kPThreads, smem, s->stream>>>(
-            nblk, pf[i], s->partials + total, status);
+        launch_dependent(kpauli_energy<float>, (unsigned)grid, kPThreads, smem,
+                         s->stream, nblk, pf[i], s->partials + total, status);
       } else {
         grid = grid_of((const void*)kpauli_energy<double>, smem, 2);
-        kpauli_energy<double><<<(unsigned)grid, kPThreads, smem, s->stream>>>(
-            nblk, pd[i], s->partials + total, status);
+        launch_dependent(kpauli_energy<double>, (unsigned)grid, kPThreads, smem,
+                         s->stream, nblk, pd[i], s->partials + total, status);
       }
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -1170,11 +1174,11 @@ sv_status apply_pauli_staged(void* out, const void* in, sv_state s, const sv_pau
     ProfScope prof(s->stream, c64 ? "kdiag_apply_c64" : "kdiag_apply_c128");
     double* part = diag_energy ? s->partials + total : nullptr;
     if (c64)
-      kdiag_apply<float><<<dgrid, kDThreads, 0, s->stream>>>(
-          (float2*)out, (const float2*)in, dfs[i], i > 0 ? 1 : 0, part);
+      launch_dependent(kdiag_apply<float>, dgrid, kDThreads, 0,
+                       s->stream, (float2*)out, (const float2*)in, dfs[i], i > 0 ? 1 : 0, part);
     else
-      kdiag_apply<double><<<dgrid, kDThreads, 0, s->stream>>>(
-          (double2*)out, (const double2*)in, dds[i], i > 0 ? 1 : 0, part);
+      launch_dependent(kdiag_apply<double>, dgrid, kDThreads, 0,
+                       s->stream, (double2*)out, (const double2*)in, dds[i], i > 0 ? 1 : 0, part);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     st = check_launch("diagonal apply kernel");
     if (st) return st;

@@ -46,6 +46,7 @@ struct ThreadSum {
 
 __global__ void __launch_bounds__(kRedThreads)
     knorm_c64(const float4* __restrict__ psi, uint64_t nvec, double* __restrict__ partials) {
+  grid_dependency_wait();
   ThreadSum<float> acc;
 #pragma unroll 4
   for (uint64_t v = (uint64_t)blockIdx.x * kRedThreads + threadIdx.x; v < nvec;
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(kRedThreads)
 
 __global__ void __launch_bounds__(kRedThreads)
     knorm_c128(const double2* __restrict__ psi, uint64_t nvec, double* __restrict__ partials) {
+  grid_dependency_wait();
   double acc = 0.0;
   for (uint64_t v = (uint64_t)blockIdx.x * kRedThreads + threadIdx.x; v < nvec;
        v += (uint64_t)gridDim.x * kRedThreads) {
@@ -86,6 +88,7 @@ template <typename R, typename T2>
 __global__ void __launch_bounds__(kRedThreads)
     kexpval(const T2* __restrict__ psi, uint64_t dim, const __grid_constant__ PauliDev P,
             double* __restrict__ partials) {
+  grid_dependency_wait();
   ThreadSum<R> acc;
   for (uint64_t x = (uint64_t)blockIdx.x * kRedThreads + threadIdx.x; x < dim;
        x += (uint64_t)gridDim.x * kRedThreads) {
@@ -117,6 +120,7 @@ __global__ void __launch_bounds__(kRedThreads)
     kapply_pauli(T2* __restrict__ out, const T2* __restrict__ psi, uint64_t dim,
                  const __grid_constant__ PauliDev P, int accumulate,
                  double* __restrict__ partials) {
+  grid_dependency_wait();
   ThreadSum<R> acc;
   for (uint64_t x = (uint64_t)blockIdx.x * kRedThreads + threadIdx.x; x < dim;
        x += (uint64_t)gridDim.x * kRedThreads) {
@@ -162,6 +166,7 @@ __global__ void __launch_bounds__(kRedThreads)
 
 __global__ void __launch_bounds__(kRedThreads)
     kfinish(const double* __restrict__ src, int count, double* __restrict__ dst, int add) {
+  grid_dependency_wait();
   const double* s = src + (size_t)blockIdx.x * count;
   double acc = 0.0;
   for (int i = threadIdx.x; i < count; i += kRedThreads) acc += s[i];
@@ -206,12 +211,14 @@ sv_status launch_norm_partials(sv_state s, double* partials, int* nparts) {
   if (s->dt == SV_C64) {
     const uint64_t nvec = s->n >= 1 ? (uint64_t(1) << (s->n - 1)) : 1;
     const int g = red_blocks(nvec);
-    knorm_c64<<<g, kRedThreads, 0, s->stream>>>((const float4*)s->data, nvec, partials);
+    launch_dependent(knorm_c64, g, kRedThreads, 0,
+                     s->stream, (const float4*)s->data, nvec, partials);
     *nparts = g;
   } else {
     const uint64_t nvec = uint64_t(1) << s->n;
     const int g = red_blocks(nvec);
-    knorm_c128<<<g, kRedThreads, 0, s->stream>>>((const double2*)s->data, nvec, partials);
+    launch_dependent(knorm_c128, g, kRedThreads, 0,
+                     s->stream, (const double2*)s->data, nvec, partials);
     *nparts = g;
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -223,11 +230,11 @@ sv_status launch_expval_partials(sv_state s, const PauliDev& P, double* partials
   const int g = red_blocks(dim);
   ProfScope prof(s->stream, "kexpval");
   if (s->dt == SV_C64)
-    kexpval<float, float2><<<g, kRedThreads, 0, s->stream>>>((const float2*)s->data, dim, P,
-                                                             partials);
+    launch_dependent(kexpval<float, float2>, g, kRedThreads, 0,
+                     s->stream, (const float2*)s->data, dim, P, partials);
   else
-    kexpval<double, double2><<<g, kRedThreads, 0, s->stream>>>((const double2*)s->data, dim, P,
-                                                               partials);
+    launch_dependent(kexpval<double, double2>, g, kRedThreads, 0,
+                     s->stream, (const double2*)s->data, dim, P, partials);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   *nparts = g;
   return check_launch("expval kernel");
@@ -240,11 +247,11 @@ sv_status launch_apply_pauli(void* out, const void* in, sv_dtype dt, int n, cuda
   const int g = red_blocks(dim);
   ProfScope prof(st, "kapply_pauli");
   if (dt == SV_C64)
-    kapply_pauli<float, float2><<<g, kRedThreads, 0, st>>>((float2*)out, (const float2*)in, dim,
-                                                           P, accumulate ? 1 : 0, partials);
+    launch_dependent(kapply_pauli<float, float2>, g, kRedThreads, 0, st, (float2*)out,
+                     (const float2*)in, dim, P, accumulate ? 1 : 0, partials);
   else
-    kapply_pauli<double, double2><<<g, kRedThreads, 0, st>>>(
-        (double2*)out, (const double2*)in, dim, P, accumulate ? 1 : 0, partials);
+    launch_dependent(kapply_pauli<double, double2>, g, kRedThreads, 0, st, (double2*)out,
+                     (const double2*)in, dim, P, accumulate ? 1 : 0, partials);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   if (nparts) *nparts = g;
   return check_launch("apply_pauli kernel");
@@ -254,7 +261,7 @@ sv_status launch_finish(const double* src, int count, int slots, double* dst, cu
                         bool add_to_dst) {
   if (slots <= 0) return SV_OK;
   ProfScope prof(st, "kfinish");
-  kfinish<<<slots, kRedThreads, 0, st>>>(src, count, dst, add_to_dst ? 1 : 0);
+  launch_dependent(kfinish, slots, kRedThreads, 0, st, src, count, dst, add_to_dst ? 1 : 0);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("finish kernel");
 }
@@ -353,15 +360,15 @@ extern "C" sv_status sv_expval_noalloc(const void* dev_state, int n_qubits, sv_d
   pauli_chunks(H, &chunks);
   for (const PauliDev& P : chunks) {
     if (dtype == SV_C64)
-      kexpval<float, float2><<<g, kRedThreads, 0, st>>>((const float2*)dev_state, dim, P,
-                                                        scratch + total);
+      launch_dependent(kexpval<float, float2>, g, kRedThreads, 0, st, (const float2*)dev_state,
+                       dim, P, scratch + total);
     else
-      kexpval<double, double2><<<g, kRedThreads, 0, st>>>((const double2*)dev_state, dim, P,
-                                                          scratch + total);
+      launch_dependent(kexpval<double, double2>, g, kRedThreads, 0, st, (const double2*)dev_state,
+                       dim, P, scratch + total);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     total += g;
   }
-  kfinish<<<1, kRedThreads, 0, st>>>(scratch, total, dev_out, 0);
+  launch_dependent(kfinish, 1, kRedThreads, 0, st, scratch, total, dev_out, 0);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("sv_expval_noalloc kernels");
 }
