@@ -59,6 +59,7 @@ struct FOpDev {
 // rot), the 2x2s in bit order
 // (8 values each, row-major re/im), then the diagonal (2^k real or 2^k re/im
 // pairs).
+// Passes that run on planes have their own coefficient order (see run_planes).
 struct FLayerDev {
   uint8_t u1, dk;
   uint16_t off;
@@ -89,6 +90,7 @@ struct FusedParams {
   uint16_t gop[kFMaxGroups + 1];
   uint8_t gkind[kFMaxGroups];        // 1, 2: the group runs as layers glay[g]..glay[g+1] (2: no dense 2x2)
   uint8_t gxm[kFMaxGroups];          // layer programs: register relabelling the stores undo
+  uint8_t gtpos[kFMaxGroups][9];     // planes: chunk bits of the thread bits (and the tile bit)
   uint16_t glay[kFMaxGroups + 1];
   int ncoef;                         // coefficients in coef[] (elements of R)
   FLayerDev layers[kFMaxLayers];
@@ -555,108 +557,244 @@ __device__ __forceinline__ void run_layers(typename Cplx2<R>::T* sm, int m, cons
   }
 }
 
-// Two sub-blocks per thread (s and s + kFThreads: a slice of 2^13 amplitudes
-// in 4-qubit groups) through one layer program in rotation form (no dense
-// 2x2: the registers of two tiles fit beside the rotations, not beside the
-// 2x2 coefficients) together: each layer's coefficients are read once for
-// both, and the two tiles' operations are independent, so a warp has twice
-// the arithmetic in flight between the dependent steps of one tile
-// (rotation on bit 0, then bit 1, ..., then the diagonal).
-// The registers hold each amplitude as a (re, im) pair, so the rotation's
-// four FMAs per register pair - every one scaling both parts of an amplitude
-// by the same t - issue as two paired fp32 FMAs (fma.rn.f32x2): half the
-// instructions for the same arithmetic.  Complex64 only.
-template <int KG, int B>
-__device__ __forceinline__ void rot_bit2p(float t, float2 (&v)[2][1 << KG]) {
-  const float2 tp = make_float2(t, t), tn = make_float2(-t, -t);
+// ---- layer programs on planes ------------------------------------------------------
+// Complex64 passes whose groups are all layer programs in rotation form run
+// on 16-byte chunks: amplitudes x and x + 1 (bit 0 clear and set) as (re, re)
+// and (im, im) register pairs, all arithmetic in paired fp32 instructions.
+//
+// What bounds these passes is the number of instructions, so no step moves a
+// register:
+//  - a complex diagonal on (re, im) pairs needs the lanes swapped and every
+//    coefficient duplicated (the passes spent more instructions on moves than on
+//    FMAs); on planes it is two multiplies and two FMAs in place;
+//  - a rotation is two shears in place, p += a q, q += b p: with t the
+//    rotation's tangent, c its cosine,
+//      [[c, -s], [s, c]] = diag(c, 1/c) [[1, 0], [s c, 1]] [[1, -t], [0, 1]],
+//    and the diagonal joins the layer's.  (p - t q and q + t p, each from the
+//    old values, need a copy of one of them.)
+// The chunks are loaded and stored as 16-byte vectors, half the shared-memory
+// instructions and address XORs.
+//
+// A thread holds 16 chunks = 32 amplitudes.  A group without bit 0 spans
+// the four chunk bits of its tile and both lanes of a pair share the
+// coefficients; a group with bit 0 spans three chunk bits and the lanes (two
+// such tiles per thread), its rotation on bit 0 working between the lanes.
+// Between groups a chunk rests as (re0, re1, im0, im1); the pass's first group
+// reads and its last writes the state's (re0, im0, re1, im1), in place.
+//
+// Measured (random layered circuit, n = 28, depth 30, 49 passes): 1516 -> 1254
+// us a pass (HBM read and write: 640 us); a third fewer instructions, the
+// shared-memory pipe now the busiest (53 %), two blocks of 8 warps a SM.
+// Coefficients duplicated in shared memory for the lanes: 1437 us; read from the
+// kernel parameters: 1683 us; shears with float2 operands instead of 64-bit
+// registers (split into scalar FMAs by the compiler): 2060 us.
+//
+// Coefficients of a layer: if it rotates, (a, b) of each of the four bits,
+// then the diagonal's 16 entries: (dr, di) or dr in order (both lanes of a
+// pair take the same one, which costs no move: a paired instruction can read
+// one register for both lanes), for a group with bit 0 in the order of its
+// pairs, (dr, dr', di, di') or (dr, dr') of entries 2 p and 2 p + 1.
+// Slices of fewer than 2^12 amplitudes (states below 20 qubits) leave such
+// threads in too few warps: run_layers' 16-amplitude threads are faster there
+// (n = 18, 2^10: 12.9 against 14.5 us a pass; n = 20, 2^12: 19.2 against 17.0).
+constexpr int kPlaneQubits = 12;
+
+// A pair of fp32 lanes in one 64-bit register: the arithmetic below stays on
+// these from load to store, so that every step is one paired instruction
+// (float2 values assembled from parts were split into scalar FMAs and moves).
+typedef unsigned long long Pair;
+
+__device__ __forceinline__ Pair pair_fma(Pair a, Pair b, Pair c) {
+  Pair d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  Pair d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ Pair pair_of(float x, float y) {
+  Pair d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float2 lanes_of(Pair p) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ Pair pair_both(float x) { return pair_of(x, x); }
+__device__ __forceinline__ Pair pair_swap(Pair p) {
+  const float2 v = lanes_of(p);
+  return pair_of(v.y, v.x);
+}
+// p += a q
+__device__ __forceinline__ void pair_add(Pair& p, Pair a, Pair q) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(p) : "l"(a), "l"(q));
+}
+
+// The rotation (a, b) on bit B of the tile index
+template <int B>
+__device__ __forceinline__ void plane_rot(float a, float b, Pair (&re)[16], Pair (&im)[16]) {
+  const Pair pa = pair_both(a), pb = pair_both(b);
 #pragma unroll
-  for (int r = 0; r < (1 << KG); ++r) {
+  for (int r = 0; r < 16; ++r) {
     if (r & (1 << B)) continue;
-    const int r1 = r | (1 << B);
+    const int q = r | (1 << B);
+    pair_add(re[r], pa, re[q]);
+    pair_add(im[r], pa, im[q]);
+    pair_add(re[q], pb, re[r]);
+    pair_add(im[q], pb, im[r]);
+  }
+}
+
+// The rotation on bit 0: between the lanes of every pair
+__device__ __forceinline__ void lane_rot(float a, float b, Pair (&re)[16], Pair (&im)[16]) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const float2 a = v[u][r], c = v[u][r1];
-      v[u][r] = __ffma2_rn(tn, c, a);   // a - t c
-      v[u][r1] = __ffma2_rn(tp, a, c);  // t a + c
+  for (int r = 0; r < 16; ++r) {
+    float2 x = lanes_of(re[r]), y = lanes_of(im[r]);
+    x.x = fmaf(a, x.y, x.x);
+    y.x = fmaf(a, y.y, y.x);
+    x.y = fmaf(b, x.x, x.y);
+    y.y = fmaf(b, y.x, y.y);
+    re[r] = pair_of(x.x, x.y);
+    im[r] = pair_of(y.x, y.y);
+  }
+}
+
+// (re, im) <- (dr + i di)(re, im) in place, dn = -di
+__device__ __forceinline__ void plane_mul(Pair dr, Pair di, Pair dn, Pair& re, Pair& im) {
+  Pair t = pair_mul(di, re);
+  re = pair_mul(dr, re);
+  pair_add(re, dn, im);
+  pair_add(t, dr, im);
+  im = t;
+}
+
+// the 128-byte swizzle on 16-byte chunk indices
+__device__ __forceinline__ int chunk_swz(int q) { return q ^ ((q >> 3) & 7); }
+
+// LOW: the group holds amplitude bit 0.  xm: the program's final register
+// relabelling (register r holds group index r ^ xm).  base0: the thread's tile
+// (its swizzled chunk index with the group's bits clear); tile: the chunk bit of
+// its second tile (LOW).
+template <bool LOW>
+__device__ __forceinline__ void run_planes(ulonglong2* sm, const uint8_t* gb,
+                                           const FLayerDev* lay, int l0, int l1,
+                                           const float* coef, int xm, int base0, int tile,
+                                           bool first, bool last) {
+  constexpr int NB = LOW ? 3 : 4;  // chunk bits of a tile
+  int sw[NB], base[LOW ? 2 : 1];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) sw[i] = chunk_swz(1 << (gb[LOW ? i + 1 : i] - 1));
+  base[0] = base0;
+  if constexpr (LOW) base[1] = base0 ^ chunk_swz(1 << tile);
+  // tile index r: chunk bits in its low NB bits, then (LOW) the tile
+  auto slot = [&](int r) {
+    int o = LOW ? base[r >> 3] : base[0];
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if ((r >> i) & 1) o ^= sw[i];
+    return o;
+  };
+  Pair re[16], im[16];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const ulonglong2 v = sm[slot(r)];
+    re[r] = v.x;
+    im[r] = v.y;
+  }
+  if (first) {  // (re0, im0), (re1, im1) as loaded
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const float2 a = lanes_of(re[r]), b = lanes_of(im[r]);
+      re[r] = pair_of(a.x, b.x);
+      im[r] = pair_of(a.y, b.y);
     }
   }
-}
-
-template <int KG>
-__device__ __forceinline__ void rot_bit2p_at(int i, const float (&tv)[4], float2 (&v)[2][1 << KG]) {
-  if (i == 0) rot_bit2p<KG, 0>(tv[0], v);
-  if constexpr (KG > 1) if (i == 1) rot_bit2p<KG, (KG > 1 ? 1 : 0)>(tv[KG > 1 ? 1 : 0], v);
-  if constexpr (KG > 2) if (i == 2) rot_bit2p<KG, (KG > 2 ? 2 : 0)>(tv[KG > 2 ? 2 : 0], v);
-  if constexpr (KG > 3) if (i == 3) rot_bit2p<KG, (KG > 3 ? 3 : 0)>(tv[KG > 3 ? 3 : 0], v);
-}
-
-template <int KG>
-__device__ __forceinline__ void run_layers_x2(float2* sm, const uint8_t* gb, const FLayerDev* lay,
-                                              int l0, int l1, const float* coef, int xm) {
-  constexpr int D = 1 << KG;
-  int sw[KG], lm[KG];
-#pragma unroll
-  for (int i = 0; i < KG; ++i) {
-    sw[i] = swz<float>(1 << gb[i]);
-    lm[i] = (1 << gb[i]) - 1;
-  }
-  int sb[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    int b = threadIdx.x + u * kFThreads;
-#pragma unroll
-    for (int i = 0; i < KG; ++i) b = ((b & ~lm[i]) << 1) | (b & lm[i]);
-    sb[u] = swz<float>(b);
-  }
-  float2 v[2][D];
-#pragma unroll
-  for (int r = 0; r < D; ++r)
-#pragma unroll
-    for (int u = 0; u < 2; ++u) v[u][r] = sm[sb[u] ^ reg_off<KG>(r, sw)];
   for (int l = l0; l < l1; ++l) {
     const FLayerDev L = lay[l];
-    const float* c = coef + L.off;
+    const float4* c = reinterpret_cast<const float4*>(coef + L.off);
     if (L.rot) {
-      float tv[4];
-      load_tau4<float>(c, tv);
-      if (L.rot == (1 << KG) - 1) {  // every bit: one straight-line block
-#pragma unroll
-        for (int i = 0; i < KG; ++i) rot_bit2p_at<KG>(i, tv, v);
+      const float4 u = c[0], v = c[1];
+      if (L.rot == 15) {  // every bit: one straight-line block
+        if constexpr (LOW) {
+          lane_rot(u.x, u.y, re, im);
+          plane_rot<0>(u.z, u.w, re, im);
+          plane_rot<1>(v.x, v.y, re, im);
+          plane_rot<2>(v.z, v.w, re, im);
+        } else {
+          plane_rot<0>(u.x, u.y, re, im);
+          plane_rot<1>(u.z, u.w, re, im);
+          plane_rot<2>(v.x, v.y, re, im);
+          plane_rot<3>(v.z, v.w, re, im);
+        }
       } else {
-#pragma unroll
-        for (int i = 0; i < KG; ++i)
-          if (L.rot & (1 << i)) rot_bit2p_at<KG>(i, tv, v);
+        if (L.rot & 1) {
+          if constexpr (LOW) lane_rot(u.x, u.y, re, im); else plane_rot<0>(u.x, u.y, re, im);
+        }
+        if (L.rot & 2) plane_rot<LOW ? 0 : 1>(u.z, u.w, re, im);
+        if (L.rot & 4) plane_rot<LOW ? 1 : 2>(v.x, v.y, re, im);
+        if (L.rot & 8) plane_rot<LOW ? 2 : 3>(v.z, v.w, re, im);
       }
-      c += 4;
+      c += 2;
     }
-    if (L.dk == 1) {
+    if (L.dk == 2) {
 #pragma unroll
-      for (int r = 0; r < D; ++r) {
-        const float2 d = make_float2(c[r], c[r]);
-#pragma unroll
-        for (int u = 0; u < 2; ++u) v[u][r] = __fmul2_rn(d, v[u][r]);
+      for (int e = 0; e < 8; ++e) {
+        const float4 d = c[e];
+        if constexpr (LOW) {
+          const Pair dr = pair_of(d.x, d.y), di = pair_of(d.z, d.w), dn = pair_of(-d.z, -d.w);
+          plane_mul(dr, di, dn, re[e], im[e]);
+          plane_mul(dr, di, dn, re[8 + e], im[8 + e]);
+        } else {
+          plane_mul(pair_both(d.x), pair_both(d.y), pair_both(-d.y), re[2 * e], im[2 * e]);
+          plane_mul(pair_both(d.z), pair_both(d.w), pair_both(-d.w), re[2 * e + 1], im[2 * e + 1]);
+        }
       }
-    } else if (L.dk == 2) {
+    } else if (L.dk == 1) {
 #pragma unroll
-      for (int r = 0; r < D; ++r) {
-        const float2 d = *reinterpret_cast<const float2*>(c + 2 * r);
-        const float2 dr = make_float2(d.x, d.x), di = make_float2(-d.y, d.y);
+      for (int e = 0; e < 4; ++e) {
+        const float4 d = c[e];
+        const float dd[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {  // (dr xr - di xi, dr xi + di xr)
-          const float2 x = v[u][r];
-          v[u][r] = __ffma2_rn(di, make_float2(x.y, x.x), __fmul2_rn(dr, x));
+        for (int j = 0; j < 4; ++j) {
+          // LOW: entries 4 e .. 4 e + 3 are pairs 2 e and 2 e + 1 of both tiles
+          const int r = LOW ? 2 * e + (j & 1) + 8 * (j >> 1) : 4 * e + j;
+          const Pair f = LOW ? pair_of(dd[2 * (j & 1)], dd[2 * (j & 1) + 1]) : pair_both(dd[j]);
+          re[r] = pair_mul(f, re[r]);
+          im[r] = pair_mul(f, im[r]);
         }
       }
     }
   }
+  int xoff = 0;
 #pragma unroll
-  for (int r = 0; r < D; ++r)
+  for (int i = 0; i < NB; ++i)
+    if ((xm >> (LOW ? i + 1 : i)) & 1) xoff ^= sw[i];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      int sbr = sb[u] ^ reg_off<KG>(xm, sw);
-      asm volatile("mov.b32 %0, %1;" : "=r"(sbr) : "r"(sbr));  // store addresses recomputed
-      sm[sbr ^ reg_off<KG>(r, sw)] = v[u][r];
+  for (int u = 0; u < (LOW ? 2 : 1); ++u) {
+    base[u] ^= xoff;
+    asm volatile("" : "+r"(base[u]));  // store addresses recomputed, not kept from the loads
+  }
+  if (LOW && (xm & 1)) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      re[r] = pair_swap(re[r]);
+      im[r] = pair_swap(im[r]);
     }
+  }
+  if (last) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const float2 a = lanes_of(re[r]), b = lanes_of(im[r]);
+      re[r] = pair_of(a.x, b.x);
+      im[r] = pair_of(a.y, b.y);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 16; ++r) sm[slot(r)] = make_ulonglong2(re[r], im[r]);
 }
 
 // ---- the pass kernel ------------------------------------------------------------
@@ -810,7 +948,8 @@ __device__ __forceinline__ void issue_store(const FusedParams<R>& P, uint32_t sr
 // MODE: 0 every group a gate list, 1 mixed, 3 every group a layer program
 // (shared-memory addresses recomputed per access instead of tabulated), 4 as
 // 3 with every dense 2x2 rounded with dither (complex64, dithered rounding
-// selected for the state)
+// selected for the state), 5 every group a layer program in rotation form, on
+// planes (complex64, 4-qubit groups, blocks of 2^(m - 5) threads)
 template <typename R, int KGF, int MINB, int MODE>
 __global__ void __launch_bounds__(kFThreads, MINB)
     kfused_tma(uint64_t n_blocks, const __grid_constant__ FusedParams<R> P) {
@@ -823,11 +962,19 @@ __global__ void __launch_bounds__(kFThreads, MINB)
   const uint32_t barp = smem_addr(&bar);
   const int lane = threadIdx.x & 31;
   R* csm = reinterpret_cast<R*>(smem_raw + (sbuf - raw) + P.slice_bytes);
-  for (int i = threadIdx.x; i < P.ncoef; i += kFThreads) csm[i] = P.coef[i];
+  for (int i = threadIdx.x; i < P.ncoef; i += blockDim.x) csm[i] = P.coef[i];
   // the layer table beside the coefficients: read per layer by every thread,
   // from shared memory rather than the parameter space
   FLayerDev* lsm = reinterpret_cast<FLayerDev*>(csm + ((P.ncoef + 1) & ~1));
-  for (int i = threadIdx.x; i < P.glay[P.ngroups]; i += kFThreads) lsm[i] = P.layers[i];
+  for (int i = threadIdx.x; i < P.glay[P.ngroups]; i += blockDim.x) lsm[i] = P.layers[i];
+  // planes: every group's tile of every thread
+  uint16_t* tbase = reinterpret_cast<uint16_t*>(lsm + P.glay[P.ngroups]);
+  if constexpr (MODE == 5)
+    for (int g = 0; g < P.ngroups; ++g) {
+      int q = 0;
+      for (int i = 0; i < P.m - 5; ++i) q |= ((threadIdx.x >> i) & 1) << P.gtpos[g][i];
+      tbase[g * blockDim.x + threadIdx.x] = (uint16_t)chunk_swz(q);
+    }
   if (threadIdx.x == 0) {
     mbar_init(barp, 1);
     fence_proxy_async_smem();
@@ -860,9 +1007,16 @@ __global__ void __launch_bounds__(kFThreads, MINB)
         run_layers<KGF, R, false, true>(
             sm, P.m, P.gbits[g], lsm, P.glay[g], P.glay[g + 1], csm,
             mix32(P.dseed ^ (uint32_t)blk ^ ((uint32_t)(blk >> 32) + (uint32_t)g * 0x85ebca6bu)));
-      else if (MODE == 3 && KGF == 4 && sizeof(R) == 4 && P.m == 13 && P.gkind[g] == 2) {
-        if constexpr (sizeof(R) == 4)  // two sub-blocks per thread (complex64 slices)
-          run_layers_x2<KGF>(sm, P.gbits[g], lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g]);
+      else if constexpr (MODE == 5) {
+        ulonglong2* sm4 = reinterpret_cast<ulonglong2*>(sm);
+        const uint8_t* gb = P.gbits[g];
+        const int base = tbase[g * blockDim.x + threadIdx.x], tile = P.gtpos[g][P.m - 5];
+        if (gb[0] == 0)
+          run_planes<true>(sm4, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], base, tile,
+                           g == 0, g + 1 == P.ngroups);
+        else
+          run_planes<false>(sm4, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], base, tile,
+                            g == 0, g + 1 == P.ngroups);
       } else if (MODE == 3)
         run_layers<KGF, R, false>(sm, P.m, P.gbits[g], lsm, P.glay[g], P.glay[g + 1], csm, 0,
                                   P.gxm[g]);
@@ -1458,12 +1612,13 @@ bool build_tma(const TmaGeom& g, void* data, FusedParams<R>* P, CUtensorMap* map
 // diagonal.  All products in fp64; the coefficients are rounded with the
 // state's error feedback (drift; the layers' 2x2s and diagonals act on the
 // whole state).  With rotform every dense 2x2 is split into a scaled real
-// rotation between diagonals (see rotation_form below).  Returns 0 (and
+// rotation between diagonals (see rotation_form below); with shear too the
+// rotations are shears (see run_planes).  Returns 0 (and
 // leaves nl, nc) if the group keeps its gate list, 2 for a layer program in
 // rotation form throughout, 1 for one with dense 2x2s.
 template <typename R>
 int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>* P, int* nlp,
-                int* ncp, double* drift, bool rotform) {
+                int* ncp, double* drift, bool rotform, bool shear) {
   struct LayerH {
     int u1 = 0, dtouch = 0;
     int rot = 0, form = 0;  // rotation form: bits with scaled rotations tau[i]
@@ -1590,6 +1745,9 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       o.msq = msq / D;
       out->push_back(o);
     }
+    // Shears: S(t) = diag(1, 1 + t^2) [[1, 0], [t / (1 + t^2), 1]] [[1, -t], [0, 1]];
+    // the diagonal, as diag(c, 1/c) / c with c = 1 / sqrt(1 + t^2), joins the
+    // layer's (on the registers, so after the relabelling below).
     // One rotation shape on the device: [[t, -1], [1, t]] = X Z S(-t) with
     // S(t) = [[1, -t], [t, 1]].  X on a bit relabels the registers instead of
     // moving them (mask M: register p holds logical index p ^ M; X S(t) X =
@@ -1606,6 +1764,9 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       cd Dl[32];
       for (int r = 0; r < D; ++r) {
         Dl[r] = o.Dg[r];
+        for (int t = 0; t < k && shear; ++t)  // register of logical index r: r ^ M ^ F
+          if ((o.rot >> t) & 1 && (((r ^ M ^ F) >> t) & 1))
+            Dl[r] = scl(Dl[r], 1.0 + o.tau[t] * o.tau[t]);
         for (int t = 0; t < k; ++t)
           if ((F >> t) & 1) Dl[r] = scl(Dl[r], ((r >> t) & 1) ? 1.0 : -1.0);  // -Z_t
       }
@@ -1709,13 +1870,19 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       }
       const int dk = one ? 0 : real ? 1 : 2;
       dks.push_back(dk);
-      need += h.rot ? 4 : 0;
+      need += h.rot ? (shear ? 8 : 4) : 0;
       need += 8 * __builtin_popcount(h.u1);
       need += dk == 0 ? 0 : dk == 1 ? D : 2 * D;
       need = (need + 3) & ~3;  // 16-byte alignment of the next layer (float)
     }
     if (nl + (int)L.size() > kFMaxLayers || nc + need > cap) return 0;
     double* fb = sizeof(R) == 4 ? drift : nullptr;
+    auto round_diag = [&](LayerH& h) {
+      if (shear)
+        feedback_round_entries(h.Dg, D, fb);
+      else
+        feedback_round_diag(h.Dg, D, fb, h.msq);
+    };
     for (size_t li = 0; li < L.size(); ++li) {
       LayerH& h = L[li];
       FLayerDev& d = P->layers[nl++];
@@ -1726,7 +1893,15 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       d.pad8 = 0;
       d.pad = 0;
       if (h.rot) {  // tau of bit i in slot i (0 where bit i has no rotation)
-        for (int i = 0; i < 4; ++i) P->coef[nc++] = ((h.rot >> i) & 1) ? (R)h.tau[i] : R(0);
+        for (int i = 0; i < 4; ++i) {
+          const double t = ((h.rot >> i) & 1) ? h.tau[i] : 0.0;
+          if (shear) {
+            P->coef[nc++] = (R)-t;
+            P->coef[nc++] = (R)(t / (1.0 + t * t));
+          } else {
+            P->coef[nc++] = (R)t;
+          }
+        }
       }
       for (int i = 0; i < k; ++i)
         if ((h.u1 >> i) & 1) {
@@ -1737,13 +1912,16 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
           }
         }
       if (dks[li] == 1) {  // real entries (+-1 in gate-list form: exact)
-        feedback_round_diag(h.Dg, D, fb, h.msq);
+        round_diag(h);
         for (int r = 0; r < D; ++r) P->coef[nc++] = (R)h.Dg[r].re;
       } else if (dks[li] == 2) {
-        feedback_round_diag(h.Dg, D, fb, h.msq);
-        for (int r = 0; r < D; ++r) {
+        round_diag(h);
+        const bool pairs = shear && lb[0] == 0;  // a group with bit 0, on planes
+        for (int r = 0; r < D; r += 2) {
           P->coef[nc++] = (R)h.Dg[r].re;
-          P->coef[nc++] = (R)h.Dg[r].im;
+          P->coef[nc++] = pairs ? (R)h.Dg[r + 1].re : (R)h.Dg[r].im;
+          P->coef[nc++] = pairs ? (R)h.Dg[r].im : (R)h.Dg[r + 1].re;
+          P->coef[nc++] = (R)h.Dg[r + 1].im;
         }
       }
       while (nc & 3) P->coef[nc++] = 0;
@@ -1761,7 +1939,8 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
 // otherwise a reverse-sweep pass (gate lists, plain rounding).
 template <typename R>
 bool build_params(const FusedPass& pass, const std::vector<int>& order, FusedParams<R>* P,
-                  bool forward = true, double* drift = nullptr, bool rotform = false) {
+                  bool forward = true, double* drift = nullptr, bool rotform = false,
+                  bool shear = false) {
   P->ngrad = 0;
   P->extra_tx = 0;
   P->dseed = 0;
@@ -1870,7 +2049,7 @@ bool build_params(const FusedPass& pass, const std::vector<int>& order, FusedPar
     for (int g = 0; g < P->ngroups; ++g) {
       P->glay[g] = (uint16_t)nl;
       P->gxm[g] = 0;
-      P->gkind[g] = (uint8_t)layer_group(pass, g, pos_of, P, &nl, &nc, fb, rotform);
+      P->gkind[g] = (uint8_t)layer_group(pass, g, pos_of, P, &nl, &nc, fb, rotform, shear);
       if (P->gkind[g] || !fb) continue;
       const FusedGroup& grp = pass.groups[g];
       for (size_t j = 0; j < grp.ops.size(); ++j) {
@@ -1904,6 +2083,8 @@ struct PassKernels {
   }
   template <int KG, int MINB>
   static Tma pick(int mode) {
+    if constexpr (sizeof(R) == 4 && KG == 4)
+      if (mode == 5) return kfused_tma<R, KG, MINB, 5>;
     if constexpr (sizeof(R) == 4)
       if (mode == 4) return kfused_tma<R, KG, MINB, 4>;
     return mode == 3   ? kfused_tma<R, KG, MINB, 3>
@@ -1919,6 +2100,32 @@ struct PassKernels {
     return kg <= 1 ? pick<1, MB>(mode) : kg == 2 ? pick<2, MB>(mode) : pick<3, MB>(mode);
   }
 };
+
+// The thread bits of every group on planes, as chunk bits.  A quarter warp's
+// 16-byte accesses are free of bank conflicts if its three lane bits reach all
+// eight 16-byte columns of a 128-byte row: chunk bits below 6 move column bit
+// (i mod 3) (bits 3..5 through the swizzle), so the lanes take three free chunk
+// bits of different residues where the group leaves them; the other thread bits
+// follow in order.
+template <typename R>
+void plane_threads(FusedParams<R>* P) {
+  for (int g = 0; g < P->ngroups; ++g) {
+    bool used[24] = {};
+    const bool low = P->gbits[g][0] == 0;
+    for (int i = low ? 1 : 0; i < 4; ++i) used[P->gbits[g][i] - 1] = true;
+    int k = 0;
+    for (int res = 0; res < 3; ++res)
+      for (int i = res; i < 6 && i < P->m - 1; i += 3)
+        if (!used[i]) {
+          P->gtpos[g][k++] = (uint8_t)i;
+          used[i] = true;
+          break;
+        }
+    for (int i = 0; i < P->m - 1; ++i)
+      if (!used[i]) P->gtpos[g][k++] = (uint8_t)i;
+    for (; k < 9; ++k) P->gtpos[g][k] = 0;
+  }
+}
 
 template <typename R>
 sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, RoundCtx* rc) {
@@ -1940,7 +2147,17 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
   // layer programs in rotation form, except where every dense 2x2 is to be
   // rounded with dither (that mode keeps the dense form)
   const bool dither_all = sizeof(R) == 4 && rc && rc->mode == SV_ROUNDING_DITHERED;
-  if (!build_params(pass, order, &P, true, drift, !dither_all)) {
+  // on planes where every group allows it
+  const bool want_planes = tma && sizeof(R) == 4 && kg == 4 && !dither_all &&
+                           (int)pass.S.size() >= kPlaneQubits;
+  bool built = build_params(pass, order, &P, true, drift, !dither_all, want_planes);
+  bool planes = want_planes && built;
+  for (int g = 0; g < P.ngroups; ++g) planes = planes && P.gkind[g] == 2;
+  if (!planes && want_planes) {
+    if (drift) *drift = drift0;
+    built = build_params(pass, order, &P, true, drift, !dither_all);
+  }
+  if (!built) {
     set_error("fused pass exceeds kernel capacity");
     return SV_ERR_INVALID;
   }
@@ -1950,8 +2167,9 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
     return SV_ERR_INVALID;
   }
   if (tma) tma = build_tma(geo, data, &P);
-  if (!tma && order != pass.S && drift) *drift = drift0;  // rebuilt below
-  if (!tma && order != pass.S && !build_params(pass, pass.S, &P, true, drift, !dither_all)) {
+  const bool rebuild = !tma && (order != pass.S || planes);
+  if (rebuild && drift) *drift = drift0;
+  if (rebuild && !build_params(pass, pass.S, &P, true, drift, !dither_all)) {
     set_error("fused pass exceeds kernel capacity");
     return SV_ERR_INVALID;
   }
@@ -1963,16 +2181,19 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
   if (tma) {
     int nlay = 0;
     for (int g = 0; g < P.ngroups; ++g) nlay += P.gkind[g] != 0;
-    const int mode = nlay == 0 ? 0 : nlay == P.ngroups ? (dither_all ? 4 : 3) : 1;
+    const int mode = planes ? 5 : nlay == 0 ? 0 : nlay == P.ngroups ? (dither_all ? 4 : 3) : 1;
     typename PassKernels<R>::Tma kern = PassKernels<R>::tma(kg, mode);
+    const int threads = mode == 5 ? 1 << (P.m - 5) : kFThreads;
+    if (mode == 5) plane_threads(&P);
     const size_t smem = (amp << P.m) + 1024 + sizeof(R) * (size_t)((P.ncoef + 1) & ~1) +
-                        sizeof(FLayerDev) * (size_t)P.glay[P.ngroups];
+                        sizeof(FLayerDev) * (size_t)P.glay[P.ngroups] +
+                        (mode == 5 ? sizeof(uint16_t) * (size_t)threads * P.ngroups : 0);
     // resident blocks per SM for this kernel and shared-memory size
     static std::map<std::pair<const void*, size_t>, int> resident;
     int& res = resident[{reinterpret_cast<const void*>(kern), smem}];
     if (!res) {
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kern, kFThreads, smem) != cudaSuccess ||
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kern, threads, smem) != cudaSuccess ||
           res < 1) {
         cudaGetLastError();
         res = 1;
@@ -1982,7 +2203,7 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint64_t grid = std::min<uint64_t>(nblk, (uint64_t)sms * res);
-    launch_dependent(kern, (unsigned)grid, kFThreads, smem, st, nblk, P);
+    launch_dependent(kern, (unsigned)grid, threads, smem, st, nblk, P);
   } else {
     typename PassKernels<R>::Lsu kern = PassKernels<R>::lsu(kg);
     const size_t smem = (amp << P.m) + (sizeof(uint64_t) * (((size_t(1) << (P.m - P.L)) + 1) & ~size_t(1))) +

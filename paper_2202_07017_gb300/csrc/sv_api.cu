@@ -172,6 +172,22 @@ void feedback_round_diag(cd* dg, int d, double* drift, double mean_sq) {
   *drift += std::log(t / (d * mean_sq));
 }
 
+void feedback_round_entries(cd* dg, int d, double* drift) {
+  if (!drift) return;
+  bool exact = true;
+  for (int e = 0; e < d && exact; ++e) exact = fp32_number(dg[e].re) && fp32_number(dg[e].im);
+  if (exact) return;
+  const double f = std::exp(-0.5 * *drift);
+  double t = 0.0;
+  for (int e = 0; e < d; ++e) {
+    const double m = dg[e].re * dg[e].re + dg[e].im * dg[e].im;
+    dg[e].re *= f;
+    dg[e].im *= f;
+    t += sq32(dg[e]) / m;
+  }
+  *drift += std::log(t / d);
+}
+
 void feedback_round_pair(double* c, cd* k, double* drift) {
   if (!drift || (fp32_number(*c) && fp32_number(k->re) && fp32_number(k->im))) return;
   const double f = std::exp(-0.5 * *drift);
