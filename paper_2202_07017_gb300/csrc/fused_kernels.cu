@@ -572,6 +572,12 @@ __device__ __forceinline__ void run_layers(typename Cplx2<R>::T* sm, int m, cons
 //      [[c, -s], [s, c]] = diag(c, 1/c) [[1, 0], [s c, 1]] [[1, -t], [0, 1]],
 //    and the diagonal joins the layer's.  (p - t q and q + t p, each from the
 //    old values, need a copy of one of them.)
+// Passes of X and Y rotations only (see FusedPass::lift) take three shears, p +=
+// a q, q += b p, p += a q with a = -tan(angle / 2), b = sin(angle), which need no
+// diagonal: what is left of theirs are exact powers of i.  Multiplying every
+// amplitude by one rounded factor near 1, step after step of a Trotter product,
+// moves the norm by a fixed part of a rounding each time (3.7e-5 over 57 000
+// rotations), while an FMA with an unrelated addend does not.
 // The chunks are loaded and stored as 16-byte vectors, half the shared-memory
 // instructions and address XORs.
 //
@@ -598,17 +604,13 @@ __device__ __forceinline__ void run_layers(typename Cplx2<R>::T* sm, int m, cons
 // threads in too few warps: run_layers' 16-amplitude threads are faster there
 // (n = 18, 2^10: 12.9 against 14.5 us a pass; n = 20, 2^12: 19.2 against 17.0).
 constexpr int kPlaneQubits = 12;
+constexpr int kLiftQubits = 10;  // smallest slice of passes with lift: one warp
 
 // A pair of fp32 lanes in one 64-bit register: the arithmetic below stays on
 // these from load to store, so that every step is one paired instruction
 // (float2 values assembled from parts were split into scalar FMAs and moves).
 typedef unsigned long long Pair;
 
-__device__ __forceinline__ Pair pair_fma(Pair a, Pair b, Pair c) {
-  Pair d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
 __device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
   Pair d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -635,7 +637,7 @@ __device__ __forceinline__ void pair_add(Pair& p, Pair a, Pair q) {
 }
 
 // The rotation (a, b) on bit B of the tile index
-template <int B>
+template <int B, bool LIFT>
 __device__ __forceinline__ void plane_rot(float a, float b, Pair (&re)[16], Pair (&im)[16]) {
   const Pair pa = pair_both(a), pb = pair_both(b);
 #pragma unroll
@@ -646,10 +648,15 @@ __device__ __forceinline__ void plane_rot(float a, float b, Pair (&re)[16], Pair
     pair_add(im[r], pa, im[q]);
     pair_add(re[q], pb, re[r]);
     pair_add(im[q], pb, im[r]);
+    if constexpr (LIFT) {
+      pair_add(re[r], pa, re[q]);
+      pair_add(im[r], pa, im[q]);
+    }
   }
 }
 
 // The rotation on bit 0: between the lanes of every pair
+template <bool LIFT>
 __device__ __forceinline__ void lane_rot(float a, float b, Pair (&re)[16], Pair (&im)[16]) {
 #pragma unroll
   for (int r = 0; r < 16; ++r) {
@@ -658,8 +665,41 @@ __device__ __forceinline__ void lane_rot(float a, float b, Pair (&re)[16], Pair 
     y.x = fmaf(a, y.y, y.x);
     x.y = fmaf(b, x.x, x.y);
     y.y = fmaf(b, y.x, y.y);
+    if constexpr (LIFT) {
+      x.x = fmaf(a, x.y, x.x);
+      y.x = fmaf(a, y.y, y.x);
+    }
     re[r] = pair_of(x.x, x.y);
     im[r] = pair_of(y.x, y.y);
+  }
+}
+
+// The rotations of a layer, (a, b) of its four bits in u and v
+template <bool LOW, bool LIFT>
+__device__ __forceinline__ void plane_rots(int rot, const float4& u, const float4& v,
+                                           Pair (&re)[16], Pair (&im)[16]) {
+  if (rot == 15) {  // every bit: one straight-line block
+    if constexpr (LOW) {
+      lane_rot<LIFT>(u.x, u.y, re, im);
+      plane_rot<0, LIFT>(u.z, u.w, re, im);
+      plane_rot<1, LIFT>(v.x, v.y, re, im);
+      plane_rot<2, LIFT>(v.z, v.w, re, im);
+    } else {
+      plane_rot<0, LIFT>(u.x, u.y, re, im);
+      plane_rot<1, LIFT>(u.z, u.w, re, im);
+      plane_rot<2, LIFT>(v.x, v.y, re, im);
+      plane_rot<3, LIFT>(v.z, v.w, re, im);
+    }
+  } else {
+    if (rot & 1) {
+      if constexpr (LOW)
+        lane_rot<LIFT>(u.x, u.y, re, im);
+      else
+        plane_rot<0, LIFT>(u.x, u.y, re, im);
+    }
+    if (rot & 2) plane_rot<LOW ? 0 : 1, LIFT>(u.z, u.w, re, im);
+    if (rot & 4) plane_rot<LOW ? 1 : 2, LIFT>(v.x, v.y, re, im);
+    if (rot & 8) plane_rot<LOW ? 2 : 3, LIFT>(v.z, v.w, re, im);
   }
 }
 
@@ -678,8 +718,8 @@ __device__ __forceinline__ int chunk_swz(int q) { return q ^ ((q >> 3) & 7); }
 // LOW: the group holds amplitude bit 0.  xm: the program's final register
 // relabelling (register r holds group index r ^ xm).  base0: the thread's tile
 // (its swizzled chunk index with the group's bits clear); tile: the chunk bit of
-// its second tile (LOW).
-template <bool LOW>
+// its second tile (LOW).  LIFT: the rotations take a third shear.
+template <bool LOW, bool LIFT>
 __device__ __forceinline__ void run_planes(ulonglong2* sm, const uint8_t* gb,
                                            const FLayerDev* lay, int l0, int l1,
                                            const float* coef, int xm, int base0, int tile,
@@ -718,26 +758,7 @@ __device__ __forceinline__ void run_planes(ulonglong2* sm, const uint8_t* gb,
     const float4* c = reinterpret_cast<const float4*>(coef + L.off);
     if (L.rot) {
       const float4 u = c[0], v = c[1];
-      if (L.rot == 15) {  // every bit: one straight-line block
-        if constexpr (LOW) {
-          lane_rot(u.x, u.y, re, im);
-          plane_rot<0>(u.z, u.w, re, im);
-          plane_rot<1>(v.x, v.y, re, im);
-          plane_rot<2>(v.z, v.w, re, im);
-        } else {
-          plane_rot<0>(u.x, u.y, re, im);
-          plane_rot<1>(u.z, u.w, re, im);
-          plane_rot<2>(v.x, v.y, re, im);
-          plane_rot<3>(v.z, v.w, re, im);
-        }
-      } else {
-        if (L.rot & 1) {
-          if constexpr (LOW) lane_rot(u.x, u.y, re, im); else plane_rot<0>(u.x, u.y, re, im);
-        }
-        if (L.rot & 2) plane_rot<LOW ? 0 : 1>(u.z, u.w, re, im);
-        if (L.rot & 4) plane_rot<LOW ? 1 : 2>(v.x, v.y, re, im);
-        if (L.rot & 8) plane_rot<LOW ? 2 : 3>(v.z, v.w, re, im);
-      }
+      plane_rots<LOW, LIFT>(L.rot, u, v, re, im);
       c += 2;
     }
     if (L.dk == 2) {
@@ -949,7 +970,8 @@ __device__ __forceinline__ void issue_store(const FusedParams<R>& P, uint32_t sr
 // (shared-memory addresses recomputed per access instead of tabulated), 4 as
 // 3 with every dense 2x2 rounded with dither (complex64, dithered rounding
 // selected for the state), 5 every group a layer program in rotation form, on
-// planes (complex64, 4-qubit groups, blocks of 2^(m - 5) threads)
+// planes (complex64, 4-qubit groups, blocks of 2^(m - 5) threads), 6 as 5 with
+// three shears a rotation (FusedPass::lift)
 template <typename R, int KGF, int MINB, int MODE>
 __global__ void __launch_bounds__(kFThreads, MINB)
     kfused_tma(uint64_t n_blocks, const __grid_constant__ FusedParams<R> P) {
@@ -969,7 +991,7 @@ __global__ void __launch_bounds__(kFThreads, MINB)
   for (int i = threadIdx.x; i < P.glay[P.ngroups]; i += blockDim.x) lsm[i] = P.layers[i];
   // planes: every group's tile of every thread
   uint16_t* tbase = reinterpret_cast<uint16_t*>(lsm + P.glay[P.ngroups]);
-  if constexpr (MODE == 5)
+  if constexpr (MODE >= 5)
     for (int g = 0; g < P.ngroups; ++g) {
       int q = 0;
       for (int i = 0; i < P.m - 5; ++i) q |= ((threadIdx.x >> i) & 1) << P.gtpos[g][i];
@@ -1007,15 +1029,15 @@ __global__ void __launch_bounds__(kFThreads, MINB)
         run_layers<KGF, R, false, true>(
             sm, P.m, P.gbits[g], lsm, P.glay[g], P.glay[g + 1], csm,
             mix32(P.dseed ^ (uint32_t)blk ^ ((uint32_t)(blk >> 32) + (uint32_t)g * 0x85ebca6bu)));
-      else if constexpr (MODE == 5) {
+      else if constexpr (MODE >= 5) {
         ulonglong2* sm4 = reinterpret_cast<ulonglong2*>(sm);
         const uint8_t* gb = P.gbits[g];
         const int base = tbase[g * blockDim.x + threadIdx.x], tile = P.gtpos[g][P.m - 5];
         if (gb[0] == 0)
-          run_planes<true>(sm4, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], base, tile,
+          run_planes<true, MODE == 6>(sm4, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], base, tile,
                            g == 0, g + 1 == P.ngroups);
         else
-          run_planes<false>(sm4, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], base, tile,
+          run_planes<false, MODE == 6>(sm4, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], base, tile,
                             g == 0, g + 1 == P.ngroups);
       } else if (MODE == 3)
         run_layers<KGF, R, false>(sm, P.m, P.gbits[g], lsm, P.glay[g], P.glay[g + 1], csm, 0,
@@ -1619,6 +1641,7 @@ bool build_tma(const TmaGeom& g, void* data, FusedParams<R>* P, CUtensorMap* map
 template <typename R>
 int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>* P, int* nlp,
                 int* ncp, double* drift, bool rotform, bool shear) {
+  const bool lift = shear && pass.lift;  // three shears and an exact diagonal
   struct LayerH {
     int u1 = 0, dtouch = 0;
     int rot = 0, form = 0;  // rotation form: bits with scaled rotations tau[i]
@@ -1637,6 +1660,12 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     return cd{(x.re * y.re + x.im * y.im) / d, (x.im * y.re - x.re * y.im) / d};
   };
   auto scl = [](cd x, double f) { return cd{x.re * f, x.im * f}; };
+  // components within the products' own rounding of 0, 1 or -1 made exact
+  auto snapped = [](cd x) {
+    for (double* v : {&x.re, &x.im})
+      if (std::fabs(*v - std::rint(*v)) < 1e-13) *v = std::rint(*v);
+    return x;
+  };
   // U = diag(a) S diag(b), S = [[1, -tau], [tau, 1]] (form 0, |u00| >= |u01|)
   // or [[tau, -1], [1, tau]] (form 1), tau <= 1 (a ZYZ Euler split:
   // U = e^{i phi} RZ RY RZ with RY = cos [[1, -tan], [tan, 1]]).  False if U
@@ -1714,8 +1743,10 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
         if (!decompose(h.U[t], a, b, &tau, &f)) return false;
         const double tr = (double)(R)tau;
         const double sc = std::sqrt((1.0 + tau * tau) / (1.0 + tr * tr));
-        a[0] = scl(a[0], sc);
-        a[1] = scl(a[1], sc);
+        // lift: the shears keep the norm, so A loses its modulus 1 / sqrt(1 + tau^2)
+        const double am = lift ? std::sqrt(1.0 + tau * tau) : sc;
+        a[0] = scl(a[0], am);
+        a[1] = scl(a[1], am);
         o.tau[t] = tr;
         if (f) o.form |= 1 << t;
         for (int r = 0; r < D; ++r) {
@@ -1764,14 +1795,14 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       cd Dl[32];
       for (int r = 0; r < D; ++r) {
         Dl[r] = o.Dg[r];
-        for (int t = 0; t < k && shear; ++t)  // register of logical index r: r ^ M ^ F
+        for (int t = 0; t < k && shear && !lift; ++t)  // register of logical index r: r ^ M ^ F
           if ((o.rot >> t) & 1 && (((r ^ M ^ F) >> t) & 1))
             Dl[r] = scl(Dl[r], 1.0 + o.tau[t] * o.tau[t]);
         for (int t = 0; t < k; ++t)
           if ((F >> t) & 1) Dl[r] = scl(Dl[r], ((r >> t) & 1) ? 1.0 : -1.0);  // -Z_t
       }
       M ^= F;
-      for (int p = 0; p < D; ++p) o.Dg[p] = Dl[p ^ M];
+      for (int p = 0; p < D; ++p) o.Dg[p] = lift ? snapped(Dl[p ^ M]) : Dl[p ^ M];
       o.form = 0;
     }
     *xmask = M;
@@ -1895,7 +1926,11 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       if (h.rot) {  // tau of bit i in slot i (0 where bit i has no rotation)
         for (int i = 0; i < 4; ++i) {
           const double t = ((h.rot >> i) & 1) ? h.tau[i] : 0.0;
-          if (shear) {
+          if (lift) {  // tan(angle / 2) and sin(angle) from t = tan(angle)
+            const double h = std::sqrt(1.0 + t * t);
+            P->coef[nc++] = (R)(-t / (1.0 + h));
+            P->coef[nc++] = (R)(t / h);
+          } else if (shear) {
             P->coef[nc++] = (R)-t;
             P->coef[nc++] = (R)(t / (1.0 + t * t));
           } else {
@@ -2084,7 +2119,7 @@ struct PassKernels {
   template <int KG, int MINB>
   static Tma pick(int mode) {
     if constexpr (sizeof(R) == 4 && KG == 4)
-      if (mode == 5) return kfused_tma<R, KG, MINB, 5>;
+      if (mode >= 5) return mode == 5 ? kfused_tma<R, KG, MINB, 5> : kfused_tma<R, KG, MINB, 6>;
     if constexpr (sizeof(R) == 4)
       if (mode == 4) return kfused_tma<R, KG, MINB, 4>;
     return mode == 3   ? kfused_tma<R, KG, MINB, 3>
@@ -2149,7 +2184,7 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
   const bool dither_all = sizeof(R) == 4 && rc && rc->mode == SV_ROUNDING_DITHERED;
   // on planes where every group allows it
   const bool want_planes = tma && sizeof(R) == 4 && kg == 4 && !dither_all &&
-                           (int)pass.S.size() >= kPlaneQubits;
+                           (int)pass.S.size() >= (pass.lift ? kLiftQubits : kPlaneQubits);
   bool built = build_params(pass, order, &P, true, drift, !dither_all, want_planes);
   bool planes = want_planes && built;
   for (int g = 0; g < P.ngroups; ++g) planes = planes && P.gkind[g] == 2;
@@ -2181,13 +2216,13 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
   if (tma) {
     int nlay = 0;
     for (int g = 0; g < P.ngroups; ++g) nlay += P.gkind[g] != 0;
-    const int mode = planes ? 5 : nlay == 0 ? 0 : nlay == P.ngroups ? (dither_all ? 4 : 3) : 1;
+    const int mode = planes ? (pass.lift ? 6 : 5) : nlay == 0 ? 0 : nlay == P.ngroups ? (dither_all ? 4 : 3) : 1;
     typename PassKernels<R>::Tma kern = PassKernels<R>::tma(kg, mode);
-    const int threads = mode == 5 ? 1 << (P.m - 5) : kFThreads;
-    if (mode == 5) plane_threads(&P);
+    const int threads = mode >= 5 ? 1 << (P.m - 5) : kFThreads;
+    if (mode >= 5) plane_threads(&P);
     const size_t smem = (amp << P.m) + 1024 + sizeof(R) * (size_t)((P.ncoef + 1) & ~1) +
                         sizeof(FLayerDev) * (size_t)P.glay[P.ngroups] +
-                        (mode == 5 ? sizeof(uint16_t) * (size_t)threads * P.ngroups : 0);
+                        (mode >= 5 ? sizeof(uint16_t) * (size_t)threads * P.ngroups : 0);
     // resident blocks per SM for this kernel and shared-memory size
     static std::map<std::pair<const void*, size_t>, int> resident;
     int& res = resident[{reinterpret_cast<const void*>(kern), smem}];

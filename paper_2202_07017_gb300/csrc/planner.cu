@@ -443,6 +443,23 @@ bool plan_fusion(const sv_circuit* c, const double* theta, const FusionConfig& c
   return true;
 }
 
+void plan_fusion_1q(int n, const std::vector<Gate1q>& gates, const FusionConfig& cfg,
+                    std::vector<FusionItem>* out) {
+  std::vector<FGate> F;
+  std::vector<int> last(64, -1);
+  for (size_t i = 0; i < gates.size(); ++i) {
+    FGate f;
+    f.type = FG_1Q;
+    f.t = gates[i].bit;
+    f.qmask = uint64_t(1) << f.t;
+    f.orig = (int)i;
+    f.origs.push_back((int)i);
+    for (int e = 0; e < 4; ++e) f.m[e] = gates[i].m[e];
+    push_fgate(std::move(f), &last, &F);
+  }
+  form_passes(F, n, cfg, out);
+}
+
 bool plan_fusion_reverse(const sv_circuit* c, const double* theta, int lo, int hi,
                          const std::vector<int>& slot_of, const FusionConfig& cfg,
                          std::vector<FusionItem>* out) {

@@ -264,6 +264,88 @@ static sv_status unapply_circuit_gate(sv_state s, void* psi, void* lam, const sv
   return st;
 }
 
+// Gate i of c is a rotation by a diagonal Pauli string.
+static bool diagonal_pauli(const sv_circuit* c, int i) {
+  const sv_gate& g = c->gates[i];
+  if (g.kind != SV_GATE_PAULI) return false;
+  for (int j = 0; j < g.n_tar; ++j)
+    if (((g.paulis >> (2 * j)) & 3) != 3) return false;
+  return true;
+}
+
+// End of the run of unfused diagonal rotations that starts at plan item i (i
+// itself if it is something else).  They commute and are applied together.
+static size_t diagonal_run_end(const std::vector<FusionItem>& plan, size_t i,
+                               const sv_circuit* c) {
+  while (i < plan.size() && !plan[i].is_pass && diagonal_pauli(c, plan[i].gate)) ++i;
+  return i;
+}
+
+static double gate_angle(const sv_gate& g, const double* theta) {
+  return g.param >= 0 ? theta[g.param] : g.angle;
+}
+
+// The plan's items in order on the state.
+static sv_status apply_plan(sv_state s, const sv_circuit* c, const double* theta,
+                            const std::vector<FusionItem>& plan) {
+  for (size_t i = 0; i < plan.size();) {
+    const size_t j = diagonal_run_end(plan, i, c);
+    sv_status st;
+    if (j > i) {
+      std::vector<uint64_t> zm;
+      std::vector<double> a;
+      for (; i < j; ++i) {
+        const sv_gate& g = c->gates[plan[i].gate];
+        uint64_t xm, z;
+        pauli_masks(s->n, g, &xm, &z);
+        zm.push_back(z);
+        a.push_back(0.5 * gate_angle(g, theta));
+      }
+      st = launch_diag_rotations(s->data, s->dt, s->n, s->stream, zm, a);
+    } else {
+      st = plan[i].is_pass
+               ? launch_fused_pass(s->data, s->dt, s->n, s->stream, plan[i].pass, &s->rc)
+               : apply_circuit_gate(s, c, plan[i].gate, theta);
+      ++i;
+    }
+    if (st) return st;
+  }
+  return SV_OK;
+}
+
+// The reverse plan's items in order on (psi, lam); gradients into
+// partials[slot * pstride + block].
+static sv_status unapply_plan(sv_state s, void* psi, void* lam, const sv_circuit* c,
+                              const double* theta, const std::vector<FusionItem>& plan,
+                              double* partials, int pstride) {
+  for (size_t i = 0; i < plan.size();) {
+    const size_t j = diagonal_run_end(plan, i, c);
+    std::vector<DiagGate> run;
+    for (size_t k = i; k < j; ++k) {
+      const sv_gate& g = c->gates[plan[k].gate];
+      uint64_t xm, z;
+      pauli_masks(s->n, g, &xm, &z);
+      const double a = gate_angle(g, theta);
+      if (!adjoint_diag_ok(s->n, a)) break;
+      run.push_back({z, a, plan[k].slot, g.param});
+    }
+    sv_status st;
+    if (!run.empty()) {
+      st = launch_adjoint_diag(psi, lam, s->dt, s->n, s->stream, run, partials, pstride);
+      i += run.size();
+    } else {
+      const FusionItem& it = plan[i++];
+      st = it.is_pass ? launch_fused_reverse_pass(psi, lam, s->dt, s->n, s->stream, it.pass,
+                                                  partials, pstride)
+                      : unapply_circuit_gate(s, psi, lam, c, it.gate, theta,
+                                             it.slot >= 0 ? partials + (size_t)it.slot * pstride
+                                                          : nullptr);
+    }
+    if (st) return st;
+  }
+  return SV_OK;
+}
+
 sv_status ensure_partials(sv_state s, size_t doubles) {
   if (s->partials_cap >= doubles) return SV_OK;
   if (s->partials) cudaFree(s->partials);
@@ -610,16 +692,7 @@ sv_status sv_apply_circuit(sv_state s, const sv_circuit* c, const double* theta,
   if (fuse_k > 0) {
     std::vector<FusionItem> plan;
     if (!plan_fusion(c, theta, fusion_config(s->n, s->dt, fuse_k), &plan)) return SV_ERR_INVALID;
-    for (const FusionItem& it : plan) {
-      sv_status st;
-      if (it.is_pass) {
-        st = launch_fused_pass(s->data, s->dt, s->n, s->stream, it.pass, &s->rc);
-      } else {
-        st = apply_circuit_gate(s, c, it.gate, theta);
-      }
-      if (st != SV_OK) return st;
-    }
-    return SV_OK;
+    return apply_plan(s, c, theta, plan);
   }
   for (int i = 0; i < c->n_gates; ++i) {
     sv_status st = apply_circuit_gate(s, c, i, theta);
@@ -1049,15 +1122,8 @@ sv_status sv_grad_fused(sv_state s, const sv_circuit* c, const double* theta,
     SV_CUDA_TRY(cudaMemsetAsync(s->partials, 0, sizeof(double) * (size_t)n_pg * G, s->stream));
   double* slots = s->partials + (size_t)n_pg * G;
   for (size_t i = bounds.size() - 1; i-- > 0;) {
-    for (const FusionItem& it : plans[i]) {
-      if (it.is_pass) {
-        st = launch_fused_reverse_pass(psi, lam, s->dt, s->n, s->stream, it.pass, s->partials, G);
-      } else {
-        st = unapply_circuit_gate(s, psi, lam, c, it.gate, theta,
-                                  it.slot >= 0 ? s->partials + (size_t)it.slot * G : nullptr);
-      }
-      if (st) return st;
-    }
+    st = unapply_plan(s, psi, lam, c, theta, plans[i], s->partials, G);
+    if (st) return st;
     const int k = ckpt_at(bounds[i]);
     if (k >= 0)
       SV_CUDA_TRY(cudaMemcpyAsync(psi, s->ckpt[k], s->bytes(), cudaMemcpyDeviceToDevice,

@@ -227,6 +227,7 @@ struct FusedPass {
   std::vector<int> S;        // staged bit positions, ascending; S[0..L) = 0..L-1
   int L = 0;
   std::vector<FGate> gates;  // the pass's gates (bits are global)
+  bool lift = false;         // X and Y rotations only, applied over and over: no rounded scale
   std::vector<FusedGroup> groups;
 };
 
@@ -254,6 +255,14 @@ FusionConfig fusion_config_reverse(int n, sv_dtype dt, int fuse_k);
 // set) if a matrix cannot be built.
 bool plan_fusion(const sv_circuit* c, const double* theta, const FusionConfig& cfg,
                  std::vector<FusionItem>* out);
+// Plan of uncontrolled 1-qubit gates given by their bits (gates on one bit
+// multiply); every item is a pass.
+struct Gate1q {
+  int bit;
+  cd m[4];
+};
+void plan_fusion_1q(int n, const std::vector<Gate1q>& gates, const FusionConfig& cfg,
+                    std::vector<FusionItem>* out);
 // Plan of the reverse sweep over gates [lo, hi): gates hi-1 .. lo as their
 // adjoints, each parameterised gate preceded by its FG_GRAD; slot_of[i] is
 // the gradient slot of circuit gate i (or -1).  Unfused items carry the
@@ -283,6 +292,22 @@ unsigned take_fused_status();
 // of sv_pauli_sum); rc as in launch_gate.
 sv_status launch_pauli_rotation(void* data, sv_dtype dt, int n, cudaStream_t st, uint64_t xm,
                                 uint64_t zm, double a, RoundCtx* rc = nullptr);
+// psi <- prod_k exp(-i a_k P_k) psi for diagonal strings P_k (z masks zm[k]).
+sv_status launch_diag_rotations(void* data, sv_dtype dt, int n, cudaStream_t st,
+                                const std::vector<uint64_t>& zm, const std::vector<double>& a);
+// Reverse-sweep step of a run of diagonal rotations exp(-i theta P / 2), every
+// one with adjoint_diag_ok(n, theta): un-applies the run on psi and lam and
+// writes Im<lam|P|psi> to partials[slot * pstride + block], the gates of one
+// parameter added up in the slot of one of them (the others' slots are left
+// alone; slot < 0: no gradient).
+struct DiagGate {
+  uint64_t zm;
+  double theta;
+  int slot, param;
+};
+bool adjoint_diag_ok(int n, double theta);
+sv_status launch_adjoint_diag(void* psi, void* lam, sv_dtype dt, int n, cudaStream_t st,
+                              const std::vector<DiagGate>& g, double* partials, int pstride);
 // Reverse-sweep step of U = exp(-i theta P / 2): Im<lam|P|psi> into
 // partials[0..nparts) (nparts = the 1-qubit adjoint's fixed grid), then
 // psi, lam <- U^dagger psi, U^dagger lam.
