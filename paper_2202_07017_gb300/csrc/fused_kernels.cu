@@ -63,8 +63,10 @@ struct FOpDev {
 struct FLayerDev {
   uint8_t u1, dk;
   uint16_t off;
-  uint8_t rot, pad8;
-  uint16_t pad;
+  uint8_t rot;
+  uint8_t grad;  // reverse sweeps on planes: group bits evaluated before the rotations,
+  uint8_t ev;    // their evaluations' numbers from ev on, in bit order
+  uint8_t pad;
 };
 
 template <typename R>
@@ -85,6 +87,11 @@ struct FusedParams {
   int ngroups;
   int ngrad;            // reverse sweeps: gradient operations of the pass
   int gslot[kFMaxOps];  // their gradient slots
+  // reverse sweeps on planes: evaluations of the pass, and per gradient its
+  // evaluation and its generator's X, Y and Z parts on the registers
+  int nev;
+  uint16_t gev[sizeof(R) == 4 ? kFMaxOps : 1];
+  float ggen[sizeof(R) == 4 ? kFMaxOps : 1][3];
   uint8_t gk[kFMaxGroups];
   uint8_t gbits[kFMaxGroups][5];
   uint16_t gop[kFMaxGroups + 1];
@@ -1315,6 +1322,238 @@ __device__ __forceinline__ void store_pair(uint32_t s1, uint32_t s2, const CUten
   tma_store<RANK>(m2, c, s2);
 }
 
+// ---- reverse sweep on planes ---------------------------------------------------------
+// The layer programs of run_planes on psi and lambda together: 16 chunks of
+// each per thread, one coefficient read for both, blocks of 2^(m - 5) threads.
+// What bounded the sweep was the instruction count (dense 2x2 un-applies at 16
+// FMAs per amplitude and gate, sign flips and gradients dispatched per gate); as
+// layers the un-applies are shears with one diagonal a layer, and a layer first
+// evaluates every bit that has gradients there.  Random layered circuit, n = 26,
+// depth 12: 1927 -> 1066 us a pass (HBM read and write of both states: 320 us);
+// HEA n = 20: 39 -> 23 us.  Three blocks of 4 warps a SM at 168 registers (148
+// bytes spilled); two blocks without spills: 1143 us.
+//
+// lambda is held conjugated, so that an evaluation has no negations: with c =
+// conj(lambda), the sums over the pairs (p, q) of a bit (clear, set)
+//   X = Im(c_p psi_q + c_q psi_p), Y = Re(c_q psi_p - c_p psi_q),
+//   Z = Im(c_p psi_p - c_q psi_q)
+// give Im<lambda|G|psi> of every traceless Hermitian G on the bit, so all the
+// gradients that share the place cost one evaluation; each takes its own
+// combination once, at the end of the block.
+//
+// The layer's registers at that point are B psi and B lambda, B the next
+// rotations' input phases, possibly with the bit's values exchanged (see
+// rotation_form): the host carries the generators over.
+constexpr int kAdjPlaneThreads = 128;
+constexpr int kAdjPlaneQubits = 10;
+
+// X, Y, Z sums of bit B of the tile index
+template <int B>
+__device__ __forceinline__ void plane_sums(const Pair (&pr)[16], const Pair (&pi)[16],
+                                           const Pair (&cr)[16], const Pair (&ci)[16],
+                                           float (&v)[4]) {
+  Pair x = 0, y0 = 0, y1 = 0, z0 = 0, z1 = 0;
+#pragma unroll
+  for (int p = 0; p < 16; ++p) {
+    if (p & (1 << B)) continue;
+    const int q = p | (1 << B);
+    pair_add(x, cr[p], pi[q]);
+    pair_add(y0, cr[q], pr[p]);
+    pair_add(y1, cr[p], pr[q]);
+    pair_add(z0, cr[p], pi[p]);
+    pair_add(z1, cr[q], pi[q]);
+    pair_add(x, ci[p], pr[q]);
+    pair_add(y0, ci[p], pi[q]);
+    pair_add(y1, ci[q], pi[p]);
+    pair_add(z0, ci[p], pr[p]);
+    pair_add(z1, ci[q], pr[q]);
+    pair_add(x, cr[q], pi[p]);
+    pair_add(x, ci[q], pr[p]);
+  }
+  const float2 xs = lanes_of(x), ya = lanes_of(y0), yb = lanes_of(y1), za = lanes_of(z0),
+               zb = lanes_of(z1);
+  v[0] = xs.x + xs.y;
+  v[1] = (ya.x - yb.x) + (ya.y - yb.y);
+  v[2] = (za.x - zb.x) + (za.y - zb.y);
+  v[3] = 0.f;
+}
+
+// the same for bit 0: p and q are the lanes of every pair
+__device__ __forceinline__ void lane_sums(const Pair (&pr)[16], const Pair (&pi)[16],
+                                          const Pair (&cr)[16], const Pair (&ci)[16],
+                                          float (&v)[4]) {
+  float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f;
+  Pair z = 0;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const float2 a = lanes_of(pr[r]), b = lanes_of(pi[r]), c = lanes_of(cr[r]), d = lanes_of(ci[r]);
+    x0 = fmaf(c.x, b.y, x0);
+    x1 = fmaf(c.y, b.x, x1);
+    y0 = fmaf(c.y, a.x, y0);
+    y1 = fmaf(c.x, a.y, y1);
+    pair_add(z, cr[r], pi[r]);
+    x0 = fmaf(d.x, a.y, x0);
+    x1 = fmaf(d.y, a.x, x1);
+    y0 = fmaf(d.x, b.y, y0);
+    y1 = fmaf(d.y, b.x, y1);
+    pair_add(z, ci[r], pr[r]);
+  }
+  const float2 zs = lanes_of(z);
+  v[0] = x0 + x1;
+  v[1] = y0 - y1;
+  v[2] = zs.x - zs.y;
+  v[3] = 0.f;
+}
+
+// (re0, im0), (re1, im1) <-> (re0, re1), (im0, im1)
+__device__ __forceinline__ void chunk_flip(Pair& x, Pair& y) {
+  const float2 a = lanes_of(x), b = lanes_of(y);
+  x = pair_of(a.x, b.x);
+  y = pair_of(a.y, b.y);
+}
+__device__ __forceinline__ Pair pair_neg(Pair p) { return p ^ 0x8000000080000000ull; }
+
+// One group over both slices (see run_planes); gw: this warp's evaluation sums.
+template <bool LOW>
+__device__ __forceinline__ void run_planes_adj(ulonglong2* smp, ulonglong2* sml, const uint8_t* gb,
+                                               const FLayerDev* lay, int l0, int l1,
+                                               const float* coef, int xm, int base0, int tile,
+                                               bool first, bool last, KahanAcc<float>* gw) {
+  constexpr int NB = LOW ? 3 : 4;
+  int sw[NB], base[LOW ? 2 : 1];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) sw[i] = chunk_swz(1 << (gb[LOW ? i + 1 : i] - 1));
+  base[0] = base0;
+  if constexpr (LOW) base[1] = base0 ^ chunk_swz(1 << tile);
+  auto slot = [&](int r) {
+    int o = LOW ? base[r >> 3] : base[0];
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if ((r >> i) & 1) o ^= sw[i];
+    return o;
+  };
+  Pair pr[16], pi[16], cr[16], ci[16];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const ulonglong2 v = smp[slot(r)], w = sml[slot(r)];
+    pr[r] = v.x;
+    pi[r] = v.y;
+    cr[r] = w.x;
+    ci[r] = w.y;
+  }
+  if (first) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      chunk_flip(pr[r], pi[r]);
+      chunk_flip(cr[r], ci[r]);
+      ci[r] = pair_neg(ci[r]);
+    }
+  }
+  const int lane = threadIdx.x & 31;
+  for (int l = l0; l < l1; ++l) {
+    const FLayerDev L = lay[l];
+    const float4* c = reinterpret_cast<const float4*>(coef + L.off);
+    if (L.grad) {
+      KahanAcc<float>* g = gw + 3 * L.ev;
+      auto add = [&](const float (&v)[4]) {
+        const float w = warp_sum4<float>(v, lane);
+        if ((lane & 7) == 0 && lane < 24) kahan_add(g[lane >> 3], w);
+        g += 3;
+      };
+      float v[4];
+      if (L.grad & 1) {
+        if constexpr (LOW)
+          lane_sums(pr, pi, cr, ci, v);
+        else
+          plane_sums<0>(pr, pi, cr, ci, v);
+        add(v);
+      }
+      if (L.grad & 2) {
+        plane_sums<LOW ? 0 : 1>(pr, pi, cr, ci, v);
+        add(v);
+      }
+      if (L.grad & 4) {
+        plane_sums<LOW ? 1 : 2>(pr, pi, cr, ci, v);
+        add(v);
+      }
+      if (L.grad & 8) {
+        plane_sums<LOW ? 2 : 3>(pr, pi, cr, ci, v);
+        add(v);
+      }
+    }
+    if (L.rot) {
+      const float4 u = c[0], v = c[1];
+      plane_rots<LOW, false>(L.rot, u, v, pr, pi);
+      plane_rots<LOW, false>(L.rot, u, v, cr, ci);
+      c += 2;
+    }
+    if (L.dk == 2) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float4 d = c[e];
+        if constexpr (LOW) {
+          const Pair dr = pair_of(d.x, d.y), di = pair_of(d.z, d.w), dn = pair_of(-d.z, -d.w);
+          plane_mul(dr, di, dn, pr[e], pi[e]);
+          plane_mul(dr, di, dn, pr[8 + e], pi[8 + e]);
+          plane_mul(dr, dn, di, cr[e], ci[e]);
+          plane_mul(dr, dn, di, cr[8 + e], ci[8 + e]);
+        } else {
+          plane_mul(pair_both(d.x), pair_both(d.y), pair_both(-d.y), pr[2 * e], pi[2 * e]);
+          plane_mul(pair_both(d.x), pair_both(-d.y), pair_both(d.y), cr[2 * e], ci[2 * e]);
+          plane_mul(pair_both(d.z), pair_both(d.w), pair_both(-d.w), pr[2 * e + 1], pi[2 * e + 1]);
+          plane_mul(pair_both(d.z), pair_both(-d.w), pair_both(d.w), cr[2 * e + 1], ci[2 * e + 1]);
+        }
+      }
+    } else if (L.dk == 1) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float4 d = c[e];
+        const float dd[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int r = LOW ? 2 * e + (j & 1) + 8 * (j >> 1) : 4 * e + j;
+          const Pair f = LOW ? pair_of(dd[2 * (j & 1)], dd[2 * (j & 1) + 1]) : pair_both(dd[j]);
+          pr[r] = pair_mul(f, pr[r]);
+          pi[r] = pair_mul(f, pi[r]);
+          cr[r] = pair_mul(f, cr[r]);
+          ci[r] = pair_mul(f, ci[r]);
+        }
+      }
+    }
+  }
+  int xoff = 0;
+#pragma unroll
+  for (int i = 0; i < NB; ++i)
+    if ((xm >> (LOW ? i + 1 : i)) & 1) xoff ^= sw[i];
+#pragma unroll
+  for (int u = 0; u < (LOW ? 2 : 1); ++u) {
+    base[u] ^= xoff;
+    asm volatile("" : "+r"(base[u]));
+  }
+  if (LOW && (xm & 1)) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      pr[r] = pair_swap(pr[r]);
+      pi[r] = pair_swap(pi[r]);
+      cr[r] = pair_swap(cr[r]);
+      ci[r] = pair_swap(ci[r]);
+    }
+  }
+  if (last) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      ci[r] = pair_neg(ci[r]);
+      chunk_flip(pr[r], pi[r]);
+      chunk_flip(cr[r], ci[r]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    smp[slot(r)] = make_ulonglong2(pr[r], pi[r]);
+    sml[slot(r)] = make_ulonglong2(cr[r], ci[r]);
+  }
+}
+
 // Shared memory of a reverse-sweep block after its two slices: the per-warp
 // gradient accumulators, then the operation list, then the gradient
 // generators (each part 16-byte aligned).
@@ -1422,6 +1661,121 @@ __global__ void __launch_bounds__(kFThreads, MINB)
     for (int w = 0; w < nw; ++w) {
       const KahanAcc<R> a = gacc[w * P.ngrad + j];
       t += (double)a.s - (double)a.c;
+    }
+    partials[(size_t)P.gslot[j] * pstride + blockIdx.x] = t;
+  }
+}
+
+
+// Shared memory of a block on planes after its two slices: the per-warp
+// evaluation sums, the coefficients, the layer table, the threads' tiles.
+__host__ __device__ constexpr size_t adj_plane_coef(int nev, int warps) {
+  return (sizeof(KahanAcc<float>) * 3 * (size_t)nev * warps + 15) & ~size_t(15);
+}
+__host__ __device__ constexpr size_t adj_plane_tail(int nev, int ncoef, int nlay, int ngroups,
+                                                    int threads) {
+  return adj_plane_coef(nev, threads / 32) + sizeof(float) * (size_t)((ncoef + 1) & ~1) +
+         sizeof(FLayerDev) * (size_t)nlay + sizeof(uint16_t) * (size_t)ngroups * threads;
+}
+
+__global__ void __launch_bounds__(kAdjPlaneThreads, 3)
+    kfused_adj_planes(uint64_t n_blocks, const __grid_constant__ FusedParams<float> P,
+                      double* __restrict__ partials, int pstride) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bar;
+  const uint32_t raw = smem_addr(smem_raw);
+  const uint32_t sbuf = (raw + 1023u) & ~1023u;
+  const uint32_t sbuf2 = sbuf + P.slice_bytes;  // slice bytes are a multiple of 1024
+  ulonglong2* smp = reinterpret_cast<ulonglong2*>(smem_raw + (sbuf - raw));
+  ulonglong2* sml = reinterpret_cast<ulonglong2*>(smem_raw + (sbuf2 - raw));
+  unsigned char* tail = smem_raw + (sbuf2 - raw) + P.slice_bytes;
+  KahanAcc<float>* gacc = reinterpret_cast<KahanAcc<float>*>(tail);
+  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* csm = reinterpret_cast<float*>(tail + adj_plane_coef(P.nev, nw));
+  FLayerDev* lsm = reinterpret_cast<FLayerDev*>(csm + ((P.ncoef + 1) & ~1));
+  const int nlay = P.glay[P.ngroups];
+  uint16_t* tbase = reinterpret_cast<uint16_t*>(lsm + nlay);
+  for (int i = threadIdx.x; i < nw * 3 * P.nev; i += blockDim.x) gacc[i] = KahanAcc<float>{0, 0};
+  for (int i = threadIdx.x; i < P.ncoef; i += blockDim.x) csm[i] = P.coef[i];
+  for (int i = threadIdx.x; i < nlay; i += blockDim.x) lsm[i] = P.layers[i];
+  for (int g = 0; g < P.ngroups; ++g) {
+    int q = 0;
+    for (int i = 0; i < P.m - 5; ++i) q |= ((threadIdx.x >> i) & 1) << P.gtpos[g][i];
+    tbase[g * blockDim.x + threadIdx.x] = (uint16_t)chunk_swz(q);
+  }
+  const uint32_t barp = smem_addr(&bar);
+  if (threadIdx.x == 0) {
+    mbar_init(barp, 1);
+    fence_proxy_async_smem();
+  }
+  grid_dependency_wait();  // the parameters are the only input so far
+  __syncthreads();
+  uint32_t parity = 0;
+  for (uint64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
+    const uint64_t base = insert_zeros(blk, P.blk);
+    if (threadIdx.x < 32) {
+      bulk_wait_read_all();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_expect_tx(barp, 2 * P.slice_bytes);
+      __syncwarp();
+      for (int k = lane; k < P.ncopies; k += 32) {
+        int c[5];
+        box_coords(P, base, k, c);
+        const uint32_t off = (uint32_t)k * P.box_bytes;
+        switch (P.rank) {
+          case 2: load_pair<2>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c, barp); break;
+          case 3: load_pair<3>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c, barp); break;
+          case 4: load_pair<4>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c, barp); break;
+          default: load_pair<5>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c, barp); break;
+        }
+      }
+      prefetch_next(P, blk, n_blocks, lane, true);
+    }
+    const bool ok = mbar_wait_bounded(barp, parity);
+    parity ^= 1;
+    if (__syncthreads_or(!ok)) {
+      if (threadIdx.x == 0) atomicOr(&g_fused_status, kWaitTimeout);
+      break;
+    }
+    for (int g = 0; g < P.ngroups; ++g) {
+      const uint8_t* gb = P.gbits[g];
+      const int tb = tbase[g * blockDim.x + threadIdx.x], tile = P.gtpos[g][P.m - 5];
+      if (gb[0] == 0)
+        run_planes_adj<true>(smp, sml, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], tb, tile,
+                             g == 0, g + 1 == P.ngroups, gacc + warp * 3 * P.nev);
+      else
+        run_planes_adj<false>(smp, sml, gb, lsm, P.glay[g], P.glay[g + 1], csm, P.gxm[g], tb, tile,
+                              g == 0, g + 1 == P.ngroups, gacc + warp * 3 * P.nev);
+      if (g + 1 < P.ngroups) __syncthreads();
+    }
+    fence_proxy_async_smem();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      for (int k = lane; k < P.ncopies; k += 32) {
+        int c[5];
+        box_coords(P, base, k, c);
+        const uint32_t off = (uint32_t)k * P.box_bytes;
+        switch (P.rank) {
+          case 2: store_pair<2>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c); break;
+          case 3: store_pair<3>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c); break;
+          case 4: store_pair<4>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c); break;
+          default: store_pair<5>(sbuf + off, sbuf2 + off, &P.tmap, &P.tmap2, c); break;
+        }
+      }
+      bulk_commit();
+    }
+  }
+  if (threadIdx.x < 32) bulk_wait_all();
+  __syncthreads();
+  for (int j = threadIdx.x; j < P.ngrad; j += blockDim.x) {
+    double t = 0.0;
+    for (int i = 0; i < 3; ++i) {
+      double e = 0.0;
+      for (int w = 0; w < nw; ++w) {
+        const KahanAcc<float> a = gacc[(w * P.nev + P.gev[j]) * 3 + i];
+        e += (double)a.s - (double)a.c;
+      }
+      t += (double)P.ggen[j][i] * e;
     }
     partials[(size_t)P.gslot[j] * pstride + blockIdx.x] = t;
   }
@@ -1626,6 +1980,13 @@ bool build_tma(const TmaGeom& g, void* data, FusedParams<R>* P, CUtensorMap* map
   return true;
 }
 
+// Generator i of an FG_GRAD: (a, d, re b, im b) of [[a, b], [conj b, d]].
+void gradient_generator(const FGate& f, int i, double* g) {
+  static const double kPauli[4][4] = {{0, 0, 0, 0}, {0, 0, 1, 0}, {0, 0, 0, -1}, {1, -1, 0, 0}};
+  const double m[4] = {f.m[0].re, f.m[3].re, f.m[1].re, f.m[1].im};
+  for (int e = 0; e < 4; ++e) g[e] = f.ng > 1 ? f.gen[i][e] : f.pauli ? kPauli[f.pauli][e] : m[e];
+}
+
 // Rewrites group g, if its gates are uncontrolled 1-qubit gates and diagonal
 // gates (phases on subspaces, controlled diagonal 1-qubit gates), as a layer
 // program: a 1-qubit gate joins the open layer unless the layer's diagonal
@@ -1635,24 +1996,30 @@ bool build_tma(const TmaGeom& g, void* data, FusedParams<R>* P, CUtensorMap* map
 // state's error feedback (drift; the layers' 2x2s and diagonals act on the
 // whole state).  With rotform every dense 2x2 is split into a scaled real
 // rotation between diagonals (see rotation_form below); with shear too the
-// rotations are shears (see run_planes).  Returns 0 (and
+// rotations are shears (see run_planes).  events (reverse sweeps on planes):
+// gradients on uncontrolled bits become evaluations, counted there, and entries
+// of gslot, gev and ggen.  Returns 0 (and
 // leaves nl, nc) if the group keeps its gate list, 2 for a layer program in
 // rotation form throughout, 1 for one with dense 2x2s.
 template <typename R>
 int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>* P, int* nlp,
-                int* ncp, double* drift, bool rotform, bool shear) {
+                int* ncp, double* drift, bool rotform, bool shear, int* events = nullptr) {
   const bool lift = shear && pass.lift;  // three shears and an exact diagonal
   struct LayerH {
     int u1 = 0, dtouch = 0;
     int rot = 0, form = 0;  // rotation form: bits with scaled rotations tau[i]
+    int grad = 0;           // reverse sweeps: bits evaluated before the rotations
+    int flip = 0;           // rotation form: register relabelling in force before the rotations
+    cd ph[5];               // rotation form: input phase ratio b0 / b1 of bit i's rotation
     double tau[5] = {0, 0, 0, 0, 0};
     double msq = 1.0;  // exact mean squared modulus of Dg
     cd U[5][4];
     cd Dg[32];
     LayerH() {
       for (int r = 0; r < 32; ++r) Dg[r] = {1.0, 0.0};
+      for (int i = 0; i < 5; ++i) ph[i] = {1.0, 0.0};
     }
-    bool empty() const { return !u1 && !dtouch; }
+    bool empty() const { return !u1 && !dtouch && !grad; }
   };
   auto cmul = [](cd a, cd b) { return cd{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; };
   auto cdiv = [](cd x, cd y) {
@@ -1735,6 +2102,7 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       const LayerH& h = in[l];
       LayerH& o = mid[l];
       o.rot = h.u1;
+      o.grad = h.grad;
       for (int t = 0; t < k; ++t) {
         if (!((h.u1 >> t) & 1)) continue;
         cd a[2], b[2];
@@ -1743,11 +2111,12 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
         if (!decompose(h.U[t], a, b, &tau, &f)) return false;
         const double tr = (double)(R)tau;
         const double sc = std::sqrt((1.0 + tau * tau) / (1.0 + tr * tr));
-        // lift: the shears keep the norm, so A loses its modulus 1 / sqrt(1 + tau^2)
-        const double am = lift ? std::sqrt(1.0 + tau * tau) : sc;
+        // shears: A's modulus 1 / sqrt(1 + tau^2) goes into their diagonal (lift: away)
+        const double am = shear ? std::sqrt(1.0 + tau * tau) : sc;
         a[0] = scl(a[0], am);
         a[1] = scl(a[1], am);
         o.tau[t] = tr;
+        o.ph[t] = cdiv(b[0], b[1]);
         if (f) o.form |= 1 << t;
         for (int r = 0; r < D; ++r) {
           A[l][r] = cmul(A[l][r], a[(r >> t) & 1]);
@@ -1776,9 +2145,12 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       o.msq = msq / D;
       out->push_back(o);
     }
-    // Shears: S(t) = diag(1, 1 + t^2) [[1, 0], [t / (1 + t^2), 1]] [[1, -t], [0, 1]];
-    // the diagonal, as diag(c, 1/c) / c with c = 1 / sqrt(1 + t^2), joins the
-    // layer's (on the registers, so after the relabelling below).
+    // Shears p += a q, q += b p with a = -t and b = t / (1 + t^2) rounded: for any
+    // a and b, diag(d0, d1) [[1, 0], [b, 1]] [[1, a], [0, 1]] diag(1, r) is a
+    // rotation with d0^2 = 1 + a b, d1^2 = -a / b, r^2 = -b / (a (1 + a b)) (r = 1 but
+    // for b's rounding).  d joins the layer's diagonal and r the one before (none
+    // before a group's first layer if that has no input phases), on the
+    // registers, so past the relabelling below.
     // One rotation shape on the device: [[t, -1], [1, t]] = X Z S(-t) with
     // S(t) = [[1, -t], [t, 1]].  X on a bit relabels the registers instead of
     // moving them (mask M: register p holds logical index p ^ M; X S(t) X =
@@ -1786,18 +2158,38 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     // after its rotations (other bits commute), and X Z = -Z X puts -Z into
     // the layer's diagonal, which is then read at p ^ M.  The group's stores
     // undo M.
+    auto shear_scales = [](double t, double* d0, double* d1, double* r) {
+      *d0 = *d1 = *r = 1.0;
+      const double a = (double)(R)-t, b = (double)(R)(t / (1.0 + t * t));
+      if (a == 0.0 || b == 0.0) return;
+      *d0 = std::sqrt(1.0 + a * b);
+      *d1 = std::sqrt(-a / b);
+      *r = std::sqrt(-b / (a * (1.0 + a * b)));
+    };
     int M = 0;
-    for (LayerH& o : *out) {
+    for (size_t li = 0; li < out->size(); ++li) {
+      LayerH& o = (*out)[li];
+      const LayerH* next = li + 1 < out->size() ? &(*out)[li + 1] : nullptr;
       const int F = o.form;
+      o.flip = M;
       for (int t = 0; t < k; ++t)
         if ((o.rot >> t) & 1)
           o.tau[t] *= (((F ^ M) >> t) & 1) ? -1.0 : 1.0;
       cd Dl[32];
       for (int r = 0; r < D; ++r) {
         Dl[r] = o.Dg[r];
-        for (int t = 0; t < k && shear && !lift; ++t)  // register of logical index r: r ^ M ^ F
-          if ((o.rot >> t) & 1 && (((r ^ M ^ F) >> t) & 1))
-            Dl[r] = scl(Dl[r], 1.0 + o.tau[t] * o.tau[t]);
+        for (int t = 0; t < k && shear && !lift; ++t) {  // register of logical index r: r ^ M ^ F
+          const bool one = ((r ^ M ^ F) >> t) & 1;
+          double d0, d1, in;
+          if ((o.rot >> t) & 1) {
+            shear_scales(o.tau[t], &d0, &d1, &in);
+            Dl[r] = scl(Dl[r], one ? d1 : d0);
+          }
+          if (next && ((next->rot >> t) & 1) && one) {
+            shear_scales(next->tau[t], &d0, &d1, &in);
+            Dl[r] = scl(Dl[r], in);
+          }
+        }
         for (int t = 0; t < k; ++t)
           if ((F >> t) & 1) Dl[r] = scl(Dl[r], ((r >> t) & 1) ? 1.0 : -1.0);  // -Z_t
       }
@@ -1818,6 +2210,7 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     bool conv = true;
     for (int oi : grp.ops) {
       const FGate& f = pass.gates[oi];
+      if (f.type == FG_GRAD && events && f.cmask == 0) continue;
       const bool diag1 = f.type == FG_1Q && f.m[1].re == 0 && f.m[1].im == 0 && f.m[2].re == 0 &&
                          f.m[2].im == 0;
       if (!(f.type == FG_PHASE || (f.type == FG_1Q && (f.cmask == 0 || diag1)))) conv = false;
@@ -1840,10 +2233,19 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     std::vector<LayerH> L(1);
     int gxm = 0;  // the rotation form's final register relabelling
     bool ok = true;
+    std::vector<std::array<int, 3>> grads;  // (operation, layer, group bit)
     for (int oi : grp.ops) {
       const FGate& f = pass.gates[oi];
       LayerH* cur = &L.back();
-      if (f.type == FG_1Q) {
+      if (f.type == FG_GRAD) {  // before the layer's rotations: nothing on the bit yet
+        const int t = gl(f.t);
+        if (((cur->dtouch | cur->u1) >> t) & 1) {
+          L.emplace_back();
+          cur = &L.back();
+        }
+        cur->grad |= 1 << t;
+        grads.push_back({oi, (int)L.size() - 1, t});
+      } else if (f.type == FG_1Q) {
         const int t = gl(f.t), cm = glmask(f.cmask);
         const bool diag = f.m[1].re == 0 && f.m[1].im == 0 && f.m[2].re == 0 && f.m[2].im == 0;
         if (diag) {
@@ -1882,12 +2284,16 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     }
     if (!ok) return 0;
     if (L.back().empty()) L.pop_back();
+    int moved = 0;  // layers that the rotation form put in front
     if (rotform) {
       std::vector<LayerH> R2;
       int xm = 0;
       if (rotation_form(L, k, &R2, &xm)) {
+        moved = (int)(R2.size() - L.size());
         L.swap(R2);
         gxm = xm;
+      } else if (events) {
+        return 0;
       }
     }
     // coefficient count and capacity
@@ -1921,7 +2327,8 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       d.dk = (uint8_t)dks[li];
       d.off = (uint16_t)nc;
       d.rot = (uint8_t)h.rot;
-      d.pad8 = 0;
+      d.grad = (uint8_t)h.grad;
+      d.ev = 0;
       d.pad = 0;
       if (h.rot) {  // tau of bit i in slot i (0 where bit i has no rotation)
         for (int i = 0; i < 4; ++i) {
@@ -1964,6 +2371,41 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     bool dense = false;
     for (const LayerH& h : L) dense = dense || h.u1 != 0;
     P->gxm[g] = (uint8_t)gxm;
+    if constexpr (sizeof(R) == 4) if (events) {
+      // evaluations numbered by layer and bit; a generator's off-diagonal on
+      // the registers: b0 conj(b1) times its own, and for an exchanged bit the
+      // two values' places swapped
+      const int lay0 = nl - (int)L.size();
+      for (size_t li = 0; li < L.size(); ++li) {
+        if (*events + __builtin_popcount(L[li].grad) > 255) return 0;
+        P->layers[lay0 + li].ev = (uint8_t)*events;
+        *events += __builtin_popcount(L[li].grad);
+      }
+      for (const auto& e : grads) {
+        const FGate& f = pass.gates[e[0]];
+        const LayerH& h = L[e[1] + moved];
+        const int t = e[2];
+        const int ev = P->layers[lay0 + e[1] + moved].ev +
+                       __builtin_popcount(h.grad & ((1 << t) - 1));
+        for (int i = 0; i < f.ng; ++i) {
+          double gen[4];
+          gradient_generator(f, i, gen);
+          cd off = cmul(h.ph[t], cd{gen[2], gen[3]});
+          double z = 0.5 * (gen[0] - gen[1]);
+          if ((h.flip >> t) & 1) {
+            off.im = -off.im;
+            z = -z;
+          }
+          if (P->ngrad >= kFMaxOps) return 0;
+          const int j = P->ngrad++;
+          P->gslot[j] = f.ng == 1 ? f.slot : f.gslots[i];
+          P->gev[j] = (uint16_t)ev;
+          P->ggen[j][0] = (float)off.re;
+          P->ggen[j][1] = (float)-off.im;
+          P->ggen[j][2] = (float)z;
+        }
+      }
+    }
     return dense ? 1 : 2;
   }
 }
@@ -2256,6 +2698,28 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
   return check_launch("fused pass kernel");
 }
 
+// A reverse-sweep pass on planes: every group as a layer program in rotation
+// form with its evaluations.  False if some group has another form (gates with
+// controls that are not diagonal, SWAP, gradients inside a control subspace, a
+// 2x2 that is not unitary) or a capacity is exceeded.
+bool build_adj_planes(const FusedPass& pass, const std::vector<int>& order,
+                      FusedParams<float>* P) {
+  if (!build_params(pass, order, P, false)) return false;
+  int pos_of[64] = {};
+  for (int i = 0; i < P->m; ++i) pos_of[order[i]] = i;
+  int nl = 0, nc = 0;
+  P->ngrad = P->nev = 0;
+  for (int g = 0; g < P->ngroups; ++g) {
+    P->glay[g] = (uint16_t)nl;
+    P->gxm[g] = 0;
+    if (layer_group(pass, g, pos_of, P, &nl, &nc, nullptr, true, true, &P->nev) != 2) return false;
+  }
+  P->glay[P->ngroups] = (uint16_t)nl;
+  P->ncoef = nc;
+  plane_threads(P);
+  return true;
+}
+
 template <typename R>
 bool adj_pass_ok(int n, const FusedPass& pass) {
   TmaGeom geo;
@@ -2276,7 +2740,13 @@ sv_status run_adj_pass(void* psi, void* lam, int n, cudaStream_t st, const Fused
     }
   const int lw = sizeof(R) == 4 ? 0 : 1;
   TmaGeom geo;
-  if (!tma_geometry(pass.S, pass.L, n, lw, &geo) || !build_params(pass, geo.order, &P, false) ||
+  const bool geo_ok = tma_geometry(pass.S, pass.L, n, lw, &geo);
+  bool planes = false;
+  if constexpr (sizeof(R) == 4)
+    planes = geo_ok && kg == 4 && (int)pass.S.size() >= kAdjPlaneQubits &&
+             (1 << ((int)pass.S.size() - 5)) <= kAdjPlaneThreads &&
+             build_adj_planes(pass, geo.order, &P);
+  if (!geo_ok || (!planes && !build_params(pass, geo.order, &P, false)) ||
       !verify_tma(geo, pass.S, n, lw, 0) ||
       !verify_tma(geo, pass.S, n, lw, (uint64_t(1) << (n - (int)pass.S.size())) - 1) ||
       !build_tma(geo, psi, &P) || !build_tma(geo, lam, &P, &P.tmap2)) {
@@ -2284,6 +2754,34 @@ sv_status run_adj_pass(void* psi, void* lam, int n, cudaStream_t st, const Fused
     return SV_ERR_UNSUPPORTED;
   }
   typedef void (*Kern)(uint64_t, const FusedParams<R>, double*, int);
+  static std::map<std::pair<const void*, size_t>, int> resident;
+  auto launch = [&](Kern kern, int threads, size_t smem) {
+    int& res = resident[{reinterpret_cast<const void*>(kern), smem}];
+    if (!res) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kern, threads, smem) != cudaSuccess ||
+          res < 1) {
+        cudaGetLastError();
+        res = 1;
+      }
+    }
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint64_t nblk = uint64_t(1) << (n - P.m);
+    const uint64_t grid = std::min<uint64_t>({nblk, (uint64_t)sms * res, (uint64_t)pstride});
+    ProfScope prof(st, sizeof(R) == 4 ? "kfused_adj_c64" : "kfused_adj_c128");
+    launch_dependent(kern, (unsigned)grid, threads, smem, st, nblk, P, partials, pstride);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return check_launch("fused reverse pass kernel");
+  };
+  if constexpr (sizeof(R) == 4)
+    if (planes) {
+      const int threads = 1 << (P.m - 5);
+      return launch(kfused_adj_planes, threads,
+                    1024 + 2 * (size_t)P.slice_bytes +
+                        adj_plane_tail(P.nev, P.ncoef, P.glay[P.ngroups], P.ngroups, threads));
+    }
   constexpr int MB = sizeof(R) == 4 ? 3 : 1;
   constexpr int KMAX = sizeof(R) == 4 ? 4 : 3;  // two 2^k tiles of complex128 above 3 spill
   if (kg > KMAX) {
@@ -2298,26 +2796,8 @@ sv_status run_adj_pass(void* psi, void* lam, int n, cudaStream_t st, const Fused
                     : kg == 2 ? kfused_adj<R, 2, MB>
                     : kg == 3 ? kfused_adj<R, 3, MB>
                               : kfused_adj<R, (KMAX > 3 ? 4 : 3), 2>;
-  const size_t smem = 1024 + 2 * (size_t)P.slice_bytes + adj_tail_bytes<R>(P.ngrad, P.gop[P.ngroups]);
-  static std::map<std::pair<const void*, size_t>, int> resident;
-  int& res = resident[{reinterpret_cast<const void*>(kern), smem}];
-  if (!res) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kern, kFThreads, smem) != cudaSuccess ||
-        res < 1) {
-      cudaGetLastError();
-      res = 1;
-    }
-  }
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t nblk = uint64_t(1) << (n - P.m);
-  const uint64_t grid = std::min<uint64_t>({nblk, (uint64_t)sms * res, (uint64_t)pstride});
-  ProfScope prof(st, sizeof(R) == 4 ? "kfused_adj_c64" : "kfused_adj_c128");
-  launch_dependent(kern, (unsigned)grid, kFThreads, smem, st, nblk, P, partials, pstride);
-  g_launches.fetch_add(1, std::memory_order_relaxed);
-  return check_launch("fused reverse pass kernel");
+  return launch(kern, kFThreads,
+                1024 + 2 * (size_t)P.slice_bytes + adj_tail_bytes<R>(P.ngrad, P.gop[P.ngroups]));
 }
 
 static_assert(sizeof(FusedParams<double>) <= 32000, "kernel parameters above the launch limit");
