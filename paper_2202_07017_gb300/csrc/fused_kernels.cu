@@ -2074,6 +2074,8 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
         a[1] = cdiv(u[2], b[0]);
       }
     }
+    for (cd* x : {&b[0], &b[1]})  // an input phase moved to an earlier gate: exactly none
+      if (std::fabs(x->re - 1.0) < 1e-13 && std::fabs(x->im) < 1e-13) *x = {1.0, 0.0};
     const double S[4] = {*form ? *tau : 1.0, -(*form ? 1.0 : *tau), *form ? 1.0 : *tau,
                          *form ? *tau : 1.0};
     for (int i = 0; i < 2; ++i)

@@ -24,6 +24,7 @@
 //      unscheduled gate it overlaps is scheduled and the union stays within
 //      fuse_k qubits).
 #include <algorithm>
+#include <cmath>
 
 #include "sv_internal.cuh"
 
@@ -78,6 +79,7 @@ FGate classify(const sv_gate& g, int i, int n, const HostMatrix& G, int kmax) {
       for (int q = 0; q < 4; ++q)
         if (q == perm[r] ? !is_one(G.at(r, q)) : !is_zero(G.at(r, q))) swap = false;
   }
+  f.diag = diag;
   if (diag && ones) {
     f.type = FG_PHASE;
     f.cmask = f.qmask;
@@ -118,21 +120,6 @@ void push_fgate(FGate f, std::vector<int>* last, std::vector<FGate>* out) {
     if ((out->back().qmask >> b) & 1) (*last)[b] = (int)out->size() - 1;
 }
 
-bool to_fgates(const sv_circuit* c, const double* theta, int kmax, std::vector<FGate>* out) {
-  const int n = c->n_qubits;
-  std::vector<int> last(64, -1);
-  HostMatrix G;
-  for (int i = 0; i < c->n_gates; ++i) {
-    const sv_gate& g = c->gates[i];
-    if (!gate_matrix(g, theta, c->mat_pool, &G)) {
-      set_error("gate %d: cannot build matrix", i);
-      return false;
-    }
-    push_fgate(classify(g, i, n, G, kmax), &last, out);
-  }
-  return true;
-}
-
 // 2x2 complex products (row-major)
 void mul2(const cd* a, const cd* b, cd* out) {  // out = a b
   for (int i = 0; i < 2; ++i)
@@ -158,6 +145,97 @@ void generator_of(const FGate& g, double* out) {
     out[2] = g.m[1].re;
     out[3] = g.m[1].im;
   }
+}
+
+bool is_unitary2(const cd* u) {
+  for (int i = 0; i < 2; ++i)
+    for (int j = i; j < 2; ++j) {
+      double re = 0, im = 0;
+      for (int r = 0; r < 2; ++r) {  // (U^dagger U)_ij
+        const cd x = u[r * 2 + i], y = u[r * 2 + j];
+        re += x.re * y.re + x.im * y.im;
+        im += x.re * y.im - x.im * y.re;
+      }
+      if (std::fabs(re - (i == j ? 1.0 : 0.0)) > 1e-12 || std::fabs(im) > 1e-12) return false;
+    }
+  return true;
+}
+
+// Input phases moved back.  A rotation U = A S B between diagonals (see
+// rotation_form in fused_kernels.cu) needs B applied before S: as the first gate of a
+// register group that is a diagonal of its own over the whole state.  B
+// commutes with the diagonal gates between U and the previous uncontrolled
+// 1-qubit gate V on the qubit, so V takes it: V <- diag(1, beta) V, U <- U
+// diag(1, 1 / beta), beta = -u01 conj(u00) / |u01 u00|, whatever pass V is in.
+// Generators of gradients on the qubit in between are carried over.  A register
+// group then starts with a diagonal only for a qubit's first gate: random layered
+// circuit, n = 28, depth 30 (159 groups of 442 layers), 1255 -> 1211 us a pass.
+void move_input_phases(std::vector<FGate>* F) {
+  struct Before {
+    int gate = -1;           // the previous uncontrolled 1-qubit gate on the bit
+    std::vector<int> grads;  // gradients on the bit since
+  };
+  std::vector<Before> before(64);
+  for (int j = 0; j < (int)F->size(); ++j) {
+    FGate& f = (*F)[j];
+    if (f.type == FG_GRAD && f.cmask == 0) {
+      before[f.t].grads.push_back(j);
+      continue;
+    }
+    if (f.type == FG_1Q && f.cmask == 0 && !(is_zero(f.m[1]) && is_zero(f.m[2]))) {
+      Before& b = before[f.t];
+      const cd u = f.m[0], w = f.m[1];
+      const double d = std::hypot(u.re, u.im) * std::hypot(w.re, w.im);
+      const cd beta{-(w.re * u.re + w.im * u.im) / d, -(w.im * u.re - w.re * u.im) / d};
+      if (b.gate >= 0 && d > 1e-10 && is_unitary2(f.m) && !is_one(beta)) {
+        const cd in[4] = {{1, 0}, {0, 0}, {0, 0}, beta};
+        const cd out[4] = {{1, 0}, {0, 0}, {0, 0}, {beta.re, -beta.im}};
+        mul2_left(in, (*F)[b.gate].m);
+        cd r[4];
+        mul2(f.m, out, r);
+        for (int e = 0; e < 4; ++e) f.m[e] = r[e];
+        for (int g : b.grads) {
+          FGate& h = (*F)[g];
+          if (h.ng == 1) generator_of(h, h.gen[0]);
+          for (int i = 0; i < h.ng; ++i) {  // off-diagonal times conj(beta)
+            double* q = h.gen[i];
+            const double re = q[2] * beta.re + q[3] * beta.im, im = q[3] * beta.re - q[2] * beta.im;
+            q[2] = re;
+            q[3] = im;
+          }
+          if (h.ng == 1) {
+            const double* q = h.gen[0];
+            h.pauli = 0;
+            h.m[0] = {q[0], 0};
+            h.m[1] = {q[2], q[3]};
+            h.m[2] = {q[2], -q[3]};
+            h.m[3] = {q[1], 0};
+          }
+        }
+      }
+      b.gate = j;
+      b.grads.clear();
+      continue;
+    }
+    if (f.diag || (f.type == FG_1Q && f.cmask == 0)) continue;  // commutes
+    for (int t = 0; t < 64; ++t)
+      if ((f.qmask >> t) & 1) before[t] = Before();
+  }
+}
+
+bool to_fgates(const sv_circuit* c, const double* theta, int kmax, std::vector<FGate>* out) {
+  const int n = c->n_qubits;
+  std::vector<int> last(64, -1);
+  HostMatrix G;
+  for (int i = 0; i < c->n_gates; ++i) {
+    const sv_gate& g = c->gates[i];
+    if (!gate_matrix(g, theta, c->mat_pool, &G)) {
+      set_error("gate %d: cannot build matrix", i);
+      return false;
+    }
+    push_fgate(classify(g, i, n, G, kmax), &last, out);
+  }
+  return true;
 }
 
 // Reverse sweep over [lo, hi): gate hi-1 first, each as its adjoint, a
@@ -439,6 +517,7 @@ bool plan_fusion(const sv_circuit* c, const double* theta, const FusionConfig& c
                  std::vector<FusionItem>* out) {
   std::vector<FGate> F;
   if (!to_fgates(c, theta, std::min(cfg.fuse_k, cfg.m), &F)) return false;
+  move_input_phases(&F);
   form_passes(F, c->n_qubits, cfg, out);
   return true;
 }
@@ -466,6 +545,7 @@ bool plan_fusion_reverse(const sv_circuit* c, const double* theta, int lo, int h
   std::vector<FGate> F;
   if (!to_fgates_reverse(c, theta, lo, hi, slot_of, std::min(cfg.fuse_k, cfg.m), &F))
     return false;
+  move_input_phases(&F);
   form_passes(F, c->n_qubits, cfg, out);
   return true;
 }

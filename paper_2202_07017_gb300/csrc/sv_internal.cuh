@@ -212,6 +212,7 @@ struct FGate {
   uint64_t qmask = 0;  // every bit the gate touches (targets and controls)
   uint64_t cmask = 0;  // control bits (FG_1Q, FG_SWAP); all bits for FG_PHASE
   int t = 0, a = 0, b = 0;  // FG_1Q target bit; FG_SWAP bits
+  bool diag = false;   // the gate's matrix is diagonal
   cd m[4] = {};        // FG_1Q: 2x2 row-major; FG_PHASE: m[0] = phase
   int orig = -1;       // index of the (last merged) circuit gate
   std::vector<int> origs;  // every circuit gate folded into this one
