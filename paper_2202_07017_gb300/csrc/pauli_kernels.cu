@@ -44,6 +44,9 @@ constexpr int kPThreads = 512;
 constexpr int kPMaxTerms = 96;
 constexpr int kPMaxGroups = 16;
 constexpr int kPG = 4;  // bits of a register tile
+constexpr int kDKeys = 16;
+constexpr int kDTerms = 64;
+constexpr int kDThreads = 256;
 
 // kind of an off-diagonal term inside its group
 enum { PT_GENERAL = 0, PT_XBIT = 1, PT_YBIT = 2 };
@@ -453,6 +456,166 @@ __global__ void __launch_bounds__(kPThreads, 1)
   if (threadIdx.x == 0) partials[blockIdx.x] = e;
 }
 
+// ---- X terms of complex64 states on 16-byte chunks -------------------------------------
+// kpauli_xbits is bound by its reads of the slice from shared memory (one per
+// group of four bits, 8 bytes at a time) and their instructions.  Here a
+// thread's tile is 16 chunks of two amplitudes, read as 16-byte vectors: three
+// groups cover the 12 chunk bits of a 2^13 slice and amplitude bit 0 comes with
+// the first, and the pair sums are paired fp32 FMAs on (re, im).  One half of
+// the block's warps takes groups 0 and 2, the other group 1 (all three in 8
+// warps: latency-bound, no faster than 8-byte reads).  n = 29: 1014 -> 726 us
+// a pass (one read: 640 us).
+constexpr int kXCGroups = 3;
+
+struct XChunkDev {
+  SliceDev geo;
+  int ngroups;
+  uint8_t gbits[kXCGroups][4];  // chunk bits of the group, ascending
+  uint8_t tpos[kXCGroups][8];   // chunk bits of the thread bits
+  double w0, w[4 * kXCGroups];  // 2 sum c_k over the terms on bit 0, on bit i of group g
+};
+
+typedef unsigned long long PairP;
+__device__ __forceinline__ void fma2_add(PairP& d, PairP a, PairP b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 lanes2(PairP p) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float lane_sum(PairP p) {
+  const float2 v = lanes2(p);
+  return v.x + v.y;
+}
+__device__ __forceinline__ int cswz(int q) { return q ^ ((q >> 3) & 7); }
+
+__global__ void __launch_bounds__(kPThreads, 1)
+    kpauli_xchunks(uint64_t n_blocks, const __grid_constant__ XChunkDev P,
+                   double* __restrict__ partials, unsigned* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bars[kXBuf];   // full: the slice's bytes have landed
+  __shared__ __align__(8) uint64_t ebars[kXBuf];  // empty: every warp is done with it
+  constexpr int kWarps = kPThreads / 32;
+  const uint32_t raw = smem_addr(smem_raw);
+  const uint32_t sbuf0 = (raw + 1023u) & ~1023u;  // slice bytes: multiples of 1024
+  const uint32_t sbytes = P.geo.slice_bytes;
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int j = 0; j < kXBuf; ++j) {
+      mbar_init(smem_addr(&bars[j]), 1);
+      mbar_init(smem_addr(&ebars[j]), kWarps);
+    }
+    fence_proxy_async_smem();
+  }
+  // the half's groups g0 and g0 + 2; at most one tile per thread and group
+  // (slices of up to 2^13 amplitudes)
+  const int half = threadIdx.x / (kPThreads / 2), t = threadIdx.x % (kPThreads / 2);
+  const bool live = t < (1 << (P.geo.m - 5));
+  int tile[2], sw[2][4];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int g = half + 2 * j < kXCGroups ? half + 2 * j : 0;
+    int q = 0;
+    for (int i = 0; i < P.geo.m - 5; ++i) q |= ((t >> i) & 1) << P.tpos[g][i];
+    tile[j] = cswz(q);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sw[j][i] = cswz(1 << P.gbits[g][i]);
+  }
+  grid_dependency_wait();
+  __syncthreads();
+  CompSum<float> acc[2][4], acc0;
+  // bit j: buffer j.  used: filled before (its refill waits until every warp
+  // released the previous fill); eparity: phase of its empty barrier
+  uint32_t parity = 0, pending = 0, used = 0, eparity = 0;
+  for (int j = 0; j < kXBuf - 1; ++j) {
+    const uint64_t b = blockIdx.x + (uint64_t)j * gridDim.x;
+    if (b < n_blocks) {
+      if (threadIdx.x < 32)
+        issue_slice<float>(P.geo, b, sbuf0 + (uint32_t)j * sbytes, smem_addr(&bars[j]), lane);
+      pending |= 1u << j;
+      used |= 1u << j;
+    }
+  }
+  int cur = 0;
+  for (uint64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
+    // slice blk + (kXBuf - 1) grid strides into the buffer of the previous
+    // iteration, once all warps have released it: no block-wide barrier, the
+    // other warps run on into the slices already loaded
+    const int nxt = cur == 0 ? kXBuf - 1 : cur - 1;
+    const uint64_t nb = blk + (uint64_t)(kXBuf - 1) * gridDim.x;
+    if (nb < n_blocks) {
+      if (threadIdx.x < 32) {
+        bool free_ok = true;
+        if ((used >> nxt) & 1)
+          free_ok = mbar_wait_bounded(smem_addr(&ebars[nxt]), (eparity >> nxt) & 1);
+        if (free_ok)
+          issue_slice<float>(P.geo, nb, sbuf0 + (uint32_t)nxt * sbytes, smem_addr(&bars[nxt]), lane);
+        else if (lane == 0)
+          atomicOr(status, kWaitTimeout);
+      }
+      if ((used >> nxt) & 1) eparity ^= 1u << nxt;
+      used |= 1u << nxt;
+      pending |= 1u << nxt;
+    }
+    const bool ok = mbar_wait_bounded(smem_addr(&bars[cur]), (parity >> cur) & 1);
+    parity ^= 1u << cur;
+    pending &= ~(1u << cur);
+    if (!ok) {  // this warp stops; the others give up at their own bounded waits
+      if (lane == 0) atomicOr(status, kWaitTimeout);
+      break;
+    }
+    const ulonglong2* sm =
+        reinterpret_cast<const ulonglong2*>(smem_raw + (sbuf0 + (uint32_t)cur * sbytes - raw));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (!live || half + 2 * j >= P.ngroups) break;
+      PairP a[16], b[16];  // amplitudes 2 q and 2 q + 1 as (re, im)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        int o = tile[j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if ((r >> i) & 1) o ^= sw[j][i];
+        const ulonglong2 v = sm[o];
+        a[r] = v.x;
+        b[r] = v.y;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        PairP x = 0, y = 0;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          if (r & (1 << i)) continue;
+          fma2_add(x, a[r], a[r | (1 << i)]);
+          fma2_add(y, b[r], b[r | (1 << i)]);
+        }
+        acc[j][i].add(lane_sum(x) + lane_sum(y));
+      }
+      if (j == 0 && half == 0) {
+        PairP x = 0;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) fma2_add(x, a[r], b[r]);
+        acc0.add(lane_sum(x));
+      }
+    }
+    __syncwarp();  // this warp is done with the buffer
+    if (lane == 0) mbar_arrive(smem_addr(&ebars[cur]));
+    cur = cur + 1 == kXBuf ? 0 : cur + 1;
+  }
+  // copies still in flight (a block that gave up): wait for them, bounded
+  for (int j = 0; j < kXBuf; ++j)
+    if ((pending >> j) & 1) mbar_wait_bounded(smem_addr(&bars[j]), (parity >> j) & 1);
+  double e = P.w0 * acc0.value();
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (half + 2 * j < kXCGroups) e += P.w[4 * (half + 2 * j) + i] * acc[j][i].value();
+  e = block_sum(e);
+  if (threadIdx.x == 0) partials[blockIdx.x] = e;
+}
+
 // ---- diagonal terms: one streaming read -----------------------------------------------
 // The diagonal part of H, E_d = sum_x |psi_x|^2 d(x), d(x) = sum_k c_k
 // (-1)^{popcount(x & z_k)}, read with coalesced 16-byte loads and no shared
@@ -466,9 +629,6 @@ __global__ void __launch_bounds__(kPThreads, 1)
 // W the Walsh-Hadamard transform of the tile's |psi|^2; at the end each term
 // takes c_k (-1)^{popcount(t & z_k's thread bits)} times its key's sum.  A
 // launch serves up to kDKeys keys (terms that share a key share its sum).
-constexpr int kDKeys = 16;
-constexpr int kDTerms = 64;
-constexpr int kDThreads = 256;
 
 template <typename R>
 struct DiagDev {
@@ -882,6 +1042,53 @@ bool lean_pass(const PauliPassDev<R>& P, XPassDev* X) {
   return true;
 }
 
+// The lean pass p of a complex64 state as kpauli_xchunks takes it.  false: more
+// than kXCGroups groups of chunk bits, or fewer than four of them.
+bool chunk_pass(const PauliPassDev<float>& P, XChunkDev* X) {
+  const int nc = P.geo.m - 1;  // chunk bits
+  if (nc < 4 || nc > 12) return false;
+  *X = XChunkDev{};
+  X->geo = P.geo;
+  double wl[24] = {};
+  for (int g = 0; g < P.ngroups; ++g)
+    for (int k = P.xstart[g]; k < P.xstart[g + 1]; ++k)
+      wl[P.gbits[g][P.terms[k].bit]] += 2.0 * (double)P.terms[k].cre;
+  X->w0 = wl[0];
+  std::vector<int> need;
+  for (int q = 0; q < nc; ++q)
+    if (wl[q + 1] != 0.0) need.push_back(q);
+  X->ngroups = std::max(1, ((int)need.size() + 3) / 4);
+  for (int g = 0; g < X->ngroups; ++g) {
+    std::vector<int> bits(need.begin() + std::min<size_t>(need.size(), 4 * g),
+                          need.begin() + std::min<size_t>(need.size(), 4 * g + 4));
+    const size_t own = bits.size();
+    for (int q = 0; q < nc && bits.size() < 4; ++q)
+      if (std::find(bits.begin(), bits.end(), q) == bits.end()) bits.push_back(q);
+    std::vector<int> sorted = bits;
+    std::sort(sorted.begin(), sorted.end());
+    bool used[24] = {};
+    for (int i = 0; i < 4; ++i) {
+      X->gbits[g][i] = (uint8_t)sorted[i];
+      used[sorted[i]] = true;
+      for (size_t j = 0; j < own; ++j)
+        if (bits[j] == sorted[i]) X->w[4 * g + i] = wl[sorted[i] + 1];
+    }
+    // a quarter warp's three lane bits on three different 16-byte column bits
+    // (chunk bit i < 6 moves column bit i mod 3), the other thread bits in order
+    int k = 0;
+    for (int res = 0; res < 3; ++res)
+      for (int i = res; i < 6 && i < nc; i += 3)
+        if (!used[i]) {
+          X->tpos[g][k++] = (uint8_t)i;
+          used[i] = true;
+          break;
+        }
+    for (int i = 0; i < nc; ++i)
+      if (!used[i]) X->tpos[g][k++] = (uint8_t)i;
+  }
+  return true;
+}
+
 // The diagonal terms of T (x mask 0) as launches of kdiag_energy /
 // kdiag_apply: up to kDKeys keys (tile pattern rho, iteration mask zJ) and
 // kDTerms terms each, keys with rho = 0 first; tb thread bits.
@@ -1062,7 +1269,12 @@ sv_status expval_staged(sv_state s, const sv_pauli_sum* H, double* dst) {
   std::vector<char> is_lean(passes.size());
   for (size_t i = 0; i < passes.size(); ++i)
     is_lean[i] = c64 ? lean_pass<float>(pf[i], &lean[i]) : lean_pass<double>(pd[i], &lean[i]);
-  const size_t smem_x = kXBuf * (size_t(8) << lw << m) + 1024;  // the lean kernel's buffers
+  const size_t smem_x = kXBuf * (size_t(8) << lw << m) + 1024;  // the lean kernels' buffers
+  // complex64: lean passes on chunks
+  std::vector<XChunkDev> chunked(passes.size());
+  std::vector<char> is_chunked(passes.size());
+  for (size_t i = 0; i < passes.size(); ++i)
+    is_chunked[i] = c64 && is_lean[i] && chunk_pass(pf[i], &chunked[i]);
   auto grid_of = [&](const void* kern, size_t bytes, int nbuf) -> uint64_t {
     int& res = resident[{kern, bytes}];
     if (!res) {
@@ -1095,17 +1307,16 @@ sv_status expval_staged(sv_state s, const sv_pauli_sum* H, double* dst) {
   }
   for (size_t i = 0; i < passes.size(); ++i) {
     uint64_t grid;
-    if (is_lean[i]) {
-      ProfScope prof(s->stream, c64 ? "kpauli_xbits_c64" : "kpauli_xbits_c128");
-      if (c64) {
-        grid = grid_of((const void*)kpauli_xbits<float>, smem_x, kXBuf);
-        launch_dependent(kpauli_xbits<float>, (unsigned)grid, kPThreads, smem_x,
-                         s->stream, nblk, lean[i], s->partials + total, status);
-      } else {
-        grid = grid_of((const void*)kpauli_xbits<double>, smem_x, kXBuf);
-        launch_dependent(kpauli_xbits<double>, (unsigned)grid, kPThreads, smem_x,
-                         s->stream, nblk, lean[i], s->partials + total, status);
-      }
+    if (is_chunked[i]) {
+      ProfScope prof(s->stream, "kpauli_xbits_c64");
+      grid = grid_of((const void*)kpauli_xchunks, smem_x, kXBuf);
+      launch_dependent(kpauli_xchunks, (unsigned)grid, kPThreads, smem_x, s->stream, nblk,
+                       chunked[i], s->partials + total, status);
+    } else if (is_lean[i] && !c64) {
+      ProfScope prof(s->stream, "kpauli_xbits_c128");
+      grid = grid_of((const void*)kpauli_xbits<double>, smem_x, kXBuf);
+      launch_dependent(kpauli_xbits<double>, (unsigned)grid, kPThreads, smem_x, s->stream, nblk,
+                       lean[i], s->partials + total, status);
     } else {
       ProfScope prof(s->stream, c64 ? "kpauli_energy_c64" : "kpauli_energy_c128");
       if (c64) {
