@@ -18,12 +18,17 @@
 // and rounds P = sum / 2^120 to fp64.
 //
 // Sampling for caller-given uniforms u (the random numbers are inputs):
-// exact chunk sums (a warp per 1024 amplitudes, one HBM pass), an exact
-// prefix scan of the chunk sums, then one warp per shot: T = floor(u *
-// total) exactly, binary search for the first chunk prefix above T, and a
-// scan of that chunk 32 amplitudes at a time (warp prefix sum) for the first
-// x with c(x) > T.  Outcomes are projected onto the measured qubits (the
-// marginal of a subset is the projection of full samples).
+// exact chunk sums (128 amplitudes, four lanes a chunk, one HBM pass), an exact
+// prefix scan of the chunk sums, then per shot T = floor(u * total) exactly and a
+// binary search for the first chunk prefix above T (a thread per shot: the
+// searches' dependent loads overlap across the threads), and a warp per shot
+// for the first x of that chunk with c(x) > T: each lane sums its share, one
+// warp prefix sum finds the lane, and its own running sum the amplitude.
+// Outcomes are projected onto the measured qubits (the marginal of a subset is
+// the projection of full samples).  Chunks of 1024 amplitudes, searched and
+// scanned 32 amplitudes at a time by a warp per shot: 3.54 ms for 10^6 shots at
+// n = 27, now 0.85 ms.  Chunk sums at n = 27: 525 -> 312 us, ten marginals 968 ->
+// 414 us (HBM: 160 us; bound by the exact squares' integer instructions).
 #include <algorithm>
 #include <vector>
 
@@ -32,7 +37,9 @@
 namespace sv {
 namespace {
 
-constexpr int kChunkBits = 10;
+// Chunk size: 2^7 amplitudes, more above 31 qubits to keep the chunk sums at
+// 2^24 (256 MiB).
+int chunk_bits(int n) { return std::max(1, std::min(n, std::max(7, n - 24))); }
 
 struct U128 {
   uint64_t lo, hi;
@@ -63,10 +70,18 @@ __device__ __forceinline__ U128 shift128(U128 x, int sh) {
   return {(x.lo >> r) | (x.hi << (64 - r)), x.hi >> r};
 }
 
-// q(v) = floor(v^2 2^120)
+// q(v) = floor(v^2 2^120).  2^-37 <= |v| < 2^-5, as most amplitudes are, is a
+// left shift by less than 64: a third of the general form's instructions, which
+// bound these kernels.
 __device__ __forceinline__ U128 q120(float v) {
   const uint32_t b = __float_as_uint(v) & 0x7fffffffu;
   const int e = (int)(b >> 23);
+  if ((unsigned)(e - 90) < 32u) {
+    const uint32_t m = (b & 0x7fffffu) | 0x800000u;  // v = m 2^(e - 150)
+    const uint64_t sq = (uint64_t)m * m;
+    const int sh = 2 * (e - 90);  // 0..62
+    return {sq << sh, (sq >> 1) >> (63 - sh)};
+  }
   if (e == 0) return {0, 0};  // zero or subnormal: v^2 2^120 < 1
   const uint64_t m = (b & 0x7fffffu) | 0x800000u;  // v = m 2^(e - 150)
   return shift128(U128{m * m, 0}, 2 * (e - 150) + 120);
@@ -92,6 +107,10 @@ __device__ __forceinline__ U128 qvec(const double2 a) { return add128(q120(a.x),
 
 __device__ __forceinline__ U128 shfl_xor128(U128 v, int o) {
   return {__shfl_xor_sync(0xffffffffu, v.lo, o), __shfl_xor_sync(0xffffffffu, v.hi, o)};
+}
+
+__device__ __forceinline__ U128 shfl_up128(U128 v, int o) {
+  return {__shfl_up_sync(0xffffffffu, v.lo, o), __shfl_up_sync(0xffffffffu, v.hi, o)};
 }
 
 __device__ __forceinline__ U128 warp_sum128(U128 v) {
@@ -141,20 +160,26 @@ __global__ void __launch_bounds__(kRedThreads)
   uint64_t rbits = 0;
   for (int j = 0; j < m; ++j)
     if ((r >> (m - 1 - j)) & 1) rbits |= uint64_t(1) << mpos[j];
-  const uint64_t len = (per_bin + slices - 1) / slices;
-  const uint64_t e0 = (uint64_t)c * len, e1 = e0 + len < per_bin ? e0 + len : per_bin;
+  // slices: a power of two of at least kRedThreads elements, or one slice, so
+  // that an element's index is the disjoint union of its block-uniform part and
+  // the thread's, and the zero-bit insertion of the thread's part is done once
+  const uint64_t len = per_bin / slices;
+  const uint64_t e0 = (uint64_t)c * len, e1 = e0 + len;
+  const uint64_t mine = insert_zeros((uint64_t)threadIdx.x, rest) | rbits;
   U128 acc = {0, 0};
   constexpr int U = 8;  // loads in flight per thread
-  for (uint64_t e = e0 + threadIdx.x; e < e1; e += (uint64_t)kRedThreads * U) {
+  uint64_t off[U];      // their places behind the first's
+#pragma unroll
+  for (int k = 0; k < U; ++k) off[k] = insert_zeros((uint64_t)k * kRedThreads, rest);
+  for (uint64_t e = e0; e < e1; e += (uint64_t)kRedThreads * U) {
+    const uint64_t at = insert_zeros(e, rest) | mine;
     T2 v[U];
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const uint64_t ek = e + (uint64_t)k * kRedThreads;
-      if (ek < e1) v[k] = psi[insert_zeros(ek, rest) | rbits];
-    }
+    for (int k = 0; k < U; ++k)
+      if (e + (uint64_t)k * kRedThreads + threadIdx.x < e1) v[k] = psi[at | off[k]];
 #pragma unroll
     for (int k = 0; k < U; ++k)
-      if (e + (uint64_t)k * kRedThreads < e1) acc = add128(acc, qamp(v[k]));
+      if (e + (uint64_t)k * kRedThreads + threadIdx.x < e1) acc = add128(acc, qamp(v[k]));
   }
   acc = warp_sum128(acc);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
@@ -178,29 +203,30 @@ __global__ void kprob_finish(const U128* __restrict__ partials, int slices, uint
            7.52316384526264005099991383822e-37;  // 2^-120
 }
 
-// sums[k] = exact sum over chunk k (2^vbits vectors of 16 bytes), a warp per chunk
+// sums[k] = exact sum over chunk k (2^vbits vectors of 16 bytes), four lanes a chunk
 template <typename V>
 __global__ void __launch_bounds__(kRedThreads)
     kchunk_sums(const V* __restrict__ psi, int vbits, uint64_t K, U128* __restrict__ sums) {
   grid_dependency_wait();
-  const uint64_t k = (uint64_t)blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (k >= K) return;
-  const V* c = psi + (k << vbits);
+  const uint64_t k = ((uint64_t)blockIdx.x * kRedThreads + threadIdx.x) >> 2;
+  const int part = threadIdx.x & 3;
+  const bool live = k < K;
+  const V* c = psi + ((live ? k : 0) << vbits);
   const int nv = 1 << vbits;
   U128 acc = {0, 0};
-  constexpr int U = 16;
-  for (int i0 = lane; i0 < nv; i0 += 32 * U) {
+  constexpr int U = 8;
+  for (int i0 = part; i0 < nv; i0 += 4 * U) {
     V v[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (i0 + 32 * u < nv) v[u] = c[i0 + 32 * u];
+      if (i0 + 4 * u < nv) v[u] = c[i0 + 4 * u];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (i0 + 32 * u < nv) acc = add128(acc, qvec(v[u]));
+      if (i0 + 4 * u < nv) acc = add128(acc, qvec(v[u]));
   }
-  acc = warp_sum128(acc);
-  if (lane == 0) sums[k] = acc;
+  acc = add128(acc, shfl_xor128(acc, 1));
+  acc = add128(acc, shfl_xor128(acc, 2));
+  if (live && part == 0) sums[k] = acc;
 }
 
 // inclusive prefix sums in place (exact, so any order gives the same values)
@@ -216,12 +242,21 @@ __global__ void __launch_bounds__(1024) kscan(U128* __restrict__ v, uint64_t K) 
   }
   tot[threadIdx.x] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {  // exclusive sums of the 1024 totals: 32 per lane, then over the lanes
     U128 run = {0, 0};
-    for (int t = 0; t < 1024; ++t) {
-      const U128 x = tot[t];
-      tot[t] = run;
-      run = add128(run, x);
+    for (int t = 0; t < 32; ++t) run = add128(run, tot[32 * threadIdx.x + t]);
+    U128 off = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const U128 y = shfl_up128(off, o);
+      if ((int)threadIdx.x >= o) off = add128(off, y);
+    }
+    off = shfl_up128(off, 1);
+    if (threadIdx.x == 0) off = {0, 0};
+    for (int t = 0; t < 32; ++t) {
+      const U128 x = tot[32 * threadIdx.x + t];
+      tot[32 * threadIdx.x + t] = off;
+      off = add128(off, x);
     }
   }
   __syncthreads();
@@ -268,7 +303,24 @@ __global__ void __launch_bounds__(1024) kscan_add(U128* __restrict__ v, uint64_t
   v[i] = add128(v[i], scanned_totals[blockIdx.x - 1]);
 }
 
-// One warp per shot.
+// chunk[s] = first chunk whose inclusive prefix exceeds shot s's threshold
+__global__ void __launch_bounds__(kRedThreads)
+    kshot_chunks(const U128* __restrict__ prefix, uint64_t K, const double* __restrict__ u,
+                 int64_t nshots, uint64_t* __restrict__ chunk) {
+  grid_dependency_wait();
+  const int64_t s = (int64_t)blockIdx.x * kRedThreads + threadIdx.x;
+  if (s >= nshots) return;
+  const U128 T = frac_mul(u[s], prefix[K - 1]);
+  uint64_t lo = 0, hi = K - 1;
+  while (lo < hi) {
+    const uint64_t mid = lo + (hi - lo) / 2;
+    if (gt128(prefix[mid], T)) hi = mid; else lo = mid + 1;
+  }
+  chunk[s] = lo;
+}
+
+// One warp per shot: the first amplitude of its chunk (out[s] on entry) whose
+// cumulative sum exceeds the threshold, projected onto the measured bits.
 template <typename T2>
 __global__ void __launch_bounds__(kRedThreads)
     kshots(const T2* __restrict__ psi, int cbits, const U128* __restrict__ prefix, uint64_t K,
@@ -278,28 +330,46 @@ __global__ void __launch_bounds__(kRedThreads)
   const int64_t s = (int64_t)blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (s >= nshots) return;
+  const uint64_t lo = out[s];
   const U128 T = frac_mul(u[s], prefix[K - 1]);
-  uint64_t lo = 0, hi = K - 1;  // first chunk whose prefix exceeds T
-  while (lo < hi) {
-    const uint64_t mid = lo + (hi - lo) / 2;
-    if (gt128(prefix[mid], T)) hi = mid; else lo = mid + 1;
-  }
   U128 acc = lo ? prefix[lo - 1] : U128{0, 0};
   const uint64_t base = lo << cbits;
   const int len = 1 << cbits;
+  constexpr int U = 4;  // amplitudes per lane and step
   uint64_t x = base + len - 1;
-  for (int i0 = 0; i0 < len; i0 += 32) {
-    const int i = i0 + lane;
-    U128 incl = i < len ? qamp(psi[base + i]) : U128{0, 0};
+  for (int i0 = 0; i0 < len; i0 += 32 * U) {
+    U128 q[U], incl = {0, 0};
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int i = i0 + U * lane + k;
+      q[k] = i < len ? qamp(psi[base + i]) : U128{0, 0};
+      incl = add128(incl, q[k]);
+    }
+    const U128 own = incl;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const U128 y = {__shfl_up_sync(0xffffffffu, incl.lo, o),
-                      __shfl_up_sync(0xffffffffu, incl.hi, o)};
+      const U128 y = shfl_up128(incl, o);
       if (lane >= o) incl = add128(incl, y);
     }
     const unsigned over = __ballot_sync(0xffffffffu, gt128(add128(acc, incl), T));
     if (over) {
-      x = base + i0 + (__ffs(over) - 1);
+      const int f = __ffs(over) - 1;
+      // lane f: the first of its amplitudes past T (its own sums; the last one
+      // reaches incl, so one is)
+      U128 run = add128(acc, incl);
+      run.hi -= own.hi + (run.lo < own.lo ? 1 : 0);
+      run.lo -= own.lo;
+      int j = U - 1;
+      bool found = false;
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        run = add128(run, q[k]);
+        if (!found && gt128(run, T)) {
+          j = k;
+          found = true;
+        }
+      }
+      x = base + i0 + U * f + __shfl_sync(0xffffffffu, j, f);
       break;
     }
     acc = add128(acc, U128{__shfl_sync(0xffffffffu, incl.lo, 31),
@@ -348,7 +418,9 @@ sv_status sv_probabilities(sv_state s, const int* qubits, int n_meas, double* ou
     pos.push_back(mpos[j]);
   }
   const uint64_t bins = uint64_t(1) << m, per_bin = uint64_t(1) << (n - m);
-  const int slices = (int)std::max<uint64_t>(1, std::min<uint64_t>(2432 / bins, per_bin / 2048));
+  // blocks for several waves over the SMs, each with at least 2048 elements of its bin
+  int slices = 1;
+  while (slices * bins < 2432 && per_bin / (2 * slices) >= 2048) slices *= 2;
   const size_t nparts = bins * slices;
   // partials (2 doubles each), then the bins, then the measured positions
   sv_status st = ensure_partials(s, 2 * nparts + bins + 64);
@@ -396,7 +468,7 @@ sv_status sv_sample(sv_state s, const int* qubits, int n_meas, int64_t n_shots,
     }
   if (n_shots == 0) return SV_OK;
   const int n = s->n, m = n_meas;
-  const int cbits = std::max(1, std::min(n, kChunkBits));
+  const int cbits = chunk_bits(n);
   const uint64_t K = uint64_t(1) << (n - cbits);
   int mpos[64];
   for (int j = 0; j < m; ++j) mpos[j] = n - 1 - qubits[j];
@@ -416,7 +488,7 @@ sv_status sv_sample(sv_state s, const int* qubits, int n_meas, int64_t n_shots,
                               s->stream));
   {
     ProfScope prof(s->stream, "kchunk_sums");
-    const unsigned g = (unsigned)((K + kRedThreads / 32 - 1) / (kRedThreads / 32));
+    const unsigned g = (unsigned)((K + kRedThreads / 4 - 1) / (kRedThreads / 4));
     if (s->dt == SV_C64)  // 2 amplitudes per 16-byte vector
       launch_dependent(kchunk_sums<float4>, g, kRedThreads, 0,
                        s->stream, (const float4*)s->data, cbits - 1, K, prefix);
@@ -436,6 +508,12 @@ sv_status sv_sample(sv_state s, const int* qubits, int n_meas, int64_t n_shots,
       launch_dependent(kscan_add, (unsigned)nb, 1024, 0, s->stream, prefix, K, btot);
       g_launches.fetch_add(3, std::memory_order_relaxed);
     }
+  }
+  {
+    ProfScope prof(s->stream, "kshot_chunks");
+    const unsigned g = (unsigned)((n_shots + kRedThreads - 1) / kRedThreads);
+    launch_dependent(kshot_chunks, g, kRedThreads, 0, s->stream, prefix, K, du, n_shots, dout);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
   }
   {
     ProfScope prof(s->stream, "kshots");
