@@ -15,10 +15,11 @@
 //      all-ones subspace, SWAP with controls, or "alone" for anything else
 //      or anything wider than fuse_k qubits); consecutive uncontrolled
 //      1-qubit gates on one qubit are multiplied into one 2x2 in fp64;
-//   2. a pass grows S greedily from the earliest remaining gate, taking
-//      every later gate whose qubits fit in S and that no skipped earlier
-//      gate overlaps; unused places in S are filled with the lowest free
-//      bits (longer contiguous runs);
+//   2. a pass's S is grown greedily from the earliest remaining gate (unused
+//      places filled with the lowest free bits, for longer contiguous runs), or
+//      is the low run plus a contiguous window of high bits, whichever takes more
+//      gates: every remaining gate whose qubits lie in S and that no skipped
+//      earlier gate overlaps;
 //   3. the pass's gates are list-scheduled into register groups of at
 //      most fuse_k qubits (a gate joins the open group when every earlier
 //      unscheduled gate it overlaps is scheduled and the union stays within
@@ -394,6 +395,7 @@ FusionConfig fusion_config(int n, sv_dtype dt, int fuse_k) {
   // keep at least 2^8 blocks for mid-size states, down to 2^10 amplitudes
   if (n > 10) m = std::max(std::min(m, n - 8), std::min(n, 10));
   c.m = m;
+  c.max_layers = dt == SV_C64 ? 72 : 40;  // 40 fp32 or 36 fp64 coefficients a layer
   c.L = std::min(dt == SV_C64 ? 5 : 4, m);
   if (c.m - c.L < fuse_k) c.L = std::max(1, c.m - fuse_k);
   return c;
@@ -411,17 +413,65 @@ FusionConfig fusion_config_reverse(int n, sv_dtype dt, int fuse_k) {
 
 namespace {
 
+// Layers that the group's operations make as a layer program: a 1-qubit gate
+// or gradient on a bit that a diagonal of the layer has touched starts the next.
+int count_layers(const std::vector<FGate>& F, const std::vector<int>& members) {
+  int layers = 1;
+  uint64_t touched = 0;
+  for (int j : members) {
+    const FGate& f = F[j];
+    if (f.type != FG_1Q && f.type != FG_GRAD) {
+      touched |= f.qmask;
+    } else if (touched & f.qmask) {
+      ++layers;
+      touched = 0;
+    }
+  }
+  return layers;
+}
+
 // Passes (steps 2 and 3 of the planning) over the operation list F.
 void form_passes(const std::vector<FGate>& F, int n, const FusionConfig& cfg,
                  std::vector<FusionItem>* out) {
-  std::vector<char> done(F.size(), 0);
   const uint64_t lowL = (cfg.L >= 64) ? ~uint64_t(0) : ((uint64_t(1) << cfg.L) - 1);
-  size_t first = 0;
+  uint64_t active = 0;
+  for (const FGate& f : F) active |= f.qmask;
+  std::vector<int> rem(F.size());  // operations not yet planned, in order
+  for (size_t j = 0; j < F.size(); ++j) rem[j] = (int)j;
+  size_t head = 0;  // rem[0..head) are planned
   out->clear();
-  while (true) {
-    while (first < F.size() && done[first]) ++first;
-    if (first == F.size()) break;
-    const FGate& f0 = F[first];
+  // The operations of a pass that stages S, in order: those inside S that no
+  // skipped earlier one overlaps; at most `scan` operations looked at.  grow: S
+  // takes the bits of every operation met, up to m.
+  auto collect = [&](uint64_t* S, bool grow, size_t scan, std::vector<int>* take) {
+    uint64_t blocked = 0;
+    int nS = popc(*S), ngrads = 0, ops = 0, count = 0;
+    for (size_t i = head; i < rem.size() && scan > 0; ++i, --scan) {
+      const FGate& f = F[rem[i]];
+      bool ok = f.type != FG_ALONE && !(f.qmask & blocked) && count < cfg.max_ops &&
+                (f.type != FG_GRAD || ngrads + f.ng <= cfg.max_grads);
+      if (ok) {
+        const uint64_t need = f.qmask & ~*S;
+        if (need && (!grow || nS + popc(need) > cfg.m)) {
+          ok = false;
+        } else {
+          *S |= need;
+          nS += popc(need);
+        }
+      }
+      if (ok) {
+        ++count;
+        if (take) take->push_back((int)i);
+        if (f.type == FG_GRAD) ngrads += f.ng; else ++ops;
+      } else {
+        blocked |= f.qmask;
+        if (!(active & ~blocked & (grow && nS < cfg.m ? ~uint64_t(0) : *S))) break;
+      }
+    }
+    return ops;
+  };
+  while (head < rem.size()) {
+    const FGate& f0 = F[rem[head]];
     if (f0.type == FG_ALONE || popc(f0.qmask & ~lowL) > cfg.m - cfg.L) {
       for (int o : f0.origs) {
         FusionItem it;
@@ -430,43 +480,32 @@ void form_passes(const std::vector<FGate>& F, int n, const FusionConfig& cfg,
         it.slot = f0.slot;
         out->push_back(it);
       }
-      done[first] = 1;
+      ++head;
       continue;
     }
-    // 2. grow S from the earliest remaining gate
-    uint64_t S = lowL, blocked = 0;
-    int nS = cfg.L, ngrads = 0;
-    std::vector<int> take;
-    for (size_t j = first; j < F.size(); ++j) {
-      if (done[j]) continue;
-      const FGate& f = F[j];
-      bool ok = f.type != FG_ALONE && !(f.qmask & blocked) && (int)take.size() < cfg.max_ops &&
-                (f.type != FG_GRAD || ngrads + f.ng <= cfg.max_grads);
-      if (ok) {
-        const uint64_t need = f.qmask & ~S;
-        if (nS + popc(need) > cfg.m) {
-          ok = false;
-        } else {
-          S |= need;
-          nS += popc(need);
-        }
+    // 2. the staged set: grown greedily from the earliest remaining operation,
+    // or the contiguous window of high bits that takes more operations.  On
+    // circuits of neighbouring gates a greedy set spreads over many short runs of
+    // qubits, whose light cones close after a layer or two: a random layered
+    // circuit of depth 30 on 28 qubits takes 49 passes, with windows 24.
+    uint64_t S = lowL;
+    int best = collect(&S, true, F.size(), nullptr);
+    for (int b = 0; b < n && popc(S) < cfg.m; ++b) S |= uint64_t(1) << b;
+    const int w = cfg.m - cfg.L;
+    for (int lo = cfg.L; lo + w <= n && n > cfg.m; ++lo) {
+      uint64_t W = lowL | (((uint64_t(1) << w) - 1) << lo);
+      const int ops = collect(&W, false, 2048, nullptr);
+      if (ops > best) {
+        best = ops;
+        S = W;
       }
-      if (ok) {
-        take.push_back((int)j);
-        if (f.type == FG_GRAD) ngrads += f.ng;
-      } else
-        blocked |= f.qmask;
     }
-    for (int b = 0; b < n && nS < cfg.m; ++b)
-      if (!((S >> b) & 1)) {
-        S |= uint64_t(1) << b;
-        ++nS;
-      }
+    std::vector<int> take;
+    collect(&S, false, F.size(), &take);
     // 3. register groups by list scheduling
     std::vector<int> pending = take;
     std::vector<FusedGroup> groups;
     std::vector<int> placed;
-    std::vector<FusionItem> none;
     FusionItem item;
     item.is_pass = true;
     FusedPass& P = item.pass;
@@ -474,11 +513,12 @@ void form_passes(const std::vector<FGate>& F, int n, const FusionConfig& cfg,
       if ((S >> b) & 1) P.S.push_back(b);
     P.L = 0;
     while (P.L < (int)P.S.size() && P.S[P.L] == P.L) ++P.L;
+    int layers = 0;
     while (!pending.empty() && (int)groups.size() < cfg.max_groups) {
-      uint64_t gq = F[pending[0]].qmask, acc = 0;
+      uint64_t gq = F[rem[pending[0]]].qmask, acc = 0;
       std::vector<int> members, rest;
       for (int j : pending) {
-        const FGate& f = F[j];
+        const FGate& f = F[rem[j]];
         if (!(f.qmask & acc) && popc(gq | f.qmask) <= cfg.fuse_k) {
           gq |= f.qmask;
           members.push_back(j);
@@ -487,6 +527,11 @@ void form_passes(const std::vector<FGate>& F, int n, const FusionConfig& cfg,
           rest.push_back(j);
         }
       }
+      // a pass holds so many layers' coefficients; the rest waits for the next
+      std::vector<int> ids;
+      for (int j : members) ids.push_back(rem[j]);
+      layers += count_layers(F, ids) + 1;  // and one for input phases
+      if (layers > cfg.max_layers && !groups.empty()) break;
       // pad every group to the same width (one kernel instantiation per
       // pass; padded bits only widen the thread's tile)
       const int width = std::min<int>(cfg.fuse_k, (int)P.S.size());
@@ -499,14 +544,25 @@ void form_passes(const std::vector<FGate>& F, int n, const FusionConfig& cfg,
         if ((gq >> b) & 1) grp.bits[grp.k++] = local_of(P.S, b);
       for (int j : members) {
         grp.ops.push_back((int)P.gates.size());
-        P.gates.push_back(F[j]);
+        P.gates.push_back(F[rem[j]]);
         placed.push_back(j);
       }
       groups.push_back(grp);
       pending.swap(rest);
     }
     P.groups = groups;
-    for (int j : placed) done[j] = 1;
+    // drop the placed operations; the others up to the last one move up to head's side
+    std::sort(placed.begin(), placed.end());
+    size_t q = placed.size();
+    size_t dst = placed.empty() ? head : (size_t)placed.back() + 1;
+    for (size_t i = dst; i-- > head;) {
+      if (q > 0 && (size_t)placed[q - 1] == i) {
+        --q;
+        continue;
+      }
+      rem[--dst] = rem[i];
+    }
+    head = dst;
     out->push_back(std::move(item));
   }
 }

@@ -246,6 +246,7 @@ struct FusionConfig {
   int max_ops = 200;         // gate capacity of one pass
   int max_grads = 200;       // gradient capacity of one pass (reverse sweeps)
   int max_groups = 64;       // group capacity of one pass
+  int max_layers = 72;       // layer capacity of one pass (coefficients of 4-qubit layers)
 };
 
 FusionConfig fusion_config(int n, sv_dtype dt, int fuse_k);
