@@ -43,6 +43,7 @@ static_assert(SV_BATCH_MAX_QUBITS < 31, "term masks are packed in 31 bits");
 struct BCirc {
   int n, ngates, gate0, ngroups, group0, nparams, nterms, term0;
   int ndiag;  // terms[term0 .. term0 + ndiag) are diagonal (no X or Y factor)
+  int nsign, sign0;  // real-amplitude lists: sign patterns rsigns[sign0 .. sign0 + nsign)
 };
 struct BGateDesc {
   int kind;   // SV_GATE_* (1-qubit kinds)
@@ -72,6 +73,9 @@ struct BatchArgs {
   const BGroup* groups;
   const BOp* ops;
   const BTerm* terms;
+  const BGroup* rgroups;   // the same groups over rops: the real-amplitude kernel's lists
+  const BOp* rops;
+  const uint32_t* rsigns;
   const int* order;      // items, longest first
   const int* item_circ;  // circuit of each item
   const int* theta_off;  // parameter offset of each item
@@ -111,7 +115,10 @@ __device__ __forceinline__ double ksum_value(float2 a) { return (double)a.x - (d
 // Arithmetic classes of a gate's 2x2 matrix: the work per pair drops from 16
 // multiply-adds (dense) to 8 (real: H, X, RY; imaginary off-diagonal: Y, RX;
 // diagonal: RZ), to 4 on one amplitude (phase: U1) or to a sign flip (Z, CZ).
-enum { BC_DENSE = 0, BC_REAL = 1, BC_IMOFF = 2, BC_DIAG = 3, BC_PHASE = 4, BC_NEG = 5 };
+// The real-amplitude kernel's lists also have BC_ROT (RY without controls) and
+// BC_SIGN (a run of sign flips as one pattern, gi its index).
+enum { BC_DENSE = 0, BC_REAL = 1, BC_IMOFF = 2, BC_DIAG = 3, BC_PHASE = 4, BC_NEG = 5,
+       BC_ROT = 6, BC_SIGN = 7 };
 
 // (a, b) <- M (a, b) for every register pair on group bit B (with controls cm
 // when CTRL).
@@ -725,8 +732,99 @@ __device__ __forceinline__ float re_grad(int cm, const float (&p)[1 << K], const
     default: CALL(4); break; \
   }
 
+// The register tile is held as pairs of group bit 0's values (group indices 2 p
+// and 2 p + 1), so that the operations on the other bits are paired fp32
+// instructions whatever the group's place in memory.  An RY without controls is
+// three shears in place, x += a y, y += b x, x += a y with a = -tan(angle / 2) and b =
+// sin(angle), the angle taken modulo pi (a sign of the whole state, which neither
+// the energy nor a gradient sees) so that |a| <= 1; a run of CZs is one
+// multiplication by its sign pattern.  C3's HEA (n = 14, 10 layers): 64 FMAs and 32
+// flips with their dispatches per tile for a rotation and four CZs before, 24 and 16 now;
+// 1024 parameter sets 4.39 -> 3.16 ms (16 warps of 128 registers an SM: the issue slots are
+// half used, and ALU work - tile addresses, signs of the terms - is the busiest pipe).
+template <int K, int B>
+__device__ __forceinline__ void re2_rot(float a, float b, Pair (&v)[1 << (K - 1)]) {
+  if constexpr (B == 0) {
+#pragma unroll
+    for (int p = 0; p < (1 << (K - 1)); ++p) {
+      float2 x = lanes_of(v[p]);
+      x.x = fmaf(a, x.y, x.x);
+      x.y = fmaf(b, x.x, x.y);
+      x.x = fmaf(a, x.y, x.x);
+      v[p] = pair_of(x.x, x.y);
+    }
+  } else {
+    const Pair pa = pair_both(a), pb = pair_both(b);
+#pragma unroll
+    for (int p = 0; p < (1 << (K - 1)); ++p) {
+      if (p & (1 << (B - 1))) continue;
+      const int q = p | (1 << (B - 1));
+      pair_add(v[p], pa, v[q]);
+      pair_add(v[q], pb, v[p]);
+      pair_add(v[p], pa, v[q]);
+    }
+  }
+}
+
+// RY's gradient without controls: sum of l1 p0 - l0 p1 over the pairs of group bit B
+template <int K, int B>
+__device__ __forceinline__ float re2_grad(const Pair (&p)[1 << (K - 1)],
+                                          const Pair (&l)[1 << (K - 1)]) {
+  if constexpr (B == 0) {
+    float x = 0.f, y = 0.f;
+#pragma unroll
+    for (int i = 0; i < (1 << (K - 1)); ++i) {
+      const float2 u = lanes_of(p[i]), w = lanes_of(l[i]);
+      x = fmaf(w.y, u.x, x);
+      y = fmaf(w.x, u.y, y);
+    }
+    return x - y;
+  } else {
+    Pair x = 0, y = 0;
+#pragma unroll
+    for (int i = 0; i < (1 << (K - 1)); ++i) {
+      if (i & (1 << (B - 1))) continue;
+      const int j = i | (1 << (B - 1));
+      pair_add(x, l[j], p[i]);
+      pair_add(y, l[i], p[j]);
+    }
+    const float2 u = lanes_of(x), w = lanes_of(y);
+    return (u.x - w.x) + (u.y - w.y);
+  }
+}
+
 template <int K>
-__device__ void group_fwd_re(float* psi, int n, const BGroup& g, const BOp* ops, const float* mats) {
+__device__ __forceinline__ void re2_signs(const float* sg, Pair (&v)[1 << (K - 1)]) {
+  const ulonglong2* s = reinterpret_cast<const ulonglong2*>(sg);
+#pragma unroll
+  for (int i = 0; i < (1 << (K - 2)); ++i) {
+    const ulonglong2 x = s[i];
+    v[2 * i] = pair_mul(x.x, v[2 * i]);
+    v[2 * i + 1] = pair_mul(x.y, v[2 * i + 1]);
+  }
+}
+
+// any other operation (see re_apply) on the tile as single values
+template <int K, bool DAG>
+__device__ __forceinline__ void re2_other(const BOp& op, const float* M, Pair (&v)[1 << (K - 1)]) {
+  float w[1 << K];
+#pragma unroll
+  for (int p = 0; p < (1 << (K - 1)); ++p) {
+    const float2 x = lanes_of(v[p]);
+    w[2 * p] = x.x;
+    w[2 * p + 1] = x.y;
+  }
+#define SV_OTHER(BB) \
+  if constexpr (BB < K) re_apply<K, BB, DAG>(op, M, w)
+  SV_RE_BITS(op.b0, SV_OTHER)
+#undef SV_OTHER
+#pragma unroll
+  for (int p = 0; p < (1 << (K - 1)); ++p) v[p] = pair_of(w[2 * p], w[2 * p + 1]);
+}
+
+template <int K>
+__device__ void group_fwd_re(float* psi, int n, const BGroup& g, const BOp* ops, const float* mats,
+                             const float* signs) {
   int off[1 << K], lm[K];
   group_offsets_swzr<K>(g, off, lm);
   const int kk = g.k;
@@ -734,26 +832,37 @@ __device__ void group_fwd_re(float* psi, int n, const BGroup& g, const BOp* ops,
   const int width = 1 << kk;
   for (int s = threadIdx.x; s < nsub; s += blockDim.x) {
     const int b = swzr(sub_base<K>(s, lm, kk));
-    float v[1 << K];
+    Pair v[1 << (K - 1)];
 #pragma unroll
-    for (int r = 0; r < (1 << K); ++r) v[r] = r < width ? psi[b ^ off[r]] : 0.f;
+    for (int p = 0; p < (1 << (K - 1)); ++p)
+      v[p] = pair_of(2 * p < width ? psi[b ^ off[2 * p]] : 0.f,
+                     2 * p + 1 < width ? psi[b ^ off[2 * p + 1]] : 0.f);
     for (int o = g.op0; o < g.op1; ++o) {
       const BOp op = ops[o];
-      const float* M = mats + 8 * op.gi;
+      if (op.cls == BC_ROT) {
+        const float a = mats[8 * op.gi + 1], c = mats[8 * op.gi + 3];
 #define SV_FWD_RE(BB) \
-  if constexpr (BB < K) re_apply<K, BB, false>(op, M, v)
-      SV_RE_BITS(op.b0, SV_FWD_RE)
+  if constexpr (BB < K) re2_rot<K, BB>(a, c, v)
+        SV_RE_BITS(op.b0, SV_FWD_RE)
 #undef SV_FWD_RE
+      } else if (op.cls == BC_SIGN) {
+        re2_signs<K>(signs + 32 * op.gi, v);
+      } else {
+        re2_other<K, false>(op, mats + 8 * op.gi, v);
+      }
     }
 #pragma unroll
-    for (int r = 0; r < (1 << K); ++r)
-      if (r < width) psi[b ^ off[r]] = v[r];
+    for (int p = 0; p < (1 << (K - 1)); ++p) {
+      const float2 x = lanes_of(v[p]);
+      if (2 * p < width) psi[b ^ off[2 * p]] = x.x;
+      if (2 * p + 1 < width) psi[b ^ off[2 * p + 1]] = x.y;
+    }
   }
 }
 
 template <int K>
 __device__ void group_bwd_re(float* psi, float* lam, int n, const BGroup& g, const BOp* ops,
-                             const float* mats, float2* wpart) {
+                             const float* mats, const float* signs, float2* wpart) {
   int off[1 << K], lm[K];
   group_offsets_swzr<K>(g, off, lm);
   const int kk = g.k;
@@ -766,43 +875,80 @@ __device__ void group_bwd_re(float* psi, float* lam, int n, const BGroup& g, con
     const int s = threadIdx.x + it * blockDim.x;
     const bool live = s < nsub;
     const int b = live ? swzr(sub_base<K>(s, lm, kk)) : 0;
-    float p[1 << K], l[1 << K];
+    Pair p[1 << (K - 1)], l[1 << (K - 1)];
 #pragma unroll
-    for (int r = 0; r < (1 << K); ++r) {
-      const bool in = live && r < width;
-      p[r] = in ? psi[b ^ off[r]] : 0.f;
-      l[r] = in ? lam[b ^ off[r]] : 0.f;
+    for (int r = 0; r < (1 << (K - 1)); ++r) {
+      const bool in0 = live && 2 * r < width, in1 = live && 2 * r + 1 < width;
+      p[r] = pair_of(in0 ? psi[b ^ off[2 * r]] : 0.f, in1 ? psi[b ^ off[2 * r + 1]] : 0.f);
+      l[r] = pair_of(in0 ? lam[b ^ off[2 * r]] : 0.f, in1 ? lam[b ^ off[2 * r + 1]] : 0.f);
     }
     for (int o = g.op1 - 1; o >= g.op0; --o) {
       const BOp op = ops[o];
-      const float* M = mats + 8 * op.gi;
-      if (op.pauli) {  // RY: generator Y
-        float c = 0.f;
+      if (op.cls == BC_ROT) {
+        if (op.pauli) {  // RY: generator Y
+          float c = 0.f;
 #define SV_GRAD_RE(BB) \
-  if constexpr (BB < K) c = re_grad<K, BB>(op.cm, p, l)
-        SV_RE_BITS(op.b0, SV_GRAD_RE)
+  if constexpr (BB < K) c = re2_grad<K, BB>(p, l)
+          SV_RE_BITS(op.b0, SV_GRAD_RE)
 #undef SV_GRAD_RE
-        c = warp_sum_f(c);
-        if (lane == 0) ksum_add(wpart[warp * kBMaxParams + op.param], c);
-      }
-#define SV_BWD_RE(BB)                        \
-  if constexpr (BB < K) {                    \
-    re_apply<K, BB, true>(op, M, p);         \
-    re_apply<K, BB, true>(op, M, l);         \
+          c = warp_sum_f(c);
+          if (lane == 0) ksum_add(wpart[warp * kBMaxParams + op.param], c);
+        }
+        const float a = -mats[8 * op.gi + 1], c = -mats[8 * op.gi + 3];
+#define SV_BWD_RE(BB)            \
+  if constexpr (BB < K) {        \
+    re2_rot<K, BB>(a, c, p);     \
+    re2_rot<K, BB>(a, c, l);     \
   }
-      SV_RE_BITS(op.b0, SV_BWD_RE)
+        SV_RE_BITS(op.b0, SV_BWD_RE)
 #undef SV_BWD_RE
+      } else if (op.cls == BC_SIGN) {
+        re2_signs<K>(signs + 32 * op.gi, p);
+        re2_signs<K>(signs + 32 * op.gi, l);
+      } else {
+        const float* M = mats + 8 * op.gi;
+        if (op.pauli) {  // controlled RY
+          float u[1 << K], w[1 << K], c = 0.f;
+#pragma unroll
+          for (int r = 0; r < (1 << (K - 1)); ++r) {
+            const float2 x = lanes_of(p[r]), y = lanes_of(l[r]);
+            u[2 * r] = x.x;
+            u[2 * r + 1] = x.y;
+            w[2 * r] = y.x;
+            w[2 * r + 1] = y.y;
+          }
+#define SV_GRAD_RE(BB) \
+  if constexpr (BB < K) c = re_grad<K, BB>(op.cm, u, w)
+          SV_RE_BITS(op.b0, SV_GRAD_RE)
+#undef SV_GRAD_RE
+          c = warp_sum_f(c);
+          if (lane == 0) ksum_add(wpart[warp * kBMaxParams + op.param], c);
+        }
+        re2_other<K, true>(op, M, p);
+        re2_other<K, true>(op, M, l);
+      }
     }
     if (live) {
 #pragma unroll
-      for (int r = 0; r < (1 << K); ++r)
-        if (r < width) {
-          psi[b ^ off[r]] = p[r];
-          lam[b ^ off[r]] = l[r];
+      for (int r = 0; r < (1 << (K - 1)); ++r) {
+        const float2 x = lanes_of(p[r]), y = lanes_of(l[r]);
+        if (2 * r < width) {
+          psi[b ^ off[2 * r]] = x.x;
+          lam[b ^ off[2 * r]] = y.x;
         }
+        if (2 * r + 1 < width) {
+          psi[b ^ off[2 * r + 1]] = x.y;
+          lam[b ^ off[2 * r + 1]] = y.y;
+        }
+      }
     }
   }
 }
+
+// Sign patterns of one circuit's real-amplitude lists in shared memory, 32 floats
+// each; a circuit with more keeps its single flips.
+constexpr int kBMaxSigns = 96;
+constexpr size_t kBSignBytes = sizeof(float) * 32 * kBMaxSigns;
 
 // Real states in shared memory: psi for items up to kBSmemQubits + 1 qubits,
 // lambda beside it up to kBSmemQubits; larger states in the block's global
@@ -818,7 +964,8 @@ __global__ void __launch_bounds__(MAXT, MINB) kbatch_re(const BatchArgs A) {
   BGroup* sgrp = reinterpret_cast<BGroup*>(dyn_smem + kBOpsBytes);
   int2* sterm = reinterpret_cast<int2*>(dyn_smem + kBOpsBytes + kBGroupBytes);
   float* scoef = reinterpret_cast<float*>(dyn_smem + kBOpsBytes + kBGroupBytes + kBTermBytes);
-  float* dyn_state = reinterpret_cast<float*>(dyn_smem + kBCacheBytes);
+  float* ssign = reinterpret_cast<float*>(dyn_smem + kBCacheBytes);
+  float* dyn_state = reinterpret_cast<float*>(dyn_smem + kBCacheBytes + kBSignBytes);
   constexpr int kSm = kBSmemQubits + 1;  // 2^15 floats = kBSmemStateBytes
   const int nwarps = blockDim.x >> 5;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -849,21 +996,27 @@ __global__ void __launch_bounds__(MAXT, MINB) kbatch_re(const BatchArgs A) {
         case SV_GATE_Z: m[3] = -1; break;
         default: m[0] = c; m[1] = -s; m[2] = s; m[3] = c; break;  // RY
       }
-      for (int e = 0; e < 4; ++e) {
-        mats[8 * gi + 2 * e] = (float)m[e];
-        mats[8 * gi + 2 * e + 1] = 0.f;
+      for (int e = 0; e < 4; ++e) mats[8 * gi + 2 * e] = (float)m[e];
+      // RY as shears (see re2_rot): cos >= 0 up to the state's sign
+      if (c < 0) {
+        c = -c;
+        s = -s;
       }
+      mats[8 * gi + 1] = (float)(-s / (1.0 + c));
+      mats[8 * gi + 3] = (float)s;
     }
     for (int x = threadIdx.x; x < dim; x += blockDim.x) psi[x] = x == 0 ? 1.f : 0.f;
     for (int i = threadIdx.x; i < nwarps * kBMaxParams; i += blockDim.x)
       wpart[i] = make_float2(0.f, 0.f);
     {
       const int ng = C.ngroups;
-      const int op_base = ng ? A.groups[C.group0].op0 : 0;
-      const int nops = ng ? A.groups[C.group0 + ng - 1].op1 - op_base : 0;
-      for (int i = threadIdx.x; i < nops; i += blockDim.x) sops[i] = A.ops[op_base + i];
+      const int op_base = ng ? A.rgroups[C.group0].op0 : 0;
+      const int nops = ng ? A.rgroups[C.group0 + ng - 1].op1 - op_base : 0;
+      for (int i = threadIdx.x; i < nops; i += blockDim.x) sops[i] = A.rops[op_base + i];
+      for (int i = threadIdx.x; i < 32 * C.nsign; i += blockDim.x)
+        ssign[i] = (A.rsigns[C.sign0 + (i >> 5)] >> (i & 31)) & 1 ? -1.f : 1.f;
       for (int i = threadIdx.x; i < ng; i += blockDim.x) {
-        BGroup G = A.groups[C.group0 + i];
+        BGroup G = A.rgroups[C.group0 + i];
         G.op0 -= op_base;
         G.op1 -= op_base;
         sgrp[i] = G;
@@ -877,7 +1030,7 @@ __global__ void __launch_bounds__(MAXT, MINB) kbatch_re(const BatchArgs A) {
     }
     __syncthreads();
     for (int gg = 0; gg < C.ngroups; ++gg) {
-      group_fwd_re<K>(psi, C.n, sgrp[gg], sops, mats);
+      group_fwd_re<K>(psi, C.n, sgrp[gg], sops, mats, ssign);
       __syncthreads();
     }
     // lambda = H psi, E = <psi|lambda>
@@ -900,7 +1053,7 @@ __global__ void __launch_bounds__(MAXT, MINB) kbatch_re(const BatchArgs A) {
     if (lane == 0) red[warp] = e;
     __syncthreads();
     for (int gg = C.ngroups - 1; gg >= 0; --gg) {
-      group_bwd_re<K>(psi, lam, C.n, sgrp[gg], sops, mats, wpart);
+      group_bwd_re<K>(psi, lam, C.n, sgrp[gg], sops, mats, ssign, wpart);
       __syncthreads();
     }
     const int toff = A.theta_off[item];
@@ -1259,6 +1412,9 @@ struct sv_batch_s {
   sv::BGroup* groups = nullptr;
   sv::BOp* ops = nullptr;
   sv::BTerm* terms = nullptr;
+  sv::BGroup* rgroups = nullptr;  // real-amplitude lists (batches that may run kbatch_re)
+  sv::BOp* rops = nullptr;
+  uint32_t* rsigns = nullptr;
   int* order = nullptr;
   int* item_circ = nullptr;
   int* theta_off = nullptr;
@@ -1280,6 +1436,9 @@ struct HostPlan {
   std::vector<BGroup> groups;
   std::vector<BOp> ops;
   std::vector<BTerm> terms;
+  std::vector<BGroup> rgroups;  // filled by real_lists
+  std::vector<BOp> rops;
+  std::vector<uint32_t> rsigns;
 };
 
 int popc64(uint64_t x) { return __builtin_popcountll(x); }
@@ -1380,6 +1539,54 @@ bool plan_circuit(const sv_circuit* c, const sv_pauli_sum* H, int k, HostPlan* P
   return P->ops.size() < (size_t)0x7fffffff;
 }
 
+// The real-amplitude kernel's lists of every circuit of P: RYs without controls as
+// rotations, and each run of sign flips with nothing else on their bits in
+// between as one pattern over the group's 2^k indices.
+void real_lists(HostPlan* P) {
+  for (BCirc& C : P->circs) {
+    for (int merge = 1; merge >= 0; --merge) {
+      const size_t o0 = P->rops.size(), s0 = P->rsigns.size(), g0 = P->rgroups.size();
+      for (int g = C.group0; g < C.group0 + C.ngroups; ++g) {
+        BGroup G = P->groups[g];
+        const int a = G.op0, b = G.op1;
+        G.op0 = (int32_t)P->rops.size();
+        int open = -1, dirty = 0;  // the last pattern, and bits touched since
+        for (int o = a; o < b; ++o) {
+          BOp op = P->ops[o];
+          const int bits = op.cm | (1 << op.b0);
+          if (op.cls == BC_NEG && merge) {
+            if (open < 0 || (bits & dirty)) {
+              open = (int)P->rsigns.size();
+              dirty = 0;
+              P->rsigns.push_back(0);
+              BOp sg{};
+              sg.cls = BC_SIGN;
+              sg.param = -1;
+              sg.gi = (int16_t)(open - (int)s0);
+              P->rops.push_back(sg);
+            }
+            for (int r = 0; r < (1 << G.k); ++r)
+              if ((r & bits) == bits) P->rsigns[open] ^= 1u << r;
+            continue;
+          }
+          dirty |= bits;
+          if (op.cls == BC_REAL && op.cm == 0 && P->gates[C.gate0 + op.gi].kind == SV_GATE_RY)
+            op.cls = BC_ROT;
+          P->rops.push_back(op);
+        }
+        G.op1 = (int32_t)P->rops.size();
+        P->rgroups.push_back(G);
+      }
+      C.sign0 = (int)s0;
+      C.nsign = (int)(P->rsigns.size() - s0);
+      if (C.nsign <= kBMaxSigns) break;
+      P->rops.resize(o0);
+      P->rsigns.resize(s0);
+      P->rgroups.resize(g0);
+    }
+  }
+}
+
 template <typename T>
 sv_status upload(T** dst, const std::vector<T>& v) {
   const size_t bytes = std::max<size_t>(1, v.size()) * sizeof(T);
@@ -1389,8 +1596,8 @@ sv_status upload(T** dst, const std::vector<T>& v) {
 }
 
 void free_batch(sv_batch b) {
-  void* ptrs[] = {b->circs, b->gates, b->groups, b->ops, b->terms, b->order,
-                  b->item_circ, b->theta_off, b->queue, b->work};
+  void* ptrs[] = {b->circs, b->gates, b->groups, b->ops, b->terms, b->rgroups,
+                  b->rops, b->rsigns, b->order, b->item_circ, b->theta_off, b->queue, b->work};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
@@ -1425,6 +1632,9 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
   A.groups = b->groups;
   A.ops = b->ops;
   A.terms = b->terms;
+  A.rgroups = b->rgroups;
+  A.rops = b->rops;
+  A.rsigns = b->rsigns;
   A.order = b->order;
   A.item_circ = b->item_circ;
   A.theta_off = b->theta_off;
@@ -1438,14 +1648,15 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
   SV_CUDA_TRY(cudaMemsetAsync(b->queue, 0, sizeof(int), st));
   if (re) {
     BatchKernel kern = real_kernel_for(k);
+    constexpr size_t smem = kBCacheBytes + kBSignBytes + kBSmemStateBytes;
     static bool attr[6] = {false, false, false, false, false, false};
     if (!attr[k]) {
-      SV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(kBCacheBytes + kBSmemStateBytes)));
+      SV_CUDA_TRY(
+          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       attr[k] = true;
     }
     ProfScope prof(st, "kbatch_re");
-    kern<<<blocks, 512, kBCacheBytes + kBSmemStateBytes, st>>>(A);
+    kern<<<blocks, 512, smem, st>>>(A);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return check_launch("batch kernel (real amplitudes)");
   }
@@ -1691,15 +1902,20 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
         set_error("sv_batch_create: a gate does not fit a register group of %d qubits", k);
         return SV_ERR_INVALID;
       }
-    void* olds[] = {b->circs, b->gates, b->groups, b->ops, b->terms};
+    if (all_real) real_lists(&P);
+    void* olds[] = {b->circs, b->gates, b->groups, b->ops, b->terms, b->rgroups, b->rops, b->rsigns};
     for (void* p : olds)
       if (p) cudaFree(p);
     b->circs = nullptr; b->gates = nullptr; b->groups = nullptr; b->ops = nullptr; b->terms = nullptr;
+    b->rgroups = nullptr; b->rops = nullptr; b->rsigns = nullptr;
     sv_status s2 = upload(&b->circs, P.circs);
     if (!s2) s2 = upload(&b->gates, P.gates);
     if (!s2) s2 = upload(&b->groups, P.groups);
     if (!s2) s2 = upload(&b->ops, P.ops);
     if (!s2) s2 = upload(&b->terms, P.terms);
+    if (!s2 && all_real) s2 = upload(&b->rgroups, P.rgroups);
+    if (!s2 && all_real) s2 = upload(&b->rops, P.rops);
+    if (!s2 && all_real) s2 = upload(&b->rsigns, P.rsigns);
     return s2;
   };
   double* th = nullptr;

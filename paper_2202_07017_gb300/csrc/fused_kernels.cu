@@ -615,36 +615,6 @@ __device__ __forceinline__ void run_layers(typename Cplx2<R>::T* sm, int m, cons
 constexpr int kPlaneQubits = 12;
 constexpr int kLiftQubits = 10;  // smallest slice of passes with lift: one warp
 
-// A pair of fp32 lanes in one 64-bit register: the arithmetic below stays on
-// these from load to store, so that every step is one paired instruction
-// (float2 values assembled from parts were split into scalar FMAs and moves).
-typedef unsigned long long Pair;
-
-__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
-  Pair d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ Pair pair_of(float x, float y) {
-  Pair d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
-  return d;
-}
-__device__ __forceinline__ float2 lanes_of(Pair p) {
-  float2 v;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ Pair pair_both(float x) { return pair_of(x, x); }
-__device__ __forceinline__ Pair pair_swap(Pair p) {
-  const float2 v = lanes_of(p);
-  return pair_of(v.y, v.x);
-}
-// p += a q
-__device__ __forceinline__ void pair_add(Pair& p, Pair a, Pair q) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(p) : "l"(a), "l"(q));
-}
-
 // The rotation (a, b) on bit B of the tile index
 template <int B, bool LIFT>
 __device__ __forceinline__ void plane_rot(float a, float b, Pair (&re)[16], Pair (&im)[16]) {

@@ -475,17 +475,8 @@ struct XChunkDev {
   double w0, w[4 * kXCGroups];  // 2 sum c_k over the terms on bit 0, on bit i of group g
 };
 
-typedef unsigned long long PairP;
-__device__ __forceinline__ void fma2_add(PairP& d, PairP a, PairP b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ float2 lanes2(PairP p) {
-  float2 v;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ float lane_sum(PairP p) {
-  const float2 v = lanes2(p);
+__device__ __forceinline__ float lane_sum(Pair p) {
+  const float2 v = lanes_of(p);
   return v.x + v.y;
 }
 __device__ __forceinline__ int cswz(int q) { return q ^ ((q >> 3) & 7); }
@@ -570,7 +561,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       if (!live || half + 2 * j >= P.ngroups) break;
-      PairP a[16], b[16];  // amplitudes 2 q and 2 q + 1 as (re, im)
+      Pair a[16], b[16];  // amplitudes 2 q and 2 q + 1 as (re, im)
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
         int o = tile[j];
@@ -583,19 +574,19 @@ __global__ void __launch_bounds__(kPThreads, 1)
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        PairP x = 0, y = 0;
+        Pair x = 0, y = 0;
 #pragma unroll
         for (int r = 0; r < 16; ++r) {
           if (r & (1 << i)) continue;
-          fma2_add(x, a[r], a[r | (1 << i)]);
-          fma2_add(y, b[r], b[r | (1 << i)]);
+          pair_add(x, a[r], a[r | (1 << i)]);
+          pair_add(y, b[r], b[r | (1 << i)]);
         }
         acc[j][i].add(lane_sum(x) + lane_sum(y));
       }
       if (j == 0 && half == 0) {
-        PairP x = 0;
+        Pair x = 0;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) fma2_add(x, a[r], b[r]);
+        for (int r = 0; r < 16; ++r) pair_add(x, a[r], b[r]);
         acc0.add(lane_sum(x));
       }
     }

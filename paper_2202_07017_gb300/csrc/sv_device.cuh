@@ -155,6 +155,36 @@ __device__ __forceinline__ void mv2_dither(const M2<float>& g, float& ar, float&
   bi = nbi;
 }
 
+// A pair of fp32 lanes in one 64-bit register: the arithmetic below stays on
+// these from load to store, so that every step is one paired instruction
+// (float2 values assembled from parts were split into scalar FMAs and moves).
+typedef unsigned long long Pair;
+
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  Pair d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ Pair pair_of(float x, float y) {
+  Pair d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float2 lanes_of(Pair p) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ Pair pair_both(float x) { return pair_of(x, x); }
+__device__ __forceinline__ Pair pair_swap(Pair p) {
+  const float2 v = lanes_of(p);
+  return pair_of(v.y, v.x);
+}
+// p += a q
+__device__ __forceinline__ void pair_add(Pair& p, Pair a, Pair q) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(p) : "l"(a), "l"(q));
+}
+
 // A thread's running sum: compensated (Kahan) in fp32 for complex64 kernels
 // (GB300 issues fp64 at a small fraction of the fp32 rate, so the per-unit
 // additions stay in fp32 and s - c meets the fp64 block sum once), plain fp64
