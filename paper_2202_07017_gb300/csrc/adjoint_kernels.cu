@@ -105,10 +105,13 @@ __global__ void __launch_bounds__(kRedThreads)
   }
 }
 
-template <typename I, int PAULI>
+// Bound by fp64 issue.  SK: the un-applied gate as shears (see shear2; 6 fp64
+// instructions per state and pair instead of 16): n = 21, RY and RZ, 65 -> 33.6 us
+// a gate (HBM and L2: 128 MiB of states, read and written).
+template <typename I, int PAULI, int SK>
 __global__ void __launch_bounds__(kRedThreads)
     kadj_c128(double2* __restrict__ psi, double2* __restrict__ lam, I n_units, Ins<I> ins,
-              I tmask, I cmask, M2<double> g, double* __restrict__ partials) {
+              I tmask, I cmask, M2<double> g, Shear2 h, double* __restrict__ partials) {
   grid_dependency_wait();
   double acc = 0.0;
   for (I u = (I)blockIdx.x * kRedThreads + threadIdx.x; u < n_units;
@@ -116,8 +119,13 @@ __global__ void __launch_bounds__(kRedThreads)
     const I lo = insert_zeros(u, ins) | cmask, hi = lo | tmask;
     double2 p0 = psi[lo], p1 = psi[hi], l0 = lam[lo], l1 = lam[hi];
     if (PAULI) acc += im_lpp<PAULI>(l0.x, l0.y, l1.x, l1.y, p0.x, p0.y, p1.x, p1.y);
-    mv2<MK_DENSE>(g, p0.x, p0.y, p1.x, p1.y);
-    mv2<MK_DENSE>(g, l0.x, l0.y, l1.x, l1.y);
+    if constexpr (SK != SK_NONE) {
+      shear2<SK>(h, p0.x, p0.y, p1.x, p1.y);
+      shear2<SK>(h, l0.x, l0.y, l1.x, l1.y);
+    } else {
+      mv2<MK_DENSE>(g, p0.x, p0.y, p1.x, p1.y);
+      mv2<MK_DENSE>(g, l0.x, l0.y, l1.x, l1.y);
+    }
     psi[lo] = p0;
     psi[hi] = p1;
     lam[lo] = l0;
@@ -166,8 +174,13 @@ void run_adj(void* psi, void* lam, sv_dtype dt, int n, cudaStream_t st, int tp, 
     }
     Ins<I> ins = make_ins<I>(pos);
     const I nu = I(1) << (n - (int)pos.size());
-    launch_dependent(kadj_c128<I, PAULI>, grid, kRedThreads, 0, st, (double2*)psi, (double2*)lam,
-                     nu, ins, I(1) << tp, cmask, to_m2<double>(G), partials);
+    const Shear2 h = make_shear2(G);
+    const auto kern = h.kind == SK_REAL     ? kadj_c128<I, PAULI, SK_REAL>
+                      : h.kind == SK_IMOFF  ? kadj_c128<I, PAULI, SK_IMOFF>
+                      : h.kind == SK_PHASES ? kadj_c128<I, PAULI, SK_PHASES>
+                                            : kadj_c128<I, PAULI, SK_NONE>;
+    launch_dependent(kern, grid, kRedThreads, 0, st, (double2*)psi, (double2*)lam, nu, ins,
+                     I(1) << tp, cmask, to_m2<double>(G), h, partials);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }

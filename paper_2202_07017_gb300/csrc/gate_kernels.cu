@@ -136,10 +136,12 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ---- complex128 1-qubit: one amplitude per vector ---------------------------------
-template <typename I, int MK, int ITEMS>
+// Bound by fp64 issue.  H at n = 27: 1046 us with the products, 812 with
+// shears (HBM: 641 us).
+template <typename I, int MK, int SK, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     k1q_c128_pair(double2* __restrict__ psi, I n_units, Ins<I> ins, I tmask, I cmask,
-                  M2<double> g) {
+                  M2<double> g, Shear2 h) {
   const int T = block_threads<ITEMS>();
   const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
   grid_dependency_wait();
@@ -159,7 +161,10 @@ __global__ void __launch_bounds__(kThreads)
     const I u = base + (I)(it * T);
     if (u < n_units) {
       double2 x = a[it], y = b[it];
-      mv2<MK>(g, x.x, x.y, y.x, y.y);
+      if constexpr (SK != SK_NONE)
+        shear2<SK>(h, x.x, x.y, y.x, y.y);
+      else
+        mv2<MK>(g, x.x, x.y, y.x, y.y);
       psi[lo[it]] = x;
       psi[lo[it] | tmask] = y;
     }
@@ -196,10 +201,12 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-template <typename I, int PK, int ITEMS>
+// SH: a phase of modulus 1 as shears.  Controlled phases at n = 27: 274 us, now
+// 213 (HBM: 160 us).
+template <typename I, int PK, bool SH, int ITEMS>
 __global__ void __launch_bounds__(kThreads)
     kphase_c128(double2* __restrict__ psi, I n_units, Ins<I> ins, I omask, double c,
-                double s) {
+                double s, Shear h) {
   const int T = block_threads<ITEMS>();
   const I base = (I)blockIdx.x * (I)(T * ITEMS) + (I)threadIdx.x;
   grid_dependency_wait();
@@ -218,7 +225,10 @@ __global__ void __launch_bounds__(kThreads)
     const I u = base + (I)(it * T);
     if (u < n_units) {
       double2 x = a[it];
-      rot<PK>(c, s, x.x, x.y);
+      if constexpr (SH)
+        shear_rot(h, x.x, x.y);
+      else
+        rot<PK>(c, s, x.x, x.y);
       psi[v[it]] = x;
     }
   }
@@ -526,9 +536,9 @@ void run_1q_c64(float4* psi, int n, cudaStream_t st, int t, int nc, const int* c
   }
 }
 
-template <typename I, int MK>
+template <typename I, int MK, int SK>
 void run_1q_c128(double2* psi, int n, cudaStream_t st, int t, int nc, const int* cp,
-                 const M2<double>& g) {
+                 const M2<double>& g, const Shear2& h) {
   std::vector<int> pos{t};
   I cmask = 0;
   for (int j = 0; j < nc; ++j) {
@@ -539,10 +549,10 @@ void run_1q_c128(double2* psi, int n, cudaStream_t st, int t, int nc, const int*
   const I tmask = I(1) << t;
   const I nu = I(1) << (n - (int)pos.size());
   const Shape sh = shape_for(nu, items_pair());
-    with_items(sh, [&](auto it) {
+  with_items(sh, [&](auto it) {
     constexpr int IT = decltype(it)::value;
-    launch_k(k1q_c128_pair<I, MK, IT>, "k1q_c128_pair", sh, st, psi, nu, ins,
-             tmask, cmask, g);
+    launch_k(k1q_c128_pair<I, MK, SK, IT>, "k1q_c128_pair", sh, st, psi, nu, ins, tmask, cmask, g,
+             h);
   });
 }
 
@@ -562,11 +572,18 @@ void run_1q(void* data, sv_dtype dt, int n, cudaStream_t st, int t, int nc, cons
   } else {
     double2* psi = (double2*)data;
     M2<double> g = to_m2<double>(G);
+    const Shear2 h = make_shear2(G);
+    switch (h.kind) {
+      case SK_REAL: run_1q_c128<I, MK_DENSE, SK_REAL>(psi, n, st, t, nc, cp, g, h); return;
+      case SK_IMOFF: run_1q_c128<I, MK_DENSE, SK_IMOFF>(psi, n, st, t, nc, cp, g, h); return;
+      case SK_PHASES: run_1q_c128<I, MK_DENSE, SK_PHASES>(psi, n, st, t, nc, cp, g, h); return;
+      default: break;
+    }
     switch (mk) {
-      case MK_DIAG: run_1q_c128<I, MK_DIAG>(psi, n, st, t, nc, cp, g); break;
-      case MK_REAL: run_1q_c128<I, MK_REAL>(psi, n, st, t, nc, cp, g); break;
-      case MK_IMOFF: run_1q_c128<I, MK_IMOFF>(psi, n, st, t, nc, cp, g); break;
-      default: run_1q_c128<I, MK_DENSE>(psi, n, st, t, nc, cp, g); break;
+      case MK_DIAG: run_1q_c128<I, MK_DIAG, SK_NONE>(psi, n, st, t, nc, cp, g, h); break;
+      case MK_REAL: run_1q_c128<I, MK_REAL, SK_NONE>(psi, n, st, t, nc, cp, g, h); break;
+      case MK_IMOFF: run_1q_c128<I, MK_IMOFF, SK_NONE>(psi, n, st, t, nc, cp, g, h); break;
+      default: run_1q_c128<I, MK_DENSE, SK_NONE>(psi, n, st, t, nc, cp, g, h); break;
     }
   }
 }
@@ -591,6 +608,8 @@ void run_phase_pk(void* data, sv_dtype dt, int n, cudaStream_t st, const std::ve
     });
   } else {
     double2* psi = (double2*)data;
+    Shear h{};
+    const bool shears = make_shear(ph.re, ph.im, &h);
     I omask = 0;
     for (int b : bits) omask |= I(1) << b;
     Ins<I> ins = make_ins<I>(bits);
@@ -598,8 +617,12 @@ void run_phase_pk(void* data, sv_dtype dt, int n, cudaStream_t st, const std::ve
     const Shape sh = shape_for(nu, items_single());
     with_items(sh, [&](auto it) {
       constexpr int IT = decltype(it)::value;
-      launch_k(kphase_c128<I, PK, IT>, "kphase_c128", sh, st, psi, nu, ins, omask,
-               ph.re, ph.im);
+      if (PK == PK_GEN && shears)
+        launch_k(kphase_c128<I, PK, PK == PK_GEN, IT>, "kphase_c128", sh, st, psi, nu, ins, omask,
+                 ph.re, ph.im, h);
+      else
+        launch_k(kphase_c128<I, PK, false, IT>, "kphase_c128", sh, st, psi, nu, ins, omask, ph.re,
+                 ph.im, h);
     });
   }
 }

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 #include <vector>
 
@@ -85,6 +86,90 @@ __device__ __forceinline__ void mv2(const M2<R>& g, R& ar, R& ai, R& br, R& bi) 
   ai = nai;
   br = nbr;
   bi = nbi;
+}
+
+// ---- complex128: rotations as shears ------------------------------------------------
+// GB300 issues fp64 at 1/64 of its fp32 rate, so complex128 gates are bound by
+// their fp64 instructions.  A rotation by an angle of at most pi / 4 is three
+// shears, x += a y, y += b x, x += a y with a = -tan(angle / 2), b = sin(angle): three
+// FMAs where the products take four instructions; whole quarter turns k come off
+// first, exactly and without fp64 arithmetic.
+struct Shear {
+  double a, b;
+  int k;
+};
+
+// (x, y) <- the rotation of (x, y); i^k by selects and sign bits, without branches
+// (which would keep a thread's other units from overlapping this one's FMAs:
+// 274 -> 394 us a phase kernel at n = 27 instead of 213)
+__device__ __forceinline__ void shear_rot(const Shear& h, double& x, double& y) {
+  const long long sx = (long long)((unsigned)(h.k + 1) & 2u) << 62, sy = (long long)(h.k & 2) << 62;
+  const double u = (h.k & 1) ? y : x, v = (h.k & 1) ? x : y;
+  x = __longlong_as_double(__double_as_longlong(u) ^ sx);
+  y = __longlong_as_double(__double_as_longlong(v) ^ sy);
+  x = fma(h.a, y, x);
+  y = fma(h.b, x, y);
+  x = fma(h.a, y, x);
+}
+
+// (a, b) <- G (a, b) for the 2x2s that are rotations: SK_REAL [[c, -s], [s, c]]
+// (h[0]; refl: of (a, -b), as H), SK_IMOFF [[c, i s], [i s, c]] (h[0], RX), SK_PHASES
+// diag(e^{i f}, e^{i g}) (h[0], h[1], RZ).  SK_NONE: none of them.
+enum { SK_NONE = 0, SK_REAL = 1, SK_IMOFF = 2, SK_PHASES = 3 };
+struct Shear2 {
+  int kind, refl;
+  Shear h[2];
+};
+
+template <int SK>
+__device__ __forceinline__ void shear2(const Shear2& g, double& ar, double& ai, double& br,
+                                       double& bi) {
+  if (SK == SK_REAL) {
+    // sign bits, not negations (which would go through the fp64 pipe)
+    const long long sg = (long long)g.refl << 63;
+    br = __longlong_as_double(__double_as_longlong(br) ^ sg);
+    bi = __longlong_as_double(__double_as_longlong(bi) ^ sg);
+    shear_rot(g.h[0], ar, br);
+    shear_rot(g.h[0], ai, bi);
+  } else if (SK == SK_IMOFF) {
+    shear_rot(g.h[0], ar, bi);
+    shear_rot(g.h[0], br, ai);
+  } else {
+    shear_rot(g.h[0], ar, ai);
+    shear_rot(g.h[1], br, bi);
+  }
+}
+
+// The shears of cos + i sin; false unless it has modulus 1 to fp64 rounding.
+inline bool make_shear(double c, double s, Shear* h) {
+  if (!(std::fabs(c * c + s * s - 1.0) < 4e-15)) return false;
+  int k = 0;  // (c, s) = i^k (c', s') with c' >= |s'|
+  while (k < 4 && !(c > 0 && c >= std::fabs(s))) {
+    const double t = c;  // times -i
+    c = s;
+    s = -t;
+    ++k;
+  }
+  *h = {-s / (1.0 + c), s, k & 3};
+  return k < 4;
+}
+
+// The shear form of a 2x2, kind SK_NONE if it has none.
+inline Shear2 make_shear2(const HostMatrix& G) {
+  Shear2 g{};
+  const cd u = G.at(0, 0), v = G.at(0, 1), w = G.at(1, 0), x = G.at(1, 1);
+  const bool real = u.im == 0 && v.im == 0 && w.im == 0 && x.im == 0;
+  if (v.re == 0 && v.im == 0 && w.re == 0 && w.im == 0) {
+    if (make_shear(u.re, u.im, &g.h[0]) && make_shear(x.re, x.im, &g.h[1])) g.kind = SK_PHASES;
+  } else if (real && v.re == -w.re && u.re == x.re) {
+    if (make_shear(u.re, w.re, &g.h[0])) g.kind = SK_REAL;
+  } else if (real && v.re == w.re && u.re == -x.re) {
+    g.refl = 1;
+    if (make_shear(u.re, w.re, &g.h[0])) g.kind = SK_REAL;
+  } else if (u.im == 0 && x.im == 0 && v.re == 0 && w.re == 0 && u.re == x.re && v.im == w.im) {
+    if (make_shear(u.re, v.im, &g.h[0])) g.kind = SK_IMOFF;
+  }
+  return g;
 }
 
 // ---- complex64: dithered rounding ---------------------------------------------
