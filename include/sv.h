@@ -369,8 +369,9 @@ sv_status sv_grad_fused(sv_state s, const sv_circuit* c, const double* theta,
  * hamiltonians[item_circuit[i]] and the adjoint gradient dE_i/dtheta.  All
  * items run in one persistent kernel whose thread blocks pull items from an
  * atomic queue (longest first); each block keeps its item's two states in a
- * workspace slot that stays in L1/L2, or (a variant the autotuner may pick)
- * psi of up to 14 qubits and lambda of up to 13 in shared memory.  Energies
+ * workspace slot that stays in L1/L2, or (variants the autotuner may pick)
+ * in shared memory as far as they fit: psi of up to 14 qubits and lambda of up
+ * to 13 with one block per SM.  Energies
  * and gradients accumulate per warp in compensated fp32 and across warps in
  * fp64, in a fixed order.  A batch whose gates are all real (H X Z RY, with
  * controls) and whose terms are all real matrices (an even number of Y
@@ -390,14 +391,13 @@ sv_status sv_grad_fused(sv_state s, const sv_circuit* c, const double* theta,
  * sv_batch_create uploads the descriptors and allocates the workspace.
  * tune = 0: single blocks of 256 threads, 2 per SM, register groups of k = 4
  * qubits, states in a global workspace slot per block.  tune = 1: the
- * autotuner times every (register-group width k in {2,3,4}, kernel: those
- * single blocks with 128/256/512 threads and 1/2/4/8 blocks per SM, single
- * blocks of 512 threads keeping psi (and lambda up to 13 qubits) in shared
- * memory up to 14 qubits, or two-block clusters of 512 threads that split each item's psi and lambda by
- * their top bit over the pair and keep them in shared memory up to 14 qubits,
- * k <= 3) on the batch and keeps the fastest (this synchronises the device).
- * For a real batch the autotuner also times the real-amplitude kernel
- * (single blocks of 512 threads, k in {3,4,5}).
+ * autotuner times on the batch, and keeps the fastest of (this synchronises the
+ * device): those single blocks with k in {2,3,4}, 128 or 256 threads and 2, 4 or 8
+ * per SM; single blocks of 512, 256 or 128 threads, 1, 2 or 4 per SM, keeping states
+ * in shared memory as far as they fit; and two-block clusters of 512 threads that
+ * split each item's psi and lambda by their top bit over the pair and keep them in
+ * shared memory up to 14 qubits, k <= 3.  For a real batch the autotuner also times
+ * the real-amplitude kernel (512, 256 or 128 threads, k in {3,4,5}).
  * tune = 2: the cluster kernel with k = 3 (the tune = 0 tile if a gate has 3
  * controls); tune = 3: single blocks of 512 threads with states in shared
  * memory, k = 4; tune = 4: the real-amplitude kernel, k = 4 (SV_ERR_INVALID

@@ -36,25 +36,25 @@ namespace {
 
 constexpr int kBMaxGates = 480;    // gates of one circuit (static smem stays < 48 KB)
 constexpr int kBMaxParams = 256;   // parameters of one circuit
-constexpr int kBMaxWarps = 16;     // 512 threads
 constexpr int kBMaxTerms = 64;     // Pauli terms of one Hamiltonian
 static_assert(SV_BATCH_MAX_QUBITS < 31, "term masks are packed in 31 bits");
 
 struct BCirc {
   int n, ngates, gate0, ngroups, group0, nparams, nterms, term0;
   int ndiag;  // terms[term0 .. term0 + ndiag) are diagonal (no X or Y factor)
-  int nsign, sign0;  // real-amplitude lists: sign patterns rsigns[sign0 .. sign0 + nsign)
+  int nsign, sign0;  // the single-block kernels' sign patterns, rsigns[sign0 .. sign0 + nsign)
 };
 struct BGateDesc {
   int kind;   // SV_GATE_* (1-qubit kinds)
   int param;  // -1: fixed angle
   double angle;
+  int free_rot;  // RX, RY or RZ without controls
 };
-struct BGroup {
+struct alignas(16) BGroup {
   uint8_t k, bits[5];
   int32_t op0, op1;
 };
-struct BOp {
+struct alignas(8) BOp {
   uint8_t b0;     // group-local target index
   uint8_t cm;     // group-local control mask
   uint8_t pauli;  // generator for gradients: 0 none, 1 X, 2 Y, 3 Z
@@ -73,7 +73,7 @@ struct BatchArgs {
   const BGroup* groups;
   const BOp* ops;
   const BTerm* terms;
-  const BGroup* rgroups;   // the same groups over rops: the real-amplitude kernel's lists
+  const BGroup* rgroups;   // the same groups over rops: the single-block kernels' lists
   const BOp* rops;
   const uint32_t* rsigns;
   const int* order;      // items, longest first
@@ -85,6 +85,10 @@ struct BatchArgs {
   double* grad;
   float2* work;          // gridDim.x slots of 2 x 2^nmax amplitudes
   int* queue;
+  // the single-block kernels' dynamic shared memory (byte offsets, see BSmem)
+  int o_mats, o_wpart, o_ops, o_grp, o_term, o_tcoef, o_sign, o_state;
+  int pstride;       // gradient partials of one warp
+  int state_floats;  // floats of state memory from o_state
 };
 
 __device__ __forceinline__ float warp_sum_f(float v) {
@@ -115,10 +119,10 @@ __device__ __forceinline__ double ksum_value(float2 a) { return (double)a.x - (d
 // Arithmetic classes of a gate's 2x2 matrix: the work per pair drops from 16
 // multiply-adds (dense) to 8 (real: H, X, RY; imaginary off-diagonal: Y, RX;
 // diagonal: RZ), to 4 on one amplitude (phase: U1) or to a sign flip (Z, CZ).
-// The real-amplitude kernel's lists also have BC_ROT (RY without controls) and
-// BC_SIGN (a run of sign flips as one pattern, gi its index).
+// The single-block kernels' lists also have BC_SIGN (a run of sign flips as one
+// pattern, gi its index) and rotations without controls.
 enum { BC_DENSE = 0, BC_REAL = 1, BC_IMOFF = 2, BC_DIAG = 3, BC_PHASE = 4, BC_NEG = 5,
-       BC_ROT = 6, BC_SIGN = 7 };
+       BC_SIGN = 6, BC_ROT = 7, BC_RX = 8, BC_RZ = 9 };
 
 // (a, b) <- M (a, b) for every register pair on group bit B (with controls cm
 // when CTRL).
@@ -235,63 +239,6 @@ __device__ __forceinline__ void pair_apply_dag(int cls, const float* M, int cm,
   pair_apply<K, B>(cls, h, cm, re, im);
 }
 
-// M^dagger on the pairs of two tiles (psi and lambda) behind one dispatch
-template <int K, int B, int CLS, bool CTRL>
-__device__ __forceinline__ void pair_apply_c2(const float* h, int cm, float (&pr)[1 << K],
-                                              float (&pi)[1 << K], float (&lr)[1 << K],
-                                              float (&li)[1 << K]) {
-  pair_apply_c<K, B, CLS, CTRL>(h, cm, pr, pi);
-  pair_apply_c<K, B, CLS, CTRL>(h, cm, lr, li);
-}
-
-template <int K, int B, int CLS, int CM>
-__device__ __forceinline__ void pair_apply_cm2(const float* h, float (&pr)[1 << K],
-                                               float (&pi)[1 << K], float (&lr)[1 << K],
-                                               float (&li)[1 << K]) {
-  pair_apply_cm<K, B, CLS, CM>(h, pr, pi);
-  pair_apply_cm<K, B, CLS, CM>(h, lr, li);
-}
-
-template <int K, int B, int CLS>
-__device__ __forceinline__ void pair_apply_ctrl2(const float* h, int cm, float (&pr)[1 << K],
-                                                 float (&pi)[1 << K], float (&lr)[1 << K],
-                                                 float (&li)[1 << K]) {
-#define SV_CM_CASE(v)                                                            \
-  case v:                                                                        \
-    if constexpr (v < (1 << K)) pair_apply_cm2<K, B, CLS, v>(h, pr, pi, lr, li); \
-    break;
-  switch (cm) {
-    SV_CM_CASE(1) SV_CM_CASE(2) SV_CM_CASE(3) SV_CM_CASE(4) SV_CM_CASE(5)
-    SV_CM_CASE(6) SV_CM_CASE(7) SV_CM_CASE(8) SV_CM_CASE(9) SV_CM_CASE(10)
-    SV_CM_CASE(11) SV_CM_CASE(12) SV_CM_CASE(13) SV_CM_CASE(14) SV_CM_CASE(15)
-    default: pair_apply_c2<K, B, CLS, true>(h, cm, pr, pi, lr, li); break;
-  }
-#undef SV_CM_CASE
-}
-
-template <int K, int B>
-__device__ __forceinline__ void pair_apply_dag2(int cls, const float* M, int cm,
-                                                float (&pr)[1 << K], float (&pi)[1 << K],
-                                                float (&lr)[1 << K], float (&li)[1 << K]) {
-  const float h[8] = {M[0], -M[1], M[4], -M[5], M[2], -M[3], M[6], -M[7]};
-  if (cm) {
-    switch (cls) {
-      case BC_PHASE: pair_apply_ctrl2<K, B, BC_PHASE>(h, cm, pr, pi, lr, li); break;
-      case BC_NEG: pair_apply_ctrl2<K, B, BC_NEG>(h, cm, pr, pi, lr, li); break;
-      default: pair_apply_c2<K, B, BC_DENSE, true>(h, cm, pr, pi, lr, li); break;
-    }
-  } else {
-    switch (cls) {
-      case BC_REAL: pair_apply_c2<K, B, BC_REAL, false>(h, 0, pr, pi, lr, li); break;
-      case BC_IMOFF: pair_apply_c2<K, B, BC_IMOFF, false>(h, 0, pr, pi, lr, li); break;
-      case BC_DIAG: pair_apply_c2<K, B, BC_DIAG, false>(h, 0, pr, pi, lr, li); break;
-      case BC_PHASE: pair_apply_c2<K, B, BC_PHASE, false>(h, 0, pr, pi, lr, li); break;
-      case BC_NEG: pair_apply_c2<K, B, BC_NEG, false>(h, 0, pr, pi, lr, li); break;
-      default: pair_apply_c2<K, B, BC_DENSE, false>(h, 0, pr, pi, lr, li); break;
-    }
-  }
-}
-
 // sum over the pairs of Im( conj(l0) (P p)_0 + conj(l1) (P p)_1 )
 template <int K, int B, int PAULI, bool CTRL>
 __device__ __forceinline__ float pair_grad_c(int cm, const float (&pr)[1 << K],
@@ -350,23 +297,6 @@ __device__ void group_offsets(const BGroup& g, int (&off)[1 << K], int (&lm)[K])
   for (int i = 0; i < K; ++i) lm[i] = (1 << g.bits[i]) - 1;
 }
 
-// Storage order of a single-block item's states: amplitude x lives at
-// swzb(x) = x ^ ((x >> 4) & 15).  The map is a bijection of [0, 2^n) for every
-// n and linear over XOR, so swzb(b | off) = swzb(b) ^ swzb(off) for disjoint
-// bits.  It spreads the 16 amplitudes of a 128-byte row over the row by the
-// next four index bits: a warp whose lanes step over a register group's low
-// bits then reaches 16 different 8-byte bank pairs instead of one.
-__device__ __forceinline__ int swzb(int x) { return x ^ ((x >> 4) & 15); }
-
-template <int K>
-__device__ void group_offsets_swzb(const BGroup& g, int (&off)[1 << K], int (&lm)[K]) {
-  off[0] = 0;
-#pragma unroll
-  for (int r = 1; r < (1 << K); ++r) off[r] = off[r & (r - 1)] ^ swzb(1 << g.bits[lowbit_b(r)]);
-#pragma unroll
-  for (int i = 0; i < K; ++i) lm[i] = (1 << g.bits[i]) - 1;
-}
-
 template <int K>
 __device__ __forceinline__ int sub_base(int s, const int (&lm)[K], int kk) {
   int b = s;
@@ -376,274 +306,40 @@ __device__ __forceinline__ int sub_base(int s, const int (&lm)[K], int kk) {
   return b;
 }
 
-// forward: psi <- group ops in order
-template <int K>
-__device__ void group_fwd(float2* psi, int n, const BGroup& g, const BOp* ops, const float* mats) {
-  int off[1 << K], lm[K];
-  group_offsets_swzb<K>(g, off, lm);
-  const int kk = g.k;
-  const int nsub = 1 << (n - kk);
-  const int width = 1 << kk;
-  for (int s = threadIdx.x; s < nsub; s += blockDim.x) {
-    const int b = swzb(sub_base<K>(s, lm, kk));
-    float re[1 << K], im[1 << K];
-#pragma unroll
-    for (int r = 0; r < (1 << K); ++r)
-      if (r < width) {
-        const float2 v = psi[b ^ off[r]];
-        re[r] = v.x;
-        im[r] = v.y;
-      }
-    for (int o = g.op0; o < g.op1; ++o) {
-      const BOp op = ops[o];
-      const float* M = mats + 8 * op.gi;
-#define SV_FWD(BB) \
-  if constexpr (BB < K) pair_apply<K, BB>(op.cls, M, op.cm, re, im)
-      SV_BIT_SWITCH(op.b0, SV_FWD)
-#undef SV_FWD
-    }
-#pragma unroll
-    for (int r = 0; r < (1 << K); ++r)
-      if (r < width) psi[b ^ off[r]] = make_float2(re[r], im[r]);
-  }
-}
+// Slices of the index range that one thread of apply_terms takes.
+__device__ __forceinline__ int term_slices(int n) { return n >= 10 ? 8 : 2; }
 
-// backward: for ops in reverse, gradient contribution then un-apply on both
-template <int K>
-__device__ void group_bwd(float2* psi, float2* lam, int n, const BGroup& g, const BOp* ops,
-                          const float* mats, float2* wpart) {
-  int off[1 << K], lm[K];
-  group_offsets_swzb<K>(g, off, lm);
-  const int kk = g.k;
-  const int nsub = 1 << (n - kk);
-  const int width = 1 << kk;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // every lane of a warp runs the same number of iterations (warp sums)
-  const int iters = (nsub + blockDim.x - 1) / blockDim.x;
-  for (int it = 0; it < iters; ++it) {
-    const int s = threadIdx.x + it * blockDim.x;
-    const bool live = s < nsub;
-    const int b = live ? swzb(sub_base<K>(s, lm, kk)) : 0;
-    float pr[1 << K], pi[1 << K], lr[1 << K], li[1 << K];
-#pragma unroll
-    for (int r = 0; r < (1 << K); ++r) {
-      pr[r] = pi[r] = lr[r] = li[r] = 0.f;
-      if (live && r < width) {
-        const float2 v = psi[b ^ off[r]], w = lam[b ^ off[r]];
-        pr[r] = v.x;
-        pi[r] = v.y;
-        lr[r] = w.x;
-        li[r] = w.y;
-      }
-    }
-    for (int o = g.op1 - 1; o >= g.op0; --o) {
-      const BOp op = ops[o];
-      const float* M = mats + 8 * op.gi;
-      if (op.pauli) {
-        float c = 0.f;
-#define SV_GRAD(BB) \
-  if constexpr (BB < K) c = pair_grad<K, BB>(op.pauli, op.cm, pr, pi, lr, li)
-        SV_BIT_SWITCH(op.b0, SV_GRAD)
-#undef SV_GRAD
-        c = warp_sum_f(c);
-        if (lane == 0) ksum_add(wpart[warp * kBMaxParams + op.param], c);
-      }
-#define SV_BWD(BB) \
-  if constexpr (BB < K) pair_apply_dag2<K, BB>(op.cls, M, op.cm, pr, pi, lr, li)
-      SV_BIT_SWITCH(op.b0, SV_BWD)
-#undef SV_BWD
-    }
-    if (live) {
-#pragma unroll
-      for (int r = 0; r < (1 << K); ++r)
-        if (r < width) {
-          psi[b ^ off[r]] = make_float2(pr[r], pi[r]);
-          lam[b ^ off[r]] = make_float2(lr[r], li[r]);
-        }
-    }
-  }
-}
-
-// SMS: the block also owns kBSmemStateBytes of dynamic shared memory and
-// keeps psi there for items of up to 14 qubits (and lambda beside it for up
-// to 13), the rest in its global workspace slot.
-constexpr int kBSmemQubits = 14;
-constexpr size_t kBSmemStateBytes = sizeof(float2) << kBSmemQubits;
-// Every block also caches its item's operation and group descriptors in
-// dynamic shared memory (they are read once per operation per sub-block).
-constexpr size_t kBOpsBytes = sizeof(BOp) * kBMaxGates;
-constexpr size_t kBGroupBytes = sizeof(BGroup) * kBMaxGates;
-constexpr size_t kBTermBytes = sizeof(BTerm) * kBMaxTerms;
-constexpr size_t kBCacheBytes = kBOpsBytes + kBGroupBytes + kBTermBytes + sizeof(float2) * kBMaxTerms;
-
-template <int K, int MAXT, int MINB, bool SMS = false>
-__global__ void __launch_bounds__(MAXT, MINB) kbatch(const BatchArgs A) {
-  __shared__ float mats[8 * kBMaxGates];
-  __shared__ float2 wpart[(MAXT / 32) * kBMaxParams];  // per warp and parameter: (sum, comp)
-  __shared__ double red[MAXT / 32];
-  __shared__ int s_item;
-  extern __shared__ __align__(16) unsigned char dyn_smem[];
-  BOp* sops = reinterpret_cast<BOp*>(dyn_smem);
-  BGroup* sgrp = reinterpret_cast<BGroup*>(dyn_smem + kBOpsBytes);
-  // per term: (swzb(x mask), z mask | parity of (x mask & z mask) << 31)
-  int2* sterm = reinterpret_cast<int2*>(dyn_smem + kBOpsBytes + kBGroupBytes);
-  // the terms' coefficients rounded to fp32 once per item (a conversion from
-  // fp64 per term and amplitude would occupy GB300's slow fp64 pipe)
-  float2* scoef = reinterpret_cast<float2*>(dyn_smem + kBOpsBytes + kBGroupBytes + kBTermBytes);
-  float2* dyn_state = reinterpret_cast<float2*>(dyn_smem + kBCacheBytes);
-  const int nwarps = blockDim.x >> 5;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float2* const gpsi = A.work + (size_t)blockIdx.x * (size_t(2) << A.nmax);
-  float2* const glam = gpsi + (size_t(1) << A.nmax);
-  while (true) {
-    if (threadIdx.x == 0) s_item = atomicAdd(A.queue, 1);
-    __syncthreads();
-    const int slot = s_item;
-    if (slot >= A.n_items) break;
-    const int item = A.order[slot];
-    const BCirc C = A.circs[A.item_circ[item]];
-    const double* th = A.theta + A.theta_off[item];
-    const int dim = 1 << C.n;
-    float2* psi = gpsi;
-    float2* lam = glam;
-    if constexpr (SMS) {
-      if (C.n <= kBSmemQubits) psi = dyn_state;
-      if (C.n < kBSmemQubits) lam = dyn_state + (1 << (kBSmemQubits - 1));
-    }
-    // gate matrices (fp64 trigonometry, rounded once), psi = |0...0>, zero partials
-    for (int gi = threadIdx.x; gi < C.ngates; gi += blockDim.x) {
-      const BGateDesc d = A.gates[C.gate0 + gi];
-      const double a = d.param >= 0 ? th[d.param] : d.angle;
-      double s, c;
-      sincos(0.5 * a, &s, &c);
-      double m[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      const double r2 = 0.70710678118654752440;
-      switch (d.kind) {
-        case SV_GATE_H: m[0] = r2; m[2] = r2; m[4] = r2; m[6] = -r2; break;
-        case SV_GATE_X: m[2] = 1; m[4] = 1; break;
-        case SV_GATE_Y: m[3] = -1; m[5] = 1; break;
-        case SV_GATE_Z: m[0] = 1; m[6] = -1; break;
-        case SV_GATE_RX: m[0] = c; m[3] = -s; m[5] = -s; m[6] = c; break;
-        case SV_GATE_RY: m[0] = c; m[2] = -s; m[4] = s; m[6] = c; break;
-        case SV_GATE_RZ: m[0] = c; m[1] = -s; m[6] = c; m[7] = s; break;
-        default: {  // U1: diag(1, e^{ia})
-          double sa, ca;
-          sincos(a, &sa, &ca);
-          m[0] = 1; m[6] = ca; m[7] = sa;
-        }
-      }
-      for (int e = 0; e < 8; ++e) mats[8 * gi + e] = (float)m[e];
-    }
-    // |0...0>: swzb(0) = 0 and swzb maps every other index to a nonzero one
-    for (int x = threadIdx.x; x < dim; x += blockDim.x) psi[x] = make_float2(x == 0 ? 1.f : 0.f, 0.f);
-    for (int i = threadIdx.x; i < nwarps * kBMaxParams; i += blockDim.x)
-      wpart[i] = make_float2(0.f, 0.f);
-    {  // this item's groups and operations, operation indices rebased to the cache
-      const int ng = C.ngroups;
-      const int op_base = ng ? A.groups[C.group0].op0 : 0;
-      const int nops = ng ? A.groups[C.group0 + ng - 1].op1 - op_base : 0;
-      for (int i = threadIdx.x; i < nops; i += blockDim.x) sops[i] = A.ops[op_base + i];
-      for (int i = threadIdx.x; i < ng; i += blockDim.x) {
-        BGroup G = A.groups[C.group0 + i];
-        G.op0 -= op_base;
-        G.op1 -= op_base;
-        sgrp[i] = G;
-      }
-      for (int t = threadIdx.x; t < C.nterms; t += blockDim.x) {
-        const BTerm T = A.terms[C.term0 + t];
-        const int xm = (int)T.xm, zm = (int)T.zm;  // n <= SV_BATCH_MAX_QUBITS < 31
-        sterm[t] = make_int2(swzb(xm), (int)((unsigned)zm | ((unsigned)__popc(xm & zm) << 31)));
-        scoef[t] = make_float2((float)T.cre, (float)T.cim);
-      }
-    }
-    __syncthreads();
-    // forward
-    for (int gg = 0; gg < C.ngroups; ++gg) {
-      group_fwd<K>(psi, C.n, sgrp[gg], sops, mats);
-      __syncthreads();
-    }
-    // lambda = H psi, E = Re <psi|lambda> (logical index x, stored at swzb(x))
-    float2 ek = make_float2(0.f, 0.f);
-    for (int x = threadIdx.x; x < dim; x += blockDim.x) {
-      const int px = swzb(x);
-      const float2 a = psi[px];
-      // sign of term t at x: parity of ((x ^ xm) & zm) = parity(x & zm) ^ parity(xm & zm)
-      float dr = 0.f, di = 0.f;
-      for (int t = 0; t < C.ndiag; ++t) {
-        const int2 q = sterm[t];
-        const float2 cf = scoef[t];
-        if (__popc(x & q.y) & 1) {  // bit 31 (parity of xm & zm) is 0 here
-          dr -= cf.x;
-          di -= cf.y;
-        } else {
-          dr += cf.x;
-          di += cf.y;
-        }
-      }
-      float orr = dr * a.x - di * a.y, oi = dr * a.y + di * a.x;
-      for (int t = C.ndiag; t < C.nterms; ++t) {
-        const int2 q = sterm[t];
-        const float2 b = psi[px ^ q.x];
-        const float2 cf = scoef[t];
-        const float sr = cf.x * b.x - cf.y * b.y, si = cf.x * b.y + cf.y * b.x;
-        if ((__popc(x & q.y) + ((unsigned)q.y >> 31)) & 1) {
-          orr -= sr;
-          oi -= si;
-        } else {
-          orr += sr;
-          oi += si;
-        }
-      }
-      lam[px] = make_float2(orr, oi);
-      ksum_add(ek, a.x * orr + a.y * oi);
-    }
-    double e = warp_sum_d(ksum_value(ek));
-    if (lane == 0) red[warp] = e;
-    __syncthreads();
-    // reverse sweep
-    for (int gg = C.ngroups - 1; gg >= 0; --gg) {
-      group_bwd<K>(psi, lam, C.n, sgrp[gg], sops, mats, wpart);
-      __syncthreads();
-    }
-    const int toff = A.theta_off[item];
-    for (int p = threadIdx.x; p < C.nparams; p += blockDim.x) {
-      double g = 0.0;
-      for (int w = 0; w < nwarps; ++w) g += ksum_value(wpart[w * kBMaxParams + p]);
-      A.grad[toff + p] = g;
-    }
-    if (threadIdx.x == 0) {
-      double E = 0.0;
-      for (int w = 0; w < nwarps; ++w) E += red[w];
-      A.energy[item] = E;
-    }
-    __syncthreads();
-  }
-}
-
-// ---- real-amplitude batches ------------------------------------------------------
-// Gates whose matrices are real (H, X, Z, RY and their controlled forms)
-// map |0...0> to real states, and a Hamiltonian whose terms are real
-// matrices (coefficient times i^{#Y} real, as for the transverse-field Ising
-// model) maps a real state to a real lambda = H psi.  A batch made only of
-// such items runs psi and lambda as real vectors: half the bytes and half the
-// multiply-adds of the complex kernel, and both states of an n = 14 item
-// (2 x 64 KiB) in shared memory.  The only parameterised kind is then RY
-// (generator Y), whose gradient Im<lambda|Y|psi> is the real sum of
-// l1 p0 - l0 p1 over the pairs of its target bit.
+// ---- single-block items ------------------------------------------------------------
+// An item's state is one plane of 2^n real parts and, when CX, a second plane of
+// imaginary parts.  Batches made of real gates and terms run with one plane: H, X, Z, RY
+// and their controlled forms map |0...0> to real states, and a Hamiltonian whose
+// terms are real matrices (coefficient times i^{#Y} real, as for the
+// transverse-field Ising model) maps a real state to a real lambda = H psi.  That
+// is half the bytes and half the multiply-adds, and both states of an n = 14
+// item (2 x 64 KiB) in shared memory.
 //
-// Storage order: amplitude x lives at swzr(x) = x ^ ((x >> 5) & 31), which
-// spreads the 32 amplitudes of a 128-byte row over the row by the next five
-// index bits (a bijection of [0, 2^n), linear over XOR).
+// Storage order: amplitude x of a plane lives at swzr(x) = x ^ ((x >> 5) & 31),
+// which spreads the 32 values of a 128-byte row over the row by the next five
+// index bits (a bijection of [0, 2^n), linear over XOR): a warp whose lanes step
+// over a register group's low bits reaches 32 banks.
+//
+// Register tile: pairs of group bit 0's values (group indices 2 p and 2 p + 1), so
+// that the operations on the other bits are paired fp32 instructions whatever the
+// group's place in memory.  A rotation without controls is three shears in place:
+// RY x += a y, y += b x, x += a y with a = -tan(angle / 4) and b = sin(angle / 2), and
+// RX the same between a and i b; the half angle is taken modulo pi (a sign of the
+// whole state, which neither the energy nor a gradient sees) so that |a| <= 1.  RZ
+// is the one phase e^{i angle} on the upper half (a phase of the whole state
+// dropped).  A run of CZs is one multiplication by its sign pattern.  Per tile of 16 or
+// 32 amplitudes a rotation costs 24 paired FMAs in place of 64 (RX, RY) or 128 (RZ)
+// single ones: 768 parameter sets of the n = 11, 6-layer random layered circuit and 192
+// mixed items 0.85 -> 0.66 ms, 1024 sets of the n = 14 real ansatz 4.4 -> 3.05 ms.
 __device__ __forceinline__ int swzr(int x) { return x ^ ((x >> 5) & 31); }
 
-template <int K>
-__device__ void group_offsets_swzr(const BGroup& g, int (&off)[1 << K], int (&lm)[K]) {
-  off[0] = 0;
-#pragma unroll
-  for (int r = 1; r < (1 << K); ++r) off[r] = off[r & (r - 1)] ^ swzr(1 << g.bits[lowbit_b(r)]);
-#pragma unroll
-  for (int i = 0; i < K; ++i) lm[i] = (1 << g.bits[i]) - 1;
-}
+template <int K, bool CX>
+struct Tile {
+  Pair r[1 << (K - 1)], i[CX ? 1 << (K - 1) : 1];
+};
 
 // (a, b) <- [[g0, g1], [g2, g3]] (a, b) on the pairs of group bit B (inside the
 // group-local control mask cm when CTRL); NEG: b <- -b
@@ -665,41 +361,12 @@ __device__ __forceinline__ void re_pairs(float g0, float g1, float g2, float g3,
   }
 }
 
-// sign flip under a control mask fixed at compile time (CZ and its kin)
-template <int K, int B, int CM>
-__device__ __forceinline__ void re_neg_cm(float (&v)[1 << K]) {
-  if constexpr (!((CM >> B) & 1)) {
-#pragma unroll
-    for (int r = 0; r < (1 << K); ++r) {
-      if (r & (1 << B)) continue;
-      if ((r & CM) != CM) continue;
-      v[r | (1 << B)] = -v[r | (1 << B)];
-    }
-  }
-}
-
-template <int K, int B>
-__device__ __forceinline__ void re_neg(int cm, float (&v)[1 << K]) {
-#define SV_RE_CM(c)                                          \
-  case c:                                                    \
-    if constexpr (c < (1 << K)) re_neg_cm<K, B, c>(v);       \
-    break;
-  switch (cm) {
-    SV_RE_CM(0) SV_RE_CM(1) SV_RE_CM(2) SV_RE_CM(3) SV_RE_CM(4) SV_RE_CM(5) SV_RE_CM(6)
-    SV_RE_CM(7) SV_RE_CM(8) SV_RE_CM(9) SV_RE_CM(10) SV_RE_CM(11) SV_RE_CM(12) SV_RE_CM(13)
-    SV_RE_CM(14) SV_RE_CM(15) SV_RE_CM(16) SV_RE_CM(17) SV_RE_CM(18) SV_RE_CM(20)
-    SV_RE_CM(24)
-    default: re_pairs<K, B, true, true>(0.f, 0.f, 0.f, 0.f, cm, v); break;
-  }
-#undef SV_RE_CM
-}
-
 // operation (cls BC_REAL or BC_NEG) with matrix M (8 floats, re/im) or, when
 // DAG, its transpose
 template <int K, int B, bool DAG>
 __device__ __forceinline__ void re_apply(const BOp& op, const float* M, float (&v)[1 << K]) {
   if (op.cls == BC_NEG) {
-    re_neg<K, B>(op.cm, v);
+    re_pairs<K, B, true, true>(0.f, 0.f, 0.f, 0.f, op.cm, v);
     return;
   }
   const float g0 = M[0], g1 = DAG ? M[4] : M[2], g2 = DAG ? M[2] : M[4], g3 = M[6];
@@ -723,27 +390,24 @@ __device__ __forceinline__ float re_grad(int cm, const float (&p)[1 << K], const
   return acc;
 }
 
-#define SV_RE_BITS(B, CALL) \
-  switch (B) {              \
-    case 0: CALL(0); break; \
-    case 1: CALL(1); break; \
-    case 2: CALL(2); break; \
-    case 3: CALL(3); break; \
-    default: CALL(4); break; \
+template <int K>
+__device__ __forceinline__ void unpack(const Pair (&v)[1 << (K - 1)], float (&w)[1 << K]) {
+#pragma unroll
+  for (int p = 0; p < (1 << (K - 1)); ++p) {
+    const float2 x = lanes_of(v[p]);
+    w[2 * p] = x.x;
+    w[2 * p + 1] = x.y;
   }
+}
+template <int K>
+__device__ __forceinline__ void repack(const float (&w)[1 << K], Pair (&v)[1 << (K - 1)]) {
+#pragma unroll
+  for (int p = 0; p < (1 << (K - 1)); ++p) v[p] = pair_of(w[2 * p], w[2 * p + 1]);
+}
 
-// The register tile is held as pairs of group bit 0's values (group indices 2 p
-// and 2 p + 1), so that the operations on the other bits are paired fp32
-// instructions whatever the group's place in memory.  An RY without controls is
-// three shears in place, x += a y, y += b x, x += a y with a = -tan(angle / 2) and b =
-// sin(angle), the angle taken modulo pi (a sign of the whole state, which neither
-// the energy nor a gradient sees) so that |a| <= 1; a run of CZs is one
-// multiplication by its sign pattern.  C3's HEA (n = 14, 10 layers): 64 FMAs and 32
-// flips with their dispatches per tile for a rotation and four CZs before, 24 and 16 now;
-// 1024 parameter sets 4.39 -> 3.16 ms (16 warps of 128 registers an SM: the issue slots are
-// half used, and ALU work - tile addresses, signs of the terms - is the busiest pipe).
+// x += a y, y += b x, x += a y on group bit B of one plane
 template <int K, int B>
-__device__ __forceinline__ void re2_rot(float a, float b, Pair (&v)[1 << (K - 1)]) {
+__device__ __forceinline__ void plane_rot(float a, float b, Pair (&v)[1 << (K - 1)]) {
   if constexpr (B == 0) {
 #pragma unroll
     for (int p = 0; p < (1 << (K - 1)); ++p) {
@@ -766,211 +430,531 @@ __device__ __forceinline__ void re2_rot(float a, float b, Pair (&v)[1 << (K - 1)
   }
 }
 
-// RY's gradient without controls: sum of l1 p0 - l0 p1 over the pairs of group bit B
+// RX: the shears between a and y = i b, (re y, im y) = (-im b, re b)
 template <int K, int B>
-__device__ __forceinline__ float re2_grad(const Pair (&p)[1 << (K - 1)],
-                                          const Pair (&l)[1 << (K - 1)]) {
+__device__ __forceinline__ void rx_rot(float a, float b, Tile<K, true>& t) {
+  if constexpr (B == 0) {
+#pragma unroll
+    for (int p = 0; p < (1 << (K - 1)); ++p) {
+      float2 r = lanes_of(t.r[p]), i = lanes_of(t.i[p]);
+      r.x = fmaf(-a, i.y, r.x);
+      i.x = fmaf(a, r.y, i.x);
+      i.y = fmaf(-b, r.x, i.y);
+      r.y = fmaf(b, i.x, r.y);
+      r.x = fmaf(-a, i.y, r.x);
+      i.x = fmaf(a, r.y, i.x);
+      t.r[p] = pair_of(r.x, r.y);
+      t.i[p] = pair_of(i.x, i.y);
+    }
+  } else {
+    const Pair pa = pair_both(a), na = pair_both(-a), pb = pair_both(b), nb = pair_both(-b);
+#pragma unroll
+    for (int p = 0; p < (1 << (K - 1)); ++p) {
+      if (p & (1 << (B - 1))) continue;
+      const int q = p | (1 << (B - 1));
+      pair_add(t.r[p], na, t.i[q]);
+      pair_add(t.i[p], pa, t.r[q]);
+      pair_add(t.i[q], nb, t.r[p]);
+      pair_add(t.r[q], pb, t.i[p]);
+      pair_add(t.r[p], na, t.i[q]);
+      pair_add(t.i[p], pa, t.r[q]);
+    }
+  }
+}
+
+// RZ up to a phase of the whole state: the upper half times c + i s
+template <int K, int B>
+__device__ __forceinline__ void rz_rot(float c, float s, Tile<K, true>& t) {
+  if constexpr (B == 0) {
+#pragma unroll
+    for (int p = 0; p < (1 << (K - 1)); ++p) {
+      float2 r = lanes_of(t.r[p]), i = lanes_of(t.i[p]);
+      const float u = c * r.y;
+      const float w = c * i.y;
+      i.y = fmaf(s, r.y, w);
+      r.y = fmaf(-s, lanes_of(t.i[p]).y, u);
+      t.r[p] = pair_of(r.x, r.y);
+      t.i[p] = pair_of(i.x, i.y);
+    }
+  } else {
+    const Pair pc = pair_both(c), ps = pair_both(s), ns = pair_both(-s);
+#pragma unroll
+    for (int q = 0; q < (1 << (K - 1)); ++q) {
+      if (!(q & (1 << (B - 1)))) continue;
+      const Pair r = t.r[q], i = t.i[q];
+      t.r[q] = pair_mul(pc, r);
+      pair_add(t.r[q], ns, i);
+      t.i[q] = pair_mul(pc, i);
+      pair_add(t.i[q], ps, r);
+    }
+  }
+}
+
+// Im <l|P|p> over the tile for a generator without controls: Y on one plane, and X
+// and Z (and the other plane's part of Y) with both
+template <int K, int B, bool CX>
+__device__ __forceinline__ float tile_grad_y(const Tile<K, CX>& p, const Tile<K, CX>& l) {
   if constexpr (B == 0) {
     float x = 0.f, y = 0.f;
 #pragma unroll
-    for (int i = 0; i < (1 << (K - 1)); ++i) {
-      const float2 u = lanes_of(p[i]), w = lanes_of(l[i]);
+    for (int k = 0; k < (1 << (K - 1)); ++k) {
+      const float2 u = lanes_of(p.r[k]), w = lanes_of(l.r[k]);
       x = fmaf(w.y, u.x, x);
       y = fmaf(w.x, u.y, y);
+      if constexpr (CX) {
+        const float2 v = lanes_of(p.i[k]), z = lanes_of(l.i[k]);
+        x = fmaf(z.y, v.x, x);
+        y = fmaf(z.x, v.y, y);
+      }
     }
     return x - y;
   } else {
     Pair x = 0, y = 0;
 #pragma unroll
-    for (int i = 0; i < (1 << (K - 1)); ++i) {
-      if (i & (1 << (B - 1))) continue;
-      const int j = i | (1 << (B - 1));
-      pair_add(x, l[j], p[i]);
-      pair_add(y, l[i], p[j]);
+    for (int k = 0; k < (1 << (K - 1)); ++k) {
+      if (k & (1 << (B - 1))) continue;
+      const int q = k | (1 << (B - 1));
+      pair_add(x, l.r[q], p.r[k]);
+      pair_add(y, l.r[k], p.r[q]);
+      if constexpr (CX) {
+        pair_add(x, l.i[q], p.i[k]);
+        pair_add(y, l.i[k], p.i[q]);
+      }
     }
     const float2 u = lanes_of(x), w = lanes_of(y);
     return (u.x - w.x) + (u.y - w.y);
   }
 }
-
-template <int K>
-__device__ __forceinline__ void re2_signs(const float* sg, Pair (&v)[1 << (K - 1)]) {
-  const ulonglong2* s = reinterpret_cast<const ulonglong2*>(sg);
+template <int K, int B>
+__device__ __forceinline__ float tile_grad_x(const Tile<K, true>& p, const Tile<K, true>& l) {
+  if constexpr (B == 0) {
+    float x = 0.f, y = 0.f;
 #pragma unroll
-  for (int i = 0; i < (1 << (K - 2)); ++i) {
-    const ulonglong2 x = s[i];
-    v[2 * i] = pair_mul(x.x, v[2 * i]);
-    v[2 * i + 1] = pair_mul(x.y, v[2 * i + 1]);
+    for (int k = 0; k < (1 << (K - 1)); ++k) {
+      const float2 pr = lanes_of(p.r[k]), pi = lanes_of(p.i[k]);
+      const float2 lr = lanes_of(l.r[k]), li = lanes_of(l.i[k]);
+      x = fmaf(lr.x, pi.y, x);
+      y = fmaf(li.x, pr.y, y);
+      x = fmaf(lr.y, pi.x, x);
+      y = fmaf(li.y, pr.x, y);
+    }
+    return x - y;
+  } else {
+    Pair x = 0, y = 0;
+#pragma unroll
+    for (int k = 0; k < (1 << (K - 1)); ++k) {
+      if (k & (1 << (B - 1))) continue;
+      const int q = k | (1 << (B - 1));
+      pair_add(x, l.r[k], p.i[q]);
+      pair_add(y, l.i[k], p.r[q]);
+      pair_add(x, l.r[q], p.i[k]);
+      pair_add(y, l.i[q], p.r[k]);
+    }
+    const float2 u = lanes_of(x), w = lanes_of(y);
+    return (u.x - w.x) + (u.y - w.y);
+  }
+}
+template <int K, int B>
+__device__ __forceinline__ float tile_grad_z(const Tile<K, true>& p, const Tile<K, true>& l) {
+  // x: l_r p_i, y: l_i p_r, the lower half's minus the upper half's
+  Pair x0 = 0, y0 = 0, x1 = 0, y1 = 0;
+#pragma unroll
+  for (int k = 0; k < (1 << (K - 1)); ++k) {
+    const bool up = B > 0 && (k & (1 << (B > 0 ? B - 1 : 0)));
+    pair_add(up ? x1 : x0, l.r[k], p.i[k]);
+    pair_add(up ? y1 : y0, l.i[k], p.r[k]);
+  }
+  const float2 a = lanes_of(x0), b = lanes_of(y0);
+  if constexpr (B == 0) {
+    return (a.x - b.x) - (a.y - b.y);
+  } else {
+    const float2 c = lanes_of(x1), d = lanes_of(y1);
+    return ((a.x - b.x) + (a.y - b.y)) - ((c.x - d.x) + (c.y - d.y));
   }
 }
 
-// any other operation (see re_apply) on the tile as single values
-template <int K, bool DAG>
-__device__ __forceinline__ void re2_other(const BOp& op, const float* M, Pair (&v)[1 << (K - 1)]) {
-  float w[1 << K];
+template <int K, int B, bool CX>
+__device__ __forceinline__ float tile_grad(int pauli, const Tile<K, CX>& p, const Tile<K, CX>& l) {
+  if constexpr (CX) {
+    if (pauli == 1) return tile_grad_x<K, B>(p, l);
+    if (pauli == 3) return tile_grad_z<K, B>(p, l);
+  }
+  return tile_grad_y<K, B, CX>(p, l);
+}
+
+// a rotation without controls; DAG: its inverse
+template <int K, int B, bool CX, bool DAG>
+__device__ __forceinline__ void tile_rot(int cls, float a, float b, Tile<K, CX>& t) {
+  if constexpr (CX) {
+    if (cls == BC_RZ) {
+      rz_rot<K, B>(a, DAG ? -b : b, t);
+      return;
+    }
+    if (cls == BC_RX) {
+      rx_rot<K, B>(DAG ? -a : a, DAG ? -b : b, t);
+      return;
+    }
+    plane_rot<K, B>(DAG ? -a : a, DAG ? -b : b, t.i);
+  }
+  plane_rot<K, B>(DAG ? -a : a, DAG ? -b : b, t.r);
+}
+
+template <int K, bool CX>
+__device__ __forceinline__ void tile_signs(const float* sg, Tile<K, CX>& t) {
+  const Pair* s = reinterpret_cast<const Pair*>(sg);
 #pragma unroll
   for (int p = 0; p < (1 << (K - 1)); ++p) {
-    const float2 x = lanes_of(v[p]);
-    w[2 * p] = x.x;
-    w[2 * p + 1] = x.y;
+    t.r[p] = pair_mul(s[p], t.r[p]);
+    if constexpr (CX) t.i[p] = pair_mul(s[p], t.i[p]);
   }
+}
+template <int K, bool CX>
+__device__ __forceinline__ void tile_signs2(const float* sg, Tile<K, CX>& t, Tile<K, CX>& u) {
+  const Pair* s = reinterpret_cast<const Pair*>(sg);
+#pragma unroll
+  for (int p = 0; p < (1 << (K - 1)); ++p) {
+    const Pair x = s[p];
+    t.r[p] = pair_mul(x, t.r[p]);
+    u.r[p] = pair_mul(x, u.r[p]);
+    if constexpr (CX) {
+      t.i[p] = pair_mul(x, t.i[p]);
+      u.i[p] = pair_mul(x, u.i[p]);
+    }
+  }
+}
+
+#define SV_TILE_BITS(B, CALL) \
+  switch (B) {                \
+    case 0: CALL(0); break;   \
+    case 1: CALL(1); break;   \
+    case 2: CALL(2); break;   \
+    case 3: CALL(3); break;   \
+    default: CALL(4); break;  \
+  }
+
+// any other operation, on the tile as single values
+template <int K, bool CX, bool DAG>
+__device__ __forceinline__ void tile_other(const BOp& op, const float* M, Tile<K, CX>& t) {
+  float w[1 << K];
+  unpack<K>(t.r, w);
+  if constexpr (CX) {
+    float u[1 << K];
+    unpack<K>(t.i, u);
+#define SV_OTHER(BB)                                                   \
+  if constexpr (BB < K) {                                              \
+    if constexpr (DAG)                                                 \
+      pair_apply_dag<K, BB>(op.cls, M, op.cm, w, u);                   \
+    else                                                               \
+      pair_apply<K, BB>(op.cls, M, op.cm, w, u);                       \
+  }
+    SV_TILE_BITS(op.b0, SV_OTHER)
+#undef SV_OTHER
+    repack<K>(u, t.i);
+  } else {
 #define SV_OTHER(BB) \
   if constexpr (BB < K) re_apply<K, BB, DAG>(op, M, w)
-  SV_RE_BITS(op.b0, SV_OTHER)
+    SV_TILE_BITS(op.b0, SV_OTHER)
 #undef SV_OTHER
-#pragma unroll
-  for (int p = 0; p < (1 << (K - 1)); ++p) v[p] = pair_of(w[2 * p], w[2 * p + 1]);
+  }
+  repack<K>(w, t.r);
 }
 
+// the gradient of a controlled rotation
+template <int K, bool CX>
+__device__ __forceinline__ float tile_other_grad(const BOp& op, const Tile<K, CX>& p,
+                                                 const Tile<K, CX>& l) {
+  float u[1 << K], w[1 << K], c = 0.f;
+  unpack<K>(p.r, u);
+  unpack<K>(l.r, w);
+  if constexpr (CX) {
+    float v[1 << K], z[1 << K];
+    unpack<K>(p.i, v);
+    unpack<K>(l.i, z);
+#define SV_OTHER(BB) \
+  if constexpr (BB < K) c = pair_grad<K, BB>(op.pauli, op.cm, u, v, w, z)
+    SV_TILE_BITS(op.b0, SV_OTHER)
+#undef SV_OTHER
+  } else {
+#define SV_OTHER(BB) \
+  if constexpr (BB < K) c = re_grad<K, BB>(op.cm, u, w)
+    SV_TILE_BITS(op.b0, SV_OTHER)
+#undef SV_OTHER
+  }
+  return c;
+}
+
+// A group's places: pl.step[i] the byte offset of its bit i in storage order (XORed), pl.low
+// the bits' low masks.
 template <int K>
-__device__ void group_fwd_re(float* psi, int n, const BGroup& g, const BOp* ops, const float* mats,
-                             const float* signs) {
-  int off[1 << K], lm[K];
-  group_offsets_swzr<K>(g, off, lm);
-  const int kk = g.k;
-  const int nsub = 1 << (n - kk);
-  const int width = 1 << kk;
-  for (int s = threadIdx.x; s < nsub; s += blockDim.x) {
-    const int b = swzr(sub_base<K>(s, lm, kk));
-    Pair v[1 << (K - 1)];
+struct Places {
+  int step[K], low[K];
+};
+template <int K>
+__device__ __forceinline__ Places<K> group_places(const BGroup& g) {
+  Places<K> pl;
 #pragma unroll
-    for (int p = 0; p < (1 << (K - 1)); ++p)
-      v[p] = pair_of(2 * p < width ? psi[b ^ off[2 * p]] : 0.f,
-                     2 * p + 1 < width ? psi[b ^ off[2 * p + 1]] : 0.f);
+  for (int i = 0; i < K; ++i) {
+    pl.step[i] = swzr(1 << g.bits[i]) * (int)sizeof(float);
+    pl.low[i] = (1 << g.bits[i]) - 1;
+  }
+  return pl;
+}
+
+// The tile at byte offset b, in Gray-code order: one XOR an address, and no table of
+// 2^K offsets to keep in registers across the operations.
+template <int K, bool CX>
+__device__ __forceinline__ void tile_load(const float* st, int b, const Places<K>& pl, int plane,
+                                          Tile<K, CX>& t) {
+  const char* re = reinterpret_cast<const char*>(st);
+  const char* im = reinterpret_cast<const char*>(st + plane);
+#pragma unroll
+  for (int k = 0; k < (1 << (K - 1)); ++k) {
+    const int p = k ^ (k >> 1);
+    if (k) b ^= pl.step[1 + lowbit_b(k)];
+    const int c = b ^ pl.step[0];
+    t.r[p] = pair_of(*reinterpret_cast<const float*>(re + b), *reinterpret_cast<const float*>(re + c));
+    if constexpr (CX)
+      t.i[p] =
+          pair_of(*reinterpret_cast<const float*>(im + b), *reinterpret_cast<const float*>(im + c));
+  }
+}
+template <int K, bool CX>
+__device__ __forceinline__ void tile_store(float* st, int b, const Places<K>& pl, int plane,
+                                           const Tile<K, CX>& t) {
+  char* re = reinterpret_cast<char*>(st);
+  char* im = reinterpret_cast<char*>(st + plane);
+  asm volatile("" : "+r"(b));  // the addresses are formed again, not kept from the loads
+#pragma unroll
+  for (int k = 0; k < (1 << (K - 1)); ++k) {
+    const int p = k ^ (k >> 1);
+    if (k) b ^= pl.step[1 + lowbit_b(k)];
+    const int c = b ^ pl.step[0];
+    const float2 v = lanes_of(t.r[p]);
+    *reinterpret_cast<float*>(re + b) = v.x;
+    *reinterpret_cast<float*>(re + c) = v.y;
+    if constexpr (CX) {
+      const float2 w = lanes_of(t.i[p]);
+      *reinterpret_cast<float*>(im + b) = w.x;
+      *reinterpret_cast<float*>(im + c) = w.y;
+    }
+  }
+}
+
+// Per block: the item's gate matrices, operations, groups, terms and sign patterns,
+// and per-warp gradient sums, in dynamic shared memory sized by the batch.
+struct BSmem {
+  float* mats;    // 8 floats a gate; a rotation without controls: its two coefficients
+  float2* wpart;  // per warp and parameter: (sum, compensation)
+  BOp* ops;
+  BGroup* grp;
+  int2* term;     // (swzr(x mask), z mask | (an odd number of Y factors) << 31)
+  float* tcoef;   // 8 a term: the coefficient times the sign of slice j's high bits
+  float* sign;    // patterns of 2^K values
+};
+
+// forward: psi <- group ops in order
+template <int K, bool CX>
+__device__ __forceinline__ void group_fwd(float* psi, int np, const BGroup& g, const BSmem& S) {
+  const Places<K> pl = group_places<K>(g);
+  const int nsub = 1 << (np - K);
+  for (int s = threadIdx.x; s < nsub; s += blockDim.x) {
+    const int b = swzr(sub_base<K>(s, pl.low, K)) * (int)sizeof(float);
+    Tile<K, CX> t;
+    tile_load<K, CX>(psi, b, pl, 1 << np, t);
     for (int o = g.op0; o < g.op1; ++o) {
-      const BOp op = ops[o];
-      if (op.cls == BC_ROT) {
-        const float a = mats[8 * op.gi + 1], c = mats[8 * op.gi + 3];
-#define SV_FWD_RE(BB) \
-  if constexpr (BB < K) re2_rot<K, BB>(a, c, v)
-        SV_RE_BITS(op.b0, SV_FWD_RE)
-#undef SV_FWD_RE
+      const BOp op = S.ops[o];
+      const float* M = S.mats + 8 * op.gi;
+      if (op.cls >= BC_ROT) {
+        const float2 ab = *reinterpret_cast<const float2*>(M);
+#define SV_ROT(BB) \
+  if constexpr (BB < K) tile_rot<K, BB, CX, false>(op.cls, ab.x, ab.y, t)
+        SV_TILE_BITS(op.b0, SV_ROT)
+#undef SV_ROT
       } else if (op.cls == BC_SIGN) {
-        re2_signs<K>(signs + 32 * op.gi, v);
+        tile_signs<K, CX>(S.sign + (op.gi << K), t);
       } else {
-        re2_other<K, false>(op, mats + 8 * op.gi, v);
+        tile_other<K, CX, false>(op, M, t);
       }
     }
-#pragma unroll
-    for (int p = 0; p < (1 << (K - 1)); ++p) {
-      const float2 x = lanes_of(v[p]);
-      if (2 * p < width) psi[b ^ off[2 * p]] = x.x;
-      if (2 * p + 1 < width) psi[b ^ off[2 * p + 1]] = x.y;
-    }
+    tile_store<K, CX>(psi, b, pl, 1 << np, t);
   }
 }
 
-template <int K>
-__device__ void group_bwd_re(float* psi, float* lam, int n, const BGroup& g, const BOp* ops,
-                             const float* mats, const float* signs, float2* wpart) {
-  int off[1 << K], lm[K];
-  group_offsets_swzr<K>(g, off, lm);
-  const int kk = g.k;
-  const int nsub = 1 << (n - kk);
-  const int width = 1 << kk;
+// backward: for ops in reverse, gradient contribution then un-apply on both
+template <int K, bool CX>
+__device__ __forceinline__ void group_bwd(float* psi, float* lam, int np, int pstride,
+                                          const BGroup& g, const BSmem& S) {
+  const Places<K> pl = group_places<K>(g);
+  const int nsub = 1 << (np - K);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // every lane of a warp runs the same number of iterations (warp sums)
-  const int iters = (nsub + blockDim.x - 1) / blockDim.x;
-  for (int it = 0; it < iters; ++it) {
-    const int s = threadIdx.x + it * blockDim.x;
+  for (int s0 = threadIdx.x - lane; s0 < nsub; s0 += blockDim.x) {
+    const int s = s0 + lane;
     const bool live = s < nsub;
-    const int b = live ? swzr(sub_base<K>(s, lm, kk)) : 0;
-    Pair p[1 << (K - 1)], l[1 << (K - 1)];
-#pragma unroll
-    for (int r = 0; r < (1 << (K - 1)); ++r) {
-      const bool in0 = live && 2 * r < width, in1 = live && 2 * r + 1 < width;
-      p[r] = pair_of(in0 ? psi[b ^ off[2 * r]] : 0.f, in1 ? psi[b ^ off[2 * r + 1]] : 0.f);
-      l[r] = pair_of(in0 ? lam[b ^ off[2 * r]] : 0.f, in1 ? lam[b ^ off[2 * r + 1]] : 0.f);
+    const int b = live ? swzr(sub_base<K>(s, pl.low, K)) * (int)sizeof(float) : 0;
+    Tile<K, CX> p{}, l{};
+    if (live) {
+      tile_load<K, CX>(psi, b, pl, 1 << np, p);
+      tile_load<K, CX>(lam, b, pl, 1 << np, l);
     }
     for (int o = g.op1 - 1; o >= g.op0; --o) {
-      const BOp op = ops[o];
-      if (op.cls == BC_ROT) {
-        if (op.pauli) {  // RY: generator Y
-          float c = 0.f;
-#define SV_GRAD_RE(BB) \
-  if constexpr (BB < K) c = re2_grad<K, BB>(p, l)
-          SV_RE_BITS(op.b0, SV_GRAD_RE)
-#undef SV_GRAD_RE
-          c = warp_sum_f(c);
-          if (lane == 0) ksum_add(wpart[warp * kBMaxParams + op.param], c);
-        }
-        const float a = -mats[8 * op.gi + 1], c = -mats[8 * op.gi + 3];
-#define SV_BWD_RE(BB)            \
-  if constexpr (BB < K) {        \
-    re2_rot<K, BB>(a, c, p);     \
-    re2_rot<K, BB>(a, c, l);     \
+      const BOp op = S.ops[o];
+      const float* M = S.mats + 8 * op.gi;
+      float c = 0.f;
+      if (op.cls >= BC_ROT) {
+        const float2 ab = *reinterpret_cast<const float2*>(M);
+#define SV_ROT(BB)                                               \
+  if constexpr (BB < K) {                                        \
+    if (op.pauli) c = tile_grad<K, BB, CX>(op.pauli, p, l);      \
+    tile_rot<K, BB, CX, true>(op.cls, ab.x, ab.y, p);            \
+    tile_rot<K, BB, CX, true>(op.cls, ab.x, ab.y, l);            \
   }
-        SV_RE_BITS(op.b0, SV_BWD_RE)
-#undef SV_BWD_RE
+        SV_TILE_BITS(op.b0, SV_ROT)
+#undef SV_ROT
       } else if (op.cls == BC_SIGN) {
-        re2_signs<K>(signs + 32 * op.gi, p);
-        re2_signs<K>(signs + 32 * op.gi, l);
+        tile_signs2<K, CX>(S.sign + (op.gi << K), p, l);
       } else {
-        const float* M = mats + 8 * op.gi;
-        if (op.pauli) {  // controlled RY
-          float u[1 << K], w[1 << K], c = 0.f;
-#pragma unroll
-          for (int r = 0; r < (1 << (K - 1)); ++r) {
-            const float2 x = lanes_of(p[r]), y = lanes_of(l[r]);
-            u[2 * r] = x.x;
-            u[2 * r + 1] = x.y;
-            w[2 * r] = y.x;
-            w[2 * r + 1] = y.y;
-          }
-#define SV_GRAD_RE(BB) \
-  if constexpr (BB < K) c = re_grad<K, BB>(op.cm, u, w)
-          SV_RE_BITS(op.b0, SV_GRAD_RE)
-#undef SV_GRAD_RE
-          c = warp_sum_f(c);
-          if (lane == 0) ksum_add(wpart[warp * kBMaxParams + op.param], c);
-        }
-        re2_other<K, true>(op, M, p);
-        re2_other<K, true>(op, M, l);
+        if (op.pauli) c = tile_other_grad<K, CX>(op, p, l);
+        tile_other<K, CX, true>(op, M, p);
+        tile_other<K, CX, true>(op, M, l);
+      }
+      if (op.pauli) {
+        c = warp_sum_f(c);
+        if (lane == 0) ksum_add(S.wpart[warp * pstride + op.param], c);
       }
     }
     if (live) {
-#pragma unroll
-      for (int r = 0; r < (1 << (K - 1)); ++r) {
-        const float2 x = lanes_of(p[r]), y = lanes_of(l[r]);
-        if (2 * r < width) {
-          psi[b ^ off[2 * r]] = x.x;
-          lam[b ^ off[2 * r]] = y.x;
-        }
-        if (2 * r + 1 < width) {
-          psi[b ^ off[2 * r + 1]] = x.y;
-          lam[b ^ off[2 * r + 1]] = y.y;
-        }
-      }
+      tile_store<K, CX>(psi, b, pl, 1 << np, p);
+      tile_store<K, CX>(lam, b, pl, 1 << np, l);
     }
   }
 }
 
-// Sign patterns of one circuit's real-amplitude lists in shared memory, 32 floats
-// each; a circuit with more keeps its single flips.
-constexpr int kBMaxSigns = 96;
-constexpr size_t kBSignBytes = sizeof(float) * 32 * kBMaxSigns;
+// lambda = H psi and this thread's part of E = Re <psi|lambda>.  A thread takes the J
+// amplitudes x0 + j 2^n / J, so that a term's sign is one parity of x0 times
+// a sign of j that the whole block shares (in tcoef): 2^14 amplitudes with
+// 27 terms took about a fifth of a real item's instructions with a parity per
+// amplitude and term.
+template <int J, bool CX>
+__device__ __forceinline__ void apply_terms(const float* psi, float* lam, const BCirc& C, int np,
+                                            const BSmem& S, float2& ek) {
+  const int d = (1 << C.n) / J, plane = 1 << np;
+  int off[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) off[j] = swzr(j * d);
+  for (int x0 = threadIdx.x; x0 < d; x0 += blockDim.x) {
+    const int p0 = swzr(x0);
+    Pair dg[J / 2], ar[J / 2], ai[CX ? J / 2 : 1], sr[J / 2], si[CX ? J / 2 : 1];
+#pragma unroll
+    for (int k = 0; k < J / 2; ++k) {
+      dg[k] = 0;
+      const float* x = psi + (p0 ^ off[2 * k]);
+      const float* y = psi + (p0 ^ off[2 * k + 1]);
+      ar[k] = pair_of(*x, *y);
+      if constexpr (CX) ai[k] = pair_of(x[plane], y[plane]);
+    }
+    for (int t = 0; t < C.ndiag; ++t) {
+      const Pair sg = pair_both(__popc(x0 & S.term[t].y) & 1 ? -1.f : 1.f);
+      const Pair* cf = reinterpret_cast<const Pair*>(S.tcoef + 8 * t);
+#pragma unroll
+      for (int k = 0; k < J / 2; ++k) pair_add(dg[k], sg, cf[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < J / 2; ++k) {
+      sr[k] = pair_mul(dg[k], ar[k]);
+      if constexpr (CX) si[k] = pair_mul(dg[k], ai[k]);
+    }
+    for (int t = C.ndiag; t < C.nterms; ++t) {
+      const int2 q = S.term[t];
+      const int odd = __popc(x0 & q.y) & 1;
+      const Pair sg = pair_both(odd ? -1.f : 1.f);
+      const Pair* cf = reinterpret_cast<const Pair*>(S.tcoef + 8 * t);
+      const int pt = p0 ^ q.x;
+#pragma unroll
+      for (int k = 0; k < J / 2; ++k) {
+        const Pair w = pair_mul(sg, cf[k]);
+        const float* x = psi + (pt ^ off[2 * k]);
+        const float* y = psi + (pt ^ off[2 * k + 1]);
+        const Pair br = pair_of(*x, *y);
+        if constexpr (CX) {
+          const Pair bi = pair_of(x[plane], y[plane]);
+          if (q.y < 0) {  // an odd number of Y factors: i times real
+            pair_add(sr[k], pair_mul(pair_both(-1.f), w), bi);
+            pair_add(si[k], w, br);
+          } else {
+            pair_add(sr[k], w, br);
+            pair_add(si[k], w, bi);
+          }
+        } else {
+          pair_add(sr[k], w, br);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < J / 2; ++k) {
+      float* x = lam + (p0 ^ off[2 * k]);
+      float* y = lam + (p0 ^ off[2 * k + 1]);
+      const float2 o = lanes_of(sr[k]), a = lanes_of(ar[k]);
+      *x = o.x;
+      *y = o.y;
+      float e0 = a.x * o.x, e1 = a.y * o.y;
+      if constexpr (CX) {
+        const float2 oi = lanes_of(si[k]), aa = lanes_of(ai[k]);
+        x[plane] = oi.x;
+        y[plane] = oi.y;
+        e0 = fmaf(aa.x, oi.x, e0);
+        e1 = fmaf(aa.y, oi.y, e1);
+      }
+      ksum_add(ek, e0);
+      ksum_add(ek, e1);
+    }
+  }
+}
 
-// Real states in shared memory: psi for items up to kBSmemQubits + 1 qubits,
-// lambda beside it up to kBSmemQubits; larger states in the block's global
-// workspace slot (read as 4 x 2^nmax floats).
-template <int K, int MAXT, int MINB>
-__global__ void __launch_bounds__(MAXT, MINB) kbatch_re(const BatchArgs A) {
-  __shared__ float mats[8 * kBMaxGates];
-  __shared__ float2 wpart[(MAXT / 32) * kBMaxParams];  // per warp and parameter: (sum, comp)
+// forward pass, lambda and the reverse sweep of one item; returns this thread's energy
+template <int K, bool CX>
+__device__ __forceinline__ double run_item(float* psi, float* lam, const BCirc& C, int pstride,
+                                           const BSmem& S) {
+  const int np = max(C.n, K);
+  // |0...0>: swzr(0) = 0 and swzr maps every other index to a nonzero one
+  for (int x = threadIdx.x; x < ((CX ? 2 : 1) << np); x += blockDim.x) psi[x] = x == 0 ? 1.f : 0.f;
+  if (C.n < K)  // the tile is wider than the state: what lies beyond stays zero
+    for (int x = threadIdx.x; x < ((CX ? 2 : 1) << np); x += blockDim.x) lam[x] = 0.f;
+  __syncthreads();
+  for (int gg = 0; gg < C.ngroups; ++gg) {
+    group_fwd<K, CX>(psi, np, S.grp[gg], S);
+    __syncthreads();
+  }
+  float2 ek = make_float2(0.f, 0.f);
+  if (term_slices(C.n) == 8)
+    apply_terms<8, CX>(psi, lam, C, np, S, ek);
+  else
+    apply_terms<2, CX>(psi, lam, C, np, S, ek);
+  __syncthreads();
+  for (int gg = C.ngroups - 1; gg >= 0; --gg) {
+    group_bwd<K, CX>(psi, lam, np, pstride, S.grp[gg], S);
+    __syncthreads();
+  }
+  return ksum_value(ek);
+}
+
+template <int K, int MAXT, int MINB, bool CX, bool SMS>
+__global__ void __launch_bounds__(MAXT, MINB) kbatch(const BatchArgs A) {
   __shared__ double red[MAXT / 32];
   __shared__ int s_item;
   extern __shared__ __align__(16) unsigned char dyn_smem[];
-  BOp* sops = reinterpret_cast<BOp*>(dyn_smem);
-  BGroup* sgrp = reinterpret_cast<BGroup*>(dyn_smem + kBOpsBytes);
-  int2* sterm = reinterpret_cast<int2*>(dyn_smem + kBOpsBytes + kBGroupBytes);
-  float* scoef = reinterpret_cast<float*>(dyn_smem + kBOpsBytes + kBGroupBytes + kBTermBytes);
-  float* ssign = reinterpret_cast<float*>(dyn_smem + kBCacheBytes);
-  float* dyn_state = reinterpret_cast<float*>(dyn_smem + kBCacheBytes + kBSignBytes);
-  constexpr int kSm = kBSmemQubits + 1;  // 2^15 floats = kBSmemStateBytes
+  const BSmem S = {reinterpret_cast<float*>(dyn_smem + A.o_mats),
+                   reinterpret_cast<float2*>(dyn_smem + A.o_wpart),
+                   reinterpret_cast<BOp*>(dyn_smem + A.o_ops),
+                   reinterpret_cast<BGroup*>(dyn_smem + A.o_grp),
+                   reinterpret_cast<int2*>(dyn_smem + A.o_term),
+                   reinterpret_cast<float*>(dyn_smem + A.o_tcoef),
+                   reinterpret_cast<float*>(dyn_smem + A.o_sign)};
+  float* const dyn_state = reinterpret_cast<float*>(dyn_smem + A.o_state);
   const int nwarps = blockDim.x >> 5;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* const gpsi = reinterpret_cast<float*>(A.work + (size_t)blockIdx.x * (size_t(2) << A.nmax));
-  float* const glam = gpsi + (size_t(1) << A.nmax);
+  float* const glam = gpsi + (size_t(2) << A.nmax);
   while (true) {
     if (threadIdx.x == 0) s_item = atomicAdd(A.queue, 1);
     __syncthreads();
@@ -979,87 +963,85 @@ __global__ void __launch_bounds__(MAXT, MINB) kbatch_re(const BatchArgs A) {
     const int item = A.order[slot];
     const BCirc C = A.circs[A.item_circ[item]];
     const double* th = A.theta + A.theta_off[item];
-    const int dim = 1 << C.n;
-    float* psi = C.n <= kSm ? dyn_state : gpsi;
-    float* lam = C.n < kSm ? dyn_state + (1 << (kSm - 1)) : glam;
-    // gate matrices (fp64 trigonometry, rounded once): real kinds only
+    // gate matrices (fp64 trigonometry, rounded once), zero partials
     for (int gi = threadIdx.x; gi < C.ngates; gi += blockDim.x) {
       const BGateDesc d = A.gates[C.gate0 + gi];
       const double a = d.param >= 0 ? th[d.param] : d.angle;
       double s, c;
-      sincos(0.5 * a, &s, &c);
-      double m[4] = {1, 0, 0, 1};
+      sincos(d.kind == SV_GATE_U1 || (d.free_rot && d.kind == SV_GATE_RZ) ? a : 0.5 * a, &s, &c);
+      double m[8] = {0, 0, 0, 0, 0, 0, 0, 0};
       const double r2 = 0.70710678118654752440;
-      switch (d.kind) {
-        case SV_GATE_H: m[0] = r2; m[1] = r2; m[2] = r2; m[3] = -r2; break;
-        case SV_GATE_X: m[0] = 0; m[1] = 1; m[2] = 1; m[3] = 0; break;
-        case SV_GATE_Z: m[3] = -1; break;
-        default: m[0] = c; m[1] = -s; m[2] = s; m[3] = c; break;  // RY
+      if (d.free_rot) {
+        if (d.kind == SV_GATE_RZ) {
+          m[0] = c;
+          m[1] = s;
+        } else {
+          if (c < 0) {
+            c = -c;
+            s = -s;
+          }
+          m[0] = -s / (1.0 + c);
+          m[1] = s;
+        }
+      } else {
+        switch (d.kind) {
+          case SV_GATE_H: m[0] = r2; m[2] = r2; m[4] = r2; m[6] = -r2; break;
+          case SV_GATE_X: m[2] = 1; m[4] = 1; break;
+          case SV_GATE_Y: m[3] = -1; m[5] = 1; break;
+          case SV_GATE_Z: m[0] = 1; m[6] = -1; break;
+          case SV_GATE_RX: m[0] = c; m[3] = -s; m[5] = -s; m[6] = c; break;
+          case SV_GATE_RY: m[0] = c; m[2] = -s; m[4] = s; m[6] = c; break;
+          case SV_GATE_RZ: m[0] = c; m[1] = -s; m[6] = c; m[7] = s; break;
+          default: m[0] = 1; m[6] = c; m[7] = s;  // U1: diag(1, e^{ia})
+        }
       }
-      for (int e = 0; e < 4; ++e) mats[8 * gi + 2 * e] = (float)m[e];
-      // RY as shears (see re2_rot): cos >= 0 up to the state's sign
-      if (c < 0) {
-        c = -c;
-        s = -s;
-      }
-      mats[8 * gi + 1] = (float)(-s / (1.0 + c));
-      mats[8 * gi + 3] = (float)s;
+      for (int e = 0; e < 8; ++e) S.mats[8 * gi + e] = (float)m[e];
     }
-    for (int x = threadIdx.x; x < dim; x += blockDim.x) psi[x] = x == 0 ? 1.f : 0.f;
-    for (int i = threadIdx.x; i < nwarps * kBMaxParams; i += blockDim.x)
-      wpart[i] = make_float2(0.f, 0.f);
-    {
+    for (int i = threadIdx.x; i < nwarps * A.pstride; i += blockDim.x)
+      S.wpart[i] = make_float2(0.f, 0.f);
+    {  // this item's groups and operations, operation indices rebased to the cache
       const int ng = C.ngroups;
       const int op_base = ng ? A.rgroups[C.group0].op0 : 0;
       const int nops = ng ? A.rgroups[C.group0 + ng - 1].op1 - op_base : 0;
-      for (int i = threadIdx.x; i < nops; i += blockDim.x) sops[i] = A.rops[op_base + i];
-      for (int i = threadIdx.x; i < 32 * C.nsign; i += blockDim.x)
-        ssign[i] = (A.rsigns[C.sign0 + (i >> 5)] >> (i & 31)) & 1 ? -1.f : 1.f;
+      for (int i = threadIdx.x; i < nops; i += blockDim.x) S.ops[i] = A.rops[op_base + i];
+      for (int i = threadIdx.x; i < (C.nsign << K); i += blockDim.x)
+        S.sign[i] = (A.rsigns[C.sign0 + (i >> K)] >> (i & ((1 << K) - 1))) & 1 ? -1.f : 1.f;
       for (int i = threadIdx.x; i < ng; i += blockDim.x) {
         BGroup G = A.rgroups[C.group0 + i];
         G.op0 -= op_base;
         G.op1 -= op_base;
-        sgrp[i] = G;
+        for (int k = G.k; k < K; ++k) G.bits[k] = (uint8_t)k;  // n < K: the group is the state
+        S.grp[i] = G;
       }
+      const int js = term_slices(C.n), dlog = C.n - (js == 8 ? 3 : 1);
       for (int t = threadIdx.x; t < C.nterms; t += blockDim.x) {
         const BTerm T = A.terms[C.term0 + t];
-        const int xm = (int)T.xm, zm = (int)T.zm;
-        sterm[t] = make_int2(swzr(xm), (int)((unsigned)zm | ((unsigned)__popc(xm & zm) << 31)));
-        scoef[t] = (float)T.cre;  // a real batch has cim = 0
+        const int xm = (int)T.xm, zm = (int)T.zm;  // n <= SV_BATCH_MAX_QUBITS < 30
+        const bool imag = __popc(xm & zm) & 1;     // i^{#Y} imaginary
+        S.term[t] = make_int2(swzr(xm), (int)((unsigned)zm | ((unsigned)imag << 31)));
+        // sign at x: the parity of (x ^ xm) & zm
+        const float c = (float)(imag ? -T.cim : T.cre);
+        for (int j = 0; j < 8; ++j)
+          S.tcoef[8 * t + j] = __popc((j << dlog) & zm) & 1 ? -c : c;
       }
     }
-    __syncthreads();
-    for (int gg = 0; gg < C.ngroups; ++gg) {
-      group_fwd_re<K>(psi, C.n, sgrp[gg], sops, mats, ssign);
-      __syncthreads();
+    const int size = (CX ? 2 : 1) << max(C.n, K);  // floats of one state
+    double e;
+    if constexpr (SMS) {
+      if (2 * size <= A.state_floats)
+        e = run_item<K, CX>(dyn_state, dyn_state + size, C, A.pstride, S);
+      else
+        e = run_item<K, CX>(size <= A.state_floats ? dyn_state : gpsi, glam, C, A.pstride, S);
+    } else {
+      e = run_item<K, CX>(gpsi, glam, C, A.pstride, S);
     }
-    // lambda = H psi, E = <psi|lambda>
-    float2 ek = make_float2(0.f, 0.f);
-    for (int x = threadIdx.x; x < dim; x += blockDim.x) {
-      const int px = swzr(x);
-      const float a = psi[px];
-      float d = 0.f;
-      for (int t = 0; t < C.ndiag; ++t) d += (__popc(x & sterm[t].y) & 1) ? -scoef[t] : scoef[t];
-      float o = d * a;
-      for (int t = C.ndiag; t < C.nterms; ++t) {
-        const int2 q = sterm[t];
-        const float sb = scoef[t] * psi[px ^ q.x];
-        o += ((__popc(x & q.y) + ((unsigned)q.y >> 31)) & 1) ? -sb : sb;
-      }
-      lam[px] = o;
-      ksum_add(ek, a * o);
-    }
-    double e = warp_sum_d(ksum_value(ek));
+    e = warp_sum_d(e);
     if (lane == 0) red[warp] = e;
     __syncthreads();
-    for (int gg = C.ngroups - 1; gg >= 0; --gg) {
-      group_bwd_re<K>(psi, lam, C.n, sgrp[gg], sops, mats, ssign, wpart);
-      __syncthreads();
-    }
     const int toff = A.theta_off[item];
     for (int p = threadIdx.x; p < C.nparams; p += blockDim.x) {
       double g = 0.0;
-      for (int w = 0; w < nwarps; ++w) g += ksum_value(wpart[w * kBMaxParams + p]);
+      for (int w = 0; w < nwarps; ++w) g += ksum_value(S.wpart[w * A.pstride + p]);
       A.grad[toff + p] = g;
     }
     if (threadIdx.x == 0) {
@@ -1412,7 +1394,7 @@ struct sv_batch_s {
   sv::BGroup* groups = nullptr;
   sv::BOp* ops = nullptr;
   sv::BTerm* terms = nullptr;
-  sv::BGroup* rgroups = nullptr;  // real-amplitude lists (batches that may run kbatch_re)
+  sv::BGroup* rgroups = nullptr;  // the single-block kernels' lists
   sv::BOp* rops = nullptr;
   uint32_t* rsigns = nullptr;
   int* order = nullptr;
@@ -1421,6 +1403,8 @@ struct sv_batch_s {
   int* queue = nullptr;
   float2* work = nullptr;
   size_t work_slots = 0;
+  // the largest of the batch's circuits, for the blocks' shared memory
+  int max_gates = 0, max_params = 0, max_ops = 0, max_groups = 0, max_terms = 0, max_signs = 0;
   std::vector<int> h_theta_off;
   // captured graph
   cudaGraphExec_t gexec = nullptr;
@@ -1436,7 +1420,7 @@ struct HostPlan {
   std::vector<BGroup> groups;
   std::vector<BOp> ops;
   std::vector<BTerm> terms;
-  std::vector<BGroup> rgroups;  // filled by real_lists
+  std::vector<BGroup> rgroups;  // filled by tile_lists
   std::vector<BOp> rops;
   std::vector<uint32_t> rsigns;
 };
@@ -1459,7 +1443,8 @@ bool plan_circuit(const sv_circuit* c, const sv_pauli_sum* H, int k, HostPlan* P
   std::vector<uint64_t> qm(c->n_gates);
   for (int i = 0; i < c->n_gates; ++i) {
     const sv_gate& g = c->gates[i];
-    BGateDesc d{g.kind, g.param, g.angle};
+    const bool rot = g.kind == SV_GATE_RX || g.kind == SV_GATE_RY || g.kind == SV_GATE_RZ;
+    BGateDesc d{g.kind, g.param, g.angle, rot && g.n_ctrl == 0};
     P->gates.push_back(d);
     uint64_t m = uint64_t(1) << (n - 1 - g.targets[0]);
     for (int j = 0; j < g.n_ctrl; ++j) m |= uint64_t(1) << (n - 1 - g.controls[j]);
@@ -1539,10 +1524,13 @@ bool plan_circuit(const sv_circuit* c, const sv_pauli_sum* H, int k, HostPlan* P
   return P->ops.size() < (size_t)0x7fffffff;
 }
 
-// The real-amplitude kernel's lists of every circuit of P: RYs without controls as
-// rotations, and each run of sign flips with nothing else on their bits in
-// between as one pattern over the group's 2^k indices.
-void real_lists(HostPlan* P) {
+// A circuit with more patterns keeps its single flips.
+constexpr int kBMaxSigns = 96;
+
+// The single-block kernels' lists of every circuit of P: rotations without controls,
+// and each run of sign flips with no other than diagonal operations on their bits
+// in between as one pattern over the group's 2^k indices.
+void tile_lists(HostPlan* P) {
   for (BCirc& C : P->circs) {
     for (int merge = 1; merge >= 0; --merge) {
       const size_t o0 = P->rops.size(), s0 = P->rsigns.size(), g0 = P->rgroups.size();
@@ -1569,9 +1557,10 @@ void real_lists(HostPlan* P) {
               if ((r & bits) == bits) P->rsigns[open] ^= 1u << r;
             continue;
           }
-          dirty |= bits;
-          if (op.cls == BC_REAL && op.cm == 0 && P->gates[C.gate0 + op.gi].kind == SV_GATE_RY)
-            op.cls = BC_ROT;
+          if (op.cls != BC_DIAG && op.cls != BC_PHASE) dirty |= bits;
+          const BGateDesc& d = P->gates[C.gate0 + op.gi];
+          if (d.free_rot)
+            op.cls = d.kind == SV_GATE_RX ? BC_RX : d.kind == SV_GATE_RY ? BC_ROT : BC_RZ;
           P->rops.push_back(op);
         }
         G.op1 = (int32_t)P->rops.size();
@@ -1604,23 +1593,66 @@ void free_batch(sv_batch b) {
 }
 
 typedef void (*BatchKernel)(const BatchArgs);
-// Kernel variants by (group width, threads per block, resident blocks per
-// SM): more resident blocks need fewer registers and less shared memory.
-BatchKernel smem_kernel_for(int k) {
-  return k == 2 ? kbatch<2, 512, 1, true> : k == 3 ? kbatch<3, 512, 1, true> : kbatch<4, 512, 1, true>;
+// Kernel variants by (group width, threads per block, resident blocks per SM).
+// With states in shared memory: 2^k amplitudes a thread make a group of an n-qubit
+// item one round of a block of 2^(n - k) threads, so items of 11 qubits want four blocks of
+// 128 threads an SM and items of 14 one of 512.
+BatchKernel real_kernel_for(int k, int threads) {
+  if (threads <= 128) return k <= 4 ? kbatch<4, 128, 4, false, true> : kbatch<5, 128, 4, false, true>;
+  if (threads <= 256) return k <= 4 ? kbatch<4, 256, 2, false, true> : kbatch<5, 256, 2, false, true>;
+  return k <= 3   ? kbatch<3, 512, 1, false, true>
+         : k == 4 ? kbatch<4, 512, 1, false, true>
+                  : kbatch<5, 512, 1, false, true>;
 }
+BatchKernel smem_kernel_for(int k, int threads) {
+  if (threads <= 128) return k <= 3 ? kbatch<3, 128, 4, true, true> : kbatch<4, 128, 4, true, true>;
+  if (threads <= 256) return k <= 3 ? kbatch<3, 256, 2, true, true> : kbatch<4, 256, 2, true, true>;
+  return k == 2   ? kbatch<2, 512, 1, true, true>
+         : k == 3 ? kbatch<3, 512, 1, true, true>
+                  : kbatch<4, 512, 1, true, true>;
+}
+// states in the global workspace
 BatchKernel kernel_for(int k, int threads, int per_sm) {
-  if (threads >= 512) return k == 2 ? kbatch<2, 512, 1> : k == 3 ? kbatch<3, 512, 1> : kbatch<4, 512, 1>;
-  if (threads <= 128) return k == 2 ? kbatch<2, 128, 8> : kbatch<3, 128, 8>;
-  if (per_sm >= 4) return k == 2 ? kbatch<2, 256, 4> : kbatch<3, 256, 4>;
-  return k == 2 ? kbatch<2, 256, 2> : k == 3 ? kbatch<3, 256, 2> : kbatch<4, 256, 2>;
+  if (threads <= 128) return k == 2 ? kbatch<2, 128, 8, true, false> : kbatch<3, 128, 8, true, false>;
+  if (per_sm >= 4) return k == 2 ? kbatch<2, 256, 4, true, false> : kbatch<3, 256, 4, true, false>;
+  return k == 2   ? kbatch<2, 256, 2, true, false>
+         : k == 3 ? kbatch<3, 256, 2, true, false>
+                  : kbatch<4, 256, 2, true, false>;
 }
 
 // register groups of 2 or 3 qubits (4 would spill at 512 threads per block)
 BatchKernel cluster_kernel_for(int k) { return k == 2 ? kbatch_cl<2> : kbatch_cl<3>; }
 
-BatchKernel real_kernel_for(int k) {
-  return k <= 3 ? kbatch_re<3, 512, 1> : k == 4 ? kbatch_re<4, 512, 1> : kbatch_re<5, 512, 1>;
+// Offsets of a block's shared memory (see BSmem) for this batch and group width k, and
+// the state memory that `per_sm` resident blocks leave it (a power of two, no
+// more than the largest item wants); returns the bytes.
+size_t block_smem(sv_batch b, int k, int threads, int per_sm, bool states, bool re, BatchArgs* A) {
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 15) & ~size_t(15);
+    return (int)o;
+  };
+  A->o_mats = take(sizeof(float) * 8 * b->max_gates);
+  A->o_wpart = take(sizeof(float2) * (threads / 32) * b->max_params);
+  A->o_ops = take(sizeof(BOp) * b->max_ops);
+  A->o_grp = take(sizeof(BGroup) * b->max_groups);
+  A->o_term = take(sizeof(int2) * b->max_terms);
+  A->o_tcoef = take(sizeof(float) * 8 * b->max_terms);
+  A->o_sign = take((sizeof(float) << k) * b->max_signs);
+  A->o_state = (int)at;
+  A->pstride = b->max_params;
+  A->state_floats = 0;
+  if (states) {
+    // 228 KiB an SM, 1 KiB of it and the static variables taken by each block
+    const size_t budget = (size_t)228 * 1024 / per_sm - 1024 - 512;
+    const size_t want = size_t(re ? 2 : 4) << std::max(b->nmax, k);
+    size_t f = 0;
+    for (size_t c = 64; c <= want && at + sizeof(float) * c <= budget; c *= 2) f = c;
+    A->state_floats = (int)f;
+    at += sizeof(float) * f;
+  }
+  return at;
 }
 
 sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* grad,
@@ -1639,27 +1671,13 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
   A.item_circ = b->item_circ;
   A.theta_off = b->theta_off;
   A.n_items = b->n_items;
-  A.nmax = b->nmax;
+  A.nmax = std::max(b->nmax, 5);  // a tile of 2^k amplitudes at least
   A.theta = theta;
   A.energy = energy;
   A.grad = grad;
   A.work = b->work;
   A.queue = b->queue;
   SV_CUDA_TRY(cudaMemsetAsync(b->queue, 0, sizeof(int), st));
-  if (re) {
-    BatchKernel kern = real_kernel_for(k);
-    constexpr size_t smem = kBCacheBytes + kBSignBytes + kBSmemStateBytes;
-    static bool attr[6] = {false, false, false, false, false, false};
-    if (!attr[k]) {
-      SV_CUDA_TRY(
-          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      attr[k] = true;
-    }
-    ProfScope prof(st, "kbatch_re");
-    kern<<<blocks, 512, smem, st>>>(A);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return check_launch("batch kernel (real amplitudes)");
-  }
   if (cl) {
     BatchKernel kern = cluster_kernel_for(k);
     static bool attr[5] = {false, false, false, false, false};
@@ -1673,34 +1691,28 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return check_launch("batch cluster kernel");
   }
-  if (sms) {
-    BatchKernel kern = smem_kernel_for(k);
-    static bool attr[5] = {false, false, false, false, false};
-    if (!attr[k]) {
-      SV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(kBCacheBytes + kBSmemStateBytes)));
-      attr[k] = true;
-    }
-    ProfScope prof(st, "kbatch_smem");
-    kern<<<blocks, 512, kBCacheBytes + kBSmemStateBytes, st>>>(A);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return check_launch("batch kernel (shared-memory states)");
-  }
-  BatchKernel kern = kernel_for(k, threads, std::max(1, blocks / std::max(1, b->sms)));
+  const int per_sm = std::max(1, blocks / std::max(1, b->sms));
+  BatchKernel kern = re    ? real_kernel_for(k, threads)
+                     : sms ? smem_kernel_for(k, threads)
+                           : kernel_for(k, threads, per_sm);
+  const size_t smem = block_smem(b, k, threads, per_sm, re || sms, re, &A);
   {
-    // static (matrices, partials) + dynamic (descriptor cache) shared memory
-    // can exceed the 48 KiB default: opt in once per kernel variant
+    // opt in to more than the default 48 KiB, to the most any batch has asked for
     static std::mutex mu;
-    static std::vector<BatchKernel> done;
+    static std::vector<std::pair<BatchKernel, size_t>> done;
     std::lock_guard<std::mutex> lk(mu);
-    if (std::find(done.begin(), done.end(), kern) == done.end()) {
-      SV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kBCacheBytes));
-      done.push_back(kern);
+    auto it = std::find_if(done.begin(), done.end(), [&](const auto& d) { return d.first == kern; });
+    if (it == done.end() || it->second < smem) {
+      SV_CUDA_TRY(
+          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      if (it == done.end())
+        done.push_back({kern, smem});
+      else
+        it->second = smem;
     }
   }
-  ProfScope prof(st, "kbatch");
-  kern<<<blocks, threads, kBCacheBytes, st>>>(A);
+  ProfScope prof(st, re ? "kbatch_re" : sms ? "kbatch_smem" : "kbatch");
+  kern<<<blocks, threads, smem, st>>>(A);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("batch kernel");
 }
@@ -1836,8 +1848,8 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
   struct Cand {
     int k, threads, per_sm;
     bool cl;          // two-block clusters (per_sm = 1, threads = kClThreads)
-    bool sms = false; // states in shared memory up to 14 qubits (512 threads, 1 per SM)
-    bool re = false;  // real amplitudes (kbatch_re, 512 threads, 1 per SM)
+    bool sms = false; // states in shared memory as far as they fit
+    bool re = false;  // real amplitudes
   };
   // real batch: every gate real (H, X, Z, RY, with controls) and every term a
   // real matrix (an even number of Y factors)
@@ -1861,16 +1873,19 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
     }
     cands.push_back({std::max(4, width), 512, 1, false, true, true});
   } else if (tune == 1) {
-    if (all_real)
-      for (int kr = std::max(3, width); kr <= 5; ++kr) cands.push_back({kr, 512, 1, false, true, true});
-    const Cand all[] = {{2, 512, 1, false, true}, {3, 512, 1, false, true}, {4, 512, 1, false, true},
+    const Cand all[] = {{3, 512, 1, false, true, true}, {4, 512, 1, false, true, true},
+                        {4, 256, 2, false, true, true}, {4, 128, 4, false, true, true},
+                        {5, 512, 1, false, true, true}, {5, 256, 2, false, true, true},
+                        {5, 128, 4, false, true, true},
+                        {2, 512, 1, false, true}, {3, 512, 1, false, true}, {4, 512, 1, false, true},
+                        {3, 256, 2, false, true}, {4, 256, 2, false, true},
+                        {3, 128, 4, false, true}, {4, 128, 4, false, true},
                         {2, kClThreads, 1, true}, {3, kClThreads, 1, true},
-                        {2, 512, 1, false}, {3, 512, 1, false}, {4, 512, 1, false},
                         {2, 256, 2, false}, {3, 256, 2, false}, {4, 256, 2, false},
                         {2, 256, 4, false}, {3, 256, 4, false}, {2, 128, 8, false},
                         {3, 128, 8, false}};
     for (const Cand& c : all)
-      if (c.k >= width) cands.push_back(c);
+      if (c.k >= width && (!c.re || all_real)) cands.push_back(c);
   } else if (tune == 2 && width <= 3) {
     cands.push_back({3, kClThreads, 1, true});
   } else if (tune == 3) {
@@ -1889,7 +1904,7 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
   if (!st) st = upload(&b->theta_off, toff);
   if (!st) {
     cudaError_t e = cudaMalloc(&b->queue, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&b->work, b->work_slots * (sizeof(float2) << (nmax + 1)));
+    if (e == cudaSuccess) e = cudaMalloc(&b->work, b->work_slots * (sizeof(float2) << (std::max(nmax, 5) + 1)));
     if (e != cudaSuccess) {
       set_error("sv_batch_create: %s", cudaGetErrorString(e));
       st = e == cudaErrorMemoryAllocation ? SV_ERR_OOM : SV_ERR_CUDA;
@@ -1902,7 +1917,18 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
         set_error("sv_batch_create: a gate does not fit a register group of %d qubits", k);
         return SV_ERR_INVALID;
       }
-    if (all_real) real_lists(&P);
+    tile_lists(&P);
+    b->max_gates = b->max_params = b->max_ops = b->max_groups = b->max_terms = b->max_signs = 1;
+    for (const BCirc& C : P.circs) {
+      b->max_gates = std::max(b->max_gates, C.ngates);
+      b->max_params = std::max(b->max_params, C.nparams);
+      b->max_terms = std::max(b->max_terms, C.nterms);
+      b->max_groups = std::max(b->max_groups, C.ngroups);
+      b->max_signs = std::max(b->max_signs, C.nsign);
+      if (C.ngroups)
+        b->max_ops = std::max(b->max_ops, P.rgroups[C.group0 + C.ngroups - 1].op1 -
+                                              P.rgroups[C.group0].op0);
+    }
     void* olds[] = {b->circs, b->gates, b->groups, b->ops, b->terms, b->rgroups, b->rops, b->rsigns};
     for (void* p : olds)
       if (p) cudaFree(p);
@@ -1913,9 +1939,9 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
     if (!s2) s2 = upload(&b->groups, P.groups);
     if (!s2) s2 = upload(&b->ops, P.ops);
     if (!s2) s2 = upload(&b->terms, P.terms);
-    if (!s2 && all_real) s2 = upload(&b->rgroups, P.rgroups);
-    if (!s2 && all_real) s2 = upload(&b->rops, P.rops);
-    if (!s2 && all_real) s2 = upload(&b->rsigns, P.rsigns);
+    if (!s2) s2 = upload(&b->rgroups, P.rgroups);
+    if (!s2) s2 = upload(&b->rops, P.rops);
+    if (!s2) s2 = upload(&b->rsigns, P.rsigns);
     return s2;
   };
   double* th = nullptr;
