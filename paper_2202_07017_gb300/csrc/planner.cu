@@ -186,7 +186,7 @@ void move_input_phases(std::vector<FGate>* F) {
     if (f.type == FG_1Q && f.cmask == 0 && !(is_zero(f.m[1]) && is_zero(f.m[2]))) {
       Before& b = before[f.t];
       const cd u = f.m[0], w = f.m[1];
-      const double d = std::hypot(u.re, u.im) * std::hypot(w.re, w.im);
+      const double d = std::sqrt((u.re * u.re + u.im * u.im) * (w.re * w.re + w.im * w.im));
       const cd beta{-(w.re * u.re + w.im * u.im) / d, -(w.im * u.re - w.re * u.im) / d};
       if (b.gate >= 0 && d > 1e-10 && is_unitary2(f.m) && !is_one(beta)) {
         const cd in[4] = {{1, 0}, {0, 0}, {0, 0}, beta};
@@ -489,7 +489,7 @@ void form_passes(const std::vector<FGate>& F, int n, const FusionConfig& cfg,
     // qubits, whose light cones close after a layer or two: a random layered
     // circuit of depth 30 on 28 qubits takes 49 passes, with windows 24.
     uint64_t S = lowL;
-    int best = collect(&S, true, F.size(), nullptr);
+    int best = n > cfg.m ? collect(&S, true, F.size(), nullptr) : 0;  // or every qubit
     for (int b = 0; b < n && popc(S) < cfg.m; ++b) S |= uint64_t(1) << b;
     const int w = cfg.m - cfg.L;
     for (int lo = cfg.L; lo + w <= n && n > cfg.m; ++lo) {
