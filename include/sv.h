@@ -369,15 +369,14 @@ sv_status sv_grad_fused(sv_state s, const sv_circuit* c, const double* theta,
  * hamiltonians[item_circuit[i]] and the adjoint gradient dE_i/dtheta.  All
  * items run in one persistent kernel whose thread blocks pull items from an
  * atomic queue (longest first); each block keeps its item's two states in a
- * workspace slot that stays in L1/L2, or (variants the autotuner may pick)
- * in shared memory as far as they fit: psi of up to 14 qubits and lambda of up
- * to 13 with one block per SM.  Energies
- * and gradients accumulate per warp in compensated fp32 and across warps in
- * fp64, in a fixed order.  A batch whose gates are all real (H X Z RY, with
- * controls) and whose terms are all real matrices (an even number of Y
- * factors) keeps real states: a variant the autotuner may pick carries psi
- * and lambda as fp32 real vectors (psi of up to 15 qubits and lambda of up to
- * 14 in shared memory), with the same results up to rounding.
+ * workspace slot that stays in L1/L2, or (variants the autotuner may pick) in
+ * shared memory: up to 13 qubits in one block and up to 15 over four.  Energies and
+ * gradients accumulate per warp in compensated fp32 and across warps in fp64, in a
+ * fixed order.  A batch whose gates are all real (H X Z RY, with controls) and
+ * whose terms are all real matrices (an even number of Y factors) keeps real
+ * states: a variant the autotuner may pick carries psi and lambda as fp32 real
+ * vectors (up to 14 qubits in one block's shared memory, up to 16 over four), with
+ * the same results up to rounding.
  *
  * Limits: <= SV_BATCH_MAX_QUBITS qubits, <= 480 gates and <= 256
  * parameters per circuit, <= 64 Pauli terms per Hamiltonian; gates are the
@@ -393,11 +392,12 @@ sv_status sv_grad_fused(sv_state s, const sv_circuit* c, const double* theta,
  * qubits, states in a global workspace slot per block.  tune = 1: the
  * autotuner times on the batch, and keeps the fastest of (this synchronises the
  * device): those single blocks with k in {2,3,4}, 128 or 256 threads and 2, 4 or 8
- * per SM; single blocks of 512, 256 or 128 threads, 1, 2 or 4 per SM, keeping states
- * in shared memory as far as they fit; and two-block clusters of 512 threads that
- * split each item's psi and lambda by their top bit over the pair and keep them in
- * shared memory up to 14 qubits, k <= 3.  For a real batch the autotuner also times
- * the real-amplitude kernel (512, 256 or 128 threads, k in {3,4,5}).
+ * per SM; one block of 512 threads per SM with states in shared memory, items of
+ * few qubits side by side in teams of 64 to 256 threads and items of two more
+ * qubits than a block holds over clusters of four blocks; and two-block clusters
+ * of 512 threads that split each item's psi and lambda by their top bit over the
+ * pair and keep them in shared memory up to 14 qubits, k <= 3.  For a real batch the
+ * autotuner also times the real-amplitude kernel (k in {3,4,5}).
  * tune = 2: the cluster kernel with k = 3 (the tune = 0 tile if a gate has 3
  * controls); tune = 3: single blocks of 512 threads with states in shared
  * memory, k = 4; tune = 4: the real-amplitude kernel, k = 4 (SV_ERR_INVALID

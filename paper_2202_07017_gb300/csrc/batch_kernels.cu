@@ -42,7 +42,9 @@ static_assert(SV_BATCH_MAX_QUBITS < 31, "term masks are packed in 31 bits");
 struct BCirc {
   int n, ngates, gate0, ngroups, group0, nparams, nterms, term0;
   int ndiag;  // terms[term0 .. term0 + ndiag) are diagonal (no X or Y factor)
-  int nsign, sign0;  // the single-block kernels' sign patterns, rsigns[sign0 .. sign0 + nsign)
+  // the single-block kernels' sign patterns rsigns[sign0 .. sign0 + nsign), rotations
+  // rots[rot0 .. rot0 + nrot) and other gates gens[gen0 .. gen0 + ngen)
+  int nsign, sign0, nrot, rot0, ngen, gen0;
 };
 struct BGateDesc {
   int kind;   // SV_GATE_* (1-qubit kinds)
@@ -50,6 +52,20 @@ struct BGateDesc {
   double angle;
   int free_rot;  // RX, RY or RZ without controls
 };
+struct BRot {  // a rotation without controls in the single-block kernels' lists
+  int kind, param;
+  double angle;
+};
+// One size class of items: teams of `ts` threads, 512 / ts of them in a block at once,
+// each with `stride` bytes of shared memory (byte offsets o_*, see BSmem).
+struct BPhase {
+  int first, count;  // items order[first .. first + count)
+  int ts, stride;
+  int o_mats, o_wpart, o_ops, o_grp, o_term, o_tcoef, o_sign, o_state;
+  int pstride;       // gradient partials of one warp
+  int state_floats;  // floats of state memory from o_state
+};
+constexpr int kBPhases = 4;
 struct alignas(16) BGroup {
   uint8_t k, bits[5];
   int32_t op0, op1;
@@ -76,6 +92,8 @@ struct BatchArgs {
   const BGroup* rgroups;   // the same groups over rops: the single-block kernels' lists
   const BOp* rops;
   const uint32_t* rsigns;
+  const BRot* rots;
+  const BGateDesc* gens;
   const int* order;      // items, longest first
   const int* item_circ;  // circuit of each item
   const int* theta_off;  // parameter offset of each item
@@ -85,10 +103,8 @@ struct BatchArgs {
   double* grad;
   float2* work;          // gridDim.x slots of 2 x 2^nmax amplitudes
   int* queue;
-  // the single-block kernels' dynamic shared memory (byte offsets, see BSmem)
-  int o_mats, o_wpart, o_ops, o_grp, o_term, o_tcoef, o_sign, o_state;
-  int pstride;       // gradient partials of one warp
-  int state_floats;  // floats of state memory from o_state
+  int n_phases;
+  BPhase phase[kBPhases], wide;  // queue[0 .. kBPhases), and queue[kBPhases] for the wide items
 };
 
 __device__ __forceinline__ float warp_sum_f(float v) {
@@ -120,9 +136,10 @@ __device__ __forceinline__ double ksum_value(float2 a) { return (double)a.x - (d
 // multiply-adds (dense) to 8 (real: H, X, RY; imaginary off-diagonal: Y, RX;
 // diagonal: RZ), to 4 on one amplitude (phase: U1) or to a sign flip (Z, CZ).
 // The single-block kernels' lists also have BC_SIGN (a run of sign flips as one
-// pattern, gi its index) and rotations without controls.
+// pattern, gi its index) and BC_RUN (cm rotations without controls from rotation gi on,
+// bit 3 b + 0, 1, 2 of param for an RX, RY, RZ on group bit b, in that order).
 enum { BC_DENSE = 0, BC_REAL = 1, BC_IMOFF = 2, BC_DIAG = 3, BC_PHASE = 4, BC_NEG = 5,
-       BC_SIGN = 6, BC_ROT = 7, BC_RX = 8, BC_RZ = 9 };
+       BC_SIGN = 6, BC_RUN = 7 };
 
 // (a, b) <- M (a, b) for every register pair on group bit B (with controls cm
 // when CTRL).
@@ -306,6 +323,17 @@ __device__ __forceinline__ int sub_base(int s, const int (&lm)[K], int kk) {
   return b;
 }
 
+template <int I, int N, typename F>
+__device__ __forceinline__ void static_for(const F& f) {
+  if constexpr (I < N) {
+    f(std::integral_constant<int, I>());
+    static_for<I + 1, N>(f);
+  }
+}
+
+// Byte offsets and masks of a state split over a cluster carry the block's rank from here.
+constexpr int kRankShift = 28;
+
 // Slices of the index range that one thread of apply_terms takes.
 __device__ __forceinline__ int term_slices(int n) { return n >= 10 ? 8 : 2; }
 
@@ -333,7 +361,7 @@ __device__ __forceinline__ int term_slices(int n) { return n >= 10 ? 8 : 2; }
 // dropped).  A run of CZs is one multiplication by its sign pattern.  Per tile of 16 or
 // 32 amplitudes a rotation costs 24 paired FMAs in place of 64 (RX, RY) or 128 (RZ)
 // single ones: 768 parameter sets of the n = 11, 6-layer random layered circuit and 192
-// mixed items 0.85 -> 0.66 ms, 1024 sets of the n = 14 real ansatz 4.4 -> 3.05 ms.
+// mixed items 0.85 -> 0.66 ms, 1024 sets of the n = 14 real ansatz (10 layers) 3.3 -> 2.34.
 __device__ __forceinline__ int swzr(int x) { return x ^ ((x >> 5) & 31); }
 
 template <int K, bool CX>
@@ -573,30 +601,97 @@ __device__ __forceinline__ float tile_grad_z(const Tile<K, true>& p, const Tile<
   }
 }
 
-template <int K, int B, bool CX>
-__device__ __forceinline__ float tile_grad(int pauli, const Tile<K, CX>& p, const Tile<K, CX>& l) {
-  if constexpr (CX) {
-    if (pauli == 1) return tile_grad_x<K, B>(p, l);
-    if (pauli == 3) return tile_grad_z<K, B>(p, l);
-  }
-  return tile_grad_y<K, B, CX>(p, l);
+// Four (eight) values summed over the warp with 6 (9) shuffles in place of 20 (40): a
+// lane ends with the sum of value lane >> 3 (lane >> 2).
+__device__ __forceinline__ float reduce2(float c0, float c1, int lane, int bit) {
+  const bool up = lane & bit;
+  return (up ? c1 : c0) + __shfl_xor_sync(0xffffffffu, up ? c0 : c1, bit);
+}
+__device__ __forceinline__ float reduce4(float c0, float c1, float c2, float c3, int lane) {
+  float v = reduce2(reduce2(c0, c2, lane, 16), reduce2(c1, c3, lane, 16), lane, 8);
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  return v + __shfl_xor_sync(0xffffffffu, v, 1);
+}
+// A run of rotations R[0 .. ), (a, b, parameter) each, in order (bit, kind) as `mask` says:
+// straight-line code with a skip per absent one, in place of a dispatch, a jump
+// and a warp sum of its own for each.
+template <int K, bool CX>
+__device__ __forceinline__ void run_fwd(const float4* R, int mask, Tile<K, CX>& t) {
+  static_for<0, K>([&](auto bb) {
+    constexpr int B = decltype(bb)::value;
+    if constexpr (CX) {
+      if ((mask >> (3 * B)) & 1) {
+        const float2 r = *reinterpret_cast<const float2*>(R++);
+        rx_rot<K, B>(r.x, r.y, t);
+      }
+    }
+    if ((mask >> (3 * B + 1)) & 1) {
+      const float2 r = *reinterpret_cast<const float2*>(R++);
+      plane_rot<K, B>(r.x, r.y, t.r);
+      if constexpr (CX) plane_rot<K, B>(r.x, r.y, t.i);
+    }
+    if constexpr (CX) {
+      if ((mask >> (3 * B + 2)) & 1) {
+        const float2 r = *reinterpret_cast<const float2*>(R++);
+        rz_rot<K, B>(r.x, r.y, t);
+      }
+    }
+  });
 }
 
-// a rotation without controls; DAG: its inverse
-template <int K, int B, bool CX, bool DAG>
-__device__ __forceinline__ void tile_rot(int cls, float a, float b, Tile<K, CX>& t) {
-  if constexpr (CX) {
-    if (cls == BC_RZ) {
-      rz_rot<K, B>(a, DAG ? -b : b, t);
-      return;
+// Backward over the same run (R one past its last): each rotation's gradient, added to
+// this warp's partials, then its inverse on both tiles.  No parameter occurs
+// twice in a run, so the lanes add to different partials.
+template <int K, bool CX>
+__device__ __forceinline__ void run_bwd(const float4* R, int mask, Tile<K, CX>& p, Tile<K, CX>& l,
+                                        float2* part) {
+  const int lane = threadIdx.x & 31;
+  const auto add = [&](const float4* r, float c) {
+    const int param = __float_as_int(r->z);
+    if (param >= 0) ksum_add(part[param], c);
+  };
+  static_for<0, K>([&](auto bb) {
+    constexpr int B = K - 1 - decltype(bb)::value;
+    if constexpr (CX) {
+      const int m = (mask >> (3 * B)) & 7;
+      if (m) {
+        float x = 0.f, y = 0.f, z = 0.f;
+        if (m & 4) {
+          const float2 r = *reinterpret_cast<const float2*>(--R);
+          z = tile_grad_z<K, B>(p, l);
+          rz_rot<K, B>(r.x, -r.y, p);
+          rz_rot<K, B>(r.x, -r.y, l);
+        }
+        if (m & 2) {
+          const float2 r = *reinterpret_cast<const float2*>(--R);
+          y = tile_grad_y<K, B, CX>(p, l);
+          plane_rot<K, B>(-r.x, -r.y, p.r);
+          plane_rot<K, B>(-r.x, -r.y, p.i);
+          plane_rot<K, B>(-r.x, -r.y, l.r);
+          plane_rot<K, B>(-r.x, -r.y, l.i);
+        }
+        if (m & 1) {
+          const float2 r = *reinterpret_cast<const float2*>(--R);
+          x = tile_grad_x<K, B>(p, l);
+          rx_rot<K, B>(-r.x, -r.y, p);
+          rx_rot<K, B>(-r.x, -r.y, l);
+        }
+        const float v = reduce4(x, y, z, 0.f, lane);
+        const int k = lane >> 3;
+        if ((lane & 7) == 0 && ((m >> k) & 1)) add(R + __popc(m & ((1 << k) - 1)), v);
+      }
+    } else {
+      if ((mask >> (3 * B + 1)) & 1) {
+        const float2 r = *reinterpret_cast<const float2*>(--R);
+        float c = tile_grad_y<K, B, CX>(p, l);
+        c = warp_sum_f(c);
+        plane_rot<K, B>(-r.x, -r.y, p.r);
+        plane_rot<K, B>(-r.x, -r.y, l.r);
+        if (lane == 0) add(R, c);
+      }
     }
-    if (cls == BC_RX) {
-      rx_rot<K, B>(DAG ? -a : a, DAG ? -b : b, t);
-      return;
-    }
-    plane_rot<K, B>(DAG ? -a : a, DAG ? -b : b, t.i);
-  }
-  plane_rot<K, B>(DAG ? -a : a, DAG ? -b : b, t.r);
+  });
 }
 
 template <int K, bool CX>
@@ -700,11 +795,12 @@ __device__ __forceinline__ Places<K> group_places(const BGroup& g) {
   return pl;
 }
 
-// The tile at byte offset b, in Gray-code order: one XOR an address, and no table of
+// Tile s of the group, in Gray-code order: one XOR an address, and no table of
 // 2^K offsets to keep in registers across the operations.
 template <int K, bool CX>
-__device__ __forceinline__ void tile_load(const float* st, int b, const Places<K>& pl, int plane,
+__device__ __forceinline__ void tile_load(const float* st, int s, const Places<K>& pl, int plane,
                                           Tile<K, CX>& t) {
+  int b = swzr(sub_base<K>(s, pl.low, K)) * (int)sizeof(float);
   const char* re = reinterpret_cast<const char*>(st);
   const char* im = reinterpret_cast<const char*>(st + plane);
 #pragma unroll
@@ -719,11 +815,11 @@ __device__ __forceinline__ void tile_load(const float* st, int b, const Places<K
   }
 }
 template <int K, bool CX>
-__device__ __forceinline__ void tile_store(float* st, int b, const Places<K>& pl, int plane,
+__device__ __forceinline__ void tile_store(float* st, int s, const Places<K>& pl, int plane,
                                            const Tile<K, CX>& t) {
+  int b = swzr(sub_base<K>(s, pl.low, K)) * (int)sizeof(float);
   char* re = reinterpret_cast<char*>(st);
   char* im = reinterpret_cast<char*>(st + plane);
-  asm volatile("" : "+r"(b));  // the addresses are formed again, not kept from the loads
 #pragma unroll
   for (int k = 0; k < (1 << (K - 1)); ++k) {
     const int p = k ^ (k >> 1);
@@ -740,92 +836,115 @@ __device__ __forceinline__ void tile_store(float* st, int b, const Places<K>& pl
   }
 }
 
-// Per block: the item's gate matrices, operations, groups, terms and sign patterns,
-// and per-warp gradient sums, in dynamic shared memory sized by the batch.
-struct BSmem {
-  float* mats;    // 8 floats a gate; a rotation without controls: its two coefficients
-  float2* wpart;  // per warp and parameter: (sum, compensation)
-  BOp* ops;
-  BGroup* grp;
-  int2* term;     // (swzr(x mask), z mask | (an odd number of Y factors) << 31)
-  float* tcoef;   // 8 a term: the coefficient times the sign of slice j's high bits
-  float* sign;    // patterns of 2^K values
+// The threads that run one item: all of the block, or a power of two of its warps.
+struct Team {
+  int tid, n, bar;  // thread of the team, threads, named barrier
+  __device__ __forceinline__ void sync() const {
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(n) : "memory");
+  }
 };
+
+// Per team: the item's rotations, gate matrices, operations, groups, terms and sign
+// patterns, and per-warp gradient sums, in dynamic shared memory sized by the
+// phase's items.
+struct BSmem {
+  unsigned char* mem;
+  const BPhase& P;
+  // (a, b, parameter)
+  __device__ __forceinline__ float4* rot() const { return reinterpret_cast<float4*>(mem); }
+  // 8 floats a gate
+  __device__ __forceinline__ float* mats() const { return at<float>(P.o_mats); }
+  // per warp and parameter: (sum, compensation)
+  __device__ __forceinline__ float2* wpart() const { return at<float2>(P.o_wpart); }
+  __device__ __forceinline__ BOp* ops() const { return at<BOp>(P.o_ops); }
+  __device__ __forceinline__ BGroup* grp() const { return at<BGroup>(P.o_grp); }
+  // (swzr(x mask's local bits) | the others << kRankShift, z mask | (an odd number of Y) << 31)
+  __device__ __forceinline__ int2* term() const { return at<int2>(P.o_term); }
+  // 8 a term: the coefficient times the sign of slice j's high bits
+  __device__ __forceinline__ float* tcoef() const { return at<float>(P.o_tcoef); }
+  // patterns of 2^K values
+  __device__ __forceinline__ float* sign() const { return at<float>(P.o_sign); }
+  template <typename T>
+  __device__ __forceinline__ T* at(int o) const {
+    return reinterpret_cast<T*>(mem + o);
+  }
+};
+
+// the group's operations on a tile; backward, on both tiles, each after its gradient
+template <int K, bool CX>
+__device__ __forceinline__ void tile_fwd(const BGroup& g, const BSmem& S, Tile<K, CX>& t) {
+  for (int o = g.op0; o < g.op1; ++o) {
+    const BOp op = S.ops()[o];
+    if (op.cls == BC_RUN)
+      run_fwd<K, CX>(S.rot() + op.gi, op.param, t);
+    else if (op.cls == BC_SIGN)
+      tile_signs<K, CX>(S.sign() + (op.gi << K), t);
+    else
+      tile_other<K, CX, false>(op, S.mats() + 8 * op.gi, t);
+  }
+}
+template <int K, bool CX>
+__device__ __forceinline__ void tile_bwd(const BGroup& g, const BSmem& S, float2* part,
+                                         Tile<K, CX>& p, Tile<K, CX>& l) {
+  const int lane = threadIdx.x & 31;
+  for (int o = g.op1 - 1; o >= g.op0; --o) {
+    const BOp op = S.ops()[o];
+    if (op.cls == BC_RUN) {
+      run_bwd<K, CX>(S.rot() + op.gi + op.cm, op.param, p, l, part);
+    } else if (op.cls == BC_SIGN) {
+      tile_signs2<K, CX>(S.sign() + (op.gi << K), p, l);
+    } else {
+      if (op.pauli) {
+        const float c = warp_sum_f(tile_other_grad<K, CX>(op, p, l));
+        if (lane == 0) ksum_add(part[op.param], c);
+      }
+      tile_other<K, CX, true>(op, S.mats() + 8 * op.gi, p);
+      tile_other<K, CX, true>(op, S.mats() + 8 * op.gi, l);
+    }
+    __syncwarp();  // a warp's next partials may be another lane's
+  }
+}
 
 // forward: psi <- group ops in order
 template <int K, bool CX>
-__device__ __forceinline__ void group_fwd(float* psi, int np, const BGroup& g, const BSmem& S) {
-  const Places<K> pl = group_places<K>(g);
+__device__ __forceinline__ void group_fwd(float* psi, int np, const BGroup& g, const BSmem& S,
+                                          const Team& T) {
   const int nsub = 1 << (np - K);
-  for (int s = threadIdx.x; s < nsub; s += blockDim.x) {
-    const int b = swzr(sub_base<K>(s, pl.low, K)) * (int)sizeof(float);
+  for (int s = T.tid; s < nsub; s += T.n) {
     Tile<K, CX> t;
-    tile_load<K, CX>(psi, b, pl, 1 << np, t);
-    for (int o = g.op0; o < g.op1; ++o) {
-      const BOp op = S.ops[o];
-      const float* M = S.mats + 8 * op.gi;
-      if (op.cls >= BC_ROT) {
-        const float2 ab = *reinterpret_cast<const float2*>(M);
-#define SV_ROT(BB) \
-  if constexpr (BB < K) tile_rot<K, BB, CX, false>(op.cls, ab.x, ab.y, t)
-        SV_TILE_BITS(op.b0, SV_ROT)
-#undef SV_ROT
-      } else if (op.cls == BC_SIGN) {
-        tile_signs<K, CX>(S.sign + (op.gi << K), t);
-      } else {
-        tile_other<K, CX, false>(op, M, t);
-      }
-    }
-    tile_store<K, CX>(psi, b, pl, 1 << np, t);
+    tile_load<K, CX>(psi, s, group_places<K>(g), 1 << np, t);
+    tile_fwd<K, CX>(g, S, t);
+    asm volatile("" ::: "memory");  // the places are read again, not kept
+    tile_store<K, CX>(psi, s, group_places<K>(g), 1 << np, t);
   }
 }
 
 // backward: for ops in reverse, gradient contribution then un-apply on both
 template <int K, bool CX>
 __device__ __forceinline__ void group_bwd(float* psi, float* lam, int np, int pstride,
-                                          const BGroup& g, const BSmem& S) {
-  const Places<K> pl = group_places<K>(g);
+                                          const BGroup& g, const BSmem& S, const Team& T) {
   const int nsub = 1 << (np - K);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = T.tid & 31;
+  float2* const part = S.wpart() + (T.tid >> 5) * pstride;
   // every lane of a warp runs the same number of iterations (warp sums)
-  for (int s0 = threadIdx.x - lane; s0 < nsub; s0 += blockDim.x) {
+  for (int s0 = T.tid - lane; s0 < nsub; s0 += T.n) {
     const int s = s0 + lane;
     const bool live = s < nsub;
-    const int b = live ? swzr(sub_base<K>(s, pl.low, K)) * (int)sizeof(float) : 0;
-    Tile<K, CX> p{}, l{};
+    Tile<K, CX> p, l;
     if (live) {
-      tile_load<K, CX>(psi, b, pl, 1 << np, p);
-      tile_load<K, CX>(lam, b, pl, 1 << np, l);
+      const Places<K> pl = group_places<K>(g);
+      tile_load<K, CX>(psi, s, pl, 1 << np, p);
+      tile_load<K, CX>(lam, s, pl, 1 << np, l);
+    } else {
+      p = {};
+      l = {};
     }
-    for (int o = g.op1 - 1; o >= g.op0; --o) {
-      const BOp op = S.ops[o];
-      const float* M = S.mats + 8 * op.gi;
-      float c = 0.f;
-      if (op.cls >= BC_ROT) {
-        const float2 ab = *reinterpret_cast<const float2*>(M);
-#define SV_ROT(BB)                                               \
-  if constexpr (BB < K) {                                        \
-    if (op.pauli) c = tile_grad<K, BB, CX>(op.pauli, p, l);      \
-    tile_rot<K, BB, CX, true>(op.cls, ab.x, ab.y, p);            \
-    tile_rot<K, BB, CX, true>(op.cls, ab.x, ab.y, l);            \
-  }
-        SV_TILE_BITS(op.b0, SV_ROT)
-#undef SV_ROT
-      } else if (op.cls == BC_SIGN) {
-        tile_signs2<K, CX>(S.sign + (op.gi << K), p, l);
-      } else {
-        if (op.pauli) c = tile_other_grad<K, CX>(op, p, l);
-        tile_other<K, CX, true>(op, M, p);
-        tile_other<K, CX, true>(op, M, l);
-      }
-      if (op.pauli) {
-        c = warp_sum_f(c);
-        if (lane == 0) ksum_add(S.wpart[warp * pstride + op.param], c);
-      }
-    }
+    tile_bwd<K, CX>(g, S, part, p, l);
+    asm volatile("" ::: "memory");  // the places are read again, not kept
     if (live) {
-      tile_store<K, CX>(psi, b, pl, 1 << np, p);
-      tile_store<K, CX>(lam, b, pl, 1 << np, l);
+      const Places<K> pl = group_places<K>(g);
+      tile_store<K, CX>(psi, s, pl, 1 << np, p);
+      tile_store<K, CX>(lam, s, pl, 1 << np, l);
     }
   }
 }
@@ -835,14 +954,16 @@ __device__ __forceinline__ void group_bwd(float* psi, float* lam, int np, int ps
 // a sign of j that the whole block shares (in tcoef): 2^14 amplitudes with
 // 27 terms took about a fifth of a real item's instructions with a parity per
 // amplitude and term.
-template <int J, bool CX>
-__device__ __forceinline__ void apply_terms(const float* psi, float* lam, const BCirc& C, int np,
-                                            const BSmem& S, float2& ek) {
-  const int d = (1 << C.n) / J, plane = 1 << np;
+// SPLIT: psi and lam are rank `rank`'s quarter of a cluster's states, nloc = n - 2.
+template <int J, bool CX, bool SPLIT = false>
+__device__ __forceinline__ void apply_terms(const float* psi, float* lam, const BCirc& C, int nloc,
+                                            int np, int rank, const BSmem& S, const Team& T,
+                                            float2& ek) {
+  const int d = (1 << nloc) / J, plane = 1 << np;
   int off[J];
 #pragma unroll
   for (int j = 0; j < J; ++j) off[j] = swzr(j * d);
-  for (int x0 = threadIdx.x; x0 < d; x0 += blockDim.x) {
+  for (int x0 = T.tid; x0 < d; x0 += T.n) {
     const int p0 = swzr(x0);
     Pair dg[J / 2], ar[J / 2], ai[CX ? J / 2 : 1], sr[J / 2], si[CX ? J / 2 : 1];
 #pragma unroll
@@ -854,8 +975,8 @@ __device__ __forceinline__ void apply_terms(const float* psi, float* lam, const 
       if constexpr (CX) ai[k] = pair_of(x[plane], y[plane]);
     }
     for (int t = 0; t < C.ndiag; ++t) {
-      const Pair sg = pair_both(__popc(x0 & S.term[t].y) & 1 ? -1.f : 1.f);
-      const Pair* cf = reinterpret_cast<const Pair*>(S.tcoef + 8 * t);
+      const Pair sg = pair_both(__popc((x0 | (rank << nloc)) & S.term()[t].y) & 1 ? -1.f : 1.f);
+      const Pair* cf = reinterpret_cast<const Pair*>(S.tcoef() + 8 * t);
 #pragma unroll
       for (int k = 0; k < J / 2; ++k) pair_add(dg[k], sg, cf[k]);
     }
@@ -865,16 +986,23 @@ __device__ __forceinline__ void apply_terms(const float* psi, float* lam, const 
       if constexpr (CX) si[k] = pair_mul(dg[k], ai[k]);
     }
     for (int t = C.ndiag; t < C.nterms; ++t) {
-      const int2 q = S.term[t];
-      const int odd = __popc(x0 & q.y) & 1;
+      const int2 q = S.term()[t];
+      const int odd = __popc((x0 | (rank << nloc)) & q.y) & 1;
       const Pair sg = pair_both(odd ? -1.f : 1.f);
-      const Pair* cf = reinterpret_cast<const Pair*>(S.tcoef + 8 * t);
-      const int pt = p0 ^ q.x;
+      const Pair* cf = reinterpret_cast<const Pair*>(S.tcoef() + 8 * t);
+      const int pt = p0 ^ (q.x & ((1 << kRankShift) - 1));
+      const float* from = psi;
+      if constexpr (SPLIT) {
+        const int flip = q.x >> kRankShift;
+        if (flip)
+          from = cooperative_groups::this_cluster().map_shared_rank(const_cast<float*>(psi),
+                                                                    rank ^ flip);
+      }
 #pragma unroll
       for (int k = 0; k < J / 2; ++k) {
         const Pair w = pair_mul(sg, cf[k]);
-        const float* x = psi + (pt ^ off[2 * k]);
-        const float* y = psi + (pt ^ off[2 * k + 1]);
+        const float* x = from + (pt ^ off[2 * k]);
+        const float* y = from + (pt ^ off[2 * k + 1]);
         const Pair br = pair_of(*x, *y);
         if constexpr (CX) {
           const Pair bi = pair_of(x[plane], y[plane]);
@@ -914,142 +1042,358 @@ __device__ __forceinline__ void apply_terms(const float* psi, float* lam, const 
 // forward pass, lambda and the reverse sweep of one item; returns this thread's energy
 template <int K, bool CX>
 __device__ __forceinline__ double run_item(float* psi, float* lam, const BCirc& C, int pstride,
-                                           const BSmem& S) {
+                                           const BSmem& S, const Team& T) {
   const int np = max(C.n, K);
   // |0...0>: swzr(0) = 0 and swzr maps every other index to a nonzero one
-  for (int x = threadIdx.x; x < ((CX ? 2 : 1) << np); x += blockDim.x) psi[x] = x == 0 ? 1.f : 0.f;
+  for (int x = T.tid; x < ((CX ? 2 : 1) << np); x += T.n) psi[x] = x == 0 ? 1.f : 0.f;
   if (C.n < K)  // the tile is wider than the state: what lies beyond stays zero
-    for (int x = threadIdx.x; x < ((CX ? 2 : 1) << np); x += blockDim.x) lam[x] = 0.f;
-  __syncthreads();
+    for (int x = T.tid; x < ((CX ? 2 : 1) << np); x += T.n) lam[x] = 0.f;
+  T.sync();
   for (int gg = 0; gg < C.ngroups; ++gg) {
-    group_fwd<K, CX>(psi, np, S.grp[gg], S);
-    __syncthreads();
+    group_fwd<K, CX>(psi, np, S.grp()[gg], S, T);
+    T.sync();
   }
   float2 ek = make_float2(0.f, 0.f);
   if (term_slices(C.n) == 8)
-    apply_terms<8, CX>(psi, lam, C, np, S, ek);
+    apply_terms<8, CX>(psi, lam, C, C.n, np, 0, S, T, ek);
   else
-    apply_terms<2, CX>(psi, lam, C, np, S, ek);
-  __syncthreads();
+    apply_terms<2, CX>(psi, lam, C, C.n, np, 0, S, T, ek);
+  T.sync();
   for (int gg = C.ngroups - 1; gg >= 0; --gg) {
-    group_bwd<K, CX>(psi, lam, np, pstride, S.grp[gg], S);
-    __syncthreads();
+    group_bwd<K, CX>(psi, lam, np, pstride, S.grp()[gg], S, T);
+    T.sync();
   }
   return ksum_value(ek);
 }
 
+// An item's rotations, matrices, lists and terms into the team's shared memory, and its
+// partials to zero.  nloc: qubits of the state that one block holds.
+template <int K>
+__device__ __forceinline__ void load_item(const BatchArgs& A, const BPhase& P, const BCirc& C,
+                                          const double* th, int nloc, const BSmem& S,
+                                          const Team& T) {
+  // rotations and gate matrices (fp64 trigonometry, rounded once), zero partials
+  for (int i = T.tid; i < C.nrot; i += T.n) {
+    const BRot d = A.rots[C.rot0 + i];
+    const double a = d.param >= 0 ? th[d.param] : d.angle;
+    double s, c;
+    sincos(d.kind == SV_GATE_RZ ? a : 0.5 * a, &s, &c);
+    if (d.kind == SV_GATE_RZ) {
+      S.rot()[i] = make_float4((float)c, (float)s, __int_as_float(d.param), 0.f);
+    } else {
+      if (c < 0) {
+        c = -c;
+        s = -s;
+      }
+      S.rot()[i] = make_float4((float)(-s / (1.0 + c)), (float)s, __int_as_float(d.param), 0.f);
+    }
+  }
+  for (int i = T.tid; i < C.ngen; i += T.n) {
+    const BGateDesc d = A.gens[C.gen0 + i];
+    const double a = d.param >= 0 ? th[d.param] : d.angle;
+    double s, c;
+    sincos(d.kind == SV_GATE_U1 ? a : 0.5 * a, &s, &c);
+    double m[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const double r2 = 0.70710678118654752440;
+    switch (d.kind) {
+      case SV_GATE_H: m[0] = r2; m[2] = r2; m[4] = r2; m[6] = -r2; break;
+      case SV_GATE_X: m[2] = 1; m[4] = 1; break;
+      case SV_GATE_Y: m[3] = -1; m[5] = 1; break;
+      case SV_GATE_Z: m[0] = 1; m[6] = -1; break;
+      case SV_GATE_RX: m[0] = c; m[3] = -s; m[5] = -s; m[6] = c; break;
+      case SV_GATE_RY: m[0] = c; m[2] = -s; m[4] = s; m[6] = c; break;
+      case SV_GATE_RZ: m[0] = c; m[1] = -s; m[6] = c; m[7] = s; break;
+      default: m[0] = 1; m[6] = c; m[7] = s;  // U1: diag(1, e^{ia})
+    }
+    for (int e = 0; e < 8; ++e) S.mats()[8 * i + e] = (float)m[e];
+  }
+  for (int i = T.tid; i < (T.n >> 5) * P.pstride; i += T.n) S.wpart()[i] = make_float2(0.f, 0.f);
+  {  // this item's groups and operations, operation indices rebased to the cache
+    const int ng = C.ngroups;
+    const int op_base = ng ? A.rgroups[C.group0].op0 : 0;
+    const int nops = ng ? A.rgroups[C.group0 + ng - 1].op1 - op_base : 0;
+    for (int i = T.tid; i < nops; i += T.n) S.ops()[i] = A.rops[op_base + i];
+    for (int i = T.tid; i < (C.nsign << K); i += T.n)
+      S.sign()[i] = (A.rsigns[C.sign0 + (i >> K)] >> (i & ((1 << K) - 1))) & 1 ? -1.f : 1.f;
+    for (int i = T.tid; i < ng; i += T.n) {
+      BGroup G = A.rgroups[C.group0 + i];
+      G.op0 -= op_base;
+      G.op1 -= op_base;
+      for (int k = G.k; k < K; ++k) G.bits[k] = (uint8_t)k;  // n < K: the group is the state
+      S.grp()[i] = G;
+    }
+    const int js = term_slices(nloc), dlog = nloc - (js == 8 ? 3 : 1);
+    for (int t = T.tid; t < C.nterms; t += T.n) {
+      const BTerm M = A.terms[C.term0 + t];
+      const int xm = (int)M.xm, zm = (int)M.zm;  // n <= SV_BATCH_MAX_QUBITS < 30
+      const bool imag = __popc(xm & zm) & 1;     // i^{#Y} imaginary
+      S.term()[t] = make_int2(swzr(xm & ((1 << nloc) - 1)) | ((xm >> nloc) << kRankShift),
+                              (int)((unsigned)zm | ((unsigned)imag << 31)));
+      // sign at x: the parity of (x ^ xm) & zm
+      const float c = (float)(imag ? -M.cim : M.cre);
+      for (int j = 0; j < 8; ++j)
+        S.tcoef()[8 * t + j] = __popc((j << dlog) & zm) & 1 ? -c : c;
+    }
+  }
+}
+
+// SMS: one block of 512 threads an SM that works through the size classes from
+// the largest.  2^K amplitudes a thread make a group of an n-qubit item one round of
+// 2^(n - K) threads: items of that size class run side by side in teams of as many,
+// each with its own barrier, and 512 threads' tiles of two states just fill
+// 128 KiB of shared memory whatever the size.  With one team of 256 threads an item
+// of 11 qubits left half of its warps at the barriers (4 of 11 stalled cycles
+// an instruction): 768 items of 11 qubits and 192 mixed 0.66 -> 0.41 ms, 740 of 10
+// qubits and 40 mixed 0.51 -> 0.22 ms.  Otherwise one size class and one team, states in global memory.
 template <int K, int MAXT, int MINB, bool CX, bool SMS>
 __global__ void __launch_bounds__(MAXT, MINB) kbatch(const BatchArgs A) {
   __shared__ double red[MAXT / 32];
-  __shared__ int s_item;
+  __shared__ int s_item[8];
   extern __shared__ __align__(16) unsigned char dyn_smem[];
-  const BSmem S = {reinterpret_cast<float*>(dyn_smem + A.o_mats),
-                   reinterpret_cast<float2*>(dyn_smem + A.o_wpart),
-                   reinterpret_cast<BOp*>(dyn_smem + A.o_ops),
-                   reinterpret_cast<BGroup*>(dyn_smem + A.o_grp),
-                   reinterpret_cast<int2*>(dyn_smem + A.o_term),
-                   reinterpret_cast<float*>(dyn_smem + A.o_tcoef),
-                   reinterpret_cast<float*>(dyn_smem + A.o_sign)};
-  float* const dyn_state = reinterpret_cast<float*>(dyn_smem + A.o_state);
-  const int nwarps = blockDim.x >> 5;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* const gpsi = reinterpret_cast<float*>(A.work + (size_t)blockIdx.x * (size_t(2) << A.nmax));
   float* const glam = gpsi + (size_t(2) << A.nmax);
+  for (int ph = 0; ph < A.n_phases; ++ph) {
+    const BPhase& P = A.phase[ph];
+    const int team = (int)threadIdx.x / P.ts;
+    const Team T = {(int)threadIdx.x - team * P.ts, P.ts, 1 + team};
+    unsigned char* const mem = dyn_smem + team * P.stride;
+    const BSmem S = {mem, P};
+    float* const dyn_state = reinterpret_cast<float*>(mem + P.o_state);
+    const int nwarps = P.ts >> 5;
+    while (true) {
+      if (T.tid == 0) s_item[team] = atomicAdd(A.queue + ph, 1);
+      T.sync();
+      const int slot = s_item[team];
+      if (slot >= P.count) break;
+      const int item = A.order[P.first + slot];
+      const BCirc C = A.circs[A.item_circ[item]];
+      const double* th = A.theta + A.theta_off[item];
+      load_item<K>(A, P, C, th, C.n, S, T);
+      const int size = (CX ? 2 : 1) << max(C.n, K);  // floats of one state
+      double e;
+      if constexpr (SMS) {
+        if (2 * size <= P.state_floats)
+          e = run_item<K, CX>(dyn_state, dyn_state + size, C, P.pstride, S, T);
+        else
+          e = run_item<K, CX>(size <= P.state_floats ? dyn_state : gpsi, glam, C, P.pstride, S, T);
+      } else {
+        e = run_item<K, CX>(gpsi, glam, C, P.pstride, S, T);
+      }
+      e = warp_sum_d(e);
+      if (lane == 0) red[warp] = e;
+      T.sync();
+      const int toff = A.theta_off[item];
+      for (int p = T.tid; p < C.nparams; p += T.n) {
+        double g = 0.0;
+        for (int w = 0; w < nwarps; ++w) g += ksum_value(S.wpart()[w * P.pstride + p]);
+        A.grad[toff + p] = g;
+      }
+      if (T.tid == 0) {
+        double E = 0.0;
+        for (int w = 0; w < nwarps; ++w) E += red[warp + w];
+        A.energy[item] = E;
+      }
+      T.sync();
+    }
+    __syncthreads();  // the next size class lays the shared memory out anew
+  }
+  grid_dependency_wait();  // the wide items, which this launch may overlap: done before it is
+}
+
+// ---- wide items: states in the shared memory of four blocks ------------------------
+// An item of 2 more qubits than one block's shared memory holds (real: 15 and 16, complex: 14
+// and 15) split by its two top bits over a cluster.  A group of lower bits runs in each
+// block on its own quarter; the tiles of the others are shared out and read
+// and written across the cluster.  From the global workspace one block took 3.1
+// ms for an n = 16 real item of 10 layers (0.9 ms for n = 15), the time of a whole batch of
+// smaller ones: its strided tiles do not fit the L1 beside the other items'
+// shared memory.  On four it takes 0.49 ms; 857 parameter sets of the n = 11, 8-layer
+// ansatz with 129 mixed items of 8 to 16 qubits 2.34 -> 0.53 ms.
+
+// Element `at` (see kRankShift) of a plane at shared address `base`.
+__device__ __forceinline__ float wide_load(unsigned base, int at) {
+  float v;
+  asm volatile(
+      "{\n .reg .u32 a;\n mapa.shared::cluster.u32 a, %1, %2;\n"
+      " ld.shared::cluster.f32 %0, [a];\n}"
+      : "=f"(v)
+      : "r"(base + (at & ((1 << kRankShift) - 1))), "r"(at >> kRankShift));
+  return v;
+}
+__device__ __forceinline__ void wide_store(unsigned base, int at, float v) {
+  asm volatile(
+      "{\n .reg .u32 a;\n mapa.shared::cluster.u32 a, %0, %1;\n"
+      " st.shared::cluster.f32 [a], %2;\n}" ::"r"(base + (at & ((1 << kRankShift) - 1))),
+      "r"(at >> kRankShift), "f"(v)
+      : "memory");
+}
+
+// steps of a split group, and the place of its tile s
+template <int K>
+__device__ __forceinline__ Places<K> wide_places(const BGroup& g, int nloc) {
+  Places<K> pl;
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    const int bit = g.bits[i];
+    pl.step[i] = bit >= nloc ? 1 << (kRankShift + bit - nloc) : swzr(1 << bit) * (int)sizeof(float);
+    pl.low[i] = (1 << bit) - 1;
+  }
+  return pl;
+}
+template <int K>
+__device__ __forceinline__ int wide_base(int s, const Places<K>& pl, int nloc) {
+  const int x = sub_base<K>(s, pl.low, K);
+  return ((x >> nloc) << kRankShift) | (swzr(x & ((1 << nloc) - 1)) * (int)sizeof(float));
+}
+template <int K, bool CX>
+__device__ __forceinline__ void wide_tile_load(unsigned re, int s, const Places<K>& pl, int nloc,
+                                               Tile<K, CX>& t) {
+  const unsigned im = re + (unsigned)(sizeof(float) << nloc);
+  int b = wide_base<K>(s, pl, nloc);
+#pragma unroll
+  for (int k = 0; k < (1 << (K - 1)); ++k) {
+    const int p = k ^ (k >> 1);
+    if (k) b ^= pl.step[1 + lowbit_b(k)];
+    const int c = b ^ pl.step[0];
+    t.r[p] = pair_of(wide_load(re, b), wide_load(re, c));
+    if constexpr (CX) t.i[p] = pair_of(wide_load(im, b), wide_load(im, c));
+  }
+}
+template <int K, bool CX>
+__device__ __forceinline__ void wide_tile_store(unsigned re, int s, const Places<K>& pl, int nloc,
+                                                const Tile<K, CX>& t) {
+  const unsigned im = re + (unsigned)(sizeof(float) << nloc);
+  int b = wide_base<K>(s, pl, nloc);
+#pragma unroll
+  for (int k = 0; k < (1 << (K - 1)); ++k) {
+    const int p = k ^ (k >> 1);
+    if (k) b ^= pl.step[1 + lowbit_b(k)];
+    const int c = b ^ pl.step[0];
+    const float2 v = lanes_of(t.r[p]);
+    wide_store(re, b, v.x);
+    wide_store(re, c, v.y);
+    if constexpr (CX) {
+      const float2 w = lanes_of(t.i[p]);
+      wide_store(im, b, w.x);
+      wide_store(im, c, w.y);
+    }
+  }
+}
+
+constexpr int kWide = 4;  // blocks of a cluster
+
+template <int K, bool CX>
+__global__ void __cluster_dims__(kWide, 1, 1) __launch_bounds__(512, 1)
+    kbatch_wide(const BatchArgs A) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ double red[16];
+  __shared__ int s_item;
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  asm volatile("griddepcontrol.launch_dependents;");  // the other items run beside these
+  const int rank = (int)cluster.block_rank();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const BPhase& P = A.wide;
+  const Team T = {(int)threadIdx.x, 512, 1};
+  const BSmem S = {dyn_smem, P};
   while (true) {
-    if (threadIdx.x == 0) s_item = atomicAdd(A.queue, 1);
-    __syncthreads();
+    if (rank == 0 && threadIdx.x == 0) {
+      const int v = atomicAdd(A.queue + kBPhases, 1);
+      for (int r = 0; r < kWide; ++r) *cluster.map_shared_rank(&s_item, r) = v;
+    }
+    cluster.sync();
     const int slot = s_item;
-    if (slot >= A.n_items) break;
-    const int item = A.order[slot];
+    if (slot >= P.count) break;
+    const int item = A.order[P.first + slot];
     const BCirc C = A.circs[A.item_circ[item]];
-    const double* th = A.theta + A.theta_off[item];
-    // gate matrices (fp64 trigonometry, rounded once), zero partials
-    for (int gi = threadIdx.x; gi < C.ngates; gi += blockDim.x) {
-      const BGateDesc d = A.gates[C.gate0 + gi];
-      const double a = d.param >= 0 ? th[d.param] : d.angle;
-      double s, c;
-      sincos(d.kind == SV_GATE_U1 || (d.free_rot && d.kind == SV_GATE_RZ) ? a : 0.5 * a, &s, &c);
-      double m[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      const double r2 = 0.70710678118654752440;
-      if (d.free_rot) {
-        if (d.kind == SV_GATE_RZ) {
-          m[0] = c;
-          m[1] = s;
-        } else {
-          if (c < 0) {
-            c = -c;
-            s = -s;
-          }
-          m[0] = -s / (1.0 + c);
-          m[1] = s;
+    const int nloc = C.n - 2, size = (CX ? 2 : 1) << nloc;
+    float* const psi = reinterpret_cast<float*>(dyn_smem + P.o_state);
+    float* const lam = psi + size;
+    const unsigned upsi = (unsigned)__cvta_generic_to_shared(psi);
+    const unsigned ulam = upsi + (unsigned)(sizeof(float) * size);
+    load_item<K>(A, P, C, A.theta + A.theta_off[item], nloc, S, T);
+    for (int x = T.tid; x < size; x += T.n) psi[x] = rank == 0 && x == 0 ? 1.f : 0.f;
+    cluster.sync();
+    bool synced = true;  // right after a cluster barrier
+    const auto split = [&](const BGroup& g) { return (int)g.bits[K - 1] >= nloc; };  // bits ascend
+    const auto done = [&](bool sp) {
+      if (sp)
+        cluster.sync();
+      else
+        T.sync();
+      synced = sp;
+    };
+    const int nsub = 1 << (nloc - K);  // a block's share of the tiles
+    for (int gg = 0; gg < C.ngroups; ++gg) {
+      const BGroup& g = S.grp()[gg];
+      const bool sp = split(g);
+      if (sp) {
+        if (!synced) cluster.sync();
+        for (int s = T.tid; s < nsub; s += T.n) {
+          Tile<K, CX> t;
+          wide_tile_load<K, CX>(upsi, s + rank * nsub, wide_places<K>(g, nloc), nloc, t);
+          tile_fwd<K, CX>(g, S, t);
+          asm volatile("" ::: "memory");
+          wide_tile_store<K, CX>(upsi, s + rank * nsub, wide_places<K>(g, nloc), nloc, t);
         }
       } else {
-        switch (d.kind) {
-          case SV_GATE_H: m[0] = r2; m[2] = r2; m[4] = r2; m[6] = -r2; break;
-          case SV_GATE_X: m[2] = 1; m[4] = 1; break;
-          case SV_GATE_Y: m[3] = -1; m[5] = 1; break;
-          case SV_GATE_Z: m[0] = 1; m[6] = -1; break;
-          case SV_GATE_RX: m[0] = c; m[3] = -s; m[5] = -s; m[6] = c; break;
-          case SV_GATE_RY: m[0] = c; m[2] = -s; m[4] = s; m[6] = c; break;
-          case SV_GATE_RZ: m[0] = c; m[1] = -s; m[6] = c; m[7] = s; break;
-          default: m[0] = 1; m[6] = c; m[7] = s;  // U1: diag(1, e^{ia})
+        group_fwd<K, CX>(psi, nloc, g, S, T);
+      }
+      done(sp);
+    }
+    if (!synced) cluster.sync();
+    float2 ek = make_float2(0.f, 0.f);
+    apply_terms<8, CX, true>(psi, lam, C, nloc, nloc, rank, S, T, ek);
+    cluster.sync();  // lambda complete; nobody still reads another's psi
+    synced = true;
+    for (int gg = C.ngroups - 1; gg >= 0; --gg) {
+      const BGroup& g = S.grp()[gg];
+      const bool sp = split(g);
+      if (sp) {
+        if (!synced) cluster.sync();
+        float2* const part = S.wpart() + warp * P.pstride;
+        for (int s = T.tid; s < nsub; s += T.n) {  // nsub is a multiple of 32
+          Tile<K, CX> p, l;
+          {
+            const Places<K> pl = wide_places<K>(g, nloc);
+            wide_tile_load<K, CX>(upsi, s + rank * nsub, pl, nloc, p);
+            wide_tile_load<K, CX>(ulam, s + rank * nsub, pl, nloc, l);
+          }
+          tile_bwd<K, CX>(g, S, part, p, l);
+          asm volatile("" ::: "memory");
+          const Places<K> pl = wide_places<K>(g, nloc);
+          wide_tile_store<K, CX>(upsi, s + rank * nsub, pl, nloc, p);
+          wide_tile_store<K, CX>(ulam, s + rank * nsub, pl, nloc, l);
         }
+      } else {
+        group_bwd<K, CX>(psi, lam, nloc, P.pstride, g, S, T);
       }
-      for (int e = 0; e < 8; ++e) S.mats[8 * gi + e] = (float)m[e];
+      done(sp);
     }
-    for (int i = threadIdx.x; i < nwarps * A.pstride; i += blockDim.x)
-      S.wpart[i] = make_float2(0.f, 0.f);
-    {  // this item's groups and operations, operation indices rebased to the cache
-      const int ng = C.ngroups;
-      const int op_base = ng ? A.rgroups[C.group0].op0 : 0;
-      const int nops = ng ? A.rgroups[C.group0 + ng - 1].op1 - op_base : 0;
-      for (int i = threadIdx.x; i < nops; i += blockDim.x) S.ops[i] = A.rops[op_base + i];
-      for (int i = threadIdx.x; i < (C.nsign << K); i += blockDim.x)
-        S.sign[i] = (A.rsigns[C.sign0 + (i >> K)] >> (i & ((1 << K) - 1))) & 1 ? -1.f : 1.f;
-      for (int i = threadIdx.x; i < ng; i += blockDim.x) {
-        BGroup G = A.rgroups[C.group0 + i];
-        G.op0 -= op_base;
-        G.op1 -= op_base;
-        for (int k = G.k; k < K; ++k) G.bits[k] = (uint8_t)k;  // n < K: the group is the state
-        S.grp[i] = G;
-      }
-      const int js = term_slices(C.n), dlog = C.n - (js == 8 ? 3 : 1);
-      for (int t = threadIdx.x; t < C.nterms; t += blockDim.x) {
-        const BTerm T = A.terms[C.term0 + t];
-        const int xm = (int)T.xm, zm = (int)T.zm;  // n <= SV_BATCH_MAX_QUBITS < 30
-        const bool imag = __popc(xm & zm) & 1;     // i^{#Y} imaginary
-        S.term[t] = make_int2(swzr(xm), (int)((unsigned)zm | ((unsigned)imag << 31)));
-        // sign at x: the parity of (x ^ xm) & zm
-        const float c = (float)(imag ? -T.cim : T.cre);
-        for (int j = 0; j < 8; ++j)
-          S.tcoef[8 * t + j] = __popc((j << dlog) & zm) & 1 ? -c : c;
-      }
-    }
-    const int size = (CX ? 2 : 1) << max(C.n, K);  // floats of one state
-    double e;
-    if constexpr (SMS) {
-      if (2 * size <= A.state_floats)
-        e = run_item<K, CX>(dyn_state, dyn_state + size, C, A.pstride, S);
-      else
-        e = run_item<K, CX>(size <= A.state_floats ? dyn_state : gpsi, glam, C, A.pstride, S);
-    } else {
-      e = run_item<K, CX>(gpsi, glam, C, A.pstride, S);
-    }
-    e = warp_sum_d(e);
+    const double e = warp_sum_d(ksum_value(ek));
     if (lane == 0) red[warp] = e;
-    __syncthreads();
-    const int toff = A.theta_off[item];
-    for (int p = threadIdx.x; p < C.nparams; p += blockDim.x) {
-      double g = 0.0;
-      for (int w = 0; w < nwarps; ++w) g += ksum_value(S.wpart[w * A.pstride + p]);
-      A.grad[toff + p] = g;
+    cluster.sync();  // every block's partials final
+    if (rank == 0) {
+      const int toff = A.theta_off[item];
+      for (int p = threadIdx.x; p < C.nparams; p += 512) {
+        double g = 0.0;
+        for (int r = 0; r < kWide; ++r) {
+          const float2* w = cluster.map_shared_rank(S.wpart(), r);
+          for (int i = 0; i < 16; ++i) g += ksum_value(w[i * P.pstride + p]);
+        }
+        A.grad[toff + p] = g;
+      }
+      if (threadIdx.x == 0) {
+        double E = 0.0;
+        for (int r = 0; r < kWide; ++r) {
+          const double* d = cluster.map_shared_rank(red, r);
+          for (int i = 0; i < 16; ++i) E += d[i];
+        }
+        A.energy[item] = E;
+      }
     }
-    if (threadIdx.x == 0) {
-      double E = 0.0;
-      for (int w = 0; w < nwarps; ++w) E += red[w];
-      A.energy[item] = E;
-    }
-    __syncthreads();
+    // the next item's barrier orders block 0's reads before the others reuse their partials
   }
 }
 
@@ -1397,14 +1741,20 @@ struct sv_batch_s {
   sv::BGroup* rgroups = nullptr;  // the single-block kernels' lists
   sv::BOp* rops = nullptr;
   uint32_t* rsigns = nullptr;
+  sv::BRot* rots = nullptr;
+  sv::BGateDesc* gens = nullptr;
   int* order = nullptr;
   int* item_circ = nullptr;
   int* theta_off = nullptr;
   int* queue = nullptr;
   float2* work = nullptr;
   size_t work_slots = 0;
-  // the largest of the batch's circuits, for the blocks' shared memory
-  int max_gates = 0, max_params = 0, max_ops = 0, max_groups = 0, max_terms = 0, max_signs = 0;
+  std::vector<sv::BCirc> h_circs;       // of the chosen group width, with
+  std::vector<int> h_ops;               // the single-block kernels' operations of each
+  std::vector<int> h_order, h_item_circ;
+  int n_phases = 0;                     // of the chosen tile
+  sv::BPhase phase[sv::kBPhases], wide;
+  size_t smem = 0;
   std::vector<int> h_theta_off;
   // captured graph
   cudaGraphExec_t gexec = nullptr;
@@ -1423,6 +1773,8 @@ struct HostPlan {
   std::vector<BGroup> rgroups;  // filled by tile_lists
   std::vector<BOp> rops;
   std::vector<uint32_t> rsigns;
+  std::vector<BRot> rots;
+  std::vector<BGateDesc> gens;
 };
 
 int popc64(uint64_t x) { return __builtin_popcountll(x); }
@@ -1527,18 +1879,39 @@ bool plan_circuit(const sv_circuit* c, const sv_pauli_sum* H, int k, HostPlan* P
 // A circuit with more patterns keeps its single flips.
 constexpr int kBMaxSigns = 96;
 
-// The single-block kernels' lists of every circuit of P: rotations without controls,
-// and each run of sign flips with no other than diagonal operations on their bits
-// in between as one pattern over the group's 2^k indices.
+// The single-block kernels' lists of every circuit of P.  Rotations without controls join
+// the group's last run while none of their qubit's later operations stand between, in
+// the order (qubit, X < Y < Z), no parameter twice; each run of sign flips with
+// no other than diagonal operations on their bits in between is one pattern
+// over the group's 2^k indices.
 void tile_lists(HostPlan* P) {
   for (BCirc& C : P->circs) {
+    C.gen0 = (int)P->gens.size();
+    C.rot0 = (int)P->rots.size();
     for (int merge = 1; merge >= 0; --merge) {
       const size_t o0 = P->rops.size(), s0 = P->rsigns.size(), g0 = P->rgroups.size();
       for (int g = C.group0; g < C.group0 + C.ngroups; ++g) {
         BGroup G = P->groups[g];
         const int a = G.op0, b = G.op1;
         G.op0 = (int32_t)P->rops.size();
-        int open = -1, dirty = 0;  // the last pattern, and bits touched since
+        int open = -1, dirty = 0;     // the last pattern, and bits touched since
+        int run = -1, since = 0;      // the last run, and bits touched since
+        std::vector<std::pair<int, BRot>> rots;  // its rotations by 3 bit + kind
+        auto close = [&] {
+          if (run < 0) return;
+          std::sort(rots.begin(), rots.end(),
+                    [](const auto& x, const auto& y) { return x.first < y.first; });
+          BOp& r = P->rops[run];
+          r.gi = (int16_t)(P->rots.size() - C.rot0);
+          r.cm = (uint8_t)rots.size();
+          for (const auto& x : rots) {
+            r.param = (int16_t)(r.param | (1 << x.first));
+            P->rots.push_back(x.second);
+          }
+          rots.clear();
+          run = -1;
+          since = 0;
+        };
         for (int o = a; o < b; ++o) {
           BOp op = P->ops[o];
           const int bits = op.cm | (1 << op.b0);
@@ -1553,25 +1926,49 @@ void tile_lists(HostPlan* P) {
               sg.gi = (int16_t)(open - (int)s0);
               P->rops.push_back(sg);
             }
+            since |= bits;
             for (int r = 0; r < (1 << G.k); ++r)
               if ((r & bits) == bits) P->rsigns[open] ^= 1u << r;
             continue;
           }
           if (op.cls != BC_DIAG && op.cls != BC_PHASE) dirty |= bits;
           const BGateDesc& d = P->gates[C.gate0 + op.gi];
-          if (d.free_rot)
-            op.cls = d.kind == SV_GATE_RX ? BC_RX : d.kind == SV_GATE_RY ? BC_ROT : BC_RZ;
+          if (d.free_rot) {
+            const int at = 3 * op.b0 + (d.kind == SV_GATE_RX ? 0 : d.kind == SV_GATE_RY ? 1 : 2);
+            bool join = run >= 0 && !(since & bits);
+            for (const auto& x : rots)
+              if ((x.first / 3 == op.b0 && x.first >= at) ||
+                  (d.param >= 0 && x.second.param == d.param))
+                join = false;
+            if (!join) {
+              close();
+              run = (int)P->rops.size();
+              BOp r{};
+              r.cls = BC_RUN;
+              P->rops.push_back(r);
+            }
+            rots.push_back({at, BRot{d.kind, d.param, d.angle}});
+            continue;
+          }
+          since |= bits;
+          op.gi = (int16_t)(P->gens.size() - C.gen0);
+          P->gens.push_back(d);
           P->rops.push_back(op);
         }
+        close();
         G.op1 = (int32_t)P->rops.size();
         P->rgroups.push_back(G);
       }
       C.sign0 = (int)s0;
       C.nsign = (int)(P->rsigns.size() - s0);
+      C.nrot = (int)P->rots.size() - C.rot0;
+      C.ngen = (int)P->gens.size() - C.gen0;
       if (C.nsign <= kBMaxSigns) break;
       P->rops.resize(o0);
       P->rsigns.resize(s0);
       P->rgroups.resize(g0);
+      P->rots.resize(C.rot0);
+      P->gens.resize(C.gen0);
     }
   }
 }
@@ -1586,27 +1983,25 @@ sv_status upload(T** dst, const std::vector<T>& v) {
 
 void free_batch(sv_batch b) {
   void* ptrs[] = {b->circs, b->gates, b->groups, b->ops, b->terms, b->rgroups,
-                  b->rops, b->rsigns, b->order, b->item_circ, b->theta_off, b->queue, b->work};
+                  b->rops, b->rsigns, b->rots, b->gens, b->order, b->item_circ, b->theta_off, b->queue, b->work};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
 }
 
 typedef void (*BatchKernel)(const BatchArgs);
-// Kernel variants by (group width, threads per block, resident blocks per SM).
-// With states in shared memory: 2^k amplitudes a thread make a group of an n-qubit
-// item one round of a block of 2^(n - k) threads, so items of 11 qubits want four blocks of
-// 128 threads an SM and items of 14 one of 512.
-BatchKernel real_kernel_for(int k, int threads) {
-  if (threads <= 128) return k <= 4 ? kbatch<4, 128, 4, false, true> : kbatch<5, 128, 4, false, true>;
-  if (threads <= 256) return k <= 4 ? kbatch<4, 256, 2, false, true> : kbatch<5, 256, 2, false, true>;
+// Kernel variants by group width (and threads per block, resident blocks per SM).
+BatchKernel real_kernel_for(int k) {
   return k <= 3   ? kbatch<3, 512, 1, false, true>
          : k == 4 ? kbatch<4, 512, 1, false, true>
                   : kbatch<5, 512, 1, false, true>;
 }
-BatchKernel smem_kernel_for(int k, int threads) {
-  if (threads <= 128) return k <= 3 ? kbatch<3, 128, 4, true, true> : kbatch<4, 128, 4, true, true>;
-  if (threads <= 256) return k <= 3 ? kbatch<3, 256, 2, true, true> : kbatch<4, 256, 2, true, true>;
+BatchKernel wide_kernel_for(int k, bool re) {
+  if (re)
+    return k <= 3 ? kbatch_wide<3, false> : k == 4 ? kbatch_wide<4, false> : kbatch_wide<5, false>;
+  return k == 2 ? kbatch_wide<2, true> : k == 3 ? kbatch_wide<3, true> : kbatch_wide<4, true>;
+}
+BatchKernel smem_kernel_for(int k) {
   return k == 2   ? kbatch<2, 512, 1, true, true>
          : k == 3 ? kbatch<3, 512, 1, true, true>
                   : kbatch<4, 512, 1, true, true>;
@@ -1623,36 +2018,131 @@ BatchKernel kernel_for(int k, int threads, int per_sm) {
 // register groups of 2 or 3 qubits (4 would spill at 512 threads per block)
 BatchKernel cluster_kernel_for(int k) { return k == 2 ? kbatch_cl<2> : kbatch_cl<3>; }
 
-// Offsets of a block's shared memory (see BSmem) for this batch and group width k, and
-// the state memory that `per_sm` resident blocks leave it (a power of two, no
-// more than the largest item wants); returns the bytes.
-size_t block_smem(sv_batch b, int k, int threads, int per_sm, bool states, bool re, BatchArgs* A) {
+// The shared memory of one team (see BSmem) that runs `items`, with a state memory of a
+// power of two floats that the budget leaves, no more than the largest item wants.
+// Wide: a quarter of the states.
+void team_smem(sv_batch b, const std::vector<int>& items, int k, bool re, size_t budget, bool wide,
+               BPhase* P) {
+  int rots = 1, gens = 1, params = 1, ops = 1, groups = 1, terms = 1, signs = 1, n = k;
+  for (int i : items) {
+    const BCirc& C = b->h_circs[b->h_item_circ[i]];
+    rots = std::max(rots, C.nrot);
+    gens = std::max(gens, C.ngen);
+    params = std::max(params, C.nparams);
+    ops = std::max(ops, b->h_ops[b->h_item_circ[i]]);
+    groups = std::max(groups, C.ngroups);
+    terms = std::max(terms, C.nterms);
+    signs = std::max(signs, C.nsign);
+    n = std::max(n, C.n);
+  }
   size_t at = 0;
   auto take = [&](size_t bytes) {
     const size_t o = at;
     at += (bytes + 15) & ~size_t(15);
     return (int)o;
   };
-  A->o_mats = take(sizeof(float) * 8 * b->max_gates);
-  A->o_wpart = take(sizeof(float2) * (threads / 32) * b->max_params);
-  A->o_ops = take(sizeof(BOp) * b->max_ops);
-  A->o_grp = take(sizeof(BGroup) * b->max_groups);
-  A->o_term = take(sizeof(int2) * b->max_terms);
-  A->o_tcoef = take(sizeof(float) * 8 * b->max_terms);
-  A->o_sign = take((sizeof(float) << k) * b->max_signs);
-  A->o_state = (int)at;
-  A->pstride = b->max_params;
-  A->state_floats = 0;
-  if (states) {
-    // 228 KiB an SM, 1 KiB of it and the static variables taken by each block
-    const size_t budget = (size_t)228 * 1024 / per_sm - 1024 - 512;
-    const size_t want = size_t(re ? 2 : 4) << std::max(b->nmax, k);
-    size_t f = 0;
-    for (size_t c = 64; c <= want && at + sizeof(float) * c <= budget; c *= 2) f = c;
-    A->state_floats = (int)f;
-    at += sizeof(float) * f;
+  take(sizeof(float4) * rots);
+  P->o_mats = take(sizeof(float) * 8 * gens);
+  P->o_wpart = take(sizeof(float2) * (P->ts / 32) * params);
+  P->o_ops = take(sizeof(BOp) * ops);
+  P->o_grp = take(sizeof(BGroup) * groups);
+  P->o_term = take(sizeof(int2) * terms);
+  P->o_tcoef = take(sizeof(float) * 8 * terms);
+  P->o_sign = take((sizeof(float) << k) * signs);
+  P->o_state = (int)at;
+  P->pstride = params;
+  const size_t want = size_t(re ? 2 : 4) << (wide ? n - 2 : n);
+  size_t f = 0;
+  for (size_t c = 64; c <= want && at + sizeof(float) * c <= budget; c *= 2) f = c;
+  P->state_floats = (int)f;
+  P->stride = (int)(at + sizeof(float) * f);
+  P->count = (int)items.size();
+}
+
+// The size classes of the batch for a tile, and the items' order by them.  A class of
+// teams smaller than the block holds both states of its items in shared memory;
+// items whose states do not fit go to larger teams.
+sv_status set_phases(sv_batch b, int k, int threads, bool states, bool re) {
+  const size_t budget = (size_t)227 * 1024 - 512;  // 512: the static variables
+  std::vector<int> order;
+  std::vector<char> carried(b->n_items, 0), taken(b->n_items, 0);
+  std::vector<std::vector<int>> lists;
+  b->n_phases = 0;
+  b->smem = 0;
+  b->wide = BPhase{};
+  if (!states) {
+    BPhase P{};
+    P.ts = threads;
+    team_smem(b, b->h_order, k, re, 0, false, &P);
+    b->phase[b->n_phases++] = P;
+    order = b->h_order;
+    b->smem = P.stride;
+  } else {
+    // Wide items: more than one block's 512 tiles, no more than four.  Those of twice 512 cost
+    // 1.7 SM-milliseconds on a cluster and 0.93 in one block (n = 15, 10 layers, real,
+    // where n = 14 costs 0.33), but take 0.42 and 0.93 ms: they go to clusters where one in
+    // a block would outlast half of the batch, and where they are an eighth of it or
+    // less (1024 items of n = 14 and 256 of 8 to 16: 2.86 ms in blocks, 2.76 wide;
+    // 152 items of n = 15: 0.93 in blocks, 1.76 wide).
+    double total = 0, twice = 0;
+    const auto cost = [&](int i) {
+      const BCirc& C = b->h_circs[b->h_item_circ[i]];
+      return (C.n == k + 10 ? 1.4 : 1.0) * C.ngates * (double)(1 << C.n);
+    };
+    for (int i : b->h_order) {
+      total += cost(i);
+      if (b->h_circs[b->h_item_circ[i]].n == k + 10) twice += cost(i);
+    }
+    std::vector<int> wide;
+    for (int i : b->h_order) {
+      const int n = b->h_circs[b->h_item_circ[i]].n;
+      if (n == k + 11 || (n == k + 10 && (8 * twice <= total || cost(i) * b->sms > 2 * total)))
+        wide.push_back(i);
+    }
+    if (!wide.empty()) {
+      b->wide.ts = 512;
+      team_smem(b, wide, k, re, budget, true, &b->wide);
+      int n = 0;
+      for (int i : wide) n = std::max(n, b->h_circs[b->h_item_circ[i]].n);
+      if ((size_t)b->wide.state_floats < size_t(re ? 2 : 4) << (n - 2)) {
+        b->wide = BPhase{};
+        wide.clear();
+      }
+    }
+    for (int i : wide) taken[i] = 1;
+    order = wide;
+    std::vector<BPhase> phases;  // from the smallest teams
+    for (int ts = 64; ts <= 512; ts *= 2) {
+      std::vector<int> mine;  // keeps h_order's order: longest first
+      for (int i : b->h_order) {
+        const int n = std::max(b->h_circs[b->h_item_circ[i]].n, k);
+        const int tiles = 1 << (n - k);
+        const bool fits = ts == 64 ? tiles <= 64 : ts == 512 ? tiles >= 512 : tiles == ts;
+        if ((fits && !taken[i]) || carried[i]) mine.push_back(i);
+        carried[i] = 0;
+      }
+      if (mine.empty()) continue;
+      BPhase P{};
+      P.ts = ts;
+      team_smem(b, mine, k, re, budget / (512 / ts) & ~size_t(15), false, &P);
+      int n = k;
+      for (int i : mine) n = std::max(n, b->h_circs[b->h_item_circ[i]].n);
+      if (ts < 512 && (size_t)P.state_floats < size_t(re ? 2 : 4) << n) {
+        for (int i : mine) carried[i] = 1;  // to the next class
+        continue;
+      }
+      b->smem = std::max(b->smem, (size_t)P.stride * (512 / ts));
+      phases.push_back(P);
+      lists.push_back(mine);
+    }
+    for (size_t i = phases.size(); i-- > 0;) {
+      phases[i].first = (int)order.size();
+      order.insert(order.end(), lists[i].begin(), lists[i].end());
+      b->phase[b->n_phases++] = phases[i];
+    }
   }
-  return at;
+  SV_CUDA_TRY(cudaMemcpy(b->order, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice));
+  return SV_OK;
 }
 
 sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* grad,
@@ -1667,6 +2157,11 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
   A.rgroups = b->rgroups;
   A.rops = b->rops;
   A.rsigns = b->rsigns;
+  A.rots = b->rots;
+  A.gens = b->gens;
+  A.n_phases = b->n_phases;
+  for (int i = 0; i < b->n_phases; ++i) A.phase[i] = b->phase[i];
+  A.wide = b->wide;
   A.order = b->order;
   A.item_circ = b->item_circ;
   A.theta_off = b->theta_off;
@@ -1677,7 +2172,7 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
   A.grad = grad;
   A.work = b->work;
   A.queue = b->queue;
-  SV_CUDA_TRY(cudaMemsetAsync(b->queue, 0, sizeof(int), st));
+  SV_CUDA_TRY(cudaMemsetAsync(b->queue, 0, (kBPhases + 1) * sizeof(int), st));
   if (cl) {
     BatchKernel kern = cluster_kernel_for(k);
     static bool attr[5] = {false, false, false, false, false};
@@ -1692,12 +2187,11 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
     return check_launch("batch cluster kernel");
   }
   const int per_sm = std::max(1, blocks / std::max(1, b->sms));
-  BatchKernel kern = re    ? real_kernel_for(k, threads)
-                     : sms ? smem_kernel_for(k, threads)
+  BatchKernel kern = re    ? real_kernel_for(k)
+                     : sms ? smem_kernel_for(k)
                            : kernel_for(k, threads, per_sm);
-  const size_t smem = block_smem(b, k, threads, per_sm, re || sms, re, &A);
-  {
-    // opt in to more than the default 48 KiB, to the most any batch has asked for
+  // opt in to more than the default 48 KiB, to the most any batch has asked for
+  const auto allow = [](BatchKernel kern, size_t smem) -> sv_status {
     static std::mutex mu;
     static std::vector<std::pair<BatchKernel, size_t>> done;
     std::lock_guard<std::mutex> lk(mu);
@@ -1710,9 +2204,25 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
       else
         it->second = smem;
     }
-  }
+    return SV_OK;
+  };
   ProfScope prof(st, re ? "kbatch_re" : sms ? "kbatch_smem" : "kbatch");
-  kern<<<blocks, threads, smem, st>>>(A);
+  sv_status s = allow(kern, b->smem);
+  if (s) return s;
+  if (b->wide.count > 0) {
+    BatchKernel wide = wide_kernel_for(k, re);
+    s = allow(wide, b->wide.stride);
+    if (s) return s;
+    const int clusters = std::min(b->wide.count, std::max(1, b->sms / kWide));
+    wide<<<clusters * kWide, 512, b->wide.stride, st>>>(A);
+    s = check_launch("batch kernel (wide items)");
+    if (s) return s;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (b->n_phases == 0) return SV_OK;
+    launch_dependent(kern, blocks, threads, b->smem, st, A);
+  } else {
+    kern<<<blocks, threads, b->smem, st>>>(A);
+  }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("batch kernel");
 }
@@ -1874,12 +2384,8 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
     cands.push_back({std::max(4, width), 512, 1, false, true, true});
   } else if (tune == 1) {
     const Cand all[] = {{3, 512, 1, false, true, true}, {4, 512, 1, false, true, true},
-                        {4, 256, 2, false, true, true}, {4, 128, 4, false, true, true},
-                        {5, 512, 1, false, true, true}, {5, 256, 2, false, true, true},
-                        {5, 128, 4, false, true, true},
+                        {5, 512, 1, false, true, true},
                         {2, 512, 1, false, true}, {3, 512, 1, false, true}, {4, 512, 1, false, true},
-                        {3, 256, 2, false, true}, {4, 256, 2, false, true},
-                        {3, 128, 4, false, true}, {4, 128, 4, false, true},
                         {2, kClThreads, 1, true}, {3, kClThreads, 1, true},
                         {2, 256, 2, false}, {3, 256, 2, false}, {4, 256, 2, false},
                         {2, 256, 4, false}, {3, 256, 4, false}, {2, 128, 8, false},
@@ -1899,11 +2405,13 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
   b->sms = sms;
   sv_status st = SV_OK;
   // plans per k are built on demand; start with the device buffers that do not depend on k
+  b->h_order = order;
+  b->h_item_circ = ic;
   st = upload(&b->order, order);
   if (!st) st = upload(&b->item_circ, ic);
   if (!st) st = upload(&b->theta_off, toff);
   if (!st) {
-    cudaError_t e = cudaMalloc(&b->queue, sizeof(int));
+    cudaError_t e = cudaMalloc(&b->queue, (kBPhases + 1) * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->work, b->work_slots * (sizeof(float2) << (std::max(nmax, 5) + 1)));
     if (e != cudaSuccess) {
       set_error("sv_batch_create: %s", cudaGetErrorString(e));
@@ -1918,22 +2426,17 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
         return SV_ERR_INVALID;
       }
     tile_lists(&P);
-    b->max_gates = b->max_params = b->max_ops = b->max_groups = b->max_terms = b->max_signs = 1;
-    for (const BCirc& C : P.circs) {
-      b->max_gates = std::max(b->max_gates, C.ngates);
-      b->max_params = std::max(b->max_params, C.nparams);
-      b->max_terms = std::max(b->max_terms, C.nterms);
-      b->max_groups = std::max(b->max_groups, C.ngroups);
-      b->max_signs = std::max(b->max_signs, C.nsign);
-      if (C.ngroups)
-        b->max_ops = std::max(b->max_ops, P.rgroups[C.group0 + C.ngroups - 1].op1 -
-                                              P.rgroups[C.group0].op0);
-    }
-    void* olds[] = {b->circs, b->gates, b->groups, b->ops, b->terms, b->rgroups, b->rops, b->rsigns};
+    b->h_circs = P.circs;
+    b->h_ops.clear();
+    for (const BCirc& C : P.circs)
+      b->h_ops.push_back(C.ngroups ? P.rgroups[C.group0 + C.ngroups - 1].op1 - P.rgroups[C.group0].op0
+                                   : 0);
+    void* olds[] = {b->circs, b->gates, b->groups, b->ops, b->terms, b->rgroups, b->rops, b->rsigns,
+                    b->rots, b->gens};
     for (void* p : olds)
       if (p) cudaFree(p);
     b->circs = nullptr; b->gates = nullptr; b->groups = nullptr; b->ops = nullptr; b->terms = nullptr;
-    b->rgroups = nullptr; b->rops = nullptr; b->rsigns = nullptr;
+    b->rgroups = nullptr; b->rops = nullptr; b->rsigns = nullptr; b->rots = nullptr; b->gens = nullptr;
     sv_status s2 = upload(&b->circs, P.circs);
     if (!s2) s2 = upload(&b->gates, P.gates);
     if (!s2) s2 = upload(&b->groups, P.groups);
@@ -1942,6 +2445,8 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
     if (!s2) s2 = upload(&b->rgroups, P.rgroups);
     if (!s2) s2 = upload(&b->rops, P.rops);
     if (!s2) s2 = upload(&b->rsigns, P.rsigns);
+    if (!s2) s2 = upload(&b->rots, P.rots);
+    if (!s2) s2 = upload(&b->gens, P.gens);
     return s2;
   };
   double* th = nullptr;
@@ -1972,6 +2477,8 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
         if (st) break;
       }
       const int blocks = c.cl ? 2 * (sms / 2) : sms * c.per_sm;
+      st = set_phases(b, c.k, c.threads, c.sms || c.re, c.re);
+      if (st) break;
       st = launch_batch(b, th, en, gr, 0, c.k, c.threads, blocks, c.cl, c.sms, c.re);  // warm-up
       if (st) break;
       cudaEventRecord(e0, 0);
@@ -2008,6 +2515,7 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
   if (en) cudaFree(en);
   if (gr) cudaFree(gr);
   if (!st) st = build_for_k(b->k);
+  if (!st) st = set_phases(b, b->k, b->threads, b->smem_states || b->real, b->real);
   if (!st) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
