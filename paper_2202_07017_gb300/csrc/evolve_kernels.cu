@@ -112,6 +112,41 @@ __global__ void __launch_bounds__(kEThreads)
   }
 }
 
+// complex128, a few strings: one rotation after the other as three FMAs an amplitude
+// (see Shear), where the angle sum's fp64 sine and cosine alone take about 40
+// instructions.  n = 20, one string: 73 -> 12 us, eight 89 -> 53 (n = 25: 2110 -> 1302),
+// 6 us each: up to kShearTerms of them, short of where the two cost the same.
+constexpr int kShearTerms = 12;
+struct DiagShears {
+  int nt;
+  uint64_t zm[kShearTerms];
+  Shear h[kShearTerms];
+};
+__global__ void __launch_bounds__(kEThreads)
+    kdiag_shears(double2* __restrict__ psi, uint64_t dim, const __grid_constant__ DiagShears D) {
+  grid_dependency_wait();
+  constexpr int IT = 4;
+  const uint64_t base = (uint64_t)blockIdx.x * (kEThreads * IT) + threadIdx.x;
+  double2 v[IT];
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const uint64_t i = base + (uint64_t)it * kEThreads;
+    if (i < dim) v[it] = psi[i];
+  }
+  for (int k = 0; k < D.nt; ++k) {
+    const uint64_t z = D.zm[k];
+    const Shear h = D.h[k];
+#pragma unroll
+    for (int it = 0; it < IT; ++it)
+      shear_rot(h, __popcll((base + (uint64_t)it * kEThreads) & z) & 1, v[it].x, v[it].y);
+  }
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const uint64_t i = base + (uint64_t)it * kEThreads;
+    if (i < dim) psi[i] = v[it];
+  }
+}
+
 // ---- runs of diagonal strings --------------------------------------------------------
 constexpr int kRunTerms = 256;  // terms of one kdiag_run launch
 constexpr int kAdjTerms = 128;  // terms of one kadj_diag launch
@@ -374,6 +409,51 @@ __global__ void __launch_bounds__(kEThreads)
   }
 }
 
+// A Pauli-string rotation c I + coef P of complex128 states as shears: with P's
+// i^{ny} and the strings' signs, even ny rotates (re x, im y) and (re y, im x) by
+// one angle, odd ny (re x, re y) and (im x, im y), with the angle's sign by
+// parity(y & zm) ^ (ny >> 1).  Six FMAs an amplitude pair where the products take 24
+// and more fp64 instructions: n = 20 25 -> 12.4 us.
+template <bool ODD>
+__device__ __forceinline__ void shear_pair(const Shear& h, int sign, double2& x, double2& y) {
+  if (ODD) {
+    shear_rot(h, sign, x.x, y.x);
+    shear_rot(h, sign, x.y, y.y);
+  } else {
+    shear_rot(h, sign, x.x, y.y);
+    shear_rot(h, sign, y.x, x.y);
+  }
+}
+
+template <bool ODD>
+__global__ void __launch_bounds__(kEThreads)
+    kpair_c128(double2* __restrict__ psi, uint64_t npairs, uint64_t lowmask, uint64_t xm,
+               uint64_t zm, int neg, Shear h) {
+  grid_dependency_wait();
+  constexpr int IT = 4;
+  const uint64_t base = (uint64_t)blockIdx.x * (kEThreads * IT) + threadIdx.x;
+  double2 a[IT], b[IT];
+  uint64_t xs[IT];
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const uint64_t u = base + (uint64_t)it * kEThreads;
+    xs[it] = ((u & ~lowmask) << 1) | (u & lowmask);
+    if (u < npairs) {
+      a[it] = psi[xs[it]];
+      b[it] = psi[xs[it] ^ xm];
+    }
+  }
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const uint64_t u = base + (uint64_t)it * kEThreads;
+    if (u >= npairs) continue;
+    const uint64_t y = xs[it] ^ xm;
+    shear_pair<ODD>(h, (__popcll(y & zm) & 1) ^ neg, a[it], b[it]);
+    psi[xs[it]] = a[it];
+    psi[y] = b[it];
+  }
+}
+
 // the rotated state: device data, precision, qubits, stream and the
 // complex64 rounding feedback (see feedback_round)
 struct Target {
@@ -442,6 +522,47 @@ __global__ void __launch_bounds__(kEThreads)
     }
   }
   const double t = block_sum(acc.value());
+  if (threadIdx.x == 0 && partials) partials[blockIdx.x] = t;
+}
+
+// The same step for complex128 as shears (fp64 issue bounds it: a diagonal string 9
+// instructions an amplitude pair of psi and lambda where the products take 14, the others 17 a
+// unit in place of 50): n = 20 42.7 -> 25 us (HBM and L2: 32 MiB of states read and
+// written).  KIND 0: diagonal; 1: even ny; 2: odd ny.
+template <int KIND>
+__global__ void __launch_bounds__(kEThreads)
+    kadj_pauli_c128(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t units,
+                    uint64_t lowmask, uint64_t xm, uint64_t zm, int neg, Shear h,
+                    double* __restrict__ partials) {
+  grid_dependency_wait();
+  double acc = 0.0;
+  for (uint64_t u = (uint64_t)blockIdx.x * kEThreads + threadIdx.x; u < units;
+       u += (uint64_t)gridDim.x * kEThreads) {
+    if (KIND == 0) {
+      double2 p = psi[u], l = lam[u];
+      const int odd = __popcll(u & zm) & 1;
+      acc += flip_sign(l.x * p.y - l.y * p.x, odd);
+      shear_rot(h, odd, p.x, p.y);
+      shear_rot(h, odd, l.x, l.y);
+      psi[u] = p;
+      lam[u] = l;
+    } else {
+      const uint64_t x = ((u & ~lowmask) << 1) | (u & lowmask), y = x ^ xm;
+      double2 px = psi[x], py = psi[y], lx = lam[x], ly = lam[y];
+      const int sign = (__popcll(y & zm) & 1) ^ neg;  // sx = sy for even ny, -sy for odd
+      if (KIND == 1)
+        acc += flip_sign(lx.x * py.y - lx.y * py.x + ly.x * px.y - ly.y * px.x, sign);
+      else
+        acc += flip_sign(lx.x * py.x + lx.y * py.y - ly.x * px.x - ly.y * px.y, sign);
+      shear_pair<KIND == 2>(h, sign, px, py);
+      shear_pair<KIND == 2>(h, sign, lx, ly);
+      psi[x] = px;
+      psi[y] = py;
+      lam[x] = lx;
+      lam[y] = ly;
+    }
+  }
+  const double t = block_sum(acc);
   if (threadIdx.x == 0 && partials) partials[blockIdx.x] = t;
 }
 
@@ -529,6 +650,23 @@ void run_tiles(const Target& s, const uint64_t* zm, const double* a, int cnt) {
 
 // A run of commuting diagonal rotations exp(-i a_k P_k).
 sv_status run_diags(const Target& s, const std::vector<uint64_t>& zm, const std::vector<double>& a) {
+  if (s.dt == SV_C128 && zm.size() <= (size_t)kShearTerms) {
+    DiagShears D{};
+    for (size_t k = 0; k < zm.size(); ++k) {
+      D.zm[k] = zm[k];
+      if (!make_shear(std::cos(a[k]), -std::sin(a[k]), &D.h[k])) break;  // not finite
+      ++D.nt;
+    }
+    if (D.nt == 0 && zm.empty()) return SV_OK;
+    if (D.nt == (int)zm.size()) {
+      const uint64_t dim = uint64_t(1) << s.n;
+      ProfScope prof(s.stream, "kdiag_shears_c128");
+      launch_dependent(kdiag_shears, (unsigned)((dim + kEThreads * 4 - 1) / (kEThreads * 4)),
+                       kEThreads, 0, s.stream, (double2*)s.data, dim, D);
+      g_launches.fetch_add(1, std::memory_order_relaxed);
+      return check_launch("diagonal rotations kernel");
+    }
+  }
   bool tiles = s.n >= kRunMinQubits;
   for (double x : a) tiles = tiles && fixed_point_angle(x);
   if (!tiles) {
@@ -622,8 +760,11 @@ sv_status run_pair(const Target& s, uint64_t xm, uint64_t zm, double a) {
     launch_dependent(kpair<float, float2>, g, kEThreads, 0, s.stream, (float2*)s.data, npairs,
                      lowmask, xm, zm, (float)c32, (float)k32.re, (float)k32.im);
   } else {
-    launch_dependent(kpair<double, double2>, g, kEThreads, 0, s.stream, (double2*)s.data, npairs,
-                     lowmask, xm, zm, ca, kr, ki);
+    Shear h;
+    if (!make_shear(ca, -sa, &h)) h = {ca, -sa, 0};  // not finite, and so the result
+    const unsigned g4 = (unsigned)((npairs + kEThreads * 4 - 1) / (kEThreads * 4));
+    launch_dependent((ny & 1) ? kpair_c128<true> : kpair_c128<false>, g4, kEThreads, 0, s.stream,
+                     (double2*)s.data, npairs, lowmask, xm, zm, ny >> 1, h);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_launch("pair rotation kernel");
@@ -754,12 +895,12 @@ sv_status launch_adjoint_pauli(void* psi, void* lam, sv_dtype dt, int n, cudaStr
                        (float2*)lam, units, lowmask, xm, zm, ny, (float)c, (float)kr, (float)ki,
                        partials);
   } else {
-    if (diag)
-      launch_dependent(kadj_pauli<double, double2, true>, grid, kEThreads, 0, st, (double2*)psi,
-                       (double2*)lam, units, lowmask, xm, zm, ny, c, kr, ki, partials);
-    else
-      launch_dependent(kadj_pauli<double, double2, false>, grid, kEThreads, 0, st, (double2*)psi,
-                       (double2*)lam, units, lowmask, xm, zm, ny, c, kr, ki, partials);
+    // c I + i sin i^{ny} P: the un-applied rotation's angle is +theta / 2
+    Shear h;
+    if (!make_shear(c, sn, &h)) h = {c, sn, 0};  // not finite, and so the result
+    const auto kern = diag ? kadj_pauli_c128<0> : (ny & 1) ? kadj_pauli_c128<2> : kadj_pauli_c128<1>;
+    launch_dependent(kern, grid, kEThreads, 0, st, (double2*)psi, (double2*)lam, units, lowmask, xm,
+                     zm, ny >> 1, h, partials);
   }
   g_launches.fetch_add(1, std::memory_order_relaxed);
   if (nparts) *nparts = grid;

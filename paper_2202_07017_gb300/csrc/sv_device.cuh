@@ -112,6 +112,15 @@ __device__ __forceinline__ void shear_rot(const Shear& h, double& x, double& y) 
   x = fma(h.a, y, x);
 }
 
+// the same by the opposite angle when `odd` (0 or 1)
+__device__ __forceinline__ double flip_sign(double x, int odd) {
+  return __longlong_as_double(__double_as_longlong(x) ^ ((long long)odd << 63));
+}
+__device__ __forceinline__ void shear_rot(const Shear& h, int odd, double& x, double& y) {
+  const Shear g = {flip_sign(h.a, odd), flip_sign(h.b, odd), odd ? (4 - h.k) & 3 : h.k};
+  shear_rot(g, x, y);
+}
+
 // (a, b) <- G (a, b) for the 2x2s that are rotations: SK_REAL [[c, -s], [s, c]]
 // (h[0]; refl: of (a, -b), as H), SK_IMOFF [[c, i s], [i s, c]] (h[0], RX), SK_PHASES
 // diag(e^{i f}, e^{i g}) (h[0], h[1], RZ).  SK_NONE: none of them.
