@@ -147,6 +147,44 @@ __global__ void __launch_bounds__(kEThreads)
   }
 }
 
+// complex64, up to kShearTermsF strings: the sine and cosine of one angle are rounded
+// alike on every amplitude, and a circuit that repeats it (QAOA's edges, gate by
+// gate) repeats their scale; shears have none.  QAOA, n = 14..20, energies and
+// gradients against 64 bits: 0.8..3.6e-6 before, 4.0..6.6e-7 now, with as little work.
+constexpr int kShearTermsF = 4;
+struct DiagShearsF {
+  int nt;
+  uint64_t zm[kShearTermsF];
+  ShearF h[kShearTermsF];
+};
+__global__ void __launch_bounds__(kEThreads)
+    kdiag_shears_f(float4* __restrict__ psi, uint64_t nvec, const __grid_constant__ DiagShearsF D) {
+  grid_dependency_wait();
+  constexpr int IT = 4;
+  const uint64_t base = (uint64_t)blockIdx.x * (kEThreads * IT) + threadIdx.x;
+  float4 v[IT];
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const uint64_t i = base + (uint64_t)it * kEThreads;
+    if (i < nvec) v[it] = psi[i];
+  }
+  for (int k = 0; k < D.nt; ++k) {
+    const uint64_t z = D.zm[k];
+    const ShearF h = D.h[k];
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int odd = __popcll((2 * (base + (uint64_t)it * kEThreads)) & z) & 1;
+      shear_rot(h, odd, v[it].x, v[it].y);
+      shear_rot(h, odd ^ (int)(z & 1), v[it].z, v[it].w);
+    }
+  }
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const uint64_t i = base + (uint64_t)it * kEThreads;
+    if (i < nvec) psi[i] = v[it];
+  }
+}
+
 // ---- runs of diagonal strings --------------------------------------------------------
 constexpr int kRunTerms = 256;  // terms of one kdiag_run launch
 constexpr int kAdjTerms = 128;  // terms of one kadj_diag launch
@@ -414,8 +452,8 @@ __global__ void __launch_bounds__(kEThreads)
 // one angle, odd ny (re x, re y) and (im x, im y), with the angle's sign by
 // parity(y & zm) ^ (ny >> 1).  Six FMAs an amplitude pair where the products take 24
 // and more fp64 instructions: n = 20 25 -> 12.4 us.
-template <bool ODD>
-__device__ __forceinline__ void shear_pair(const Shear& h, int sign, double2& x, double2& y) {
+template <bool ODD, typename H, typename T2>
+__device__ __forceinline__ void shear_pair(const H& h, int sign, T2& x, T2& y) {
   if (ODD) {
     shear_rot(h, sign, x.x, y.x);
     shear_rot(h, sign, x.y, y.y);
@@ -467,93 +505,42 @@ struct Target {
 // Adjoint step of a Pauli-string rotation U = exp(-i theta P / 2) in a
 // reverse sweep (P = i^{ny} X^xm Z^zm up to the sign convention above): each
 // unit first adds its part of Im<lambda|P|psi> (the gradient of theta) and
-// then un-applies U^dagger = c I + kappa P, c = cos(theta / 2),
-// kappa = i sin(theta / 2) i^{ny}, on psi and lambda.  DIAG (xm = 0): a unit
-// is one amplitude, (P v)_x = s(x) v_x; otherwise a unit is the pair
-// (x, y = x ^ xm) with bit h = top bit of xm clear in x and
+// then un-applies U^dagger on psi and lambda, as shears.  KIND 0 (xm = 0): a unit
+// is one amplitude, (P v)_x = s(x) v_x; otherwise (KIND 1 even ny, 2 odd ny) a unit
+// is the pair (x, y = x ^ xm) with bit h = top bit of xm clear in x and
 // (P v)_x = i^{ny} s(y) v_y, (P v)_y = i^{ny} s(x) v_x, s(v) =
-// (-1)^{popcount(v & zm)}.  Per-thread sums: compensated in fp32 for
-// complex64, fp64 for complex128; the block's fp64 sum goes to
+// (-1)^{popcount(v & zm)}, s(x) = s(y) (-1)^{ny}.  Per-thread sums: compensated in
+// fp32 for complex64, fp64 for complex128; the block's fp64 sum goes to
 // partials[blockIdx.x] (grid-stride loop, every block writes its slot).
-template <typename R, typename T2, bool DIAG>
+// complex128 is bound by fp64 issue: a diagonal string takes 9 instructions an
+// amplitude of psi and lambda where the products take 14, the others 17 a unit in
+// place of 50: n = 20 42.7 -> 25 us (HBM and L2: 32 MiB of states read and written).
+// complex64 loses no norm (see kdiag_shears_f); its time is the states' traffic.
+template <typename R, typename T2, int KIND>
 __global__ void __launch_bounds__(kEThreads)
     kadj_pauli(T2* __restrict__ psi, T2* __restrict__ lam, uint64_t units, uint64_t lowmask,
-               uint64_t xm, uint64_t zm, int ny, R c, R kr, R ki, double* __restrict__ partials) {
+               uint64_t xm, uint64_t zm, int neg, typename ShearOf<R>::T h,
+               double* __restrict__ partials) {
   grid_dependency_wait();
   CompSum<R> acc;
   for (uint64_t u = (uint64_t)blockIdx.x * kEThreads + threadIdx.x; u < units;
        u += (uint64_t)gridDim.x * kEThreads) {
-    if (DIAG) {
-      const uint64_t x = u;
-      T2 p = psi[x], l = lam[x];
-      const R sx = (__popcll(x & zm) & 1) ? R(-1) : R(1);
-      acc.add(sx * (l.x * p.y - l.y * p.x));  // Im conj(l) s p
-      // v <- (c + s(x) kappa) v, kappa = (kr, ki)
-      const R ar = c + sx * kr, ai = sx * ki;
-      T2 np, nl;
-      np.x = ar * p.x - ai * p.y;
-      np.y = ar * p.y + ai * p.x;
-      nl.x = ar * l.x - ai * l.y;
-      nl.y = ar * l.y + ai * l.x;
-      psi[x] = np;
-      lam[x] = nl;
-    } else {
-      const uint64_t x = ((u & ~lowmask) << 1) | (u & lowmask), y = x ^ xm;
-      const T2 px = psi[x], py = psi[y], lx = lam[x], ly = lam[y];
-      const R sx = (__popcll(x & zm) & 1) ? R(-1) : R(1);
-      const R sy = (__popcll(y & zm) & 1) ? R(-1) : R(1);
-      // w = s(y) conj(lx) py + s(x) conj(ly) px; the unit adds Im(i^{ny} w)
-      const R wr = sy * (lx.x * py.x + lx.y * py.y) + sx * (ly.x * px.x + ly.y * px.y);
-      const R wi = sy * (lx.x * py.y - lx.y * py.x) + sx * (ly.x * px.y - ly.y * px.x);
-      acc.add(ny == 0 ? wi : ny == 1 ? wr : ny == 2 ? -wi : -wr);
-      T2 npx, npy, nlx, nly;
-      npx.x = c * px.x + sy * (kr * py.x - ki * py.y);
-      npx.y = c * px.y + sy * (kr * py.y + ki * py.x);
-      npy.x = c * py.x + sx * (kr * px.x - ki * px.y);
-      npy.y = c * py.y + sx * (kr * px.y + ki * px.x);
-      nlx.x = c * lx.x + sy * (kr * ly.x - ki * ly.y);
-      nlx.y = c * lx.y + sy * (kr * ly.y + ki * ly.x);
-      nly.x = c * ly.x + sx * (kr * lx.x - ki * lx.y);
-      nly.y = c * ly.y + sx * (kr * lx.y + ki * lx.x);
-      psi[x] = npx;
-      psi[y] = npy;
-      lam[x] = nlx;
-      lam[y] = nly;
-    }
-  }
-  const double t = block_sum(acc.value());
-  if (threadIdx.x == 0 && partials) partials[blockIdx.x] = t;
-}
-
-// The same step for complex128 as shears (fp64 issue bounds it: a diagonal string 9
-// instructions an amplitude pair of psi and lambda where the products take 14, the others 17 a
-// unit in place of 50): n = 20 42.7 -> 25 us (HBM and L2: 32 MiB of states read and
-// written).  KIND 0: diagonal; 1: even ny; 2: odd ny.
-template <int KIND>
-__global__ void __launch_bounds__(kEThreads)
-    kadj_pauli_c128(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t units,
-                    uint64_t lowmask, uint64_t xm, uint64_t zm, int neg, Shear h,
-                    double* __restrict__ partials) {
-  grid_dependency_wait();
-  double acc = 0.0;
-  for (uint64_t u = (uint64_t)blockIdx.x * kEThreads + threadIdx.x; u < units;
-       u += (uint64_t)gridDim.x * kEThreads) {
     if (KIND == 0) {
-      double2 p = psi[u], l = lam[u];
+      T2 p = psi[u], l = lam[u];
       const int odd = __popcll(u & zm) & 1;
-      acc += flip_sign(l.x * p.y - l.y * p.x, odd);
+      acc.add(flip_sign(l.x * p.y - l.y * p.x, odd));
       shear_rot(h, odd, p.x, p.y);
       shear_rot(h, odd, l.x, l.y);
       psi[u] = p;
       lam[u] = l;
     } else {
       const uint64_t x = ((u & ~lowmask) << 1) | (u & lowmask), y = x ^ xm;
-      double2 px = psi[x], py = psi[y], lx = lam[x], ly = lam[y];
-      const int sign = (__popcll(y & zm) & 1) ^ neg;  // sx = sy for even ny, -sy for odd
+      T2 px = psi[x], py = psi[y], lx = lam[x], ly = lam[y];
+      const int sign = (__popcll(y & zm) & 1) ^ neg;
       if (KIND == 1)
-        acc += flip_sign(lx.x * py.y - lx.y * py.x + ly.x * px.y - ly.y * px.x, sign);
+        acc.add(flip_sign(lx.x * py.y - lx.y * py.x + ly.x * px.y - ly.y * px.x, sign));
       else
-        acc += flip_sign(lx.x * py.x + lx.y * py.y - ly.x * px.x - ly.y * px.y, sign);
+        acc.add(flip_sign(lx.x * py.x + lx.y * py.y - ly.x * px.x - ly.y * px.y, sign));
       shear_pair<KIND == 2>(h, sign, px, py);
       shear_pair<KIND == 2>(h, sign, lx, ly);
       psi[x] = px;
@@ -562,7 +549,7 @@ __global__ void __launch_bounds__(kEThreads)
       lam[y] = ly;
     }
   }
-  const double t = block_sum(acc);
+  const double t = block_sum(acc.value());
   if (threadIdx.x == 0 && partials) partials[blockIdx.x] = t;
 }
 
@@ -650,19 +637,30 @@ void run_tiles(const Target& s, const uint64_t* zm, const double* a, int cnt) {
 
 // A run of commuting diagonal rotations exp(-i a_k P_k).
 sv_status run_diags(const Target& s, const std::vector<uint64_t>& zm, const std::vector<double>& a) {
-  if (s.dt == SV_C128 && zm.size() <= (size_t)kShearTerms) {
-    DiagShears D{};
-    for (size_t k = 0; k < zm.size(); ++k) {
-      D.zm[k] = zm[k];
-      if (!make_shear(std::cos(a[k]), -std::sin(a[k]), &D.h[k])) break;  // not finite
-      ++D.nt;
-    }
-    if (D.nt == 0 && zm.empty()) return SV_OK;
-    if (D.nt == (int)zm.size()) {
-      const uint64_t dim = uint64_t(1) << s.n;
-      ProfScope prof(s.stream, "kdiag_shears_c128");
-      launch_dependent(kdiag_shears, (unsigned)((dim + kEThreads * 4 - 1) / (kEThreads * 4)),
-                       kEThreads, 0, s.stream, (double2*)s.data, dim, D);
+  if (zm.empty()) return SV_OK;
+  if (zm.size() <= (size_t)(s.dt == SV_C64 ? kShearTermsF : kShearTerms)) {
+    Shear h[kShearTerms];
+    size_t k = 0;  // stops at an angle that is not finite
+    while (k < zm.size() && make_shear(std::cos(a[k]), -std::sin(a[k]), &h[k])) ++k;
+    if (k == zm.size()) {
+      const uint64_t vecs = uint64_t(1) << (s.dt == SV_C64 ? s.n - 1 : s.n);
+      const unsigned grid = (unsigned)((vecs + kEThreads * 4 - 1) / (kEThreads * 4));
+      ProfScope prof(s.stream, s.dt == SV_C64 ? "kdiag_shears_c64" : "kdiag_shears_c128");
+      if (s.dt == SV_C64) {
+        DiagShearsF D{};
+        for (; D.nt < (int)k; ++D.nt) {
+          D.zm[D.nt] = zm[D.nt];
+          D.h[D.nt] = round_shear(h[D.nt]);
+        }
+        launch_dependent(kdiag_shears_f, grid, kEThreads, 0, s.stream, (float4*)s.data, vecs, D);
+      } else {
+        DiagShears D{};
+        for (; D.nt < (int)k; ++D.nt) {
+          D.zm[D.nt] = zm[D.nt];
+          D.h[D.nt] = h[D.nt];
+        }
+        launch_dependent(kdiag_shears, grid, kEThreads, 0, s.stream, (double2*)s.data, vecs, D);
+      }
       g_launches.fetch_add(1, std::memory_order_relaxed);
       return check_launch("diagonal rotations kernel");
     }
@@ -868,14 +866,6 @@ sv_status launch_adjoint_pauli(void* psi, void* lam, sv_dtype dt, int n, cudaStr
   const int grid = red_blocks(uint64_t(1) << (n >= 2 ? n - 2 : 0));
   const int ny = __builtin_popcountll(xm & zm) & 3;
   const double c = std::cos(0.5 * theta), sn = std::sin(0.5 * theta);
-  // kappa = i sin(theta / 2) i^{ny}
-  double kr = 0, ki = 0;
-  switch (ny) {
-    case 0: ki = sn; break;
-    case 1: kr = -sn; break;
-    case 2: ki = -sn; break;
-    default: kr = sn; break;
-  }
   const bool diag = xm == 0;
   uint64_t units = uint64_t(1) << n, lowmask = 0;
   if (!diag) {
@@ -885,20 +875,19 @@ sv_status launch_adjoint_pauli(void* psi, void* lam, sv_dtype dt, int n, cudaStr
     units >>= 1;
   }
   ProfScope prof(st, dt == SV_C64 ? "kadj_pauli_c64" : "kadj_pauli_c128");
+  // c I + i sin i^{ny} P: the un-applied rotation's angle is +theta / 2
+  Shear h;
+  if (!make_shear(c, sn, &h)) h = {c, sn, 0};  // not finite, and so the result
   if (dt == SV_C64) {
-    if (diag)
-      launch_dependent(kadj_pauli<float, float2, true>, grid, kEThreads, 0, st, (float2*)psi,
-                       (float2*)lam, units, lowmask, xm, zm, ny, (float)c, (float)kr, (float)ki,
-                       partials);
-    else
-      launch_dependent(kadj_pauli<float, float2, false>, grid, kEThreads, 0, st, (float2*)psi,
-                       (float2*)lam, units, lowmask, xm, zm, ny, (float)c, (float)kr, (float)ki,
-                       partials);
+    const auto kern = diag       ? kadj_pauli<float, float2, 0>
+                      : (ny & 1) ? kadj_pauli<float, float2, 2>
+                                 : kadj_pauli<float, float2, 1>;
+    launch_dependent(kern, grid, kEThreads, 0, st, (float2*)psi, (float2*)lam, units, lowmask, xm,
+                     zm, ny >> 1, round_shear(h), partials);
   } else {
-    // c I + i sin i^{ny} P: the un-applied rotation's angle is +theta / 2
-    Shear h;
-    if (!make_shear(c, sn, &h)) h = {c, sn, 0};  // not finite, and so the result
-    const auto kern = diag ? kadj_pauli_c128<0> : (ny & 1) ? kadj_pauli_c128<2> : kadj_pauli_c128<1>;
+    const auto kern = diag       ? kadj_pauli<double, double2, 0>
+                      : (ny & 1) ? kadj_pauli<double, double2, 2>
+                                 : kadj_pauli<double, double2, 1>;
     launch_dependent(kern, grid, kEThreads, 0, st, (double2*)psi, (double2*)lam, units, lowmask, xm,
                      zm, ny >> 1, h, partials);
   }

@@ -121,6 +121,41 @@ __device__ __forceinline__ void shear_rot(const Shear& h, int odd, double& x, do
   shear_rot(g, x, y);
 }
 
+// complex64: the shears of the angle that the rounded a makes, so that a and b are the
+// rotation's to half an ulp of b and no scale repeats with one sign
+struct ShearF {
+  float a, b;
+  int k;
+};
+template <typename R>
+struct ShearOf {
+  typedef Shear T;
+};
+template <>
+struct ShearOf<float> {
+  typedef ShearF T;
+};
+__device__ __forceinline__ float flip_sign(float x, int odd) {
+  return __uint_as_float(__float_as_uint(x) ^ ((unsigned)odd << 31));
+}
+inline ShearF round_shear(const Shear& h) {
+  const float a = (float)h.a;
+  return {a, (float)(-2.0 * a / (1.0 + (double)a * a)), h.k};
+}
+__device__ __forceinline__ void shear_rot(const ShearF& h, int odd, float& x, float& y) {
+  const int k = odd ? (4 - h.k) & 3 : h.k;
+  const unsigned s = (unsigned)odd << 31;
+  const unsigned sx = ((unsigned)(k + 1) & 2u) << 30, sy = ((unsigned)k & 2u) << 30;
+  const float u = (k & 1) ? y : x, v = (k & 1) ? x : y;
+  const float a = __uint_as_float(__float_as_uint(h.a) ^ s);
+  const float b = __uint_as_float(__float_as_uint(h.b) ^ s);
+  x = __uint_as_float(__float_as_uint(u) ^ sx);
+  y = __uint_as_float(__float_as_uint(v) ^ sy);
+  x = fmaf(a, y, x);
+  y = fmaf(b, x, y);
+  x = fmaf(a, y, x);
+}
+
 // (a, b) <- G (a, b) for the 2x2s that are rotations: SK_REAL [[c, -s], [s, c]]
 // (h[0]; refl: of (a, -b), as H), SK_IMOFF [[c, i s], [i s, c]] (h[0], RX), SK_PHASES
 // diag(e^{i f}, e^{i g}) (h[0], h[1], RZ).  SK_NONE: none of them.

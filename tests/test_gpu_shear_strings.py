@@ -73,3 +73,29 @@ def test_gradients(n):
     ref = oracle.grad_param_shift(c, theta, terms)
     assert abs(e - oracle.energy(c, theta, terms)) <= 1e-11
     assert np.max(np.abs(g - ref)) <= 1e-10 * max(1.0, np.max(np.abs(ref)))
+
+
+@pytest.mark.parametrize("n,layers", [(3, 40), (12, 12)])
+def test_complex64_keeps_the_norm(n, layers):
+    """One angle on every edge, many times, forward and back: no scale repeats."""
+    from paper_2202_07017_gb300 import State
+    oracle_threads()
+    gates = [W.Gate("H", (q,)) for q in range(n)]
+    for _ in range(layers):
+        gates += [W.Gate("PAULI", (q, (q + 1) % n), (), 0, paulis="ZZ") for q in range(n)]
+        gates += [W.Gate("PAULI", (q,), (), 1, paulis="X") for q in range(n)]
+    c, theta = W.Circuit(n, gates, 2), np.array([0.7, 2.2])
+    terms = W.tfim(n)
+    st = State(n, "c64").init(0)
+    try:
+        e, g = st.grad(c, theta, terms)
+        norm = st.init(0).apply_circuit(c, theta).norm()
+    finally:
+        st.close()
+    ref, count, scale = oracle.grad_param_shift(c, theta, terms), len(gates), sum(t[0] for t in terms)
+    # a rotation's rounding is a fraction of 2^-24 of random sign on each of `count` gates;
+    # a repeated scale would be up to 2^-24 times all of them
+    bar = 4 * math.sqrt(count) * 2.0 ** -24
+    assert abs(norm - 1) <= bar
+    assert abs(e - oracle.energy(c, theta, terms)) <= bar * scale
+    assert np.max(np.abs(g - ref)) <= bar * scale * layers * n
