@@ -595,9 +595,9 @@ def fused_layered(torch, n=33, depth=40, k=4):
     finally:
         sv_free(h)
     pass_bytes = 2 * 8 * 2 ** n
-    # arithmetic of the layer programs in rotation form: per circuit layer
-    # every qubit's RX RY RZ product is one scaled real rotation on its bit,
-    # one FMA per output component (2 per amplitude), and every 4-qubit
+    # arithmetic of the layer programs of shears: per circuit layer
+    # every qubit's RX RY RZ product is one rotation on its bit as two shears,
+    # 2 FMAs per amplitude, and every 4-qubit
     # group applies one complex diagonal (2 FMUL + 2 FFMA per amplitude)
     ffma = float(depth) * (2 * n + 4 * (n / 4)) * 2 ** n
     return {"workload": f"random layered n={n} complex64 depth {depth} ({len(c.gates)} gates), "
@@ -661,13 +661,13 @@ def qft_c128(torch, n=30, reps=2):
 
 def fp64_instructions(kernel: str, n: int) -> float:
     """fp64 arithmetic instructions per launch of the complex128 QFT kernels:
-    H (a real 2x2) costs 4 multiplies and 4 fused multiply-adds per
-    amplitude pair; a controlled U1 phase 2 multiplies and 2 FMAs per
-    touched amplitude (2^(n-2)); SWAP and initialisation none."""
+    as three shears a rotation, H costs 6 fused multiply-adds per amplitude
+    pair and a controlled U1 phase 3 per touched amplitude (2^(n-2)); SWAP and
+    initialisation none."""
     if kernel.startswith("k1q_c128"):
-        return 8.0 * 2 ** (n - 1)
+        return 6.0 * 2 ** (n - 1)
     if kernel.startswith("kphase_c128"):
-        return 4.0 * 2 ** (n - 2)
+        return 3.0 * 2 ** (n - 2)
     return 0.0
 
 

@@ -5,9 +5,10 @@
 // its Pauli-sum Hamiltonian) from an atomic queue and run each item to the
 // end inside the block - the forward pass from |0...0>, lambda = H psi and
 // E = <psi|lambda>, then the adjoint reverse sweep (dE/dtheta_j =
-// Im<lambda|P_j|psi> before U_j is un-applied on both states).  Each block
-// owns one workspace slot of two states (2 x 2^nmax complex64), small enough
-// to stay in L1/L2 while the block works on it.
+// Im<lambda|P_j|psi> before U_j is un-applied on both states).  The states
+// stay in shared memory - small items side by side in one block, large ones over
+// a cluster - or in the block's workspace slot of two states (2 x 2^nmax complex64),
+// small enough to stay in L1/L2 while the block works on it.
 //
 // Gates are applied in register groups: the host list-schedules each
 // circuit's gates into groups of at most k qubits; a thread pulls the 2^k
@@ -18,8 +19,7 @@
 // Precision: states and gate arithmetic in fp32; gate matrices from fp64
 // sincos; the energy and every gradient accumulate per thread / per warp in
 // compensated fp32 sums and across warps in fp64 (fixed order, so results
-// repeat bit for bit; the single-block kernels - the cluster kernel keeps
-// fp64 slots).
+// repeat bit for bit; the two-block cluster kernel keeps fp64 slots).
 #include <algorithm>
 #include <chrono>
 #include <cmath>
