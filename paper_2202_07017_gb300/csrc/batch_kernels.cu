@@ -1297,6 +1297,7 @@ __global__ void __cluster_dims__(kWide, 1, 1) __launch_bounds__(512, 1)
   const BPhase& P = A.wide;
   const Team T = {(int)threadIdx.x, 512, 1};
   const BSmem S = {dyn_smem, P};
+  cluster.sync();  // block 0 stores into the others' shared memory: they have to have started
   while (true) {
     if (rank == 0 && threadIdx.x == 0) {
       const int v = atomicAdd(A.queue + kBPhases, 1);
@@ -1583,6 +1584,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kClThreads, 1)
   const size_t cid = blockIdx.x / 2;
   float2* gw = A.work + cid * (size_t(2) << A.nmax);  // global slot: psi, then lambda
   int* partner_item = cluster.map_shared_rank(&s_item, 1);
+  cluster.sync();  // block 0 stores into its partner's shared memory: it has to have started
   while (true) {
     if (rank == 0 && threadIdx.x == 0) {
       const int v = atomicAdd(A.queue, 1);
