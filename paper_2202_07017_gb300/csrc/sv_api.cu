@@ -179,13 +179,16 @@ void feedback_round_entries(cd* dg, int d, double* drift) {
   if (exact) return;
   const double f = std::exp(-0.5 * *drift);
   double t = 0.0;
+  int counted = 0;
   for (int e = 0; e < d; ++e) {
     const double m = dg[e].re * dg[e].re + dg[e].im * dg[e].im;
     dg[e].re *= f;
     dg[e].im *= f;
+    if (m < 1e-70) continue;  // zero, or below fp32's normal range: no relative error to feed back
     t += sq32(dg[e]) / m;
+    ++counted;
   }
-  *drift += std::log(t / d);
+  if (counted) *drift += std::log(t / counted);
 }
 
 void feedback_round_pair(double* c, cd* k, double* drift) {

@@ -79,7 +79,8 @@ bool gate_matrix(const sv_gate& g, const double* theta, const double* pool, Host
 // form of the fused layer programs, states its own).  feedback_round_entries
 // is for a diagonal of unequal moduli between shears (see run_planes): what the
 // rounding of an entry does to the norm is its relative error, whatever its
-// modulus.  feedback_round_pair
+// modulus (zeros, as a projector among the layer's gates leaves, have none).
+// feedback_round_pair
 // treats a Pauli rotation c I + k P (P^2 = I, Hermitian) with factor
 // |c|^2 + |k|^2.
 void feedback_round(cd* m, int d, double* drift);
