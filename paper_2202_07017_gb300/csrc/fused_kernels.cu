@@ -2064,8 +2064,8 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
   // layer and layer l becomes the rotations S_l and the one diagonal
   // E_l = B_{l+1} Dg_l A_l.  tau is rounded to the state's precision and A
   // rescaled so that A S B stays unitary in fp64 (the rounding moves the
-  // rotation angle, not the norm).  False (nothing changed) if some 2x2 is
-  // not unitary.
+  // rotation angle, not the norm); not with lift, whose two coefficients come from
+  // the exact tau.  False (nothing changed) if some 2x2 is not unitary.
   auto rotation_form = [&](const std::vector<LayerH>& in, int k, std::vector<LayerH>* out,
                            int* xmask) {
     const int D = 1 << k;
@@ -2090,7 +2090,7 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
         const double am = shear ? std::sqrt(1.0 + tau * tau) : sc;
         a[0] = scl(a[0], am);
         a[1] = scl(a[1], am);
-        o.tau[t] = tr;
+        o.tau[t] = lift ? tau : tr;
         o.ph[t] = cdiv(b[0], b[1]);
         if (f) o.form |= 1 << t;
         for (int r = 0; r < D; ++r) {
@@ -2308,7 +2308,11 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       if (h.rot) {  // tau of bit i in slot i (0 where bit i has no rotation)
         for (int i = 0; i < 4; ++i) {
           const double t = ((h.rot >> i) & 1) ? h.tau[i] : 0.0;
-          if (lift) {  // tan(angle / 2) and sin(angle) from t = tan(angle)
+          // lift: tan(angle / 2) and sin(angle) from t = tan(angle), each rounded once.
+          // (From a rounded t the rms error of a rotation is 1.9e-8 in place of 1.5e-8 and of
+          // a hundred alike 1.3e-6 in place of 0.9e-6; with sin tied to the rounded tan,
+          // which keeps the norm a quarter better, 1.9e-8 and 1.3e-6.)
+          if (lift) {
             const double h = std::sqrt(1.0 + t * t);
             P->coef[nc++] = (R)(-t / (1.0 + h));
             P->coef[nc++] = (R)(t / h);
