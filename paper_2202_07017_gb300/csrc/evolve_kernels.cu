@@ -323,15 +323,39 @@ struct DiagGrads {
   uint32_t zt[kAdjTerms];
 };
 
+// to (lane 0's) += the sum of the lanes' g, each step's rounding error carried along
+__device__ __forceinline__ void warp_add(const CompSum<float>& g, CompSum<float>& to, int lane) {
+  float s = g.s, e = -g.c;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    const float x = __shfl_xor_sync(0xffffffffu, s, o);
+    e += __shfl_xor_sync(0xffffffffu, e, o);
+    const float t = s + x, b = t - s;
+    e += (s - (t - b)) + (x - b);
+    s = t;
+  }
+  if (lane == 0) {
+    to.add(s);
+    to.add(e);
+  }
+}
+__device__ __forceinline__ void warp_add(const CompSum<double>& g, CompSum<double>& to, int lane) {
+  double s = g.s;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) to.add(s);
+}
+
 // Reverse-sweep step of a run of diagonal rotations: all commute, so every
 // gradient Im<lambda|P_k|psi> = sum_x s_k(x) Im(conj(lambda_x) psi_x) comes
 // from the states before the run is un-applied.  The Walsh-Hadamard transform
 // of a tile's Im(conj(lambda) psi) gives each term's tile sum; the terms of a
 // slot (gates that share a parameter) add up in the thread before one warp
-// sum.  Per warp and slot a compensated sum (fp64 for complex128), per block
-// fp64 into partials[slot * pstride + blockIdx.x].  QAOA on a 3-regular graph,
-// n = 22, 33 ZZ gates per layer on one parameter: 33 launches of 16.5 us
-// before, one of 35 us.
+// sum.  Past the tile's transform (four additions) every sum is compensated (fp64
+// for complex128): the terms of a thread, the warp's and the warp's tiles; per block
+// fp64 into partials[slot * pstride + blockIdx.x].  With plain sums of the terms 127
+// equal ones were up to 32 * 2^-24 off.  QAOA on a 3-regular graph, n = 22, 33 ZZ gates
+// per layer on one parameter: 33 launches of 16.5 us before, one of 35 us.
 template <typename R>
 __global__ void __launch_bounds__(kEThreads, 2)
     kadj_diag(typename TurnVec<R>::T* __restrict__ psi, typename TurnVec<R>::T* __restrict__ lam,
@@ -378,14 +402,12 @@ __global__ void __launch_bounds__(kEThreads, 2)
 #pragma unroll
       for (int r = 0; r < NT; ++r) sw[r * blockDim.x + threadIdx.x] = w[r];
       for (int j = 0; j < G.ns; ++j) {
-        R g = 0;
+        CompSum<R> g;
         for (int k = G.sstart[j]; k < G.sstart[j + 1]; ++k) {
           const R a = sw[G.rho[k] * blockDim.x + threadIdx.x];
-          g += (__popc(t & G.zt[k]) & 1) ? -a : a;
+          g.add((__popc(t & G.zt[k]) & 1) ? -a : a);
         }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (lane == 0) gw[warp * G.ns + j].add(g);
+        warp_add(g, gw[warp * G.ns + j], lane);
       }
     }
     typename Turn<R>::T v[NT];
