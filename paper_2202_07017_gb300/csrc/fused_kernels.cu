@@ -1985,7 +1985,6 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     int flip = 0;           // rotation form: register relabelling in force before the rotations
     cd ph[5];               // rotation form: input phase ratio b0 / b1 of bit i's rotation
     double tau[5] = {0, 0, 0, 0, 0};
-    double msq = 1.0;  // exact mean squared modulus of Dg
     cd U[5][4];
     cd Dg[32];
     LayerH() {
@@ -2110,14 +2109,11 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
     }
     for (size_t l = 0; l < NL; ++l) {
       LayerH o = mid[l];
-      double msq = 0.0;
       for (int r = 0; r < D; ++r) {
         cd e = cmul(in[l].Dg[r], A[l][r]);
         if (l + 1 < NL) e = cmul(B[l + 1][r], e);
         o.Dg[r] = e;
-        msq += e.re * e.re + e.im * e.im;
       }
-      o.msq = msq / D;
       out->push_back(o);
     }
     // Shears p += a q, q += b p with a = -t and b = t / (1 + t^2) rounded: for any
@@ -2293,7 +2289,7 @@ int layer_group(const FusedPass& pass, int g, const int* pos_of, FusedParams<R>*
       if (shear)
         feedback_round_entries(h.Dg, D, fb);
       else
-        feedback_round_diag(h.Dg, D, fb, h.msq);
+        feedback_round_diag(h.Dg, D, fb);
     };
     for (size_t li = 0; li < L.size(); ++li) {
       LayerH& h = L[li];

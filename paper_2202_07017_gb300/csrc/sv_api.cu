@@ -140,6 +140,19 @@ double sq32(cd z) {
   const double r = (float)z.re, i = (float)z.im;
   return r * r + i * i;
 }
+// The entries by the feedback factor; what their rounding does to the sum of their
+// squares (not what the matrix itself does: it need not be unitary) to *drift.
+void scale_and_round(cd* z, int count, double* drift) {
+  const double f = std::exp(-0.5 * *drift);
+  double t = 0.0, own = 0.0;
+  for (int e = 0; e < count; ++e) {
+    own += z[e].re * z[e].re + z[e].im * z[e].im;
+    z[e].re *= f;
+    z[e].im *= f;
+    t += sq32(z[e]);
+  }
+  if (own >= 1e-70) *drift += std::log(t / own);  // else below fp32's normal range
+}
 }  // namespace
 
 void feedback_round(cd* m, int d, double* drift) {
@@ -147,29 +160,15 @@ void feedback_round(cd* m, int d, double* drift) {
   bool exact = true;
   for (int e = 0; e < d * d && exact; ++e) exact = fp32_number(m[e].re) && fp32_number(m[e].im);
   if (exact) return;
-  const double f = std::exp(-0.5 * *drift);
-  double t = 0.0;
-  for (int e = 0; e < d * d; ++e) {
-    m[e].re *= f;
-    m[e].im *= f;
-    t += sq32(m[e]);
-  }
-  *drift += std::log(t / d);
+  scale_and_round(m, d * d, drift);
 }
 
-void feedback_round_diag(cd* dg, int d, double* drift, double mean_sq) {
+void feedback_round_diag(cd* dg, int d, double* drift) {
   if (!drift) return;
   bool exact = true;
   for (int e = 0; e < d && exact; ++e) exact = fp32_number(dg[e].re) && fp32_number(dg[e].im);
   if (exact) return;
-  const double f = std::exp(-0.5 * *drift);
-  double t = 0.0;
-  for (int e = 0; e < d; ++e) {
-    dg[e].re *= f;
-    dg[e].im *= f;
-    t += sq32(dg[e]);
-  }
-  *drift += std::log(t / (d * mean_sq));
+  scale_and_round(dg, d, drift);
 }
 
 void feedback_round_entries(cd* dg, int d, double* drift) {

@@ -72,19 +72,17 @@ bool gate_matrix(const sv_gate& g, const double* theta, const double* pool, Host
 // CZ, SWAP, ...) are left untouched.
 //
 // feedback_round scales the d x d row-major matrix m in place (when drift is
-// not null and some entry is not an fp32 number) and adds the log of the
-// rounded matrix's mean squared column norm to *drift.  feedback_round_diag
-// does the same for a diagonal of d entries whose exact mean squared modulus
-// is mean_sq (1 for a unitary diagonal; a scaled one, as in the rotation
-// form of the fused layer programs, states its own).  feedback_round_entries
+// not null and some entry is not an fp32 number) and adds to *drift the log of
+// the rounded matrix's mean squared column norm over the exact one's (1 for a
+// unitary; a matrix that scales the state keeps its scale).  feedback_round_diag
+// does the same for a diagonal of d entries.  feedback_round_entries
 // is for a diagonal of unequal moduli between shears (see run_planes): what the
 // rounding of an entry does to the norm is its relative error, whatever its
 // modulus (zeros, as a projector among the layer's gates leaves, have none).
-// feedback_round_pair
-// treats a Pauli rotation c I + k P (P^2 = I, Hermitian) with factor
-// |c|^2 + |k|^2.
+// feedback_round_pair treats a Pauli rotation c I + k P (P^2 = I, Hermitian)
+// with factor |c|^2 + |k|^2.
 void feedback_round(cd* m, int d, double* drift);
-void feedback_round_diag(cd* dg, int d, double* drift, double mean_sq = 1.0);
+void feedback_round_diag(cd* dg, int d, double* drift);
 void feedback_round_entries(cd* dg, int d, double* drift);
 void feedback_round_pair(double* c, cd* k, double* drift);
 

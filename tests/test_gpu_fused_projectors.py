@@ -46,3 +46,32 @@ def _check(n, fuse_k, alone, under_control):
 @pytest.mark.parametrize("diag", sorted(DIAGONALS))
 def test_diagonals_with_zeros(n, fuse_k, diag):
     _check(n, fuse_k, *DIAGONALS[diag])
+
+
+# matrices that scale the state, as they stand: alone they are applied gate by gate,
+# in passes they multiply with the rotations beside them
+MATRICES = {"scaled": 0.6 * np.array([[0.8, -0.6], [0.6, 0.8]]), "projector": np.diag([0, 1]),
+            "diagonal": np.diag([0.3 + 0.1j, 0.7]), "damping": np.array([[1, 0], [0.1, 0.9]])}
+
+
+@pytest.mark.parametrize("n,fuse_k", [(6, 0), (12, 4), (20, 4), (20, 3)])
+@pytest.mark.parametrize("name", sorted(MATRICES))
+def test_matrices_that_are_not_unitary(n, fuse_k, name):
+    oracle_threads()
+    rng = W.SplitMix64(11 * n)
+    gates, theta = [], []
+    for layer in range(3):
+        for q in range(n):
+            theta.append(rng.angle())
+            gates.append(W.Gate(("RX", "RY", "RZ")[(q + layer) % 3], (q,), (), len(theta) - 1))
+        gates += [W.Gate("Z", (i + 1,), (i,)) for i in range(layer % 2, n - 1, 2)]
+        for q in (1, n // 2):
+            gates.append(W.Gate("MATRIX", (q,), (), matrix=MATRICES[name].astype(complex)))
+        gates += [W.Gate("H", (q,)) for q in range(n)]
+    c = W.Circuit(n, gates, len(theta))
+    psi0 = rounded(W.random_state(n, 9), "c64")
+    got = gpu_run(c, np.array(theta), psi0, "c64", fuse_k)
+    want = oracle.run(c, np.array(theta), psi0)
+    # 12 operations a qubit of at most 4 roundings each, relative to the norm; the state
+    # before a projector may be twice as long, three times over
+    assert np.linalg.norm(got - want) <= 8 * 12 * n * 4 * 2.0**-24 * np.linalg.norm(want)
