@@ -246,6 +246,7 @@ struct FusionConfig {
   int max_grads = 200;       // gradient capacity of one pass (reverse sweeps)
   int max_groups = 64;       // group capacity of one pass
   int max_layers = 72;       // layer capacity of one pass (coefficients of 4-qubit layers)
+  bool move_phases = true;   // input phases move to earlier gates (see move_input_phases)
 };
 
 FusionConfig fusion_config(int n, sv_dtype dt, int fuse_k);
