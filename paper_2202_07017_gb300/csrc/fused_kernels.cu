@@ -25,10 +25,10 @@
 // register-group accesses of a warp over the banks.
 #include <algorithm>
 #include <array>
-#include <map>
 #include <mutex>
 #include <numeric>
 
+#include "resident_cache.cuh"
 #include "slice_geom.cuh"
 #include "sv_device.cuh"
 #include "tma.cuh"
@@ -2640,6 +2640,25 @@ void plane_threads(FusedParams<R>* P) {
   }
 }
 
+// Blocks of a persistent pass kernel that the current device holds at once.
+template <typename Kern>
+uint64_t resident_blocks(Kern kern, int threads, size_t smem) {
+  static ResidentCache cache;
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int res = cache.get(reinterpret_cast<const void*>(kern), dev, threads, smem, [&] {
+    int blocks = 0;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, threads, smem) == cudaSuccess &&
+        blocks >= 1)
+      return blocks;
+    cudaGetLastError();
+    return 1;
+  });
+  return (uint64_t)sms * res;
+}
+
 template <typename R>
 sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, RoundCtx* rc) {
   double* drift = rc ? &rc->drift : nullptr;
@@ -2702,21 +2721,7 @@ sv_status run_pass(void* data, int n, cudaStream_t st, const FusedPass& pass, Ro
     const size_t smem = (amp << P.m) + 1024 + sizeof(R) * (size_t)((P.ncoef + 1) & ~1) +
                         sizeof(FLayerDev) * (size_t)P.glay[P.ngroups] +
                         (mode >= 5 ? sizeof(uint16_t) * (size_t)threads * P.ngroups : 0);
-    // resident blocks per SM for this kernel and shared-memory size
-    static std::map<std::pair<const void*, size_t>, int> resident;
-    int& res = resident[{reinterpret_cast<const void*>(kern), smem}];
-    if (!res) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kern, threads, smem) != cudaSuccess ||
-          res < 1) {
-        cudaGetLastError();
-        res = 1;
-      }
-    }
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const uint64_t grid = std::min<uint64_t>(nblk, (uint64_t)sms * res);
+    const uint64_t grid = std::min<uint64_t>(nblk, resident_blocks(kern, threads, smem));
     launch_dependent(kern, (unsigned)grid, threads, smem, st, nblk, P);
   } else {
     typename PassKernels<R>::Lsu kern = PassKernels<R>::lsu(kg);
@@ -2792,22 +2797,10 @@ sv_status run_adj_pass(void* psi, void* lam, int n, cudaStream_t st, const Fused
     return SV_ERR_UNSUPPORTED;
   }
   typedef void (*Kern)(uint64_t, const FusedParams<R>, double*, int);
-  static std::map<std::pair<const void*, size_t>, int> resident;
   auto launch = [&](Kern kern, int threads, size_t smem) {
-    int& res = resident[{reinterpret_cast<const void*>(kern), smem}];
-    if (!res) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kern, threads, smem) != cudaSuccess ||
-          res < 1) {
-        cudaGetLastError();
-        res = 1;
-      }
-    }
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint64_t nblk = uint64_t(1) << (n - P.m);
-    const uint64_t grid = std::min<uint64_t>({nblk, (uint64_t)sms * res, (uint64_t)pstride});
+    const uint64_t grid =
+        std::min<uint64_t>({nblk, resident_blocks(kern, threads, smem), (uint64_t)pstride});
     ProfScope prof(st, sizeof(R) == 4 ? "kfused_adj_c64" : "kfused_adj_c128");
     launch_dependent(kern, (unsigned)grid, threads, smem, st, nblk, P, partials, pstride);
     g_launches.fetch_add(1, std::memory_order_relaxed);

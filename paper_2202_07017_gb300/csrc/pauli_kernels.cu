@@ -33,6 +33,7 @@
 #include <mutex>
 #include <vector>
 
+#include "resident_cache.cuh"
 #include "slice_geom.cuh"
 #include "sv_device.cuh"
 #include "tma.cuh"
@@ -1237,7 +1238,7 @@ sv_status expval_staged(sv_state s, const sv_pauli_sum* H, double* dst) {
   static std::mutex mu;
   static PauliPassDev<float> Pf;
   static PauliPassDev<double> Pd;
-  static std::map<std::pair<const void*, size_t>, int> resident;
+  static ResidentCache resident;
   std::lock_guard<std::mutex> lk(mu);
   unsigned* status = nullptr;
   if (cudaGetSymbolAddress((void**)&status, g_pauli_status) != cudaSuccess) {
@@ -1267,18 +1268,18 @@ sv_status expval_staged(sv_state s, const sv_pauli_sum* H, double* dst) {
   for (size_t i = 0; i < passes.size(); ++i)
     is_chunked[i] = c64 && is_lean[i] && chunk_pass(pf[i], &chunked[i]);
   auto grid_of = [&](const void* kern, size_t bytes, int nbuf) -> uint64_t {
-    int& res = resident[{kern, bytes}];
-    if (!res) {
+    const int res = resident.get(kern, dev, kPThreads, bytes, [&] {
+      int blocks = 0;
       // the largest slice any pass stages (the attribute is per kernel, not per size)
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(nbuf * (size_t(8) << lw << (c64 ? 13 : 12)) + 1024));
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kern, kPThreads, bytes) !=
-              cudaSuccess ||
-          res < 1) {
-        cudaGetLastError();
-        res = 1;
-      }
-    }
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, kPThreads, bytes) ==
+              cudaSuccess &&
+          blocks >= 1)
+        return blocks;
+      cudaGetLastError();
+      return 1;
+    });
     return std::min<uint64_t>({nblk, (uint64_t)sms * res, (uint64_t)kRedMaxBlocks});
   };
   int total = 0;
