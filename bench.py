@@ -1050,7 +1050,7 @@ def main():
                 "bound": "hbm", "achieved_gbs": rp["achieved_gbs"], "peak_gbs": peak,
                 "frac": rp["achieved_gbs"] / peak}
         if batch is not None:
-            kname = "kbatch_re" if batch["tile"].get("real_states") else "kbatch"
+            kname = "kbatch_real" if batch["tile"].get("real_states") else "kbatch"
             rooflines[f"{kname} (C3)"] = {"bound": "shared memory (nominal)",
                                           **batch["state_traffic"]}
         for key in ("energy_sum_z", "energy_tfim"):

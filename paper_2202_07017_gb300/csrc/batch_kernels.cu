@@ -1731,8 +1731,7 @@ struct sv_batch_s {
   int k = 4, threads = 256, blocks = 0;  // chosen tile
   bool cluster = false;                  // two-block cluster kernel
   bool smem_states = false;              // single-block kernel with states in shared memory
-  bool real = false;                     // real-amplitude kernel (kbatch_re)
-  bool all_real = false;                 // every gate and term real: kbatch_re may run
+  bool real = false;                     // real amplitudes (kbatch with one plane)
   int sms = 152;
   // device buffers
   sv::BCirc* circs = nullptr;
@@ -1757,7 +1756,6 @@ struct sv_batch_s {
   int n_phases = 0;                     // of the chosen tile
   sv::BPhase phase[sv::kBPhases], wide;
   size_t smem = 0;
-  std::vector<int> h_theta_off;
   // captured graph
   cudaGraphExec_t gexec = nullptr;
   const void* g_key[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -2208,7 +2206,7 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
     }
     return SV_OK;
   };
-  ProfScope prof(st, re ? "kbatch_re" : sms ? "kbatch_smem" : "kbatch");
+  ProfScope prof(st, re ? "kbatch_real" : sms ? "kbatch_smem" : "kbatch");
   sv_status s = allow(kern, b->smem);
   if (s) return s;
   if (b->wide.count > 0) {
@@ -2233,10 +2231,6 @@ sv_status launch_batch(sv_batch b, const double* theta, double* energy, double* 
 }  // namespace sv
 
 using namespace sv;
-
-extern "C" {
-
-}  // extern "C"
 
 // Checks every circuit and Hamiltonian against the batch kernel's limits;
 // returns the largest qubit count and the widest gate (target + controls).
@@ -2343,7 +2337,6 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
   b->n_items = n_items;
   b->nmax = nmax;
   b->total_params = total;
-  b->h_theta_off = toff;
   // batch packing: longest items first (work ~ gates x 2^n)
   std::vector<int> order(n_items);
   for (int i = 0; i < n_items; ++i) order[i] = i;
@@ -2374,7 +2367,6 @@ sv_status sv_batch_create(const sv_circuit* circuits, const sv_pauli_sum* hamilt
     for (int t = 0; t < hamiltonians[c].n_terms; ++t)
       if (popc64(hamiltonians[c].xmask[t] & hamiltonians[c].zmask[t]) & 1) all_real = false;
   }
-  b->all_real = all_real;
   std::vector<Cand> cands;
   if (tune == 4) {
     if (!all_real) {

@@ -691,9 +691,6 @@ __device__ __forceinline__ void plane_mul(Pair dr, Pair di, Pair dn, Pair& re, P
   im = t;
 }
 
-// the 128-byte swizzle on 16-byte chunk indices
-__device__ __forceinline__ int chunk_swz(int q) { return q ^ ((q >> 3) & 7); }
-
 // LOW: the group holds amplitude bit 0.  xm: the program's final register
 // relabelling (register r holds group index r ^ xm).  base0: the thread's tile
 // (its swizzled chunk index with the group's bits clear); tile: the chunk bit of

@@ -18,9 +18,9 @@
 // on one bit through the tile's pair sums, other shapes through partners
 // read from the slice), its z bits giving a sign per tile (staged bits), per
 // slice (unstaged bits) and per pair (group bits).  A pass of single-X terms
-// only (a transverse field, a QAOA mixer) takes the lean kernel
-// kpauli_xbits, which keeps per-bit pair sums in registers for the whole
-// launch and weighs them once.  The planner covers the x bits by passes that
+// only (a transverse field, a QAOA mixer) takes a lean kernel (kpauli_xchunks in
+// complex64, kpauli_xbits in complex128), which keeps per-bit pair sums in registers
+// for the whole launch and weighs them once.  The planner covers the x bits by passes that
 // stage the low rows plus up to m - 4 high bits each; terms it cannot place
 // (more than four x bits, or x bits too far apart) go to the per-amplitude
 // kernel.
@@ -312,11 +312,11 @@ struct XPassDev {
 };
 
 // pair sums A_i of one group over the tile (all four bits)
-template <typename R>
-__device__ __forceinline__ void xsums(const R (&re)[16], const R (&im)[16], R (&A)[4]) {
+__device__ __forceinline__ void xsums(const double (&re)[16], const double (&im)[16],
+                                      double (&A)[4]) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    R a = 0;
+    double a = 0;
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
       if (r & (1 << i)) continue;
@@ -331,11 +331,9 @@ __device__ __forceinline__ void xsums(const R (&re)[16], const R (&im)[16], R (&
 // the current one is read.
 constexpr int kXBuf = 3;
 
-template <typename R>
 __global__ void __launch_bounds__(kPThreads, 1)
     kpauli_xbits(uint64_t n_blocks, const __grid_constant__ XPassDev P,
                  double* __restrict__ partials, unsigned* __restrict__ status) {
-  typedef typename Cplx2P<R>::T V2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[kXBuf];   // full: the slice's bytes have landed
   __shared__ __align__(8) uint64_t ebars[kXBuf];  // empty: every warp is done with it
@@ -353,7 +351,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
   }
   grid_dependency_wait();
   __syncthreads();
-  CompSum<R> acc[kPG * kXGroups];
+  CompSum<double> acc[kPG * kXGroups];
   // bit j: buffer j.  used: filled before (its refill waits until every warp
   // released the previous fill); eparity: phase of its empty barrier
   uint32_t parity = 0, pending = 0, used = 0, eparity = 0;
@@ -362,7 +360,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const uint64_t b = blockIdx.x + (uint64_t)j * gridDim.x;
     if (b < n_blocks) {
       if (threadIdx.x < 32)
-        issue_slice<R>(P.geo, b, sbuf0 + (uint32_t)j * sbytes, smem_addr(&bars[j]), lane);
+        issue_slice<double>(P.geo, b, sbuf0 + (uint32_t)j * sbytes, smem_addr(&bars[j]), lane);
       pending |= 1u << j;
       used |= 1u << j;
     }
@@ -380,7 +378,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         if ((used >> nxt) & 1)
           free_ok = mbar_wait_bounded(smem_addr(&ebars[nxt]), (eparity >> nxt) & 1);
         if (free_ok)
-          issue_slice<R>(P.geo, nb, sbuf0 + (uint32_t)nxt * sbytes, smem_addr(&bars[nxt]), lane);
+          issue_slice<double>(P.geo, nb, sbuf0 + (uint32_t)nxt * sbytes, smem_addr(&bars[nxt]), lane);
         else if (lane == 0)
           atomicOr(status, kWaitTimeout);
       }
@@ -395,14 +393,14 @@ __global__ void __launch_bounds__(kPThreads, 1)
       if (lane == 0) atomicOr(status, kWaitTimeout);
       break;
     }
-    const V2* sm = reinterpret_cast<const V2*>(smem_raw + (sbuf0 + (uint32_t)cur * sbytes - raw));
+    const double2* sm = reinterpret_cast<const double2*>(smem_raw + (sbuf0 + (uint32_t)cur * sbytes - raw));
 #pragma unroll
     for (int g = 0; g < kXGroups; ++g) {
       if (g >= P.ngroups) break;
       const uint8_t* gb = P.gbits[g];
       int sw[kPG];
 #pragma unroll
-      for (int i = 0; i < kPG; ++i) sw[i] = pswz<R>(1 << gb[i]);
+      for (int i = 0; i < kPG; ++i) sw[i] = pswz<double>(1 << gb[i]);
       for (int s = threadIdx.x; s < nsub; s += kPThreads) {
         uint32_t b = (uint32_t)s;
 #pragma unroll
@@ -410,35 +408,20 @@ __global__ void __launch_bounds__(kPThreads, 1)
           const uint32_t lm = (1u << gb[i]) - 1;
           b = ((b & ~lm) << 1) | (b & lm);
         }
-        const int sb = pswz<R>((int)b);
-        R re[16], im[16];
-        if (sizeof(R) == 4 && gb[0] == 0 && gb[3] == 3) {
-          // the tile is one 128-byte row: amplitudes 2q, 2q + 1 share a
-          // 16-byte chunk at chunk (q ^ row swizzle), read as one vector
-          // (a warp's 32 rows then spread over all banks)
-          const float4* sm4 = reinterpret_cast<const float4*>(sm);
+        const int sb = pswz<double>((int)b);
+        double re[16], im[16];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float4 v = sm4[(sb >> 1) ^ q];
-            re[2 * q] = v.x;
-            im[2 * q] = v.y;
-            re[2 * q + 1] = v.z;
-            im[2 * q + 1] = v.w;
-          }
-        } else {
+        for (int r = 0; r < 16; ++r) {
+          int o = 0;
 #pragma unroll
-          for (int r = 0; r < 16; ++r) {
-            int o = 0;
-#pragma unroll
-            for (int i = 0; i < kPG; ++i)
-              if ((r >> i) & 1) o ^= sw[i];
-            const V2 v = sm[sb ^ o];
-            re[r] = v.x;
-            im[r] = v.y;
-          }
+          for (int i = 0; i < kPG; ++i)
+            if ((r >> i) & 1) o ^= sw[i];
+          const double2 v = sm[sb ^ o];
+          re[r] = v.x;
+          im[r] = v.y;
         }
-        R A[4];
-        xsums<R>(re, im, A);
+        double A[4];
+        xsums(re, im, A);
 #pragma unroll
         for (int i = 0; i < kPG; ++i) acc[kPG * g + i].add(A[i]);
       }
@@ -458,8 +441,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
 }
 
 // ---- X terms of complex64 states on 16-byte chunks -------------------------------------
-// kpauli_xbits is bound by its reads of the slice from shared memory (one per
-// group of four bits, 8 bytes at a time) and their instructions.  Here a
+// In the form of kpauli_xbits these passes were bound by their reads of the slice from
+// shared memory (one per group of four bits, 8 bytes at a time) and their instructions.  Here a
 // thread's tile is 16 chunks of two amplitudes, read as 16-byte vectors: three
 // groups cover the 12 chunk bits of a 2^13 slice and amplitude bit 0 comes with
 // the first, and the pair sums are paired fp32 FMAs on (re, im).  One half of
@@ -480,7 +463,6 @@ __device__ __forceinline__ float lane_sum(Pair p) {
   const float2 v = lanes_of(p);
   return v.x + v.y;
 }
-__device__ __forceinline__ int cswz(int q) { return q ^ ((q >> 3) & 7); }
 
 __global__ void __launch_bounds__(kPThreads, 1)
     kpauli_xchunks(uint64_t n_blocks, const __grid_constant__ XChunkDev P,
@@ -510,9 +492,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const int g = half + 2 * j < kXCGroups ? half + 2 * j : 0;
     int q = 0;
     for (int i = 0; i < P.geo.m - 5; ++i) q |= ((t >> i) & 1) << P.tpos[g][i];
-    tile[j] = cswz(q);
+    tile[j] = chunk_swz(q);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sw[j][i] = cswz(1 << P.gbits[g][i]);
+    for (int i = 0; i < 4; ++i) sw[j][i] = chunk_swz(1 << P.gbits[g][i]);
   }
   grid_dependency_wait();
   __syncthreads();
@@ -1306,8 +1288,8 @@ sv_status expval_staged(sv_state s, const sv_pauli_sum* H, double* dst) {
                        chunked[i], s->partials + total, status);
     } else if (is_lean[i] && !c64) {
       ProfScope prof(s->stream, "kpauli_xbits_c128");
-      grid = grid_of((const void*)kpauli_xbits<double>, smem_x, kXBuf);
-      launch_dependent(kpauli_xbits<double>, (unsigned)grid, kPThreads, smem_x, s->stream, nblk,
+      grid = grid_of((const void*)kpauli_xbits, smem_x, kXBuf);
+      launch_dependent(kpauli_xbits, (unsigned)grid, kPThreads, smem_x, s->stream, nblk,
                        lean[i], s->partials + total, status);
     } else {
       ProfScope prof(s->stream, c64 ? "kpauli_energy_c64" : "kpauli_energy_c128");

@@ -492,7 +492,7 @@ void form_passes(std::vector<FGate>& F, int n, const FusionConfig& cfg,
     // or the contiguous window of high bits that takes more operations.  On
     // circuits of neighbouring gates a greedy set spreads over many short runs of
     // qubits, whose light cones close after a layer or two: a random layered
-    // circuit of depth 30 on 28 qubits takes 49 passes, with windows 24.
+    // circuit of depth 30 on 28 qubits takes 49 passes, with windows 23.
     uint64_t S = lowL;
     int best = n > cfg.m ? collect(&S, true, F.size(), nullptr) : 0;  // or every qubit
     for (int b = 0; b < n && popc(S) < cfg.m; ++b) S |= uint64_t(1) << b;

@@ -59,6 +59,9 @@ struct SliceDev {
 bool build_slice(const TmaGeom& g, const std::vector<int>& S, int n, int lw, void* data,
                  SliceDev* d);
 
+// the 128-byte swizzle on 16-byte chunk indices
+__device__ __forceinline__ int chunk_swz(int q) { return q ^ ((q >> 3) & 7); }
+
 __device__ __forceinline__ void slice_box_coords(const SliceDev& P, uint64_t base, int k, int* c) {
   uint64_t a = base;
   for (int j = 0; j < P.nsw; ++j)
